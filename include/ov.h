@@ -78,14 +78,19 @@ typedef enum {
    * of Eq. 7 becomes sum_i g_i v_i over the Lanczos basis.  The basis is kept in device
    * memory when min(max_iter, 1024) vectors per source fit a quarter of it (the sum is
    * then one read of the basis); otherwise a second Lanczos pass regenerates it.
-   * Same result as OV_MODE_FP64 up to rounding; vector work independent of N. */
+   * Same result as OV_MODE_FP64 up to rounding; vector work independent of N.
+   * Unitary links and |4 - m0| <= 4: the vectors of the stored basis are 58-bit integers
+   * of one scale per vector, products and sums of them exact to 2^-58 of the vector's
+   * largest component (GB300's FP64 rate is a fourteenth of its integer multiply rate);
+   * recurrence scalars and the result stay FP64.  Other links and masses: FP64 vectors. */
   OV_MODE_FP64_2PASS = 2,
   /* As OV_MODE_FP64_2PASS, always regenerating the basis (memory: three vectors per
    * source). */
   OV_MODE_FP64_REGEN = 3,
-  /* As OV_MODE_FP64_2PASS with every vector operation -- the H_W stencil, the Lanczos
-   * updates and the stored basis -- in FP32-pair (double-float) arithmetic on the FP32
-   * units: each real is an unevaluated sum of two floats (~48-bit significand), sums
+  /* As OV_MODE_FP64_2PASS; where its integer vectors do not apply (links not unitary, or
+   * |4 - m0| > 4) or a stored basis does not fit, every vector operation -- the H_W
+   * stencil, the Lanczos updates and the basis -- is in FP32-pair (double-float)
+   * arithmetic on the FP32 units: each real is an unevaluated sum of two floats (~48-bit significand), sums
    * by error-free two-sum, products by FMA-based exact products.  Recurrence scalars,
    * inner products and the quadrature sum stay FP64.  All sources run in the same
    * launches.  Accuracy ~1e-13 relative; on GB300 (FP64 at 1/58 of the FP32 rate) it

@@ -17,6 +17,28 @@ const char* const kKernelClassNames[KC_COUNT] = {"hw_kernel",         "lanczos_h
 
 // ------------------------------------------------------------ utilities
 
+static FastDiv make_div(int d) {
+  if (d <= 1) return {0, 0};
+  int l = 0;
+  while ((2LL << l) < d) ++l;  // 2^l < d <= 2^(l + 1)
+  return {(unsigned)((1ULL << (32 + l)) / (unsigned)d + 1), l};
+}
+
+Geom make_geom(const int dims[4], int bc_t) {
+  Geom g;
+  int st = 1;
+  for (int k = 0; k < 4; ++k) {
+    g.L[k] = dims[k];
+    g.st[k] = st;
+    g.dL[k] = make_div(dims[k]);
+    g.dst[k] = make_div(st);
+    st *= dims[k];
+  }
+  g.V = st;
+  g.bc_t = bc_t;
+  return g;
+}
+
 int ctx_fail(ov_ctx* ctx, int code, const std::string& msg) {
   if (ctx) ctx->err = msg;
   return code;
@@ -300,13 +322,7 @@ int ov_create(ov_ctx** out, const int dims[4], int bc_t, double m0, double r, in
   ov_ctx* ctx = new ov_ctx();
   ctx->device = device;
   DeviceGuard dg(device);
-  for (int k = 0; k < 4; ++k) ctx->g.L[k] = dims[k];
-  ctx->g.st[0] = 1;
-  ctx->g.st[1] = dims[0];
-  ctx->g.st[2] = dims[0] * dims[1];
-  ctx->g.st[3] = dims[0] * dims[1] * dims[2];
-  ctx->g.V = (int)V;
-  ctx->g.bc_t = bc_t;
+  ctx->g = make_geom(dims, bc_t);
   ctx->m0 = m0;
   ctx->r = r;
   if (cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -377,6 +393,7 @@ int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream) {
   ctx->have_c32 = false;
   ctx->have_s4 = false;
   ctx->have_df = false;
+  ctx->have_fx = false;
   return OV_OK;
 }
 

@@ -145,6 +145,10 @@ template <typename R> __device__ __forceinline__ R cnorm2(Cx<R> a) { return a.re
 
 // ------------------------------------------------------------ neighbours
 
+__device__ __forceinline__ int fast_div(int n, FastDiv d) {
+  return d.m ? (int)(__umulhi((unsigned)n, d.m) >> d.l) : n;
+}
+
 __device__ __forceinline__ void site_coords(const Geom& g, int s, int c[4]) {
   c[0] = s % g.L[0];
   int q = s / g.L[0];

@@ -5,7 +5,7 @@
 // Structure of arrays: a spinor is 12 planes of V complex numbers (plane k =
 // 3 * spin + colour), so consecutive threads (consecutive sites) read
 // consecutive 8- or 16-byte words of a plane; a gauge field is 4 x 9 planes.
-#include "common.cuh"
+#include "fixed.cuh"
 
 namespace {
 
@@ -93,6 +93,40 @@ __global__ void links_df_kernel(const double2* __restrict__ u64, float4* __restr
     const double2 v = u64[t];
     const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
     udf[t] = make_float4(rh, __double2float_rn(v.x - (double)rh), ih, __double2float_rn(v.y - (double)ih));
+  }
+}
+
+// FP64 solver links (-1/2 U, boundary sign included) -> fixed-point tiles of unit 2^-58; *bad
+// is set when a link's rows or columns exceed the norm the fixed-point bounds assume (not
+// unitary, or not finite)
+__global__ void links_fx_kernel(const double2* __restrict__ u, int4* __restrict__ ufx,
+                                int V, int* __restrict__ bad) {
+  const size_t n = 4 * fx_padded(V);
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
+    // thread -> (tile, mu, lane)
+    const size_t mu = t / kFxTile % 4, site = t / (4 * kFxTile) * kFxTile + t % kFxTile;
+    if (site >= V) continue;
+    double row[3] = {0.0, 0.0, 0.0}, col[3] = {0.0, 0.0, 0.0};
+    double2 v[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      v[e] = u[(mu * 9 + e) * V + site];
+      const double m = v[e].x * v[e].x + v[e].y * v[e].y;
+      row[e / 3] += m;
+      col[e % 3] += m;
+    }
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ok = ok && row[k] <= 0.25 * kFxRowMax && col[k] <= 0.25 * kFxRowMax;
+    if (!ok) {  // also for NaN
+      atomicOr(bad, 1);
+      continue;
+    }
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const FX re = fx_split(__double2ll_rn(ldexp(v[e].x, 58))), im = fx_split(__double2ll_rn(ldexp(v[e].y, 58)));
+      ufx[fx_index((int)site, 36) + (mu * 9 + e) * kFxTile] = make_int4(re.hi, re.lo, im.hi, im.lo);
+    }
   }
 }
 
@@ -192,6 +226,26 @@ int ensure_links_df(ov_ctx* ctx, cudaStream_t s) {
     links_df_kernel<<<grid_for(n, 256), 256, 0, s>>>(ctx->U64h, ctx->Udf, n);  // -1/2 U, signs baked in
     OV_CHECK_LAUNCH(ctx, "links_df_kernel");
     ctx->have_df = true;
+  }
+  return OV_OK;
+}
+
+int ensure_links_fx(ov_ctx* ctx, cudaStream_t s) {
+  int st = OV_OK;
+  const size_t n = (size_t)4 * ctx->g.V;
+  ctx->Ufx = (int4*)ws_get(ctx, "gauge.fx", sizeof(int4) * 36 * fx_padded(ctx->g.V), &st);
+  int* bad = (int*)ws_get(ctx, "gauge.fxbad", sizeof(int), &st);
+  if (st != OV_OK) return st;
+  if (!ctx->have_fx) {
+    cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), s);
+    if (e != cudaSuccess) return ctx_cuda(ctx, e, "clear link check");
+    links_fx_kernel<<<grid_for(n, 256), 256, 0, s>>>(ctx->U64h, ctx->Ufx, ctx->g.V, bad);
+    OV_CHECK_LAUNCH(ctx, "links_fx_kernel");
+    e = cudaMemcpyAsync(ctx->host_flag + 1, bad, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return ctx_cuda(ctx, e, "read link check");
+    ctx->fx_ok = ctx->host_flag[1] == 0;
+    ctx->have_fx = true;
   }
   return OV_OK;
 }

@@ -140,14 +140,7 @@ extern "C" int ov_apply_HW_noalloc(const int dims[4], int bc_t, double m0, const
   double2* U_soa = (double2*)base;
   double2* in_soa = (double2*)((unsigned char*)base + gauge_bytes);
   double2* out_soa = (double2*)((unsigned char*)base + gauge_bytes + spinor_bytes);
-  Geom g;
-  for (int k = 0; k < 4; ++k) g.L[k] = dims[k];
-  g.st[0] = 1;
-  g.st[1] = dims[0];
-  g.st[2] = dims[0] * dims[1];
-  g.st[3] = dims[0] * dims[1] * dims[2];
-  g.V = (int)V;
-  g.bc_t = bc_t;
+  const Geom g = make_geom(dims, bc_t);
   cudaStream_t s = (cudaStream_t)stream;
   // every byte of the scratch the stencil reads is written first in this call,
   // so nothing carried over from an earlier call is used

@@ -25,12 +25,23 @@ struct NvtxRange {
 
 // ---------------------------------------------------------------- geometry
 
+// Division by a fixed d for numerators below 2^28: (n m >> 32) >> l with m = floor(2^(32 + l)
+// / d) + 1, l = ceil(log2 d) - 1 (the error m d - 2^(32 + l) <= d <= 2^(4 + l), so the
+// quotient is exact); m = 0 stands for d = 1.
+struct FastDiv {
+  unsigned m;
+  int l;
+};
+
 struct Geom {
   int L[4];    // Lx, Ly, Lz, Lt
   int st[4];   // site strides: 1, Lx, Lx*Ly, Lx*Ly*Lz
   int V;       // sites
   int bc_t;    // +1 / -1
+  FastDiv dst[4], dL[4];  // division by st and L
 };
+
+Geom make_geom(const int dims[4], int bc_t);  // extents >= 1 of at most 2^28 sites
 
 // ---------------------------------------------------------------- workspace
 
@@ -102,6 +113,8 @@ struct ov_ctx {
   bool have_s4 = false;                // FP32 links for the spin-paired float4 layout
   float4* Udf = nullptr;               // double-float links (workspace "gauge.df") when have_df
   bool have_df = false;
+  int4* Ufx = nullptr;                 // fixed-point links (workspace "gauge.fx") when have_fx
+  bool have_fx = false, fx_ok = false; // fx_ok: every link fits the fixed-point bounds
   std::map<int, int> hw32_choice;      // nrhs -> autotuned FP32 stencil variant
   int hw32_force = -1;                 // ov_set_hw32_variant
   bool no_coop = true;                 // ov_set_persistent(ctx, 1) enables the persistent loop
@@ -169,6 +182,8 @@ void hw32_variant_info(int k, int* rt, int* comp, int* nt);
 float hw32_time_soa_variants(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int* best);
 // double-float links for the FP32-pair solve (dslash.cu)
 int ensure_links_df(ov_ctx* ctx, cudaStream_t s);
+// fixed-point links (dslash.cu); sets ctx->fx_ok
+int ensure_links_fx(ov_ctx* ctx, cudaStream_t s);
 // spin-paired float4 FP32 layout (dslash32.cu)
 int launch_pack_s4(ov_ctx* ctx, const float2* aos, float4* s4, int nrhs, cudaStream_t s);
 int launch_unpack_s4(ov_ctx* ctx, const float4* s4, float2* aos, int nrhs, cudaStream_t s);

@@ -40,7 +40,7 @@
 
 #include <cooperative_groups.h>
 
-#include "common.cuh"
+#include "fixed.cuh"
 
 namespace {
 
@@ -77,6 +77,11 @@ struct SrcState {
   double cm;      // ||U_i|| / ||U_{i-1}|| (0 at i = 1)
   double alpha_n; // alpha_i / ||U_i||: U_{i+1} = w - alpha_n U_i in one FMA per real
   float df[8];    // inv_n, cm, alpha, alpha_n as double-float (hi, lo) pairs
+  // fixed-point vectors X_i (solve_sign_stored<FX>); U_i = X_i up to a power of two
+  double n2, inv_n2;  // ||X_i||^2 in integer units and its reciprocal
+  FX dia, gam, alf;   // coefficients of X_i and X_{i-1} in w, of X_i in X_{i+1}; unit 2^-60
+  int q, k;           // w = (H X_i / 4 - ...) 2^-q;  X_{i+1} = (w - ...) 2^k
+  int e_in;           // X_1 = b 2^e_in
 };
 
 // exact double-float split of an FP64 value: hi = rn(x), lo = rn(x - hi)
@@ -177,10 +182,13 @@ struct SolveArgs {
   typename Coef<R>::T* act_z;   // [src][nshift] zeta_i
   double* part1;      // [src][nblk1]
   double* part2;      // [src][nblk2]
+  long long* bins1;   // [src][kFxBins][kFxWords] fixed point: sums of K1 and of K2
+  long long* bins2;
   unsigned* cnt;      // [src][2]
   int* done_count;
   double* hist_a;     // [src][max_iter] or null
   double* hist_b;
+  double* hist_n2;    // fixed point: ||X_i||^2
   const double2* gco; // [src][max_iter] second-pass coefficients or null
   const RegenRec<R>* rrec;  // [src][max_iter] regeneration-pass scalars or null
   const double* tol_src;  // [src] per-source tolerance or null (then SolveParams::tol)
@@ -188,6 +196,7 @@ struct SolveArgs {
   const T* U;         // links
   Geom g;
   R diag;
+  double diag4;       // (4 - m0) / 4 (fixed point)
 };
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
@@ -1116,6 +1125,472 @@ __global__ void __launch_bounds__(NT2) lanczos_init_kernel(SolveArgs<R> a, const
   }
 }
 
+// ------------------------------------------------------ fixed-point Lanczos kernels
+//
+// The recurrence on integer vectors X_i (fixed.cuh), each at a power-of-two scale of its
+// own.  With v_i = X_i / ||X_i||, H v_i = beta_{i-1} v_{i-1} + alpha_i v_i + beta_i v_{i+1}:
+//
+//   K1   w       = 2^-q H X_i / 4 - gam X_{i-1},  gam = 2^-q beta_{i-1} ||X_i|| / (4 ||X_{i-1}||)
+//        a       = <X_i, w> / ||X_i||^2,          alpha_i = 4 2^q a
+//   K2   X_{i+1} = 2^k (w - a X_i),               beta_i = 4 2^(q - k) ||X_{i+1}|| / ||X_i||
+//
+// q keeps gam at most 2 (q > 0 only while a localised source spreads); k brings
+// the largest component to just below 2^58, from the bound max |w| + |a| 2^58 that K1's
+// last block knows.  The inner products are sums of exact integer products (per thread),
+// then FP64.
+// 2^e as a double, -1022 <= e <= 1023
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+// floor(log2 |x|) of a normal number
+__device__ __forceinline__ int exponent_of(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+
+// Block maximum of an int; sh >= NT / 32 ints; a barrier must follow before sh is reused.
+template <int NT>
+__device__ __forceinline__ int block_max(int v, int* sh) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NT / 32; ++k) v = max(v, sh[k]);
+  return v;
+}
+
+// Sums over a source: integers, so that atomic additions in any order give the same result.
+// Blocks add into kFxBins bins (fewer collisions per address); the last block to arrive
+// (last_arrival) adds the bins up and clears them for the next launch.
+constexpr int kFxBins = 32;
+constexpr int kFxWords = 6;  // K1: five words of <X, w> and the maximum; K2: four words
+__device__ __forceinline__ bool last_arrival(unsigned* cnt, unsigned n) {
+  __threadfence();
+  if (atomicAdd(cnt, 1u) != n - 1) return false;
+  *cnt = 0;
+  __threadfence();
+  return true;
+}
+__device__ __forceinline__ long long warp_sum(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// A block takes one 32-site tile of `per` sources in turn (their links then come from L1).
+// Bound by the wide multiply-adds (one warp instruction per cycle and SM, 1300 per 32 sites
+// for the hops and 430 for the rest, half of the time) and the L2 latency of the neighbour
+// loads.  One source at 16^3 x 32: 63 us, where the FP64 kernel takes 227 us and the
+// double-float one 66 us; 6 sources in one launch: 6 x 45 us (links from L1).  4 blocks per
+// SM (64 registers): 375 ms per 12-source FP64 solve, 393 ms at 3.
+__global__ void __launch_bounds__(kFxNT, 4) fx_lanczos_hw_kernel(const __grid_constant__ SolveArgs<FX> a,
+                                                                 int nsrc, int per) {
+  __shared__ int red[kFxNT / 32][kFxWords];
+  __shared__ longlong2 sm[4 * 12 * kFxTile];
+  const int V = a.g.V;
+  const int nb = (V + kFxTile - 1) / kFxTile, ng = gridDim.x / nb;
+  const int tb = blockIdx.x / ng, r0 = blockIdx.x % ng * per;
+  const size_t n12 = 12 * fx_padded(V);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int s = tb * kFxTile + lane;  
+  const bool in = s < V;
+  const FxHops nbr = fx_hops(a.g, in ? s : 0, wid >> 1);
+  for (int r = r0; r < min(nsrc, r0 + per); ++r) {
+    SrcState* S = a.src + r;
+    if (S->done) continue;
+    const int i = S->iter, q = S->q;
+    int4* base = a.ring + (size_t)r * a.prm->nslots * n12;
+    const int4* Xi = base + (size_t)i * n12;  // stored basis: slot i holds X_i
+    if (in) fx_phase1(Xi, a.U, wid, s, nbr, sm + (wid >> 1) * 12 * kFxTile + lane);
+    __syncthreads();
+    // <X_i, w> = hh 2^62 + x1 2^30 + x2 2^32, w = wh 2^32 + wl with signed wl
+    long long hh = 0, x1 = 0, x2 = 0;
+    int wmax = 0;
+    if (in && wid < 6) {  // components 2 wid, 2 wid + 1
+      const bool low = wid >= 3;
+      // 2^-q diag / 4 x - gam X_{i-1} = (hh 2^60 + x 2^30) / 2^60; gamma5 = -1 on the lower spins
+      const FX dg = S->dia, nd = FX{low ? -dg.hi : dg.hi, low ? -dg.lo : dg.lo}, ng = S->gam;
+      const int4* xp = Xi + fx_index(s, 12) + 2 * wid * kFxTile;
+      longlong2* wp = reinterpret_cast<longlong2*>(const_cast<int4*>(xp + n12));
+      int4 xb[2], ub[2];
+      longlong2 t[2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        xb[j] = __ldg(xp + j * kFxTile);
+        ub[j] = i > 1 ? __ldg(xp - n12 + j * kFxTile) : make_int4(0, 0, 0, 0);
+        t[j] = fx_phase2(sm, 2 * wid + j, lane);
+      }
+      if (q > 0) {
+        const long long rq = 1LL << (q - 1);
+        for (int j = 0; j < 2; ++j) t[j] = make_longlong2((t[j].x + rq) >> q, (t[j].y + rq) >> q);
+      }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        long long w[2] = {t[j].x, t[j].y};
+        const int xv[4] = {xb[j].x, xb[j].y, xb[j].z, xb[j].w}, uv[4] = {ub[j].x, ub[j].y, ub[j].z, ub[j].w};
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          long long gh = w[c], gx = kFxHalf30;
+          fx_mac(gh, gx, nd.hi, nd.lo, xv[2 * c], xv[2 * c + 1]);
+          fx_mac(gh, gx, ng.hi, ng.lo, uv[2 * c], uv[2 * c + 1]);
+          w[c] = fx_value(gh, gx);
+          const int wl = (int)w[c], wh = (int)(w[c] >> 32) + (int)((unsigned)wl >> 31);
+          hh += (long long)xv[2 * c] * wh;
+          x1 += (long long)xv[2 * c] * wl;
+          x2 += (long long)xv[2 * c + 1] * wh;
+          wmax = max(wmax, abs(wh));
+        }
+        wp[j * kFxTile] = make_longlong2(w[0], w[1]);
+      }
+    } else if (wid < 6) {  // the padding of the last tile
+      int4* wp = base + (size_t)(i + 1) * n12 + fx_index(s, 12) + 2 * wid * kFxTile;
+      wp[0] = wp[kFxTile] = make_int4(0, 0, 0, 0);
+    }
+    // warp sums in words that cannot overflow 32 lanes: hh in 26 + 26 + 12 bits, the cross
+    // terms (below 2^-30 of hh's weight, kept to 2^-47) in 24 + 24
+    {
+      const long long xs = (x2 + (x1 >> 2)) >> 16;
+      int v[kFxWords];
+      v[0] = __reduce_add_sync(0xffffffffu, (int)(hh & 0x3ffffff));
+      v[1] = __reduce_add_sync(0xffffffffu, (int)((hh >> 26) & 0x3ffffff));
+      v[2] = __reduce_add_sync(0xffffffffu, (int)(hh >> 52));
+      v[3] = __reduce_add_sync(0xffffffffu, (int)(xs & 0xffffff));
+      v[4] = __reduce_add_sync(0xffffffffu, (int)(xs >> 24));
+      v[5] = __reduce_max_sync(0xffffffffu, wmax);
+      if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < kFxWords; ++k) red[wid][k] = v[k];
+    }
+    __syncthreads();
+    if (wid != 0) continue;  // red is next written after the next source's first barrier
+    long long* bins = a.bins1 + (size_t)r * kFxBins * kFxWords;
+    if (lane < kFxWords) {
+      long long t = red[0][lane];
+      for (int k = 1; k < kFxNT / 32; ++k) t = lane == 5 ? max(t, (long long)red[k][lane]) : t + red[k][lane];
+      long long* d = bins + (tb % kFxBins) * kFxWords + lane;
+      if (lane == 5)
+        atomicMax(d, t);
+      else
+        atomicAdd((unsigned long long*)d, (unsigned long long)t);
+    }
+    __syncwarp();
+    bool last = false;
+    if (lane == 0) last = last_arrival(a.cnt + 2 * r, nb);
+    if (!__shfl_sync(0xffffffffu, last, 0)) continue;
+    long long t[kFxWords];
+#pragma unroll
+    for (int k = 0; k < kFxWords; ++k) {
+      t[k] = __ldcg(bins + lane * kFxWords + k);
+      bins[lane * kFxWords + k] = 0;
+      if (k < 5)
+        t[k] = warp_sum(t[k]);
+      else
+        t[k] = __reduce_max_sync(0xffffffffu, (int)t[k]);
+    }
+    if (lane != 0) continue;
+    const double dot = fma((double)t[2], pow2(114), fma((double)t[1], pow2(88), (double)t[0] * pow2(62))) +
+                       fma((double)t[4], pow2(72), (double)t[3] * pow2(48));
+    const double a1 = dot * S->inv_n2;
+    const double alpha = a1 * pow2(2 + q);
+    S->alpha = alpha;
+    S->alf = fx_split(-__double2ll_rn(a1 * pow2(60)));
+    // |X_{i+1}| <= 2^k bound < 2^58
+    const double bound = fma(fabs(a1), pow2(kFxBits), (double)(t[5] + 1) * 4294967296.0);
+    S->k = kFxBits - 1 - exponent_of(bound);
+    a.hist_a[(size_t)r * a.prm->max_iter + (i - 1)] = alpha;
+    if (!isfinite(alpha)) mark_done(S, a.done_count, OV_ERR_BREAKDOWN);
+  }
+}
+
+// HBM-bound (576 B per site and source): two reads, one write, an exact integer norm; one
+// wave of blocks, two elements in flight per thread (18.6 us for one source at 16^3 x 32).
+template <>
+__global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX> a) {
+  __shared__ long long red[NT2 / 32][4];
+  const int r = blockIdx.y;
+  SrcState* S = a.src + r;
+  if (S->done) return;
+  const size_t n12 = 12 * fx_padded(a.g.V);
+  const int i = S->iter;
+  const int4* Xi = a.ring + ((size_t)r * a.prm->nslots + i) * n12;
+  int4* W = a.ring + ((size_t)r * a.prm->nslots + i + 1) * n12;
+  const FX alf = S->alf;
+  const int k = S->k;
+  const int kl = max(k, 0), kr = max(-k, 0);  // below 32 both
+  // 2^k y rounded, plus 2^29 (hi then comes out of a plain shift by 30)
+  const long long rnd = (kr > 0 ? 1LL << (kr - 1) : 0) + (kFxHalf30 << kr);
+  // ||X||^2 = n[0] 2^92 + n[1] 2^60 + n[2] 2^38 + n[3] 2^8 (what is dropped is far below 2^-53)
+  long long n[4] = {0, 0, 0, 0};
+  const size_t e0 = (size_t)blockIdx.x * NT2 + threadIdx.x, gs = (size_t)gridDim.x * NT2;
+  constexpr int B = 2;  // elements in flight per thread
+  for (size_t eb = e0; eb < n12; eb += B * gs) {
+    int4 xb[B], wb[B];
+#pragma unroll
+    for (int t = 0; t < B; ++t) {
+      const bool in = eb + t * gs < n12;
+      xb[t] = in ? __ldg(Xi + eb + t * gs) : make_int4(0, 0, 0, 0);
+      wb[t] = in ? W[eb + t * gs] : make_int4(0, 0, 0, 0);  // int64 pair (re, im)
+    }
+    long long hh = 0, xx = 0, ll = 0;  // of up to 8 reals: hh 2^60 + xx 2^30 + ll
+#pragma unroll
+    for (int t = 0; t < B; ++t) {
+      const int xv[4] = {xb[t].x, xb[t].y, xb[t].z, xb[t].w};
+      const long long wv[2] = {(long long)(((unsigned long long)(unsigned)wb[t].y << 32) | (unsigned)wb[t].x),
+                               (long long)(((unsigned long long)(unsigned)wb[t].w << 32) | (unsigned)wb[t].z)};
+      FX o[2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        // w - a X = w + (ah 2^60 + ax 2^30) / 2^60
+        long long ah = wv[c], ax = kFxHalf30;
+        fx_mac(ah, ax, alf.hi, alf.lo, xv[2 * c], xv[2 * c + 1]);
+        const long long y = fx_shr(fx_shl(fx_value(ah, ax), kl) + rnd, kr);
+        o[c].hi = (int)(y >> 30);
+        o[c].lo = ((int)y & 0x3fffffff) - (1 << 29);
+        hh += (long long)o[c].hi * o[c].hi;
+        xx += (long long)o[c].hi * (2 * o[c].lo);
+        ll += (long long)o[c].lo * o[c].lo;
+      }
+      if (eb + t * gs < n12) W[eb + t * gs] = make_int4(o[0].hi, o[0].lo, o[1].hi, o[1].lo);
+    }
+    n[0] += hh >> 32;
+    n[1] += (unsigned)hh;
+    n[2] += xx >> 8;
+    n[3] += ll >> 8;
+  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    n[j] = warp_sum(n[j]);
+    if (lane == 0) red[wid][j] = n[j];
+  }
+  __syncthreads();
+  if (wid != 0) return;
+  long long* bins = a.bins2 + (size_t)r * kFxBins * kFxWords;
+  if (lane < 4) {
+    long long t = 0;
+#pragma unroll
+    for (int j = 0; j < NT2 / 32; ++j) t += red[j][lane];
+    atomicAdd((unsigned long long*)bins + (blockIdx.x % kFxBins) * kFxWords + lane, (unsigned long long)t);
+  }
+  __syncwarp();
+  bool last = false;
+  if (lane == 0) last = last_arrival(a.cnt + 2 * r + 1, gridDim.x);
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    n[j] = warp_sum(__ldcg(bins + lane * kFxWords + j));
+    bins[lane * kFxWords + j] = 0;
+  }
+  if (lane != 0) return;
+  const double tot = fma((double)n[0], pow2(92), (double)n[1] * pow2(60)) + fma((double)n[2], pow2(38), (double)n[3] * 256.0);
+  const int q = S->q, ns = a.prm->nshift, mi = a.prm->max_iter;
+  const double ratio = tot * S->inv_n2;  // ||X_{i+1}||^2 / ||X_i||^2
+  const double beta = sqrt(ratio) * pow2(2 + q - k);
+  a.hist_b[(size_t)r * mi + (i - 1)] = beta;
+  if (i < mi) a.hist_n2[(size_t)r * mi + i] = tot;
+  const double g1 = ratio * pow2(q - k);  // beta_i ||X_{i+1}|| / (4 ||X_i||)
+  const int qn = max(0, exponent_of(g1));  // g1 2^-qn < 2
+  S->gam = fx_split(-__double2ll_rn(g1 * pow2(60 - qn)));
+  S->dia = fx_split(__double2ll_rn(a.diag4 * pow2(60 - qn)));
+  S->q = qn;
+  S->n2 = tot;
+  S->inv_n2 = __drcp_rn(tot);
+  S->n_prev = S->n_cur;
+  S->n_cur = beta;
+  S->iter = i + 1;
+  if (!isfinite(beta)) {
+    mark_done(S, a.done_count, OV_ERR_BREAKDOWN);
+  } else if (beta == 0.0) {
+    mark_done(S, a.done_count, OV_OK);
+  } else if (i >= mi || (a.prm->store && i + 2 >= a.prm->nslots)) {
+    mark_done(S, a.done_count, ns > 0 ? OV_ERR_NOT_CONVERGED : OV_OK);
+  }
+}
+
+// As the generic init, with the largest component of b for the scale of X_1 (written by
+// fx_quantize_kernel).
+template <>
+__global__ void __launch_bounds__(NT2) lanczos_init_kernel<FX>(SolveArgs<FX> a, const double2* __restrict__ b,
+                                                               double2 c0) {
+  __shared__ double sh[NT2 / 32];
+  __shared__ int shi[NT2 / 32];
+  __shared__ bool last;
+  __shared__ double tot_sh;
+  const int r = blockIdx.y;
+  const size_t n12 = (size_t)12 * a.g.V;
+  const size_t e = (size_t)blockIdx.x * NT2 + threadIdx.x;
+  double nrm = 0.0;
+  int mx = 0;
+  if (e < n12) {
+    const double2 bv = b[(size_t)r * n12 + e];
+    nrm = bv.x * bv.x + bv.y * bv.y;
+    mx = max(__double2hiint(bv.x) & 0x7fffffff, __double2hiint(bv.y) & 0x7fffffff);  // ordered as |b|
+    if (a.sacc) a.sacc[(size_t)r * n12 + e] = make_double2(c0.x * bv.x - c0.y * bv.y, c0.x * bv.y + c0.y * bv.x);
+  }
+  const double bs = block_sum<NT2>(nrm, sh);
+  mx = block_max<NT2>(mx, shi);
+  if (threadIdx.x == 0) {
+    a.part2[(size_t)r * gridDim.x + blockIdx.x] = bs;
+    atomicMax(a.bins1 + (size_t)r * kFxBins * kFxWords + 5, (long long)mx);
+    __threadfence();
+    last = (atomicAdd(a.cnt + 2 * r + 1, 1u) == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const double t = sum_partials<NT2>(a.part2 + (size_t)r * gridDim.x, gridDim.x, sh);
+  if (threadIdx.x == 0) tot_sh = t;
+  __syncthreads();
+  const double tot = tot_sh, bnorm = sqrt(tot);
+  SrcState* S = a.src + r;
+  const int ns = a.prm->nshift;
+  const bool skip = !(bnorm > 0.0) || !isfinite(bnorm);
+  for (int j = threadIdx.x; j < ns; j += NT2) {
+    ShiftState& q = a.sh[(size_t)r * ns + j];
+    q.invd = q.omega = q.zeta = make_double2(0.0, 0.0);
+    q.res2 = skip ? 0.0 : 1.0;
+    q.active = skip ? 0 : 1;
+    q.last_iter = 0;
+  }
+  if (threadIdx.x != 0) return;
+  a.cnt[2 * r + 1] = 0;
+  S->bnorm = bnorm;
+  S->inv_b2 = tot > 0.0 ? 1.0 / tot : 0.0;
+  S->n_cur = bnorm;
+  S->n_prev = 1.0;
+  S->alpha = 0.0;
+  S->iter = 1;
+  long long* mb = a.bins1 + (size_t)r * kFxBins * kFxWords + 5;
+  const int m = (int)__ldcg(mb);
+  *mb = 0;
+  S->e_in = kFxBits - 1 - ((m >> 20) - 1023);
+  S->n2 = ldexp(tot, 2 * S->e_in);
+  S->inv_n2 = 1.0 / S->n2;
+  a.hist_n2[(size_t)r * a.prm->max_iter] = S->n2;
+  S->gam = S->alf = FX{0, 0};
+  S->dia = fx_split(__double2ll_rn(a.diag4 * pow2(60)));
+  S->q = S->k = 0;
+  S->status = OV_OK;
+  S->n_act = 0;
+  S->node_updates = 0.0;
+  S->k_final = 0;
+  S->done = 0;
+  if (skip) mark_done(S, a.done_count, isfinite(bnorm) ? OV_OK : OV_ERR_BREAKDOWN);
+}
+
+// X_1 = b 2^e_in, rounded to integers
+__global__ void __launch_bounds__(NT2) fx_quantize_kernel(const __grid_constant__ SolveArgs<FX> a,
+                                                          const double2* __restrict__ b) {
+  const int r = blockIdx.y, V = a.g.V;
+  const SrcState* S = a.src + r;
+  if (S->done) return;
+  const size_t n12 = 12 * fx_padded(V);
+  const int e_in = S->e_in;
+  int4* X1 = a.ring + ((size_t)r * a.prm->nslots + 1) * n12;
+  for (size_t e = (size_t)blockIdx.x * NT2 + threadIdx.x; e < n12; e += (size_t)gridDim.x * NT2) {
+    const size_t tk = e / kFxTile;
+    const size_t site = tk / 12 * kFxTile + e % kFxTile;
+    double2 v = make_double2(0.0, 0.0);
+    if (site < V) v = b[((size_t)r * 12 + tk % 12) * V + site];
+    const FX re = fx_split(__double2ll_rn(ldexp(v.x, e_in))), im = fx_split(__double2ll_rn(ldexp(v.y, e_in)));
+    X1[e] = make_int4(re.hi, re.lo, im.hi, im.lo);
+  }
+}
+
+// sum[r][e] += scale_r sum_i G_i X_i[e] (basis_sum_kernel in fixed point): G_i = g_i / ||X_i||
+// as integers of at most 2^57; groups of 16 (8 complex) products are summed exactly, the groups in
+// FP64.  Reads 16 B per basis vector and element: HBM-bound.
+template <bool REAL>
+__global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restrict__ basis, int nslots,
+                                                           const int4* __restrict__ G, int ldg,
+                                                           const int* __restrict__ kr, const double* __restrict__ scale,
+                                                           double2* __restrict__ sum,
+                                                           int V) {
+  const int r = blockIdx.y;
+  const size_t n12 = 12 * fx_padded(V), e = (size_t)blockIdx.x * blockDim.x + threadIdx.x, tk = e / kFxTile;
+  if (e >= n12) return;
+  const size_t site = tk / 12 * kFxTile + e % kFxTile;
+  if (site >= V) return;
+  const int4* B = basis + (size_t)r * nslots * n12 + n12 + e;
+  const int4* w = G + (size_t)r * ldg;
+  const int k = kr[r];
+  double re = 0.0, im = 0.0;
+  constexpr int K = REAL ? 16 : 8;  // products whose cross terms fit 63 bits
+  for (int i0 = 0; i0 < k; i0 += K) {
+    long long rh = 0, rx = kFxHalf30, ih = 0, ix = kFxHalf30;
+    const int n = min(K, k - i0);
+#pragma unroll 8
+    for (int i = 0; i < n; ++i) {
+      const int4 g = __ldg(w + i0 + i), x = __ldg(B + (size_t)(i0 + i) * n12);
+      fx_mac(rh, rx, g.x, g.y, x.x, x.y);
+      fx_mac(ih, ix, g.x, g.y, x.z, x.w);
+      if (!REAL) {
+        fx_mac(rh, rx, -g.z, -g.w, x.z, x.w);
+        fx_mac(ih, ix, g.z, g.w, x.x, x.y);
+      }
+    }
+    re += (double)fx_value(rh, rx);
+    im += (double)fx_value(ih, ix);
+  }
+  const double sc = scale[r];
+  double2* so = sum + ((size_t)r * 12 + tk % 12) * V + site;
+  double2 sv = *so;
+  sv.x = fma(sc, re, sv.x);
+  sv.y = fma(sc, im, sv.y);
+  *so = sv;
+}
+
+// Per-node solutions from a fixed-point basis (basis_nodes_kernel): Y per (source, node) with
+// its own scale, JT nodes per thread.
+template <int JT>
+__global__ void __launch_bounds__(256) fx_basis_nodes_kernel(const int4* __restrict__ basis, int nslots,
+                                                             const int4* __restrict__ Y,
+                                                             const double* __restrict__ scale, int ns, int ldy,
+                                                             const int* __restrict__ kr, int j0, int nc,
+                                                             double2* __restrict__ X,
+                                                             int V) {
+  const int r = blockIdx.y, jt = blockIdx.z * JT;
+  const size_t n12 = 12 * fx_padded(V), e = (size_t)blockIdx.x * blockDim.x + threadIdx.x, tk = e / kFxTile;
+  if (e >= n12 || jt >= nc) return;
+  const size_t site = tk / 12 * kFxTile + e % kFxTile;
+  if (site >= V) return;
+  const int4* B = basis + (size_t)r * nslots * n12 + n12 + e;
+  const int4* Yr = Y + ((size_t)r * ns + j0 + jt) * ldy;
+  const int k = kr[r], nj = min(JT, nc - jt);
+  double re[JT], im[JT];
+#pragma unroll
+  for (int t = 0; t < JT; ++t) re[t] = im[t] = 0.0;
+  for (int i0 = 0; i0 < k; i0 += 8) {
+    long long rh[JT], rx[JT], ih[JT], ix[JT];
+#pragma unroll
+    for (int t = 0; t < JT; ++t) {
+      rh[t] = ih[t] = 0;
+      rx[t] = ix[t] = kFxHalf30;
+    }
+    const int n = min(8, k - i0);
+    for (int i = 0; i < n; ++i) {
+      const int4 x = __ldg(B + (size_t)(i0 + i) * n12);
+#pragma unroll
+      for (int t = 0; t < JT; ++t) {
+        if (t < nj) {
+          const int4 y = __ldg(Yr + (size_t)t * ldy + i0 + i);
+          fx_mac(rh[t], rx[t], y.x, y.y, x.x, x.y);
+          fx_mac(rh[t], rx[t], -y.z, -y.w, x.z, x.w);
+          fx_mac(ih[t], ix[t], y.x, y.y, x.z, x.w);
+          fx_mac(ih[t], ix[t], y.z, y.w, x.x, x.y);
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < JT; ++t) {
+      re[t] += (double)fx_value(rh[t], rx[t]);
+      im[t] += (double)fx_value(ih[t], ix[t]);
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < JT; ++t) {
+    if (t < nj) {
+      const double sc = scale[(size_t)r * ns + j0 + jt + t];
+      X[(((size_t)r * nc + jt + t) * 12 + tk % 12) * V + site] = make_double2(sc * re[t], sc * im[t]);
+    }
+  }
+}
+
 // second pass: U_1 = b again in ring slot 1 (the first pass overwrote the ring)
 template <typename R>
 __global__ void ring_reset_kernel(SolveArgs<R> a, const double2* __restrict__ b, int nsrc, int nslots) {
@@ -1147,6 +1622,7 @@ namespace {
 template <typename R> const char* coef_tag();
 template <> const char* coef_tag<double>() { return "fp64"; }
 template <> const char* coef_tag<DF>() { return "df"; }
+template <> const char* coef_tag<FX>() { return "fx"; }
 
 // a complex coefficient in the storage type of the vectors (host side)
 inline double2 host_store(double2 v, double2*) { return v; }
@@ -1160,17 +1636,24 @@ template <typename R> const typename Store<R>::T* solver_links(ov_ctx* ctx);
 template <> const double2* solver_links<double>(ov_ctx* ctx) { return ctx->U64h; }  // -1/2 U
 template <> const float2* solver_links<float>(ov_ctx* ctx) { return ctx->U32; }
 template <> const float4* solver_links<DF>(ov_ctx* ctx) { return ctx->Udf; }
+template <> const int4* solver_links<FX>(ov_ctx* ctx) { return ctx->Ufx; }
 template <typename R> R solver_real(double x) { return (R)x; }
 template <> DF solver_real<DF>(double x) {
   const float h = (float)x;
   return DF(h, (float)(x - (double)h));
 }
+template <> FX solver_real<FX>(double) { return FX{0, 0}; }  // SolveArgs::diag4 instead
+
+// Elements of one Lanczos vector: 12 planes of V, padded to whole tiles in fixed point.
+template <typename R> size_t vec_elems(size_t V) { return 12 * V; }
+template <> size_t vec_elems<FX>(size_t V) { return 12 * fx_padded(V); }
 
 template <typename R>
 struct SolveWs {
   SolveArgs<R> a{};
   int nblk1 = 0, nblk2 = 0, nblk2u = 0;
   int nslots = 3;
+  size_t nvec = 0;   // elements of one Lanczos vector (12 V, padded in fixed point)
   int nshift = 0;
   int max_iter = 0;  // row length of the per-source histories
   SolveParams* prm_dev = nullptr;
@@ -1184,7 +1667,7 @@ template <typename R>
 SolveArgs<R> args_for_sources(const SolveWs<R>& w, int r0) {
   SolveArgs<R> a = w.a;
   const size_t n12 = (size_t)12 * w.a.g.V, ns = (size_t)w.nshift, r = (size_t)r0;
-  a.ring += r * w.nslots * n12;
+  a.ring += r * w.nslots * w.nvec;
   if (a.p) a.p += r * ns * n12;
   if (a.x) a.x += r * ns * n12;
   if (a.sacc) a.sacc += r * n12;
@@ -1200,9 +1683,12 @@ SolveArgs<R> args_for_sources(const SolveWs<R>& w, int r0) {
   a.act_z += r * ns;
   a.part1 += r * w.nblk1;
   a.part2 += r * w.nblk2u;
+  if (a.bins1) a.bins1 += r * kFxBins * kFxWords;
+  if (a.bins2) a.bins2 += r * kFxBins * kFxWords;
   a.cnt += 2 * r;
   if (a.hist_a) a.hist_a += r * w.max_iter;
   if (a.hist_b) a.hist_b += r * w.max_iter;
+  if (a.hist_n2) a.hist_n2 += r * w.max_iter;
   if (a.gco) a.gco += r * w.max_iter;
   if (a.rrec) a.rrec += r * w.max_iter;
   if (a.tol_src) a.tol_src += r;
@@ -1288,9 +1774,12 @@ int setup_ws(ov_ctx* ctx, int nsrc, int ns, bool want_x, bool want_sacc, bool wa
   // HBM) when every thread would otherwise stride over more than 8 elements
   const size_t want = std::min<size_t>(8 * 152, std::max<size_t>(2 * 152, (size_t)nsrc * n12 / (NT2 * 8)));
   w->nblk2u = (int)std::min<size_t>(w->nblk2, std::max<size_t>(8, want / (size_t)nsrc));
+  if (std::is_same<R, FX>::value)  // one wave of resident blocks at most
+    w->nblk2u = (int)std::min<size_t>(w->nblk2, std::max<size_t>(8, std::min<size_t>(want, 4 * 152) / (size_t)nsrc));
   auto& a = w->a;
   w->nslots = nslots;
-  a.ring = (T*)ws_get(ctx, (t + ".ring").c_str(), sizeof(T) * (size_t)nslots * n12 * nsrc, &st);
+  w->nvec = vec_elems<R>(V);
+  a.ring = (T*)ws_get(ctx, (t + ".ring").c_str(), sizeof(T) * (size_t)nslots * w->nvec * nsrc, &st);
   // per-node direction vectors: only the vector-space form (coefficient-space: none)
   a.p = (ns && want_p) ? (T*)ws_get(ctx, (t + ".p").c_str(), sizeof(T) * n12 * (size_t)nsrc * ns, &st) : nullptr;
   a.x = (want_x && ns) ? (T*)ws_get(ctx, (t + ".x").c_str(), sizeof(T) * n12 * (size_t)nsrc * ns, &st) : nullptr;
@@ -1307,6 +1796,14 @@ int setup_ws(ov_ctx* ctx, int nsrc, int ns, bool want_x, bool want_sacc, bool wa
   a.act_z = (CT*)ws_get(ctx, (t + ".az").c_str(), sizeof(CT) * nsh, &st);
   a.part1 = (double*)ws_get(ctx, (t + ".part1").c_str(), sizeof(double) * (size_t)w->nblk1 * nsrc, &st);
   a.part2 = (double*)ws_get(ctx, (t + ".part2").c_str(), sizeof(double) * (size_t)w->nblk2 * nsrc, &st);
+  a.bins1 = a.bins2 = nullptr;
+  a.hist_n2 = nullptr;
+  if (std::is_same<R, FX>::value) {
+    const size_t nbins = (size_t)nsrc * kFxBins * kFxWords;
+    a.bins1 = (long long*)ws_get(ctx, (t + ".bins").c_str(), sizeof(long long) * 2 * nbins, &st);
+    if (a.bins1) a.bins2 = a.bins1 + nbins;
+    a.hist_n2 = (double*)ws_get(ctx, (t + ".hn").c_str(), sizeof(double) * (size_t)nsrc * max_iter, &st);
+  }
   a.cnt = (unsigned*)ws_get(ctx, (t + ".cnt").c_str(), sizeof(unsigned) * 2 * nsrc, &st);
   a.done_count = (int*)ws_get(ctx, (t + ".done").c_str(), sizeof(int), &st);
   if (want_hist) {
@@ -1322,6 +1819,7 @@ int setup_ws(ov_ctx* ctx, int nsrc, int ns, bool want_x, bool want_sacc, bool wa
   a.stencil = nullptr;
   a.g = ctx->g;
   a.diag = solver_real<R>(4.0 - ctx->m0);
+  a.diag4 = 0.25 * (4.0 - ctx->m0);
   a.U = solver_links<R>(ctx);
   return st;
 }
@@ -1338,6 +1836,21 @@ dim3 k1_grid(const SolveWs<R>& w, int n) {
   return dim3((unsigned)w.nblk1 * (unsigned)n);
 }
 
+// K1 over n sources.  Fixed point: a block takes up to kFxPerBlock sources of a tile (their
+// links then come from registers), fewer while the grid would not fill the GPU.
+constexpr int kFxPerBlock = 6;
+template <typename R>
+void launch_k1(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s) {
+  if constexpr (std::is_same<R, FX>::value) {
+    int ng = (n + kFxPerBlock - 1) / kFxPerBlock;
+    while (ng < n && (size_t)w.nblk1 * ng < 4 * 4 * 152) ++ng;
+    const int per = (n + ng - 1) / ng;
+    fx_lanczos_hw_kernel<<<(unsigned)w.nblk1 * ((n + per - 1) / per), kFxNT, 0, s>>>(a, n, per);
+  } else {
+    lanczos_hw_kernel<R><<<k1_grid(w, n), NT1, 0, s>>>(a);
+  }
+}
+
 template <typename R>
 void launch_node_check(const SolveWs<R>& w, const SolveArgs<R>& a, int nsrc, cudaStream_t s) {
   node_check_kernel<R><<<dim3(1, nsrc), NT1, 0, s>>>(a);
@@ -1350,7 +1863,7 @@ template <typename R>
 int launch_iteration(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, cudaStream_t s, int it) {
   cudaEvent_t ev;
   kt_begin(ctx, KC_LANCZOS_HW, s, &ev);
-  lanczos_hw_kernel<R><<<k1_grid(w, nsrc), NT1, 0, s>>>(w.a);
+  launch_k1<R>(w, w.a, nsrc, s);
   kt_end(ctx, KC_LANCZOS_HW, s, ev);
   kt_begin(ctx, KC_SHIFT_UPDATE, s, &ev);
   lanczos_update_kernel<R><<<dim3(w.nblk2u, nsrc), NT2, 0, s>>>(w.a);
@@ -1384,7 +1897,7 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
           ctx, w, nsrc, G,
           [&](cudaStream_t cs, const SolveArgs<R>& a, int n) {
             for (int k = 0; k < chunk; ++k) {
-              lanczos_hw_kernel<R><<<k1_grid(w, n), NT1, 0, cs>>>(a);
+              launch_k1<R>(w, a, n, cs);
               lanczos_update_kernel<R><<<dim3(w.nblk2u, n), NT2, 0, cs>>>(a);
               if (w.defer && (k + 1) % kNodeCheck == 0) launch_node_check<R>(w, a, n, cs);
             }
@@ -1431,6 +1944,8 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
 template <typename R>
 int run_coop(ov_ctx* ctx, SolveWs<R>& w, int nsrc, cudaStream_t s, double* launches) {
   if (nsrc > kCoopMaxSrc || ctx->no_coop) return OV_ERR_INVALID_ARG;
+  if constexpr (std::is_same<R, FX>::value) return OV_ERR_INVALID_ARG;  // not reached: FP64 then
+  else {
   int dev = 0, coop = 0, nsm = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
@@ -1457,6 +1972,7 @@ int run_coop(ov_ctx* ctx, SolveWs<R>& w, int nsrc, cudaStream_t s, double* launc
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "cudaLaunchCooperativeKernel");
   *launches += 1.0;
   return OV_OK;
+  }
 }
 
 template <typename R>
@@ -1476,13 +1992,16 @@ int init_solve(ov_ctx* ctx, SolveWs<R>& w, const double2* b_soa, int nsrc, int n
   }
   cudaMemsetAsync(w.a.cnt, 0, sizeof(unsigned) * 2 * nsrc, s);
   cudaMemsetAsync(w.a.done_count, 0, sizeof(int), s);
-  if (w.a.x) {
+  if (w.a.bins1) cudaMemsetAsync(w.a.bins1, 0, sizeof(long long) * 2 * kFxBins * kFxWords * nsrc, s);
+  if constexpr (!std::is_same<R, FX>::value) {  // fixed point keeps no per-node vectors
     const size_t n = (size_t)12 * ctx->g.V * nsrc * ns;
-    zero_kernel<R><<<1024, 256, 0, s>>>(w.a.x, n);
+    if (w.a.x) zero_kernel<R><<<1024, 256, 0, s>>>(w.a.x, n);
   }
   cudaEvent_t ev;
   kt_begin(ctx, KC_MISC, s, &ev);
   lanczos_init_kernel<R><<<dim3(w.nblk2, nsrc), NT2, 0, s>>>(w.a, b_soa, c0);
+  if constexpr (std::is_same<R, FX>::value)
+    fx_quantize_kernel<<<dim3(std::min(w.nblk2, 1024), nsrc), NT2, 0, s>>>(w.a, b_soa);
   kt_end(ctx, KC_MISC, s, ev);
   OV_CHECK_LAUNCH(ctx, "lanczos_init_kernel");
   return OV_OK;
@@ -1631,6 +2150,20 @@ static void fom_coefficients(const double* al, const double* be, int k, double b
   for (int i = k - 2; i >= 0; --i) yy[i] = sc.zt[i] - sc.ll[i] * yy[i + 1];
 }
 
+// Coefficients w[0..k) as fixed-point integers of at most 2^57 in out; returns the factor
+// of sum_i w_i X_i, given as (hh + x 2^-30) = 2^-60 sum_i out_i X_i.
+static double fx_coefficients(const std::complex<double>* w, int k, int4* out) {
+  double mx = 0.0;
+  for (int i = 0; i < k; ++i) mx = std::max(mx, std::max(std::fabs(w[i].real()), std::fabs(w[i].imag())));
+  if (!(mx > 0.0) || !std::isfinite(mx)) mx = 1.0;
+  const int e = 56 - std::ilogb(mx);
+  for (int i = 0; i < k; ++i) {
+    const FX re = fx_split(std::llrint(std::ldexp(w[i].real(), e))), im = fx_split(std::llrint(std::ldexp(w[i].imag(), e)));
+    out[i] = make_int4(re.hi, re.lo, im.hi, im.lo);
+  }
+  return std::ldexp(1.0, 60 - e);
+}
+
 // g = sum_j c_j (z_j - T_k)^-1 e_1 ||b|| per source, from the recorded alpha (ha) and beta
 // (hb), leading dimension ld.
 static void lanczos_sum_coefficients(const ov_ctx* ctx, int nsrc, const std::vector<int>& kr,
@@ -1661,6 +2194,7 @@ template <typename R>
 static int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int nsrc,
                              const ov_solve_opts& o, SolveOut* so, cudaStream_t s, int cap) {
   NvtxRange nvtx_("solve: stored basis");
+  constexpr bool kFix = std::is_same<R, FX>::value;
   const int ns = (int)ctx->z.size();
   const size_t n12 = (size_t)12 * ctx->g.V;
   SolveWs<R> w;
@@ -1688,6 +2222,9 @@ static int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa
   cudaError_t e = cudaMemcpyAsync(S.data(), w.a.src, sizeof(SrcState) * nsrc, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ha.data(), w.a.hist_a, sizeof(double) * ha.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hb.data(), w.a.hist_b, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, s);
+  std::vector<double> hn(kFix ? ha.size() : 0);  // fixed point: ||X_i||^2
+  if (kFix && e == cudaSuccess)
+    e = cudaMemcpyAsync(hn.data(), w.a.hist_n2, sizeof(double) * hn.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "read Lanczos history");
   std::vector<int> kr(nsrc);
@@ -1700,7 +2237,7 @@ static int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa
   lanczos_sum_coefficients(ctx, nsrc, kr, bn, ha, hb, cap, g);
   for (int r = 0; r < nsrc; ++r)
     for (int i = 0; i < kr[r]; ++i) {  // fold in 1 / ||U_i||
-      const double ni = (i == 0) ? bn[r] : hb[(size_t)r * cap + i - 1];
+      const double ni = kFix ? std::sqrt(hn[(size_t)r * cap + i]) : (i == 0) ? bn[r] : hb[(size_t)r * cap + i - 1];
       g[(size_t)r * cap + i].x /= ni;
       g[(size_t)r * cap + i].y /= ni;
     }
@@ -1718,20 +2255,39 @@ static int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa
   }
   using T = typename Store<R>::T;
   std::vector<T> gs(g.size());
-  for (size_t t = 0; t < g.size(); ++t) gs[t] = host_store(g[t], (T*)nullptr);
+  std::vector<double> gsc(nsrc, 1.0);
+  if constexpr (kFix) {
+    std::vector<std::complex<double>> gr;
+    for (int r = 0; r < nsrc; ++r) {
+      gr.resize(kr[r]);
+      for (int i = 0; i < kr[r]; ++i) gr[i] = {g[(size_t)r * cap + i].x, g[(size_t)r * cap + i].y};
+      gsc[r] = fx_coefficients(gr.data(), kr[r], gs.data() + (size_t)r * cap);
+    }
+  } else {
+    for (size_t t = 0; t < g.size(); ++t) gs[t] = host_store(g[t], (T*)nullptr);
+  }
   T* gd = (T*)ws_get(ctx, (tag + ".g").c_str(), sizeof(T) * gs.size(), &st);
   int* krd = (int*)ws_get(ctx, (tag + ".kr").c_str(), sizeof(int) * nsrc, &st);
+  double* gscd = kFix ? (double*)ws_get(ctx, (tag + ".gsc").c_str(), sizeof(double) * nsrc, &st) : nullptr;
   if (st != OV_OK) return st;
   e = cudaMemcpyAsync(gd, gs.data(), sizeof(T) * gs.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(krd, kr.data(), sizeof(int) * nsrc, cudaMemcpyHostToDevice, s);
+  if (kFix && e == cudaSuccess)
+    e = cudaMemcpyAsync(gscd, gsc.data(), sizeof(double) * nsrc, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy coefficients");
   cudaEvent_t ev;
   kt_begin(ctx, KC_BASIS_SUM, s, &ev);
-  const dim3 gsum((unsigned)((n12 + 255) / 256), nsrc);
-  if (real)
+  const dim3 gsum((unsigned)((w.nvec + 255) / 256), nsrc);
+  if constexpr (kFix) {
+    if (real)
+      fx_basis_sum_kernel<true><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, gscd, w.a.sacc, ctx->g.V);
+    else
+      fx_basis_sum_kernel<false><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, gscd, w.a.sacc, ctx->g.V);
+  } else if (real) {
     basis_sum_kernel<R, true><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, w.a.sacc, n12);
-  else
+  } else {
     basis_sum_kernel<R, false><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, w.a.sacc, n12);
+  }
   kt_end(ctx, KC_BASIS_SUM, s, ev);
   OV_CHECK_LAUNCH(ctx, "basis_sum_kernel");
   so->launches = launches + 3.0;
@@ -1778,7 +2334,13 @@ template <typename R>
 static int solve_sign_coef(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int nsrc, const ov_solve_opts& o,
                            SolveOut* so, cudaStream_t s) {
   NvtxRange nvtx_("solve: coefficient space");
-  if (o.mode == OV_MODE_FP64_REGEN) return solve_sign_regen<R>(ctx, b_soa, out_soa, nsrc, o, so, s);
+  auto regen = [&](int r0, int nb, SolveOut* sb) {
+    const size_t off = (size_t)r0 * 12 * ctx->g.V;
+    if (o.mode != OV_MODE_F32X2) return solve_sign_regen<double>(ctx, b_soa + off, out_soa + off, nb, o, sb, s);
+    const int st = ensure_links_df(ctx, s);
+    return st != OV_OK ? st : solve_sign_regen<DF>(ctx, b_soa + off, out_soa + off, nb, o, sb, s);
+  };
+  if (o.mode == OV_MODE_FP64_REGEN) return regen(0, nsrc, so);
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
   const std::string ring = std::string(coef_tag<R>()) + "s.ring";
@@ -1786,7 +2348,7 @@ static int solve_sign_coef(ov_ctx* ctx, const double2* b_soa, double2* out_soa, 
   const double held = it != ctx->bufs.end() ? (double)it->second.bytes : 0.0;
   const double budget = std::min(0.40 * (double)totalb, (double)freeb + held - 0.10 * (double)totalb);
   const size_t n12 = (size_t)12 * ctx->g.V;
-  const double per_vec = (double)n12 * sizeof(double2);
+  const double per_vec = (double)vec_elems<R>(ctx->g.V) * sizeof(double2);
   int cap = std::min(o.max_iter, ctx->coef_iter_hint > 0 ? std::max(64, ctx->coef_iter_hint * 5 / 4 + 32) : 1024);
   int r0 = 0, worst = OV_OK;
   bool first = true;
@@ -1801,7 +2363,7 @@ static int solve_sign_coef(ov_ctx* ctx, const double2* b_soa, double2* out_soa, 
     if (st == OV_ERR_OUT_OF_MEMORY || (st == OV_ERR_NOT_CONVERGED && cap < o.max_iter)) {
       cudaGetLastError();
       sb = SolveOut();
-      st = solve_sign_regen<R>(ctx, b_soa + r0 * n12, out_soa + r0 * n12, nb, o, &sb, s);
+      st = regen(r0, nb, &sb);
     }
     if (st != OV_OK && st != OV_ERR_NOT_CONVERGED) return st;
     if (st == OV_ERR_NOT_CONVERGED) worst = st;
@@ -1954,6 +2516,7 @@ template <typename R>
 static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
                       const std::vector<double2>& ch, int chunk, double2* X, double2* sums, const ov_solve_opts& o,
                       SolveOut* so, cudaStream_t s, const std::function<int(int, int)>& per_chunk) {
+  constexpr bool kFix = std::is_same<R, FX>::value;
   const size_t n12 = (size_t)12 * ctx->g.V;
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
@@ -1962,7 +2525,7 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
   const double held = it != ctx->bufs.end() ? (double)it->second.bytes : 0.0;
   const double budget = std::min(0.40 * (double)totalb, (double)freeb + held - 0.10 * (double)totalb);
   const int cap = std::min(o.max_iter, ctx->coef_iter_hint > 0 ? std::max(64, ctx->coef_iter_hint * 5 / 4 + 32) : 1024);
-  if ((double)(cap + 3) * nsrc * n12 * sizeof(double2) > budget) return OV_ERR_INVALID_ARG;
+  if ((double)(cap + 3) * nsrc * vec_elems<R>(ctx->g.V) * sizeof(double2) > budget) return OV_ERR_INVALID_ARG;
   SolveWs<R> w;
   int st = setup_ws<R>(ctx, nsrc, ns, false, true, true, cap, &w, tag.c_str(), cap + 3, false);
   if (st != OV_OK) return st;
@@ -1978,6 +2541,9 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
   cudaError_t e = cudaMemcpyAsync(S.data(), w.a.src, sizeof(SrcState) * nsrc, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ha.data(), w.a.hist_a, sizeof(double) * ha.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hb.data(), w.a.hist_b, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, s);
+  std::vector<double> hn(kFix ? ha.size() : 0);  // fixed point: ||X_i||^2
+  if (kFix && e == cudaSuccess)
+    e = cudaMemcpyAsync(hn.data(), w.a.hist_n2, sizeof(double) * hn.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "read Lanczos history");
   // FOM coefficients y^j = (z_j - T_k)^-1 e_1 ||b|| per source and node (forward LDL^T sweep,
@@ -1986,6 +2552,7 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
   std::vector<T> Yh((size_t)nsrc * ns * cap);
   std::vector<T> gh((size_t)nsrc * cap);
   std::vector<int> kr(nsrc);
+  std::vector<double> Ysc((size_t)nsrc * ns, 1.0), gsc(nsrc, 1.0);  // fixed point: factors of the sums
   FomScratch sc;
   std::vector<std::complex<double>> yy, gs;
   for (int r = 0; r < nsrc; ++r) {
@@ -1998,18 +2565,31 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
       const std::complex<double> cj(ch[(size_t)r * ns + j].x, ch[(size_t)r * ns + j].y);
       fom_coefficients(al, be, k, S[r].bnorm, zj, sc, yy);
       for (int i = 0; i < k; ++i) {
-        const double ni = (i == 0) ? S[r].bnorm : be[i - 1];
-        const std::complex<double> y = yy[i] / ni;
-        Yh[((size_t)r * ns + j) * cap + i] = host_store(make_double2(y.real(), y.imag()), (T*)nullptr);
-        gs[i] += cj * y;
+        const double ni = kFix ? std::sqrt(hn[(size_t)r * cap + i]) : (i == 0) ? S[r].bnorm : be[i - 1];
+        yy[i] /= ni;
+        if constexpr (!kFix)
+          Yh[((size_t)r * ns + j) * cap + i] = host_store(make_double2(yy[i].real(), yy[i].imag()), (T*)nullptr);
+        gs[i] += cj * yy[i];
       }
+      if constexpr (kFix)
+        Ysc[(size_t)r * ns + j] = fx_coefficients(yy.data(), k, Yh.data() + ((size_t)r * ns + j) * cap);
     }
-    for (int i = 0; i < k; ++i) gh[(size_t)r * cap + i] = host_store(make_double2(gs[i].real(), gs[i].imag()), (T*)nullptr);
+    if constexpr (kFix)
+      gsc[r] = fx_coefficients(gs.data(), k, gh.data() + (size_t)r * cap);
+    else
+      for (int i = 0; i < k; ++i) gh[(size_t)r * cap + i] = host_store(make_double2(gs[i].real(), gs[i].imag()), (T*)nullptr);
   }
   T* Yd = (T*)ws_get(ctx, (tag + ".Y").c_str(), sizeof(T) * Yh.size(), &st);
   T* gd = (T*)ws_get(ctx, (tag + ".g").c_str(), sizeof(T) * gh.size(), &st);
   int* krd = (int*)ws_get(ctx, (tag + ".kr").c_str(), sizeof(int) * nsrc, &st);
+  double* Yscd = kFix ? (double*)ws_get(ctx, (tag + ".Ysc").c_str(), sizeof(double) * Ysc.size(), &st) : nullptr;
+  double* gscd = kFix ? (double*)ws_get(ctx, (tag + ".gsc").c_str(), sizeof(double) * nsrc, &st) : nullptr;
   if (st != OV_OK) return st;
+  if (kFix) {
+    e = cudaMemcpyAsync(Yscd, Ysc.data(), sizeof(double) * Ysc.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(gscd, gsc.data(), sizeof(double) * nsrc, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy coefficient scales");
+  }
   e = cudaMemcpyAsync(Yd, Yh.data(), sizeof(T) * Yh.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(gd, gh.data(), sizeof(T) * gh.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(krd, kr.data(), sizeof(int) * nsrc, cudaMemcpyHostToDevice, s);
@@ -2017,15 +2597,21 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy node coefficients");
   cudaEvent_t ev;
   kt_begin(ctx, KC_BASIS_SUM, s, &ev);
-  basis_sum_kernel<R><<<dim3((unsigned)((n12 + 255) / 256), nsrc), 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd,
-                                                                             sums, n12);
+  const dim3 gsum((unsigned)((w.nvec + 255) / 256), nsrc);
+  if constexpr (kFix)
+    fx_basis_sum_kernel<false><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, gscd, sums, ctx->g.V);
+  else
+    basis_sum_kernel<R><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, sums, n12);
   kt_end(ctx, KC_BASIS_SUM, s, ev);
   OV_CHECK_LAUNCH(ctx, "basis_sum_kernel");
-  constexpr int JT = 8;
+  constexpr int JT = kFix ? 4 : 8;
   for (int j0 = 0; j0 < ns; j0 += chunk) {
     const int nc = std::min(chunk, ns - j0);
-    basis_nodes_kernel<R, JT><<<dim3((unsigned)((n12 + 255) / 256), nsrc, (nc + JT - 1) / JT), 256, 0, s>>>(
-        w.a.ring, cap + 3, Yd, ns, cap, krd, j0, nc, X, n12);
+    const dim3 gn((unsigned)((w.nvec + 255) / 256), nsrc, (nc + JT - 1) / JT);
+    if constexpr (kFix)
+      fx_basis_nodes_kernel<JT><<<gn, 256, 0, s>>>(w.a.ring, cap + 3, Yd, Yscd, ns, cap, krd, j0, nc, X, ctx->g.V);
+    else
+      basis_nodes_kernel<R, JT><<<gn, 256, 0, s>>>(w.a.ring, cap + 3, Yd, ns, cap, krd, j0, nc, X, n12);
     OV_CHECK_LAUNCH(ctx, "basis_nodes_kernel");
     if ((st = per_chunk(j0, nc)) != OV_OK) return st;
   }
@@ -2034,9 +2620,18 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
   return fst;
 }
 
+// Whether the stored-basis forms run in fixed point (fixed.cuh): links of norm 1 (the bounds
+// there) and |4 - m0| <= 4.  Other links and masses, and the persistent loop, keep the
+// FP64 and double-float kernels.
+static bool fixed_point_fits(ov_ctx* ctx, cudaStream_t s) {
+  return ctx->no_coop && std::fabs(4.0 - ctx->m0) <= kFxDiagMax && ensure_links_fx(ctx, s) == OV_OK && ctx->fx_ok;
+}
+
 int solve_nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
                      const std::vector<double2>& ch, int chunk, double2* X, double2* sums, const ov_solve_opts& o,
                      SolveOut* so, cudaStream_t s, const std::function<int(int, int)>& per_chunk) {
+  if (fixed_point_fits(ctx, s))
+    return nodes_coef<FX>(ctx, b_soa, nsrc, ns, zh, ch, chunk, X, sums, o, so, s, per_chunk);
   if (o.mode == OV_MODE_F32X2) {
     const int st = ensure_links_df(ctx, s);
     if (st != OV_OK) return st;
@@ -2047,6 +2642,8 @@ int solve_nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const 
 
 int solve_sign_2pass(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int nsrc, const ov_solve_opts& o,
                      SolveOut* so, cudaStream_t s) {
+  if (o.mode != OV_MODE_FP64_REGEN && fixed_point_fits(ctx, s))
+    return solve_sign_coef<FX>(ctx, b_soa, out_soa, nsrc, o, so, s);
   if (o.mode == OV_MODE_F32X2) {
     const int st = ensure_links_df(ctx, s);
     if (st != OV_OK) return st;
