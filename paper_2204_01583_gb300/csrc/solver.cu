@@ -1492,31 +1492,123 @@ __global__ void __launch_bounds__(NT2) fx_quantize_kernel(const __grid_constant_
   }
 }
 
-// sum[r][e] += scale_r sum_i G_i X_i[e] (basis_sum_kernel in fixed point): G_i = g_i / ||X_i||
-// as integers of at most 2^57; groups of 16 (8 complex) products are summed exactly, the groups in
-// FP64.  Reads 16 B per basis vector and element: HBM-bound.
-template <bool REAL>
-__global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restrict__ basis, int nslots,
-                                                           const int4* __restrict__ G, int ldg,
-                                                           const int* __restrict__ kr, const double* __restrict__ scale,
-                                                           double2* __restrict__ sum,
-                                                           int V) {
-  const int r = blockIdx.y;
-  const size_t n12 = 12 * fx_padded(V), e = (size_t)blockIdx.x * blockDim.x + threadIdx.x, tk = e / kFxTile;
-  if (e >= n12) return;
-  const size_t site = tk / 12 * kFxTile + e % kFxTile;
-  if (site >= V) return;
-  const int4* B = basis + (size_t)r * nslots * n12 + n12 + e;
-  const int4* w = G + (size_t)r * ldg;
-  const int k = kr[r];
-  double re = 0.0, im = 0.0;
-  constexpr int K = REAL ? 16 : 8;  // products whose cross terms fit 63 bits
-  for (int i0 = 0; i0 < k; i0 += K) {
-    long long rh = 0, rx = kFxHalf30, ih = 0, ix = kFxHalf30;
-    const int n = min(K, k - i0);
-#pragma unroll 8
-    for (int i = 0; i < n; ++i) {
-      const int4 g = __ldg(w + i0 + i), x = __ldg(B + (size_t)(i0 + i) * n12);
+// Coefficients y = (z_j - T_k)^-1 e_1 ||b|| of every node, one thread per node:
+//   f_k = z - alpha_k,  f_i = z - alpha_i - beta_i^2 / f_{i+1};   y_1 = ||b|| / f_1,  y_{i+1} =
+//   beta_i y_i / f_{i+1}
+// (the factorisation from the last row up: |Im f_i| >= |Im z|).  Y[r][i][j] holds 1 / f, then y
+// / ||X_i||.  A chain of k reciprocals (0.2 us each) that took 25 us per source and node on
+// the host.
+__global__ void __launch_bounds__(32) fx_node_coef_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
+                                                          double2* __restrict__ Y) {
+  const int r = blockIdx.y, j = blockIdx.x * 32 + threadIdx.x;
+  if (j >= ns) return;
+  const SrcState* S = a.src + r;
+  const int mi = a.prm->max_iter, k = S->iter - 1;
+  const double *al = a.hist_a + (size_t)r * mi, *be = a.hist_b + (size_t)r * mi, *n2 = a.hist_n2 + (size_t)r * mi;
+  double2* y = Y + (size_t)r * mi * ns + j;
+  const double2 z = a.z[(size_t)r * ns + j];
+  double2 f = make_double2(0.0, 0.0);  // 1 / f_{i+1}
+#pragma unroll 4
+  for (int i = k - 1; i >= 0; --i) {
+    const double b = be[i], b2 = i + 1 < k ? b * b : 0.0;
+    const double dx = fma(-b2, f.x, z.x - al[i]), dy = fma(-b2, f.y, z.y);
+    const double inv = __drcp_rn(fma(dx, dx, dy * dy));
+    f = make_double2(dx * inv, -dy * inv);
+    y[(size_t)i * ns] = f;
+  }
+  double2 v = make_double2(S->bnorm, 0.0);
+#pragma unroll 4
+  for (int i = 0; i < k; ++i) {
+    const double2 g = y[(size_t)i * ns];
+    const double b = i > 0 ? be[i - 1] : 1.0, rn = rsqrt(n2[i]);
+    v = cmul(v, make_double2(b * g.x, b * g.y));
+    y[(size_t)i * ns] = make_double2(v.x * rn, v.y * rn);
+  }
+}
+
+// w[0..k) at stride `ld` as integers of at most 2^57 (out), k from the whole block; returns the
+// factor of sum_i w_i X_i given as hh + x 2^-30 = 2^-60 sum_i out_i X_i.  *real: all imaginary
+// parts vanish up to rounding.
+template <int NT, typename F>
+__device__ __forceinline__ double fx_quantise(F w, int k, int4* out, bool* real, int* sh) {
+  int mr = 0, mi = 0;  // high words of the largest |re|, |im|
+  for (int i = threadIdx.x; i < k; i += NT) {
+    const double2 v = w(i);
+    mr = max(mr, __double2hiint(v.x) & 0x7fffffff);
+    mi = max(mi, __double2hiint(v.y) & 0x7fffffff);
+  }
+  mr = block_max<NT>(mr, sh);
+  __syncthreads();
+  mi = block_max<NT>(mi, sh);
+  *real = __hiloint2double(mi, 0) <= 1e-14 * __hiloint2double(mr, 0);
+  const int m = max(mr, mi) >> 20, e = m > 0 && m < 0x7ff ? 56 - (m - 1023) : 56;
+  for (int i = threadIdx.x; i < k; i += NT) {
+    const double2 v = w(i);
+    const FX re = fx_split(__double2ll_rn(ldexp(v.x, e))), im = fx_split(__double2ll_rn(ldexp(v.y, e)));
+    out[i] = make_int4(re.hi, re.lo, im.hi, im.lo);
+  }
+  return ldexp(1.0, 60 - e);
+}
+
+struct FxSumInfo {
+  double scale;
+  int k, real;
+};
+
+// G[r][i] = sum_j c_j Y[r][i][j] (one block per source) in integers.  Real coefficients come
+// from a node list closed under conjugation (basis_sum_kernel).
+constexpr int kCoefNT = 512;
+__global__ void __launch_bounds__(kCoefNT) fx_sum_coef_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
+                                                              const double2* __restrict__ Y, double2* __restrict__ g,
+                                                              int4* __restrict__ G, FxSumInfo* __restrict__ info) {
+  __shared__ int sh[kCoefNT / 32];
+  const int r = blockIdx.x, mi = a.prm->max_iter, k = a.src[r].iter - 1;
+  const double2* c = a.c + (size_t)r * ns;
+  g += (size_t)r * mi;
+  // a warp per i: lanes over the nodes
+  for (int i = threadIdx.x >> 5; i < k; i += kCoefNT / 32) {
+    const double2* y = Y + ((size_t)r * mi + i) * ns;
+    double2 t = make_double2(0.0, 0.0);
+    for (int j = threadIdx.x & 31; j < ns; j += 32) {
+      const double2 v = cmul(c[j], y[j]);
+      t.x += v.x;
+      t.y += v.y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+      t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+    }
+    if ((threadIdx.x & 31) == 0) g[i] = t;
+  }
+  __syncthreads();
+  bool real;
+  const double sc = fx_quantise<kCoefNT>([&](int i) { return g[i]; }, k, G + (size_t)r * mi, &real, sh);
+  if (threadIdx.x == 0) info[r] = {sc, k, real ? 1 : 0};
+}
+
+// Yq[r][j][i] = Y[r][i][j] in integers, one block per (node, source)
+__global__ void __launch_bounds__(128) fx_node_quant_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
+                                                            const double2* __restrict__ Y, int4* __restrict__ Yq,
+                                                            double* __restrict__ scale) {
+  __shared__ int sh[128 / 32];
+  const int r = blockIdx.y, j = blockIdx.x, mi = a.prm->max_iter, k = a.src[r].iter - 1;
+  const double2* y = Y + (size_t)r * mi * ns + j;
+  bool real;
+  const size_t o = (size_t)r * ns + j;
+  const double sc = fx_quantise<128>([&](int i) { return y[(size_t)i * ns]; }, k, Yq + o * mi, &real, sh);
+  if (threadIdx.x == 0) scale[o] = sc;
+}
+
+// K basis vectors' products added exactly, the group's sum in FP64
+template <bool REAL, int K>
+__device__ __forceinline__ void fx_sum_group(const int4* __restrict__ w, const int4* __restrict__ B, size_t n12, int n,
+                                             double& re, double& im) {
+  long long rh = 0, rx = kFxHalf30, ih = 0, ix = kFxHalf30;
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
+    if (i < n) {
+      const int4 g = __ldg(w + i), x = __ldg(B + (size_t)i * n12);
       fx_mac(rh, rx, g.x, g.y, x.x, x.y);
       fx_mac(ih, ix, g.x, g.y, x.z, x.w);
       if (!REAL) {
@@ -1524,14 +1616,39 @@ __global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restric
         fx_mac(ih, ix, g.z, g.w, x.x, x.y);
       }
     }
-    re += (double)fx_value(rh, rx);
-    im += (double)fx_value(ih, ix);
   }
-  const double sc = scale[r];
+  re += (double)fx_value(rh, rx);
+  im += (double)fx_value(ih, ix);
+}
+
+// sum[r][e] += scale_r sum_i G_i X_i[e] (basis_sum_kernel in fixed point), G_i = g_i / ||X_i|| of
+// at most 2^57: groups of 8 products are summed exactly (their cross terms fit 63 bits), the
+// groups in FP64.  Reads 16 B per basis vector and element: HBM-bound.
+__global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restrict__ basis, int nslots,
+                                                           const int4* __restrict__ G, int ldg,
+                                                           const FxSumInfo* __restrict__ info,
+                                                           double2* __restrict__ sum, int V) {
+  const int r = blockIdx.y;
+  const size_t n12 = 12 * fx_padded(V), e = (size_t)blockIdx.x * blockDim.x + threadIdx.x, tk = e / kFxTile;
+  if (e >= n12) return;
+  const size_t site = tk / 12 * kFxTile + e % kFxTile;
+  if (site >= V) return;
+  const int4* B = basis + (size_t)r * nslots * n12 + n12 + e;
+  const int4* w = G + (size_t)r * ldg;
+  const FxSumInfo f = info[r];
+  constexpr int K = 8;
+  double re = 0.0, im = 0.0;
+  int i = 0;
+  if (f.real) {
+    for (; i + K <= f.k; i += K) fx_sum_group<true, K>(w + i, B + (size_t)i * n12, n12, K, re, im);
+  } else {
+    for (; i + K <= f.k; i += K) fx_sum_group<false, K>(w + i, B + (size_t)i * n12, n12, K, re, im);
+  }
+  if (i < f.k) fx_sum_group<false, K>(w + i, B + (size_t)i * n12, n12, f.k - i, re, im);
   double2* so = sum + ((size_t)r * 12 + tk % 12) * V + site;
   double2 sv = *so;
-  sv.x = fma(sc, re, sv.x);
-  sv.y = fma(sc, im, sv.y);
+  sv.x = fma(f.scale, re, sv.x);
+  sv.y = fma(f.scale, im, sv.y);
   *so = sv;
 }
 
@@ -1541,9 +1658,8 @@ template <int JT>
 __global__ void __launch_bounds__(256) fx_basis_nodes_kernel(const int4* __restrict__ basis, int nslots,
                                                              const int4* __restrict__ Y,
                                                              const double* __restrict__ scale, int ns, int ldy,
-                                                             const int* __restrict__ kr, int j0, int nc,
-                                                             double2* __restrict__ X,
-                                                             int V) {
+                                                             const FxSumInfo* __restrict__ info, int j0, int nc,
+                                                             double2* __restrict__ X, int V) {
   const int r = blockIdx.y, jt = blockIdx.z * JT;
   const size_t n12 = 12 * fx_padded(V), e = (size_t)blockIdx.x * blockDim.x + threadIdx.x, tk = e / kFxTile;
   if (e >= n12 || jt >= nc) return;
@@ -1551,7 +1667,7 @@ __global__ void __launch_bounds__(256) fx_basis_nodes_kernel(const int4* __restr
   if (site >= V) return;
   const int4* B = basis + (size_t)r * nslots * n12 + n12 + e;
   const int4* Yr = Y + ((size_t)r * ns + j0 + jt) * ldy;
-  const int k = kr[r], nj = min(JT, nc - jt);
+  const int k = info[r].k, nj = min(JT, nc - jt);
   double re[JT], im[JT];
 #pragma unroll
   for (int t = 0; t < JT; ++t) re[t] = im[t] = 0.0;
@@ -1944,8 +2060,6 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
 template <typename R>
 int run_coop(ov_ctx* ctx, SolveWs<R>& w, int nsrc, cudaStream_t s, double* launches) {
   if (nsrc > kCoopMaxSrc || ctx->no_coop) return OV_ERR_INVALID_ARG;
-  if constexpr (std::is_same<R, FX>::value) return OV_ERR_INVALID_ARG;  // not reached: FP64 then
-  else {
   int dev = 0, coop = 0, nsm = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
@@ -1972,7 +2086,6 @@ int run_coop(ov_ctx* ctx, SolveWs<R>& w, int nsrc, cudaStream_t s, double* launc
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "cudaLaunchCooperativeKernel");
   *launches += 1.0;
   return OV_OK;
-  }
 }
 
 template <typename R>
@@ -2150,20 +2263,6 @@ static void fom_coefficients(const double* al, const double* be, int k, double b
   for (int i = k - 2; i >= 0; --i) yy[i] = sc.zt[i] - sc.ll[i] * yy[i + 1];
 }
 
-// Coefficients w[0..k) as fixed-point integers of at most 2^57 in out; returns the factor
-// of sum_i w_i X_i, given as (hh + x 2^-30) = 2^-60 sum_i out_i X_i.
-static double fx_coefficients(const std::complex<double>* w, int k, int4* out) {
-  double mx = 0.0;
-  for (int i = 0; i < k; ++i) mx = std::max(mx, std::max(std::fabs(w[i].real()), std::fabs(w[i].imag())));
-  if (!(mx > 0.0) || !std::isfinite(mx)) mx = 1.0;
-  const int e = 56 - std::ilogb(mx);
-  for (int i = 0; i < k; ++i) {
-    const FX re = fx_split(std::llrint(std::ldexp(w[i].real(), e))), im = fx_split(std::llrint(std::ldexp(w[i].imag(), e)));
-    out[i] = make_int4(re.hi, re.lo, im.hi, im.lo);
-  }
-  return std::ldexp(1.0, 60 - e);
-}
-
 // g = sum_j c_j (z_j - T_k)^-1 e_1 ||b|| per source, from the recorded alpha (ha) and beta
 // (hb), leading dimension ld.
 static void lanczos_sum_coefficients(const ov_ctx* ctx, int nsrc, const std::vector<int>& kr,
@@ -2191,10 +2290,9 @@ static void lanczos_sum_coefficients(const ov_ctx* ctx, int nsrc, const std::vec
 // Stored-basis form of OV_MODE_FP64_2PASS: pass 1 keeps U_1 .. U_k (slot i), then
 // s = c0 b + sum_i (g_i / ||U_i||) U_i in one read of the basis.
 template <typename R>
-static int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int nsrc,
+int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int nsrc,
                              const ov_solve_opts& o, SolveOut* so, cudaStream_t s, int cap) {
   NvtxRange nvtx_("solve: stored basis");
-  constexpr bool kFix = std::is_same<R, FX>::value;
   const int ns = (int)ctx->z.size();
   const size_t n12 = (size_t)12 * ctx->g.V;
   SolveWs<R> w;
@@ -2222,9 +2320,6 @@ static int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa
   cudaError_t e = cudaMemcpyAsync(S.data(), w.a.src, sizeof(SrcState) * nsrc, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ha.data(), w.a.hist_a, sizeof(double) * ha.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hb.data(), w.a.hist_b, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, s);
-  std::vector<double> hn(kFix ? ha.size() : 0);  // fixed point: ||X_i||^2
-  if (kFix && e == cudaSuccess)
-    e = cudaMemcpyAsync(hn.data(), w.a.hist_n2, sizeof(double) * hn.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "read Lanczos history");
   std::vector<int> kr(nsrc);
@@ -2237,7 +2332,7 @@ static int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa
   lanczos_sum_coefficients(ctx, nsrc, kr, bn, ha, hb, cap, g);
   for (int r = 0; r < nsrc; ++r)
     for (int i = 0; i < kr[r]; ++i) {  // fold in 1 / ||U_i||
-      const double ni = kFix ? std::sqrt(hn[(size_t)r * cap + i]) : (i == 0) ? bn[r] : hb[(size_t)r * cap + i - 1];
+      const double ni = (i == 0) ? bn[r] : hb[(size_t)r * cap + i - 1];
       g[(size_t)r * cap + i].x /= ni;
       g[(size_t)r * cap + i].y /= ni;
     }
@@ -2255,45 +2350,96 @@ static int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa
   }
   using T = typename Store<R>::T;
   std::vector<T> gs(g.size());
-  std::vector<double> gsc(nsrc, 1.0);
-  if constexpr (kFix) {
-    std::vector<std::complex<double>> gr;
-    for (int r = 0; r < nsrc; ++r) {
-      gr.resize(kr[r]);
-      for (int i = 0; i < kr[r]; ++i) gr[i] = {g[(size_t)r * cap + i].x, g[(size_t)r * cap + i].y};
-      gsc[r] = fx_coefficients(gr.data(), kr[r], gs.data() + (size_t)r * cap);
-    }
-  } else {
-    for (size_t t = 0; t < g.size(); ++t) gs[t] = host_store(g[t], (T*)nullptr);
-  }
+  for (size_t t = 0; t < g.size(); ++t) gs[t] = host_store(g[t], (T*)nullptr);
   T* gd = (T*)ws_get(ctx, (tag + ".g").c_str(), sizeof(T) * gs.size(), &st);
   int* krd = (int*)ws_get(ctx, (tag + ".kr").c_str(), sizeof(int) * nsrc, &st);
-  double* gscd = kFix ? (double*)ws_get(ctx, (tag + ".gsc").c_str(), sizeof(double) * nsrc, &st) : nullptr;
   if (st != OV_OK) return st;
   e = cudaMemcpyAsync(gd, gs.data(), sizeof(T) * gs.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(krd, kr.data(), sizeof(int) * nsrc, cudaMemcpyHostToDevice, s);
-  if (kFix && e == cudaSuccess)
-    e = cudaMemcpyAsync(gscd, gsc.data(), sizeof(double) * nsrc, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy coefficients");
   cudaEvent_t ev;
   kt_begin(ctx, KC_BASIS_SUM, s, &ev);
-  const dim3 gsum((unsigned)((w.nvec + 255) / 256), nsrc);
-  if constexpr (kFix) {
-    if (real)
-      fx_basis_sum_kernel<true><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, gscd, w.a.sacc, ctx->g.V);
-    else
-      fx_basis_sum_kernel<false><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, gscd, w.a.sacc, ctx->g.V);
-  } else if (real) {
+  const dim3 gsum((unsigned)((n12 + 255) / 256), nsrc);
+  if (real)
     basis_sum_kernel<R, true><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, w.a.sacc, n12);
-  } else {
+  else
     basis_sum_kernel<R, false><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, w.a.sacc, n12);
-  }
   kt_end(ctx, KC_BASIS_SUM, s, ev);
   OV_CHECK_LAUNCH(ctx, "basis_sum_kernel");
   so->launches = launches + 3.0;
   e = cudaMemcpyAsync(out_soa, w.a.sacc, sizeof(double2) * n12 * nsrc, cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy sum");
   return fst;
+}
+
+// Device workspace of the fixed-point coefficients.
+struct FxCoef {
+  double2 *Y = nullptr, *g = nullptr;
+  int4* G = nullptr;
+  FxSumInfo* info = nullptr;
+};
+
+// The Lanczos pass of the fixed-point forms, then (enqueued, no host read between) every node's
+// coefficients and the integer coefficients of the weighted sum.
+static int fx_lanczos(ov_ctx* ctx, SolveWs<FX>& w, FxCoef& f, const double2* b_soa, int nsrc, int ns,
+                      const std::vector<double2>& zh, const std::vector<double2>& ch, double2 c0, double2* sums,
+                      const ov_solve_opts& o, cudaStream_t s, int cap, int flavour, double* launches) {
+  int st = setup_ws<FX>(ctx, nsrc, ns, false, false, true, cap, &w, "fxs", cap + 3, false);
+  if (st != OV_OK) return st;
+  f.Y = (double2*)ws_get(ctx, "fxs.Y", sizeof(double2) * (size_t)nsrc * cap * ns, &st);
+  f.g = (double2*)ws_get(ctx, "fxs.gd", sizeof(double2) * (size_t)nsrc * cap, &st);
+  f.G = (int4*)ws_get(ctx, "fxs.g", sizeof(int4) * (size_t)nsrc * cap, &st);
+  f.info = (FxSumInfo*)ws_get(ctx, "fxs.info", sizeof(FxSumInfo) * nsrc, &st);
+  if (st != OV_OK) return st;
+  w.a.sacc = sums;  // c0 b, written by the init kernel only
+  st = init_solve<FX>(ctx, w, b_soa, nsrc, ns, zh, ch, c0, o.tol, cap, s, 0);
+  w.a.sacc = nullptr;
+  if (st != OV_OK) return st;
+  *launches = 2.0;
+  st = run_iterations<FX>(ctx, w, nsrc, ns, flavour, cap, o, s, launches);
+  if (st != OV_OK) return st;
+  cudaEvent_t ev;
+  kt_begin(ctx, KC_MISC, s, &ev);
+  fx_node_coef_kernel<<<dim3((ns + 31) / 32, nsrc), 32, 0, s>>>(w.a, ns, f.Y);
+  fx_sum_coef_kernel<<<nsrc, kCoefNT, 0, s>>>(w.a, ns, f.Y, f.g, f.G, f.info);
+  kt_end(ctx, KC_MISC, s, ev);
+  OV_CHECK_LAUNCH(ctx, "fx_node_coef_kernel");
+  *launches += 2.0;
+  return OV_OK;
+}
+
+static int launch_fx_basis_sum(ov_ctx* ctx, const SolveWs<FX>& w, const FxCoef& f, int nsrc, int cap, double2* sums,
+                               cudaStream_t s) {
+  cudaEvent_t ev;
+  kt_begin(ctx, KC_BASIS_SUM, s, &ev);
+  fx_basis_sum_kernel<<<dim3((unsigned)((w.nvec + 255) / 256), nsrc), 256, 0, s>>>(w.a.ring, cap + 3, f.G, cap, f.info,
+                                                                                sums, ctx->g.V);
+  kt_end(ctx, KC_BASIS_SUM, s, ev);
+  OV_CHECK_LAUNCH(ctx, "fx_basis_sum_kernel");
+  return OV_OK;
+}
+
+// solve_sign_stored in fixed point: the sum goes straight to out_soa, and the host waits for
+// the device once, at the end.
+template <>
+int solve_sign_stored<FX>(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int nsrc, const ov_solve_opts& o,
+                          SolveOut* so, cudaStream_t s, int cap) {
+  NvtxRange nvtx_("solve: stored basis, fixed point");
+  const int ns = (int)ctx->z.size();
+  std::vector<double2> zh, ch;
+  for (int r = 0; r < nsrc; ++r) {
+    zh.insert(zh.end(), ctx->z.begin(), ctx->z.end());
+    ch.insert(ch.end(), ctx->c.begin(), ctx->c.end());
+  }
+  SolveWs<FX> w;
+  FxCoef f;
+  double launches = 0.0;
+  int st = fx_lanczos(ctx, w, f, b_soa, nsrc, ns, zh, ch, ctx->c0, out_soa, o, s, cap, 6, &launches);
+  if (st == OV_OK) st = launch_fx_basis_sum(ctx, w, f, nsrc, cap, out_soa, s);
+  if (st != OV_OK) return st;
+  st = finish_solve<FX>(ctx, w, nsrc, ns, zh, ch, so, s);
+  so->launches = launches + 3.0;
+  return st;
 }
 
 // OV_MODE_FP64_2PASS.  Pass 1: the Lanczos process with every node's LDL^T scalar
@@ -2513,10 +2659,9 @@ static int solve_sign_regen(ov_ctx* ctx, const double2* b_soa, double2* out_soa,
 // work does not repeat per chunk.  Returns OV_ERR_INVALID_ARG when the basis does not fit
 // the store budget or the solve outgrows it (the caller uses the vector-space form).
 template <typename R>
-static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
+int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
                       const std::vector<double2>& ch, int chunk, double2* X, double2* sums, const ov_solve_opts& o,
                       SolveOut* so, cudaStream_t s, const std::function<int(int, int)>& per_chunk) {
-  constexpr bool kFix = std::is_same<R, FX>::value;
   const size_t n12 = (size_t)12 * ctx->g.V;
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
@@ -2541,9 +2686,6 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
   cudaError_t e = cudaMemcpyAsync(S.data(), w.a.src, sizeof(SrcState) * nsrc, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ha.data(), w.a.hist_a, sizeof(double) * ha.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hb.data(), w.a.hist_b, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, s);
-  std::vector<double> hn(kFix ? ha.size() : 0);  // fixed point: ||X_i||^2
-  if (kFix && e == cudaSuccess)
-    e = cudaMemcpyAsync(hn.data(), w.a.hist_n2, sizeof(double) * hn.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "read Lanczos history");
   // FOM coefficients y^j = (z_j - T_k)^-1 e_1 ||b|| per source and node (forward LDL^T sweep,
@@ -2552,7 +2694,6 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
   std::vector<T> Yh((size_t)nsrc * ns * cap);
   std::vector<T> gh((size_t)nsrc * cap);
   std::vector<int> kr(nsrc);
-  std::vector<double> Ysc((size_t)nsrc * ns, 1.0), gsc(nsrc, 1.0);  // fixed point: factors of the sums
   FomScratch sc;
   std::vector<std::complex<double>> yy, gs;
   for (int r = 0; r < nsrc; ++r) {
@@ -2565,31 +2706,18 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
       const std::complex<double> cj(ch[(size_t)r * ns + j].x, ch[(size_t)r * ns + j].y);
       fom_coefficients(al, be, k, S[r].bnorm, zj, sc, yy);
       for (int i = 0; i < k; ++i) {
-        const double ni = kFix ? std::sqrt(hn[(size_t)r * cap + i]) : (i == 0) ? S[r].bnorm : be[i - 1];
-        yy[i] /= ni;
-        if constexpr (!kFix)
-          Yh[((size_t)r * ns + j) * cap + i] = host_store(make_double2(yy[i].real(), yy[i].imag()), (T*)nullptr);
-        gs[i] += cj * yy[i];
+        const double ni = (i == 0) ? S[r].bnorm : be[i - 1];
+        const std::complex<double> y = yy[i] / ni;
+        Yh[((size_t)r * ns + j) * cap + i] = host_store(make_double2(y.real(), y.imag()), (T*)nullptr);
+        gs[i] += cj * y;
       }
-      if constexpr (kFix)
-        Ysc[(size_t)r * ns + j] = fx_coefficients(yy.data(), k, Yh.data() + ((size_t)r * ns + j) * cap);
     }
-    if constexpr (kFix)
-      gsc[r] = fx_coefficients(gs.data(), k, gh.data() + (size_t)r * cap);
-    else
-      for (int i = 0; i < k; ++i) gh[(size_t)r * cap + i] = host_store(make_double2(gs[i].real(), gs[i].imag()), (T*)nullptr);
+    for (int i = 0; i < k; ++i) gh[(size_t)r * cap + i] = host_store(make_double2(gs[i].real(), gs[i].imag()), (T*)nullptr);
   }
   T* Yd = (T*)ws_get(ctx, (tag + ".Y").c_str(), sizeof(T) * Yh.size(), &st);
   T* gd = (T*)ws_get(ctx, (tag + ".g").c_str(), sizeof(T) * gh.size(), &st);
   int* krd = (int*)ws_get(ctx, (tag + ".kr").c_str(), sizeof(int) * nsrc, &st);
-  double* Yscd = kFix ? (double*)ws_get(ctx, (tag + ".Ysc").c_str(), sizeof(double) * Ysc.size(), &st) : nullptr;
-  double* gscd = kFix ? (double*)ws_get(ctx, (tag + ".gsc").c_str(), sizeof(double) * nsrc, &st) : nullptr;
   if (st != OV_OK) return st;
-  if (kFix) {
-    e = cudaMemcpyAsync(Yscd, Ysc.data(), sizeof(double) * Ysc.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(gscd, gsc.data(), sizeof(double) * nsrc, cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy coefficient scales");
-  }
   e = cudaMemcpyAsync(Yd, Yh.data(), sizeof(T) * Yh.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(gd, gh.data(), sizeof(T) * gh.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(krd, kr.data(), sizeof(int) * nsrc, cudaMemcpyHostToDevice, s);
@@ -2597,22 +2725,51 @@ static int nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy node coefficients");
   cudaEvent_t ev;
   kt_begin(ctx, KC_BASIS_SUM, s, &ev);
-  const dim3 gsum((unsigned)((w.nvec + 255) / 256), nsrc);
-  if constexpr (kFix)
-    fx_basis_sum_kernel<false><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, gscd, sums, ctx->g.V);
-  else
-    basis_sum_kernel<R><<<gsum, 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd, sums, n12);
+  basis_sum_kernel<R><<<dim3((unsigned)((n12 + 255) / 256), nsrc), 256, 0, s>>>(w.a.ring, cap + 3, gd, cap, krd,
+                                                                             sums, n12);
   kt_end(ctx, KC_BASIS_SUM, s, ev);
   OV_CHECK_LAUNCH(ctx, "basis_sum_kernel");
-  constexpr int JT = kFix ? 4 : 8;
+  constexpr int JT = 8;
   for (int j0 = 0; j0 < ns; j0 += chunk) {
     const int nc = std::min(chunk, ns - j0);
-    const dim3 gn((unsigned)((w.nvec + 255) / 256), nsrc, (nc + JT - 1) / JT);
-    if constexpr (kFix)
-      fx_basis_nodes_kernel<JT><<<gn, 256, 0, s>>>(w.a.ring, cap + 3, Yd, Yscd, ns, cap, krd, j0, nc, X, ctx->g.V);
-    else
-      basis_nodes_kernel<R, JT><<<gn, 256, 0, s>>>(w.a.ring, cap + 3, Yd, ns, cap, krd, j0, nc, X, n12);
+    const dim3 gn((unsigned)((n12 + 255) / 256), nsrc, (nc + JT - 1) / JT);
+    basis_nodes_kernel<R, JT><<<gn, 256, 0, s>>>(w.a.ring, cap + 3, Yd, ns, cap, krd, j0, nc, X, n12);
     OV_CHECK_LAUNCH(ctx, "basis_nodes_kernel");
+    if ((st = per_chunk(j0, nc)) != OV_OK) return st;
+  }
+  so->launches = launches + 2.0 + (ns + chunk - 1) / chunk;
+  if (so->converged) ctx->coef_iter_hint = so->iterations;
+  return fst;
+}
+
+template <>
+int nodes_coef<FX>(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
+                   const std::vector<double2>& ch, int chunk, double2* X, double2* sums, const ov_solve_opts& o,
+                   SolveOut* so, cudaStream_t s, const std::function<int(int, int)>& per_chunk) {
+  size_t freeb = 0, totalb = 0;
+  cudaMemGetInfo(&freeb, &totalb);
+  auto it = ctx->bufs.find("fxs.ring");
+  const double held = it != ctx->bufs.end() ? (double)it->second.bytes : 0.0;
+  const double budget = std::min(0.40 * (double)totalb, (double)freeb + held - 0.10 * (double)totalb);
+  const int cap = std::min(o.max_iter, ctx->coef_iter_hint > 0 ? std::max(64, ctx->coef_iter_hint * 5 / 4 + 32) : 1024);
+  if ((double)(cap + 3) * nsrc * vec_elems<FX>(ctx->g.V) * sizeof(int4) > budget) return OV_ERR_INVALID_ARG;
+  SolveWs<FX> w;
+  FxCoef f;
+  double launches = 0.0;
+  int st = fx_lanczos(ctx, w, f, b_soa, nsrc, ns, zh, ch, make_double2(0.0, 0.0), sums, o, s, cap, 7, &launches);
+  int4* Yq = (int4*)ws_get(ctx, "fxs.Yq", sizeof(int4) * (size_t)nsrc * ns * cap, &st);
+  double* Ysc = (double*)ws_get(ctx, "fxs.Ysc", sizeof(double) * (size_t)nsrc * ns, &st);
+  if (st == OV_OK) st = launch_fx_basis_sum(ctx, w, f, nsrc, cap, sums, s);
+  if (st != OV_OK) return st;
+  const int fst = finish_solve<FX>(ctx, w, nsrc, ns, zh, ch, so, s);
+  if (fst != OV_OK && !(fst == OV_ERR_NOT_CONVERGED && cap >= o.max_iter)) return OV_ERR_INVALID_ARG;
+  fx_node_quant_kernel<<<dim3(ns, nsrc), 128, 0, s>>>(w.a, ns, f.Y, Yq, Ysc);
+  constexpr int JT = 4;
+  for (int j0 = 0; j0 < ns; j0 += chunk) {
+    const int nc = std::min(chunk, ns - j0);
+    fx_basis_nodes_kernel<JT><<<dim3((unsigned)((w.nvec + 255) / 256), nsrc, (nc + JT - 1) / JT), 256, 0, s>>>(
+        w.a.ring, cap + 3, Yq, Ysc, ns, cap, f.info, j0, nc, X, ctx->g.V);
+    OV_CHECK_LAUNCH(ctx, "fx_basis_nodes_kernel");
     if ((st = per_chunk(j0, nc)) != OV_OK) return st;
   }
   so->launches = launches + 2.0 + (ns + chunk - 1) / chunk;
