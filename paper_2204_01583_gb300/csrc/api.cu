@@ -107,6 +107,7 @@ void ws_release_all(ov_ctx* ctx) {
 void graphs_release(ov_ctx* ctx) {
   for (auto& kv : ctx->graphs) cudaGraphExecDestroy(kv.second);
   ctx->graphs.clear();
+  ctx->graph_launches.clear();
 }
 
 void kt_begin(ov_ctx* ctx, int cls, cudaStream_t s, cudaEvent_t* a) {

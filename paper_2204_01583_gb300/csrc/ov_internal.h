@@ -134,6 +134,7 @@ struct ov_ctx {
   std::vector<cudaStream_t> aux_streams;  // extra capture branches (source groups)
   std::vector<cudaEvent_t> cap_events;    // fork/join events of those branches
   std::map<GraphKey, cudaGraphExec_t> graphs;
+  std::map<GraphKey, double> graph_launches;  // kernels in one replay
 
   // kernel timing
   bool timing = false;

@@ -59,6 +59,13 @@ constexpr int k1_min_blocks() { return std::is_same<R, DF>::value ? 7 : 4; }
 template <typename R>
 constexpr bool kHalvedLinks = std::is_same<R, double>::value || std::is_same<R, DF>::value;
 
+// Fixed point: what the kernels of iteration i know of X_i.
+struct FxVec {
+  double n2, inv_n2;  // ||X_i||^2 in integer units and its reciprocal
+  FX dia, gam;        // coefficients of X_i and X_{i-1} in w, unit 2^-60
+  int q;              // w = (H X_i / 4) 2^-q - ...
+};
+
 struct SrcState {
   double bnorm;   // ||b||
   double inv_b2;  // 1 / ||b||^2
@@ -77,11 +84,12 @@ struct SrcState {
   double cm;      // ||U_i|| / ||U_{i-1}|| (0 at i = 1)
   double alpha_n; // alpha_i / ||U_i||: U_{i+1} = w - alpha_n U_i in one FMA per real
   float df[8];    // inv_n, cm, alpha, alpha_n as double-float (hi, lo) pairs
-  // fixed-point vectors X_i (solve_sign_stored<FX>); U_i = X_i up to a power of two
-  double n2, inv_n2;  // ||X_i||^2 in integer units and its reciprocal
-  FX dia, gam, alf;   // coefficients of X_i and X_{i-1} in w, of X_i in X_{i+1}; unit 2^-60
-  int q, k;           // w = (H X_i / 4 - ...) 2^-q;  X_{i+1} = (w - ...) 2^k
-  int e_in;           // X_1 = b 2^e_in
+  // fixed-point vectors X_i (fx_* kernels); U_i = X_i up to a power of two
+  FxVec vec[2];  // of X_i in slot i & 1: written by K1 of iteration i, read by K2 and the next K1
+  int k[2];      // X_{i+1} = (w - a X_i) 2^k, k in slot i & 1: written by K2, read by the next K1
+  int it1, it2;  // iteration K1 last ran, 0: none left to run (read by K2); iteration K1 runs
+                 // next (written by K2)
+  int e_in;      // X_1 = b 2^e_in
 };
 
 // exact double-float split of an FP64 value: hi = rn(x), lo = rn(x - hi)
@@ -182,7 +190,7 @@ struct SolveArgs {
   typename Coef<R>::T* act_z;   // [src][nshift] zeta_i
   double* part1;      // [src][nblk1]
   double* part2;      // [src][nblk2]
-  long long* bins1;   // [src][kFxBins][kFxWords] fixed point: sums of K1 and of K2
+  long long* bins1;   // [src][2][kFxBins][kFxWords] fixed point: sums of K1 and of K2, slot i & 1
   long long* bins2;
   unsigned* cnt;      // [src][2]
   int* done_count;
@@ -1155,21 +1163,73 @@ __device__ __forceinline__ int block_max(int v, int* sh) {
 }
 
 // Sums over a source: integers, so that atomic additions in any order give the same result.
-// Blocks add into kFxBins bins (fewer collisions per address); the last block to arrive
-// (last_arrival) adds the bins up and clears them for the next launch.
+// Blocks add into kFxBins bins (fewer collisions per address).  No block waits for the others:
+// every block of the next kernel adds the bins up and forms the iteration's scalars itself,
+// beside its first loads (an arrival counter, a last block's serial FP64 chain and its
+// state writes took 10 us of an iteration's 21 at 8^4).  Block 0 records them.  Two slots, by
+// the iteration's parity: the reader's block 0 clears the other one.
 constexpr int kFxBins = 32;
 constexpr int kFxWords = 6;  // K1: five words of <X, w> and the maximum; K2: four words
-__device__ __forceinline__ bool last_arrival(unsigned* cnt, unsigned n) {
-  __threadfence();
-  if (atomicAdd(cnt, 1u) != n - 1) return false;
-  *cnt = 0;
-  __threadfence();
-  return true;
+__device__ __forceinline__ long long* fx_bins(long long* bins, int r, int i) {
+  return bins + (size_t)(2 * r + (i & 1)) * kFxBins * kFxWords;
 }
 __device__ __forceinline__ long long warp_sum(long long v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// The scalars of X_i (i >= 2) from ||X_i||^2 (K2's bins of iteration i - 1); a whole warp.
+// *beta: beta_{i-1}, *tot: ||X_i||^2.
+__device__ __forceinline__ FxVec fx_vec(const SolveArgs<FX>& a, const SrcState* S, int r, int i, double* beta) {
+  const long long* bins = fx_bins(a.bins2, r, i - 1) + (threadIdx.x & 31) * kFxWords;
+  long long n[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) n[j] = warp_sum(__ldcg(bins + j));
+  const FxVec p = S->vec[(i - 1) & 1];
+  const int sh = p.q - S->k[(i - 1) & 1];
+  FxVec v;
+  v.n2 = fma((double)n[0], pow2(92), (double)n[1] * pow2(60)) + fma((double)n[2], pow2(38), (double)n[3] * 256.0);
+  v.inv_n2 = __drcp_rn(v.n2);
+  const double ratio = v.n2 * p.inv_n2;    // ||X_i||^2 / ||X_{i-1}||^2
+  *beta = sqrt(ratio) * pow2(2 + sh);
+  const double g1 = ratio * pow2(sh);      // beta_{i-1} ||X_i|| / (4 ||X_{i-1}||)
+  v.q = max(0, exponent_of(g1));           // g1 2^-q < 2
+  v.gam = fx_split(-__double2ll_rn(g1 * pow2(60 - v.q)));
+  v.dia = fx_split(__double2ll_rn(a.diag4 * pow2(60 - v.q)));
+  return v;
+}
+
+// The start of an iteration by one warp: the scalars of X_i, recorded by the one warp that has
+// `record` set.  Returns true when no iteration is left to run.
+__device__ __forceinline__ bool fx_begin(const SolveArgs<FX>& a, SrcState* S, int r, int i, bool record, FxVec* out) {
+  const int lane = threadIdx.x & 31, mi = a.prm->max_iter;
+  double beta = 1.0;
+  const FxVec v = i > 1 ? fx_vec(a, S, r, i, &beta) : S->vec[1];
+  const bool end = beta == 0.0 || i > mi;
+  *out = v;
+  if (!record) return end;
+  long long* z = fx_bins(a.bins2, r, i) + lane * kFxWords;
+#pragma unroll
+  for (int k = 0; k < kFxWords; ++k) z[k] = 0;
+  if (lane == 0) {
+    if (i > 1) {
+      S->vec[i & 1] = v;
+      a.hist_b[(size_t)r * mi + i - 2] = beta;
+      if (i <= mi) a.hist_n2[(size_t)r * mi + i - 1] = v.n2;
+    }
+    __threadfence();  // a check running beside this reads the history once it1 is 0
+    *(volatile int*)&S->it1 = end ? 0 : i;
+  }
+  return end;
+}
+
+// fx_begin ahead of K1 for grids of many blocks (one warp per source)
+__global__ void __launch_bounds__(32) fx_begin_kernel(const __grid_constant__ SolveArgs<FX> a) {
+  SrcState* S = a.src + blockIdx.x;
+  if (__any_sync(0xffffffffu, S->done)) return;
+  FxVec v;
+  fx_begin(a, S, blockIdx.x, S->it2, true, &v);
 }
 
 // A block takes one 32-site tile of `per` sources in turn (their links then come from L1).
@@ -1177,34 +1237,58 @@ __device__ __forceinline__ long long warp_sum(long long v) {
 // for the hops and 430 for the rest, half of the time) and the L2 latency of the neighbour
 // loads.  One source at 16^3 x 32: 63 us, where the FP64 kernel takes 227 us and the
 // double-float one 66 us; 6 sources in one launch: 6 x 45 us (links from L1).  4 blocks per
-// SM (64 registers): 375 ms per 12-source FP64 solve, 393 ms at 3.
-__global__ void __launch_bounds__(kFxNT, 4) fx_lanczos_hw_kernel(const __grid_constant__ SolveArgs<FX> a,
-                                                                 int nsrc, int per) {
+// SM (64 registers): 375 ms per 12-source FP64 solve, 393 ms at 3.  NT = 288, for small grids
+// where nothing else covers it: a ninth warp forms the scalars while the others run phase 1
+// (8^4, 4 sources: 8.0 -> 6.5 ms per solve against a last block's serial end); NT = 256: from
+// fx_begin_kernel (formed in every block, 16^3 x 32 took 374 ms instead of 366).
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == kFxNT ? 4 : 3) fx_lanczos_hw_kernel(const __grid_constant__ SolveArgs<FX> a,
+                                                                                int nsrc, int per) {
   __shared__ int red[kFxNT / 32][kFxWords];
+  __shared__ FxVec vec;
+  __shared__ int stop;
   __shared__ longlong2 sm[4 * 12 * kFxTile];
   const int V = a.g.V;
   const int nb = (V + kFxTile - 1) / kFxTile, ng = gridDim.x / nb;
   const int tb = blockIdx.x / ng, r0 = blockIdx.x % ng * per;
   const size_t n12 = 12 * fx_padded(V);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int s = tb * kFxTile + lane;  
+  const int s = tb * kFxTile + lane;
   const bool in = s < V;
-  const FxHops nbr = fx_hops(a.g, in ? s : 0, wid >> 1);
+  const FxHops nbr = fx_hops(a.g, in ? s : 0, (wid >> 1) & 3);
   for (int r = r0; r < min(nsrc, r0 + per); ++r) {
     SrcState* S = a.src + r;
-    if (S->done) continue;
-    const int i = S->iter, q = S->q;
+    // the check of earlier iterations may set `done` while this runs: one answer per block
+    if (__syncthreads_or(S->done)) continue;
+    const int i = S->it2, mi = a.prm->max_iter;
     int4* base = a.ring + (size_t)r * a.prm->nslots * n12;
     const int4* Xi = base + (size_t)i * n12;  // stored basis: slot i holds X_i
-    if (in) fx_phase1(Xi, a.U, wid, s, nbr, sm + (wid >> 1) * 12 * kFxTile + lane);
+    if (NT > kFxNT && wid == kFxNT / 32) {
+      FxVec v;
+      const bool end = fx_begin(a, S, r, i, tb == 0, &v);
+      if (lane == 0) {
+        vec = v;
+        stop = end;
+      }
+    }
+    if (NT == kFxNT && threadIdx.x == 0) {
+      vec = S->vec[i & 1];
+      stop = S->it1 == 0;
+    }
+    if (in && i <= mi && wid < kFxNT / 32) fx_phase1(Xi, a.U, wid, s, nbr, sm + (wid >> 1) * 12 * kFxTile + lane);
     __syncthreads();
+    if (stop) {
+      __syncthreads();
+      continue;
+    }
     // <X_i, w> = hh 2^62 + x1 2^30 + x2 2^32, w = wh 2^32 + wl with signed wl
     long long hh = 0, x1 = 0, x2 = 0;
     int wmax = 0;
     if (in && wid < 6) {  // components 2 wid, 2 wid + 1
+      const int q = vec.q;
       const bool low = wid >= 3;
       // 2^-q diag / 4 x - gam X_{i-1} = (hh 2^60 + x 2^30) / 2^60; gamma5 = -1 on the lower spins
-      const FX dg = S->dia, nd = FX{low ? -dg.hi : dg.hi, low ? -dg.lo : dg.lo}, ng = S->gam;
+      const FX dg = vec.dia, nd = FX{low ? -dg.hi : dg.hi, low ? -dg.lo : dg.lo}, ngm = vec.gam;
       const int4* xp = Xi + fx_index(s, 12) + 2 * wid * kFxTile;
       longlong2* wp = reinterpret_cast<longlong2*>(const_cast<int4*>(xp + n12));
       int4 xb[2], ub[2];
@@ -1227,7 +1311,7 @@ __global__ void __launch_bounds__(kFxNT, 4) fx_lanczos_hw_kernel(const __grid_co
         for (int c = 0; c < 2; ++c) {
           long long gh = w[c], gx = kFxHalf30;
           fx_mac(gh, gx, nd.hi, nd.lo, xv[2 * c], xv[2 * c + 1]);
-          fx_mac(gh, gx, ng.hi, ng.lo, uv[2 * c], uv[2 * c + 1]);
+          fx_mac(gh, gx, ngm.hi, ngm.lo, uv[2 * c], uv[2 * c + 1]);
           w[c] = fx_value(gh, gx);
           const int wl = (int)w[c], wh = (int)(w[c] >> 32) + (int)((unsigned)wl >> 31);
           hh += (long long)xv[2 * c] * wh;
@@ -1243,7 +1327,7 @@ __global__ void __launch_bounds__(kFxNT, 4) fx_lanczos_hw_kernel(const __grid_co
     }
     // warp sums in words that cannot overflow 32 lanes: hh in 26 + 26 + 12 bits, the cross
     // terms (below 2^-30 of hh's weight, kept to 2^-47) in 24 + 24
-    {
+    if (wid < 6) {
       const long long xs = (x2 + (x1 >> 2)) >> 16;
       int v[kFxWords];
       v[0] = __reduce_add_sync(0xffffffffu, (int)(hh & 0x3ffffff));
@@ -1257,76 +1341,85 @@ __global__ void __launch_bounds__(kFxNT, 4) fx_lanczos_hw_kernel(const __grid_co
         for (int k = 0; k < kFxWords; ++k) red[wid][k] = v[k];
     }
     __syncthreads();
-    if (wid != 0) continue;  // red is next written after the next source's first barrier
-    long long* bins = a.bins1 + (size_t)r * kFxBins * kFxWords;
-    if (lane < kFxWords) {
+    // red is next written after the next source's first barrier
+    if (wid == 0 && lane < kFxWords) {
       long long t = red[0][lane];
-      for (int k = 1; k < kFxNT / 32; ++k) t = lane == 5 ? max(t, (long long)red[k][lane]) : t + red[k][lane];
-      long long* d = bins + (tb % kFxBins) * kFxWords + lane;
+#pragma unroll
+      for (int k = 1; k < 6; ++k) t = lane == 5 ? max(t, (long long)red[k][lane]) : t + red[k][lane];
+      long long* d = fx_bins(a.bins1, r, i) + (tb % kFxBins) * kFxWords + lane;
       if (lane == 5)
         atomicMax(d, t);
       else
         atomicAdd((unsigned long long*)d, (unsigned long long)t);
     }
-    __syncwarp();
-    bool last = false;
-    if (lane == 0) last = last_arrival(a.cnt + 2 * r, nb);
-    if (!__shfl_sync(0xffffffffu, last, 0)) continue;
-    long long t[kFxWords];
-#pragma unroll
-    for (int k = 0; k < kFxWords; ++k) {
-      t[k] = __ldcg(bins + lane * kFxWords + k);
-      bins[lane * kFxWords + k] = 0;
-      if (k < 5)
-        t[k] = warp_sum(t[k]);
-      else
-        t[k] = __reduce_max_sync(0xffffffffu, (int)t[k]);
-    }
-    if (lane != 0) continue;
-    const double dot = fma((double)t[2], pow2(114), fma((double)t[1], pow2(88), (double)t[0] * pow2(62))) +
-                       fma((double)t[4], pow2(72), (double)t[3] * pow2(48));
-    const double a1 = dot * S->inv_n2;
-    const double alpha = a1 * pow2(2 + q);
-    S->alpha = alpha;
-    S->alf = fx_split(-__double2ll_rn(a1 * pow2(60)));
-    // |X_{i+1}| <= 2^k bound < 2^58
-    const double bound = fma(fabs(a1), pow2(kFxBits), (double)(t[5] + 1) * 4294967296.0);
-    S->k = kFxBits - 1 - exponent_of(bound);
-    a.hist_a[(size_t)r * a.prm->max_iter + (i - 1)] = alpha;
-    if (!isfinite(alpha)) mark_done(S, a.done_count, OV_ERR_BREAKDOWN);
   }
 }
 
 // HBM-bound (576 B per site and source): two reads, one write, an exact integer norm; one
 // wave of blocks, two elements in flight per thread (18.6 us for one source at 16^3 x 32).
+// Warp 0 forms alpha and the scale from K1's sums beside the block's first loads.
 template <>
 __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX> a) {
   __shared__ long long red[NT2 / 32][4];
+  __shared__ FX alf_sh;
+  __shared__ int k_sh;
   const int r = blockIdx.y;
   SrcState* S = a.src + r;
-  if (S->done) return;
+  const int i = S->it1;
+  if (__syncthreads_or(S->done) || i < 1) return;
   const size_t n12 = 12 * fx_padded(a.g.V);
-  const int i = S->iter;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int4* Xi = a.ring + ((size_t)r * a.prm->nslots + i) * n12;
   int4* W = a.ring + ((size_t)r * a.prm->nslots + i + 1) * n12;
-  const FX alf = S->alf;
-  const int k = S->k;
-  const int kl = max(k, 0), kr = max(-k, 0);  // below 32 both
-  // 2^k y rounded, plus 2^29 (hi then comes out of a plain shift by 30)
-  const long long rnd = (kr > 0 ? 1LL << (kr - 1) : 0) + (kFxHalf30 << kr);
-  // ||X||^2 = n[0] 2^92 + n[1] 2^60 + n[2] 2^38 + n[3] 2^8 (what is dropped is far below 2^-53)
-  long long n[4] = {0, 0, 0, 0};
   const size_t e0 = (size_t)blockIdx.x * NT2 + threadIdx.x, gs = (size_t)gridDim.x * NT2;
   constexpr int B = 2;  // elements in flight per thread
-  for (size_t eb = e0; eb < n12; eb += B * gs) {
-    int4 xb[B], wb[B];
+  int4 xb[B], wb[B];
+  auto load = [&](size_t eb) {
 #pragma unroll
     for (int t = 0; t < B; ++t) {
       const bool in = eb + t * gs < n12;
       xb[t] = in ? __ldg(Xi + eb + t * gs) : make_int4(0, 0, 0, 0);
       wb[t] = in ? W[eb + t * gs] : make_int4(0, 0, 0, 0);  // int64 pair (re, im)
     }
-    long long hh = 0, xx = 0, ll = 0;  // of up to 8 reals: hh 2^60 + xx 2^30 + ll
+  };
+  load(e0);
+  if (wid == 0) {
+    const long long* bins = fx_bins(a.bins1, r, i) + lane * kFxWords;
+    long long t[kFxWords];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) t[j] = warp_sum(__ldcg(bins + j));
+    const int m = __reduce_max_sync(0xffffffffu, (int)__ldcg(bins + 5));
+    const double dot = fma((double)t[2], pow2(114), fma((double)t[1], pow2(88), (double)t[0] * pow2(62))) +
+                       fma((double)t[4], pow2(72), (double)t[3] * pow2(48));
+    const double a1 = dot * S->vec[i & 1].inv_n2;
+    // |X_{i+1}| <= 2^k bound < 2^58
+    const double bound = fma(fabs(a1), pow2(kFxBits), (double)(m + 1LL) * 4294967296.0);
+    const int k = kFxBits - 1 - exponent_of(bound);
+    if (lane == 0) {
+      alf_sh = fx_split(-__double2ll_rn(a1 * pow2(60)));
+      k_sh = k;
+    }
+    if (blockIdx.x == 0) {
+      long long* z = fx_bins(a.bins1, r, i + 1) + lane * kFxWords;
+#pragma unroll
+      for (int j = 0; j < kFxWords; ++j) z[j] = 0;
+      if (lane == 0) {
+        S->k[i & 1] = k;
+        a.hist_a[(size_t)r * a.prm->max_iter + (i - 1)] = a1 * pow2(2 + S->vec[i & 1].q);
+        S->it2 = i + 1;
+      }
+    }
+  }
+  __syncthreads();
+  const FX alf = alf_sh;
+  const int kl = max(k_sh, 0), kr = max(-k_sh, 0);  // below 32 both
+  // 2^k y rounded, plus 2^29 (hi then comes out of a plain shift by 30)
+  const long long rnd = (kr > 0 ? 1LL << (kr - 1) : 0) + (kFxHalf30 << kr);
+  // ||X||^2 = n[0] 2^92 + n[1] 2^60 + n[2] 2^38 + n[3] 2^8 (what is dropped is far below 2^-53)
+  long long n[4] = {0, 0, 0, 0};
+  for (size_t eb = e0; eb < n12; eb += B * gs) {
+    if (eb != e0) load(eb);
+    long long hh = 0, xx = 0, ll = 0;  // of up to 4 reals: hh 2^60 + xx 2^30 + ll
 #pragma unroll
     for (int t = 0; t < B; ++t) {
       const int xv[4] = {xb[t].x, xb[t].y, xb[t].z, xb[t].w};
@@ -1352,53 +1445,104 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
     n[2] += xx >> 8;
     n[3] += ll >> 8;
   }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     n[j] = warp_sum(n[j]);
     if (lane == 0) red[wid][j] = n[j];
   }
   __syncthreads();
-  if (wid != 0) return;
-  long long* bins = a.bins2 + (size_t)r * kFxBins * kFxWords;
-  if (lane < 4) {
+  if (threadIdx.x < 4) {
     long long t = 0;
 #pragma unroll
     for (int j = 0; j < NT2 / 32; ++j) t += red[j][lane];
-    atomicAdd((unsigned long long*)bins + (blockIdx.x % kFxBins) * kFxWords + lane, (unsigned long long)t);
+    atomicAdd((unsigned long long*)fx_bins(a.bins2, r, i) + (blockIdx.x % kFxBins) * kFxWords + lane,
+              (unsigned long long)t);
   }
-  __syncwarp();
-  bool last = false;
-  if (lane == 0) last = last_arrival(a.cnt + 2 * r + 1, gridDim.x);
-  if (!__shfl_sync(0xffffffffu, last, 0)) return;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    n[j] = warp_sum(__ldcg(bins + lane * kFxWords + j));
-    bins[lane * kFxWords + j] = 0;
+}
+
+// node_check_kernel for the fixed-point forms.  It runs beside the iterations that follow it
+// (run_iterations), so that it looks at a fixed count of them: the recorded ones of whole
+// check intervals.  `final` (nothing runs beside it) takes them all, with the last beta from
+// K2's sums; so does a check that finds a source at the end of its Krylov space (beta = 0).
+// The count of iterations a source ends with does not depend on which check finds it.
+__global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constant__ SolveArgs<FX> a, int final) {
+  __shared__ int last_sh[NT1 / 32];
+  const int r = blockIdx.y;
+  SrcState* S = a.src + r;
+  if (S->done) return;  // set by this kernel only
+  const int ns = a.prm->nshift, mi = a.prm->max_iter;
+  const int ran = S->it2 - 1;  // iterations whose alpha is recorded; their betas but the last
+  int upto = ran / kNodeCheck * kNodeCheck - 1;
+  if (__syncthreads_or(*(volatile int*)&S->it1 == 0 && ran >= 1)) upto = ran;  // K1 recorded the last beta, too
+  __threadfence();
+  if (final) {
+    upto = ran;
+    if (ran >= 1 && threadIdx.x < 32) {
+      double beta;
+      const FxVec v = fx_vec(a, S, r, ran + 1, &beta);
+      if (threadIdx.x == 0) {
+        a.hist_b[(size_t)r * mi + ran - 1] = beta;
+        if (ran < mi) a.hist_n2[(size_t)r * mi + ran] = v.n2;
+        S->iter = ran + 1;
+      }
+    }
+    __syncthreads();
   }
-  if (lane != 0) return;
-  const double tot = fma((double)n[0], pow2(92), (double)n[1] * pow2(60)) + fma((double)n[2], pow2(38), (double)n[3] * 256.0);
-  const int q = S->q, ns = a.prm->nshift, mi = a.prm->max_iter;
-  const double ratio = tot * S->inv_n2;  // ||X_{i+1}||^2 / ||X_i||^2
-  const double beta = sqrt(ratio) * pow2(2 + q - k);
-  a.hist_b[(size_t)r * mi + (i - 1)] = beta;
-  if (i < mi) a.hist_n2[(size_t)r * mi + i] = tot;
-  const double g1 = ratio * pow2(q - k);  // beta_i ||X_{i+1}|| / (4 ||X_i||)
-  const int qn = max(0, exponent_of(g1));  // g1 2^-qn < 2
-  S->gam = fx_split(-__double2ll_rn(g1 * pow2(60 - qn)));
-  S->dia = fx_split(__double2ll_rn(a.diag4 * pow2(60 - qn)));
-  S->q = qn;
-  S->n2 = tot;
-  S->inv_n2 = __drcp_rn(tot);
-  S->n_prev = S->n_cur;
-  S->n_cur = beta;
-  S->iter = i + 1;
-  if (!isfinite(beta)) {
-    mark_done(S, a.done_count, OV_ERR_BREAKDOWN);
-  } else if (beta == 0.0) {
+  const double tol2 = a.prm->tol * a.prm->tol, inv_b2 = S->inv_b2;
+  const double* ha = a.hist_a + (size_t)r * mi;
+  const double* hb = a.hist_b + (size_t)r * mi;
+  int still = 0, last = 0;
+  for (int j0 = 0; j0 < ns; j0 += NT1) {
+    const int j = j0 + threadIdx.x;
+    bool act = false;
+    if (j < ns) {
+      ShiftState& q = a.sh[(size_t)r * ns + j];
+      if (q.active) {
+        const double2 zj = a.z[(size_t)r * ns + j];
+        double2 invd = q.invd, om = q.omega, zeta = q.zeta;
+        double res2 = q.res2;
+        int i = q.last_iter + 1;
+        act = true;
+        for (; i <= upto; ++i) {
+          const double alpha = __ldcg(ha + i - 1), beta = __ldcg(hb + i - 1);
+          double2 d;
+          if (i == 1) {
+            d = make_double2(zj.x - alpha, zj.y);
+            om = make_double2(S->bnorm, 0.0);
+          } else {
+            const double bp = __ldcg(hb + i - 2);
+            const double b2 = bp * bp;
+            d = make_double2(zj.x - alpha - b2 * invd.x, zj.y - b2 * invd.y);
+            om = cmul(make_double2(bp * invd.x, bp * invd.y), om);
+          }
+          const double inv = __drcp_rn(d.x * d.x + d.y * d.y);
+          invd = make_double2(d.x * inv, -d.y * inv);
+          zeta = cmul(om, invd);
+          res2 = beta * beta * inv_b2 * (zeta.x * zeta.x + zeta.y * zeta.y);
+          if (res2 <= tol2 || beta == 0.0) {
+            if (beta == 0.0) res2 = 0.0;
+            act = false;
+            break;
+          }
+        }
+        q.invd = invd;
+        q.omega = om;
+        q.zeta = zeta;
+        q.res2 = res2;
+        q.last_iter = act ? max(upto, 0) : i;
+        q.active = act ? 1 : 0;
+      }
+      last = max(last, q.last_iter);
+    }
+    still += __syncthreads_count(act);
+  }
+  last = block_max<NT1>(last, last_sh);
+  if (threadIdx.x == 0 && ns > 0 && still == 0) {
+    // The next multiple of the check interval after the last node's iteration, an even count:
+    // the iterates of an indefinite operator alternate, and the sum over an odd number of
+    // vectors is several times further off (8^4: 2.9e-13 with 367, 3.5e-14 with 368).
+    S->iter = min(ran, (last + kNodeCheck) / kNodeCheck * kNodeCheck) + 1;
     mark_done(S, a.done_count, OV_OK);
-  } else if (i >= mi || (a.prm->store && i + 2 >= a.prm->nslots)) {
-    mark_done(S, a.done_count, ns > 0 ? OV_ERR_NOT_CONVERGED : OV_OK);
   }
 }
 
@@ -1426,7 +1570,7 @@ __global__ void __launch_bounds__(NT2) lanczos_init_kernel<FX>(SolveArgs<FX> a, 
   mx = block_max<NT2>(mx, shi);
   if (threadIdx.x == 0) {
     a.part2[(size_t)r * gridDim.x + blockIdx.x] = bs;
-    atomicMax(a.bins1 + (size_t)r * kFxBins * kFxWords + 5, (long long)mx);
+    atomicMax(fx_bins(a.bins1, r, 0) + 5, (long long)mx);
     __threadfence();
     last = (atomicAdd(a.cnt + 2 * r + 1, 1u) == gridDim.x - 1);
   }
@@ -1455,16 +1599,20 @@ __global__ void __launch_bounds__(NT2) lanczos_init_kernel<FX>(SolveArgs<FX> a, 
   S->n_prev = 1.0;
   S->alpha = 0.0;
   S->iter = 1;
-  long long* mb = a.bins1 + (size_t)r * kFxBins * kFxWords + 5;
+  long long* mb = fx_bins(a.bins1, r, 0) + 5;
   const int m = (int)__ldcg(mb);
   *mb = 0;
   S->e_in = kFxBits - 1 - ((m >> 20) - 1023);
-  S->n2 = ldexp(tot, 2 * S->e_in);
-  S->inv_n2 = 1.0 / S->n2;
-  a.hist_n2[(size_t)r * a.prm->max_iter] = S->n2;
-  S->gam = S->alf = FX{0, 0};
-  S->dia = fx_split(__double2ll_rn(a.diag4 * pow2(60)));
-  S->q = S->k = 0;
+  FxVec v;
+  v.n2 = ldexp(tot, 2 * S->e_in);
+  v.inv_n2 = 1.0 / v.n2;
+  v.gam = FX{0, 0};
+  v.dia = fx_split(__double2ll_rn(a.diag4 * pow2(60)));
+  v.q = 0;
+  S->vec[1] = v;
+  S->it1 = 0;
+  S->it2 = 1;
+  a.hist_n2[(size_t)r * a.prm->max_iter] = v.n2;
   S->status = OV_OK;
   S->n_act = 0;
   S->node_updates = 0.0;
@@ -1496,8 +1644,8 @@ __global__ void __launch_bounds__(NT2) fx_quantize_kernel(const __grid_constant_
 //   f_k = z - alpha_k,  f_i = z - alpha_i - beta_i^2 / f_{i+1};   y_1 = ||b|| / f_1,  y_{i+1} =
 //   beta_i y_i / f_{i+1}
 // (the factorisation from the last row up: |Im f_i| >= |Im z|).  Y[r][i][j] holds 1 / f, then y
-// / ||X_i||.  A chain of k reciprocals (0.2 us each) that took 25 us per source and node on
-// the host.
+// / ||X_i||.  A serial chain of k complex reciprocals per thread, all nodes and sources at once
+// (on the host it took 8 us per source and node at 8^4, 2 of 10 ms of a 4-source solve).
 __global__ void __launch_bounds__(32) fx_node_coef_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
                                                           double2* __restrict__ Y) {
   const int r = blockIdx.y, j = blockIdx.x * 32 + threadIdx.x;
@@ -1799,8 +1947,8 @@ SolveArgs<R> args_for_sources(const SolveWs<R>& w, int r0) {
   a.act_z += r * ns;
   a.part1 += r * w.nblk1;
   a.part2 += r * w.nblk2u;
-  if (a.bins1) a.bins1 += r * kFxBins * kFxWords;
-  if (a.bins2) a.bins2 += r * kFxBins * kFxWords;
+  if (a.bins1) a.bins1 += r * 2 * kFxBins * kFxWords;
+  if (a.bins2) a.bins2 += r * 2 * kFxBins * kFxWords;
   a.cnt += 2 * r;
   if (a.hist_a) a.hist_a += r * w.max_iter;
   if (a.hist_b) a.hist_b += r * w.max_iter;
@@ -1820,25 +1968,29 @@ SolveArgs<R> args_for_sources(const SolveWs<R>& w, int r0) {
 // sources fits two waves (152 SMs x 4 blocks); else two, or six for double-float.
 // (8^4, 4 sources, FP64 two-pass: 23.8 / 22.6 / 22.0 ms per apply with 1 / 2 / 4 groups;
 // 16^3 x 32, 12 sources in batches of 6, 1 / 2 / 3 / 6 groups: FP64 two-pass 1385 / 1373
-// / 1374 / 1375 ms, double-float 407 / 390 / 390 / 386 ms; 16^4: 533.6 / 529.8 ms.)
+// / 1374 / 1375 ms, double-float 407 / 390 / 390 / 386 ms; 16^4: 533.6 / 529.8 ms.  Fixed
+// point: three on large lattices -- 16^3 x 32 with 1 / 2 / 3 / 4 / 6 groups 355 / 348 / 343 / 354
+// / 370 ms, 16^4 131.5 / 128.3 / 126.0 / 128.2 / 134.0 ms; 8^4 7.6 / 6.8 / 6.7 / 6.5 / 6.5 ms.)
 template <typename R>
 int source_groups(const ov_ctx* ctx, int nsrc, int nblk1) {
   int g = ctx->groups;
-  if (g <= 0) g = ((size_t)nblk1 * nsrc <= (size_t)2 * 152 * 4) ? 4 : (std::is_same<R, DF>::value ? 6 : 2);
+  if (g <= 0)
+    g = ((size_t)nblk1 * nsrc <= (size_t)2 * 152 * 4) ? 4 : std::is_same<R, DF>::value ? 6 : std::is_same<R, FX>::value ? 3 : 2;
   return std::max(1, std::min(g, nsrc));
 }
 
-// Capture body(stream, args, sources) once per source group, each group on its own branch
-// (forked from and joined back to the capture stream), and instantiate the graph.
+// Capture body(stream, side stream, fork and join events, args, sources) once per source group,
+// each group on its own branch (forked from and joined back to the capture stream; the body
+// forks and joins its side stream itself), and instantiate the graph.
 template <typename R, typename F>
 int capture_groups(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int G, F body, cudaGraphExec_t* exec) {
-  while ((int)ctx->aux_streams.size() < G) {
+  while ((int)ctx->aux_streams.size() < 2 * G) {
     cudaStream_t st = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
     if (e != cudaSuccess) return ctx_cuda(ctx, e, "cudaStreamCreate");
     ctx->aux_streams.push_back(st);
   }
-  while ((int)ctx->cap_events.size() < G) {
+  while ((int)ctx->cap_events.size() < 3 * G) {
     cudaEvent_t ev = nullptr;
     cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e != cudaSuccess) return ctx_cuda(ctx, e, "cudaEventCreate");
@@ -1852,7 +2004,8 @@ int capture_groups(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int G, F body, cu
   }
   for (int g = 0; g < G; ++g) {
     const int lo = (int)((long long)nsrc * g / G), hi = (int)((long long)nsrc * (g + 1) / G);
-    body(g == 0 ? ctx->cap_stream : ctx->aux_streams[g], args_for_sources(w, lo), hi - lo);
+    body(g == 0 ? ctx->cap_stream : ctx->aux_streams[g], ctx->aux_streams[G + g], ctx->cap_events[G + 2 * g],
+         ctx->cap_events[G + 2 * g + 1], args_for_sources(w, lo), hi - lo);
   }
   if (G > 1) {
     for (int g = 1; g < G; ++g) {
@@ -1915,7 +2068,7 @@ int setup_ws(ov_ctx* ctx, int nsrc, int ns, bool want_x, bool want_sacc, bool wa
   a.bins1 = a.bins2 = nullptr;
   a.hist_n2 = nullptr;
   if (std::is_same<R, FX>::value) {
-    const size_t nbins = (size_t)nsrc * kFxBins * kFxWords;
+    const size_t nbins = (size_t)nsrc * 2 * kFxBins * kFxWords;
     a.bins1 = (long long*)ws_get(ctx, (t + ".bins").c_str(), sizeof(long long) * 2 * nbins, &st);
     if (a.bins1) a.bins2 = a.bins1 + nbins;
     a.hist_n2 = (double*)ws_get(ctx, (t + ".hn").c_str(), sizeof(double) * (size_t)nsrc * max_iter, &st);
@@ -1953,39 +2106,55 @@ dim3 k1_grid(const SolveWs<R>& w, int n) {
 }
 
 // K1 over n sources.  Fixed point: a block takes up to kFxPerBlock sources of a tile (their
-// links then come from registers), fewer while the grid would not fill the GPU.
+// links then come from L1), fewer while the grid would not fill the GPU; grids of at most
+// three blocks per SM form the scalars themselves.  Returns the number of launches.
 constexpr int kFxPerBlock = 6;
 template <typename R>
-void launch_k1(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s) {
+int launch_k1(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s) {
   if constexpr (std::is_same<R, FX>::value) {
     int ng = (n + kFxPerBlock - 1) / kFxPerBlock;
     while (ng < n && (size_t)w.nblk1 * ng < 4 * 4 * 152) ++ng;
     const int per = (n + ng - 1) / ng;
-    fx_lanczos_hw_kernel<<<(unsigned)w.nblk1 * ((n + per - 1) / per), kFxNT, 0, s>>>(a, n, per);
+    const unsigned grid = (unsigned)w.nblk1 * ((n + per - 1) / per);
+    if (grid <= 3 * 152) {
+      fx_lanczos_hw_kernel<kFxNT + 32><<<grid, kFxNT + 32, 0, s>>>(a, n, per);
+      return 1;
+    }
+    fx_begin_kernel<<<n, 32, 0, s>>>(a);
+    fx_lanczos_hw_kernel<kFxNT><<<grid, kFxNT, 0, s>>>(a, n, per);
+    return 2;
   } else {
     lanczos_hw_kernel<R><<<k1_grid(w, n), NT1, 0, s>>>(a);
+    return 1;
   }
 }
 
 template <typename R>
-void launch_node_check(const SolveWs<R>& w, const SolveArgs<R>& a, int nsrc, cudaStream_t s) {
-  node_check_kernel<R><<<dim3(1, nsrc), NT1, 0, s>>>(a);
+void launch_node_check(const SolveWs<R>& w, const SolveArgs<R>& a, int nsrc, cudaStream_t s, bool final = false) {
+  if constexpr (std::is_same<R, FX>::value)
+    fx_node_check_kernel<<<dim3(1, nsrc), NT1, 0, s>>>(a, final);
+  else
+    node_check_kernel<R><<<dim3(1, nsrc), NT1, 0, s>>>(a);
 }
 
 // One Lanczos iteration (K1, K2); `it` counts iterations from 0 within the loop, and a
 // scalar-only form with deferred node recurrences checks its nodes after every
-// kNodeCheck-th.
+// kNodeCheck-th.  Returns the number of launches.
 template <typename R>
 int launch_iteration(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, cudaStream_t s, int it) {
   cudaEvent_t ev;
   kt_begin(ctx, KC_LANCZOS_HW, s, &ev);
-  launch_k1<R>(w, w.a, nsrc, s);
+  int n = launch_k1<R>(w, w.a, nsrc, s);
   kt_end(ctx, KC_LANCZOS_HW, s, ev);
   kt_begin(ctx, KC_SHIFT_UPDATE, s, &ev);
   lanczos_update_kernel<R><<<dim3(w.nblk2u, nsrc), NT2, 0, s>>>(w.a);
   kt_end(ctx, KC_SHIFT_UPDATE, s, ev);
-  if (w.defer && (it + 1) % kNodeCheck == 0) launch_node_check<R>(w, w.a, nsrc, s);
-  return OV_OK;
+  ++n;
+  if (w.defer && (it + 1) % kNodeCheck == 0) {
+    launch_node_check<R>(w, w.a, nsrc, s);
+    ++n;
+  }
+  return n;
 }
 
 // Run iterations until every source is done or max_iter is reached.
@@ -1999,6 +2168,7 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
   if (w.defer) chunk = (chunk + kNodeCheck - 1) / kNodeCheck * kNodeCheck;
   const bool graph = o.use_graph && !ctx->timing;
   cudaGraphExec_t exec = nullptr;
+  double graph_launches = 0.0;  // per replay
   if (graph) {
     const int G = source_groups<R>(ctx, nsrc, w.nblk1);
     GraphKey key{{(const void*)w.a.ring, (const void*)w.a.p, (const void*)w.a.x, (const void*)w.a.sacc},
@@ -2006,36 +2176,48 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
     auto it = ctx->graphs.find(key);
     if (it != ctx->graphs.end()) {
       exec = it->second;
+      graph_launches = ctx->graph_launches[key];
     } else {
       // the graph replays identical launches: every argument is a workspace pointer
       // and all per-iteration state lives in device memory
       const int st = capture_groups<R>(
           ctx, w, nsrc, G,
-          [&](cudaStream_t cs, const SolveArgs<R>& a, int n) {
+          [&](cudaStream_t cs, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, const SolveArgs<R>& a, int n) {
+            // fixed point: the node checks run on a side branch beside the next interval
+            constexpr bool beside = std::is_same<R, FX>::value;
             for (int k = 0; k < chunk; ++k) {
-              launch_k1<R>(w, a, n, cs);
+              graph_launches += launch_k1<R>(w, a, n, cs) + 1;
               lanczos_update_kernel<R><<<dim3(w.nblk2u, n), NT2, 0, cs>>>(a);
-              if (w.defer && (k + 1) % kNodeCheck == 0) launch_node_check<R>(w, a, n, cs);
+              if (!w.defer || (k + 1) % kNodeCheck != 0) continue;
+              graph_launches += 1.0;
+              if (beside) {
+                if (k >= kNodeCheck) cudaStreamWaitEvent(cs, join, 0);
+                cudaEventRecord(fork, cs);
+                cudaStreamWaitEvent(side, fork, 0);
+                launch_node_check<R>(w, a, n, side);
+                cudaEventRecord(join, side);
+              } else {
+                launch_node_check<R>(w, a, n, cs);
+              }
             }
+            if (beside && w.defer) cudaStreamWaitEvent(cs, join, 0);
           },
           &exec);
       if (st != OV_OK) return st;
       ctx->graphs[key] = exec;
+      ctx->graph_launches[key] = graph_launches;
     }
   }
-  const int G = graph ? source_groups<R>(ctx, nsrc, w.nblk1) : 1;
   int done_iters = 0;
   while (done_iters < max_iter) {
     const int n = std::min(chunk, max_iter - done_iters);
-    const int nchecks = w.defer ? (done_iters + n) / kNodeCheck - done_iters / kNodeCheck : 0;
     if (graph && n == chunk) {
       cudaError_t e = cudaGraphLaunch(exec, s);
       if (e != cudaSuccess) return ctx_cuda(ctx, e, "cudaGraphLaunch");
-      *launches += (2.0 * n + nchecks) * G;
+      *launches += graph_launches;
     } else {
-      for (int k = 0; k < n; ++k) launch_iteration<R>(ctx, w, nsrc, s, done_iters + k);
+      for (int k = 0; k < n; ++k) *launches += launch_iteration<R>(ctx, w, nsrc, s, done_iters + k);
       OV_CHECK_LAUNCH(ctx, "lanczos kernels");
-      *launches += 2.0 * n + nchecks;
     }
     done_iters += n;
     cudaError_t e = cudaMemcpyAsync(ctx->host_flag, w.a.done_count, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -2046,7 +2228,7 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
     if (*ctx->host_flag >= nsrc) break;
   }
   if (w.defer) {  // the iterations since the last check (final node residuals and status)
-    launch_node_check<R>(w, w.a, nsrc, s);
+    launch_node_check<R>(w, w.a, nsrc, s, true);
     OV_CHECK_LAUNCH(ctx, "node_check_kernel");
     *launches += 1.0;
   }
@@ -2105,7 +2287,7 @@ int init_solve(ov_ctx* ctx, SolveWs<R>& w, const double2* b_soa, int nsrc, int n
   }
   cudaMemsetAsync(w.a.cnt, 0, sizeof(unsigned) * 2 * nsrc, s);
   cudaMemsetAsync(w.a.done_count, 0, sizeof(int), s);
-  if (w.a.bins1) cudaMemsetAsync(w.a.bins1, 0, sizeof(long long) * 2 * kFxBins * kFxWords * nsrc, s);
+  if (w.a.bins1) cudaMemsetAsync(w.a.bins1, 0, sizeof(long long) * 4 * kFxBins * kFxWords * nsrc, s);
   if constexpr (!std::is_same<R, FX>::value) {  // fixed point keeps no per-node vectors
     const size_t n = (size_t)12 * ctx->g.V * nsrc * ns;
     if (w.a.x) zero_kernel<R><<<1024, 256, 0, s>>>(w.a.x, n);
@@ -2613,7 +2795,7 @@ static int solve_sign_regen(ov_ctx* ctx, const double2* b_soa, double2* out_soa,
     } else {
       st = capture_groups<R>(
           ctx, w, nsrc, G,
-          [&](cudaStream_t cs, const SolveArgs<R>& a, int n) {
+          [&](cudaStream_t cs, cudaStream_t, cudaEvent_t, cudaEvent_t, const SolveArgs<R>& a, int n) {
             for (int k = 0; k < chunk; ++k) lanczos_regen_kernel<R><<<dim3(w.nblk1, n), NT1, 0, cs>>>(a);
           },
           &exec);
