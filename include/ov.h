@@ -172,7 +172,10 @@ int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream);
 
 /* out = H_W in (Eq. 1 and the definition of H_W = gamma5 D_W(-m0) after it) for nrhs
  * spinors in the canonical layout psi[rhs][t][z][y][x][4][3], device pointers, in the
- * given precision (OV_FP64: complex double, OV_FP32: complex float).  in and out must
+ * given precision (OV_FP64: complex double, OV_FP32: complex float).  FP64 with unitary
+ * links and |4 - m0| <= 4 is computed in integers, exact to about 2^-57 of the largest
+ * component of each output's site and its eight neighbours (non-finite components
+ * propagate as in FP64 arithmetic); other links and masses in FP64.  in and out must
  * not alias.  nrhs = 0 is a no-op.  Errors: INVALID_ARG, NO_GAUGE, OUT_OF_MEMORY, CUDA. */
 int ov_apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precision, void* stream);
 

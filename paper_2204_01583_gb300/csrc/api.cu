@@ -386,6 +386,7 @@ int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream) {
   }
   st = launch_gauge_ingest(ctx, src, s);
   if (st != OV_OK) return st;
+  const bool fx = launch_links_fx(ctx, s);
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "ov_set_gauge");
   kt_collect(ctx);
@@ -394,7 +395,7 @@ int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream) {
   ctx->have_c32 = false;
   ctx->have_s4 = false;
   ctx->have_df = false;
-  ctx->have_fx = false;
+  ctx->fx_ok = fx && ctx->host_flag[1] == 0;
   return OV_OK;
 }
 
@@ -441,6 +442,11 @@ int ov_apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precision,
   cudaStream_t s = (cudaStream_t)stream;
   const size_t n = (size_t)12 * ctx->g.V * nrhs;
   int st = OV_OK;
+  if (precision == OV_FP64 && ctx->fx_ok) {
+    st = launch_hw64_fx(ctx, (const double2*)in, (double2*)out, nrhs, true, s);
+    if (st != OV_ERR_INVALID_ARG) return st;  // too many right-hand sides for one launch: below
+    st = OV_OK;
+  }
   if (precision == OV_FP64) {
     double2* a = (double2*)ws_get(ctx, "hw.a64", sizeof(double2) * n, &st);
     double2* b = (double2*)ws_get(ctx, "hw.b64", sizeof(double2) * n, &st);

@@ -198,11 +198,11 @@ __device__ __forceinline__ void mulAdag(Cx<R> h0, Cx<R> h1, Cx<R>& a0, Cx<R>& a1
 
 // One direction of the hopping term, both hops, accumulated into acc[12]
 // (acc -= 1/2 [(1 - g) U psi(x+mu) + (1 + g) U(x-mu)^dag psi(x-mu)]).
-// in: spinor planes, element (k, site) at in[k * V + site]; U: link planes.
+// in: element (k, site) at in[k ks + site ss] (planes: ks = V, ss = 1); U: link planes.
 template <int MU, typename R, bool CG = false>
 __device__ __forceinline__ void hop_dir(const typename Store<R>::T* __restrict__ in,
                                         const typename Store<R>::T* __restrict__ U, const Geom& g,
-                                        int s, const int c[4], Cx<R> acc[12]) {
+                                        int s, const int c[4], Cx<R> acc[12], size_t ks, size_t ss) {
   const int V = g.V;
 #pragma unroll
   for (int dir = 0; dir < 2; ++dir) {
@@ -213,10 +213,10 @@ __device__ __forceinline__ void hop_dir(const typename Store<R>::T* __restrict__
     Cx<R> h0[3], h1[3];
 #pragma unroll
     for (int col = 0; col < 3; ++col) {
-      Cx<R> p0 = ld<R, CG>(in + (0 * 3 + col) * (size_t)V + sn);
-      Cx<R> p1 = ld<R, CG>(in + (1 * 3 + col) * (size_t)V + sn);
-      Cx<R> p2 = ld<R, CG>(in + (2 * 3 + col) * (size_t)V + sn);
-      Cx<R> p3 = ld<R, CG>(in + (3 * 3 + col) * (size_t)V + sn);
+      Cx<R> p0 = ld<R, CG>(in + (0 * 3 + col) * ks + sn * ss);
+      Cx<R> p1 = ld<R, CG>(in + (1 * 3 + col) * ks + sn * ss);
+      Cx<R> p2 = ld<R, CG>(in + (2 * 3 + col) * ks + sn * ss);
+      Cx<R> p3 = ld<R, CG>(in + (3 * 3 + col) * ks + sn * ss);
       Cx<R> a0, a1;
       mulA<MU>(p2, p3, a0, a1);
       if (dir == 0) { h0[col] = csub(p0, a0); h1[col] = csub(p1, a1); }
@@ -344,17 +344,23 @@ __device__ __forceinline__ void hop_dir_unscaled(const typename Store<R>::T* __r
 template <typename R>
 __device__ __forceinline__ void hw_site(const typename Store<R>::T* __restrict__ in,
                                         const typename Store<R>::T* __restrict__ U, const Geom& g,
-                                        int s, R diag, Cx<R> out[12]) {
+                                        int s, R diag, Cx<R> out[12], size_t ks, size_t ss) {
   int c[4];
   site_coords(g, s, c);
 #pragma unroll
-  for (int k = 0; k < 12; ++k) out[k] = cscale(diag, ld<R>(in + k * (size_t)g.V + s));
-  hop_dir<0, R>(in, U, g, s, c, out);
-  hop_dir<1, R>(in, U, g, s, c, out);
-  hop_dir<2, R>(in, U, g, s, c, out);
-  hop_dir<3, R>(in, U, g, s, c, out);
+  for (int k = 0; k < 12; ++k) out[k] = cscale(diag, ld<R>(in + k * ks + s * ss));
+  hop_dir<0, R>(in, U, g, s, c, out, ks, ss);
+  hop_dir<1, R>(in, U, g, s, c, out, ks, ss);
+  hop_dir<2, R>(in, U, g, s, c, out, ks, ss);
+  hop_dir<3, R>(in, U, g, s, c, out, ks, ss);
 #pragma unroll
   for (int k = 6; k < 12; ++k) out[k] = cneg(out[k]);
+}
+template <typename R>
+__device__ __forceinline__ void hw_site(const typename Store<R>::T* __restrict__ in,
+                                        const typename Store<R>::T* __restrict__ U, const Geom& g,
+                                        int s, R diag, Cx<R> out[12]) {
+  hw_site<R>(in, U, g, s, diag, out, (size_t)g.V, 1);
 }
 
 // ------------------------------------------------------------ reductions

@@ -5,6 +5,8 @@
 // Structure of arrays: a spinor is 12 planes of V complex numbers (plane k =
 // 3 * spin + colour), so consecutive threads (consecutive sites) read
 // consecutive 8- or 16-byte words of a plane; a gauge field is 4 x 9 planes.
+#include <cmath>
+
 #include "fixed.cuh"
 
 namespace {
@@ -230,22 +232,18 @@ int ensure_links_df(ov_ctx* ctx, cudaStream_t s) {
   return OV_OK;
 }
 
-int ensure_links_fx(ov_ctx* ctx, cudaStream_t s) {
+bool launch_links_fx(ov_ctx* ctx, cudaStream_t s) {
+  if (!(std::fabs(4.0 - ctx->m0) <= kFxDiagMax)) return false;
   int st = OV_OK;
-  const size_t n = (size_t)4 * ctx->g.V;
-  ctx->Ufx = (int4*)ws_get(ctx, "gauge.fx", sizeof(int4) * 36 * fx_padded(ctx->g.V), &st);
+  const size_t n = 4 * fx_padded(ctx->g.V);
+  ctx->Ufx = (int4*)ws_get(ctx, "gauge.fx", sizeof(int4) * 9 * n, &st);
   int* bad = (int*)ws_get(ctx, "gauge.fxbad", sizeof(int), &st);
-  if (st != OV_OK) return st;
-  if (!ctx->have_fx) {
-    cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), s);
-    if (e != cudaSuccess) return ctx_cuda(ctx, e, "clear link check");
-    links_fx_kernel<<<grid_for(n, 256), 256, 0, s>>>(ctx->U64h, ctx->Ufx, ctx->g.V, bad);
-    OV_CHECK_LAUNCH(ctx, "links_fx_kernel");
-    e = cudaMemcpyAsync(ctx->host_flag + 1, bad, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return ctx_cuda(ctx, e, "read link check");
-    ctx->fx_ok = ctx->host_flag[1] == 0;
-    ctx->have_fx = true;
-  }
-  return OV_OK;
+  if (st != OV_OK) return false;
+  cudaMemsetAsync(bad, 0, sizeof(int), s);
+  cudaEvent_t ev;
+  kt_begin(ctx, KC_LAYOUT, s, &ev);
+  links_fx_kernel<<<grid_for(n, 256), 256, 0, s>>>(ctx->U64h, ctx->Ufx, ctx->g.V, bad);
+  kt_end(ctx, KC_LAYOUT, s, ev);
+  return cudaGetLastError() == cudaSuccess &&
+         cudaMemcpyAsync(ctx->host_flag + 1, bad, sizeof(int), cudaMemcpyDeviceToHost, s) == cudaSuccess;
 }

@@ -55,6 +55,12 @@ __device__ __forceinline__ long long fx_shr(long long v, int k) {
   const int hi = (int)(v >> 32);
   return (long long)(((unsigned long long)(unsigned)(hi >> k) << 32) | __funnelshift_r(lo, (unsigned)hi, k));
 }
+// arithmetic shift right by any k >= 0 (62 at most: the sign is left), in two steps
+struct FxShift {
+  int a, b;
+};
+__device__ __forceinline__ FxShift fx_shift(int k) { return {min(k, 31), min(max(k - 31, 0), 31)}; }
+__device__ __forceinline__ long long fx_sar(long long v, FxShift k) { return fx_shr(fx_shr(v, k.a), k.b); }
 __device__ __forceinline__ long long fx_value(long long hh, long long x) { return hh + (x >> 30); }
 constexpr long long kFxHalf30 = 1LL << 29;  // added to x before that shift: rounds to nearest
 
@@ -86,7 +92,11 @@ __device__ __forceinline__ FxProj fx_projection(int mu, int spin) {
   f.dim = neg ? -1 : 0;
   return f;
 }
-__device__ __forceinline__ long long fx_neg(long long v, int mask) { return v ^ (long long)mask; }  // -v - 1
+// v or -v; without EXACT -v - 1
+template <bool EXACT>
+__device__ __forceinline__ long long fx_neg(long long v, int mask) {
+  return EXACT ? (v ^ (long long)mask) - (long long)mask : v ^ (long long)mask;
+}
 
 template <int DIR>
 __device__ __forceinline__ int4 fx_project(const FxProj& f, int4 p, int4 q) {
@@ -127,8 +137,13 @@ __device__ __forceinline__ FxHops fx_hops(const Geom& g, int s, int mu) {
 // the vector / 4 (factor -1/2 in the links): u_f + u_b for the upper spin, -A_mu^dag (u_b -
 // u_f) for the lower one.
 constexpr int kFxNT = 256;
+// SCALED (fields with a scale per site, ov_apply_HW): u_f and u_b are shifted right by sf and
+// sb, products are rounded to nearest and negations exact, so that exact zeros stay.  The
+// Lanczos kernels round down and negate to -v - 1 (a unit of 2^-58; 3% faster).
+template <bool SCALED = false>
 __device__ __forceinline__ void fx_phase1(const int4* __restrict__ in, const int4* __restrict__ U, int mu_spin,
-                                          int s, const FxHops& nb, longlong2* out) {
+                                          int s, const FxHops& nb, longlong2* out, FxShift sf = {0, 0},
+                                          FxShift sb = {0, 0}) {
   const int mu = mu_spin >> 1, spin = mu_spin & 1;
   const FxProj f = fx_projection(mu, spin);
   longlong2* lo = out + 3 * f.lower * kFxTile;
@@ -155,7 +170,8 @@ __device__ __forceinline__ void fx_phase1(const int4* __restrict__ in, const int
     for (int i = 0; i < 3; ++i) {
       // a complex product from three real ones: re = a - b, im = c - a - b with a = l_re h_re,
       // b = l_im h_im, c = (l_re + l_im)(h_re + h_im): 27 wide multiply-adds per row, not 36
-      long long ah = 0, ax = 0, bh = 0, bx = 0, ch = 0, cx = 0;
+      constexpr long long rnd = SCALED ? kFxHalf30 : 0;
+      long long ah = 0, ax = 0, bh = 0, bx = 0, ch = 0, cx = rnd;
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
         const int4 m = l[3 * i + j];
@@ -163,7 +179,11 @@ __device__ __forceinline__ void fx_phase1(const int4* __restrict__ in, const int
         fx_mac(bh, bx, m.z, m.w, h[j].z, h[j].w);
         fx_mac(ch, cx, m.x + m.z, m.y + m.w, hs[j].x, hs[j].y);
       }
-      const longlong2 u = make_longlong2(fx_value(ah - bh, ax - bx), fx_value(ch - ah - bh, cx - ax - bx));
+      longlong2 u = make_longlong2(fx_value(ah - bh, ax - bx + rnd), fx_value(ch - ah - bh, cx - ax - bx));
+      if (SCALED) {
+        u.x = fx_sar(u.x, dir == 0 ? sf : sb);
+        u.y = fx_sar(u.y, dir == 0 ? sf : sb);
+      }
       longlong2* o = out + i * kFxTile;
       if (dir == 0) {
         *o = u;
@@ -171,7 +191,7 @@ __device__ __forceinline__ void fx_phase1(const int4* __restrict__ in, const int
         const longlong2 uf = *o;
         *o = make_longlong2(uf.x + u.x, uf.y - u.y);
         const long long dr = u.x - uf.x, di = u.y + uf.y;  // d_re, -d_im
-        lo[i * kFxTile] = make_longlong2(fx_neg(f.swap ? di : dr, f.dre), fx_neg(f.swap ? dr : di, f.dim));
+        lo[i * kFxTile] = make_longlong2(fx_neg<SCALED>(f.swap ? di : dr, f.dre), fx_neg<SCALED>(f.swap ? dr : di, f.dim));
       }
     }
   }
@@ -183,4 +203,13 @@ __device__ __forceinline__ longlong2 fx_phase2(const longlong2* sm, int k, int l
   const longlong2* p = sm + k * kFxTile + lane;
   const longlong2 x = p[0], y = p[D], z = p[2 * D], t = p[3 * D];
   return make_longlong2((x.x + y.x) + (z.x + t.x), (x.y + y.y) + (z.y + t.y));
+}
+// The same with the direction's partials shifted right by k0 .. k3.
+__device__ __forceinline__ longlong2 fx_phase2_scaled(const longlong2* sm, int k, int lane, FxShift k0, FxShift k1,
+                                                      FxShift k2, FxShift k3) {
+  constexpr int D = 12 * kFxTile;
+  const longlong2* p = sm + k * kFxTile + lane;
+  const longlong2 x = p[0], y = p[D], z = p[2 * D], t = p[3 * D];
+  return make_longlong2((fx_sar(x.x, k0) + fx_sar(y.x, k1)) + (fx_sar(z.x, k2) + fx_sar(t.x, k3)),
+                        (fx_sar(x.y, k0) + fx_sar(y.y, k1)) + (fx_sar(z.y, k2) + fx_sar(t.y, k3)));
 }

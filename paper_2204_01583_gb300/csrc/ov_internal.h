@@ -113,8 +113,8 @@ struct ov_ctx {
   bool have_s4 = false;                // FP32 links for the spin-paired float4 layout
   float4* Udf = nullptr;               // double-float links (workspace "gauge.df") when have_df
   bool have_df = false;
-  int4* Ufx = nullptr;                 // fixed-point links (workspace "gauge.fx") when have_fx
-  bool have_fx = false, fx_ok = false; // fx_ok: every link fits the fixed-point bounds
+  int4* Ufx = nullptr;                 // fixed-point links (workspace "gauge.fx") when fx_ok
+  bool fx_ok = false;                  // links and mass fit the fixed-point bounds
   std::map<int, int> hw32_choice;      // nrhs -> autotuned FP32 stencil variant
   int hw32_force = -1;                 // ov_set_hw32_variant
   bool no_coop = true;                 // ov_set_persistent(ctx, 1) enables the persistent loop
@@ -183,8 +183,11 @@ void hw32_variant_info(int k, int* rt, int* comp, int* nt);
 float hw32_time_soa_variants(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int* best);
 // double-float links for the FP32-pair solve (dslash.cu)
 int ensure_links_df(ov_ctx* ctx, cudaStream_t s);
-// fixed-point links (dslash.cu); sets ctx->fx_ok
-int ensure_links_fx(ov_ctx* ctx, cudaStream_t s);
+// Fixed-point links (dslash.cu): enqueues them and the copy of the check's verdict to
+// ctx->host_flag[1] (0: every link fits); false when they do not apply or do not fit in memory.
+bool launch_links_fx(ov_ctx* ctx, cudaStream_t s);
+// out = H_W in, FP64 fields (canonical or planes) through integers (hw64.cu); needs fx_ok
+int launch_hw64_fx(ov_ctx* ctx, const double2* in, double2* out, int nrhs, bool canonical, cudaStream_t s);
 // spin-paired float4 FP32 layout (dslash32.cu)
 int launch_pack_s4(ov_ctx* ctx, const float2* aos, float4* s4, int nrhs, cudaStream_t s);
 int launch_unpack_s4(ov_ctx* ctx, const float4* s4, float2* aos, int nrhs, cudaStream_t s);

@@ -2962,14 +2962,12 @@ int nodes_coef<FX>(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const st
 // Whether the stored-basis forms run in fixed point (fixed.cuh): links of norm 1 (the bounds
 // there) and |4 - m0| <= 4.  Other links and masses, and the persistent loop, keep the
 // FP64 and double-float kernels.
-static bool fixed_point_fits(ov_ctx* ctx, cudaStream_t s) {
-  return ctx->no_coop && std::fabs(4.0 - ctx->m0) <= kFxDiagMax && ensure_links_fx(ctx, s) == OV_OK && ctx->fx_ok;
-}
+static bool fixed_point_fits(const ov_ctx* ctx) { return ctx->no_coop && ctx->fx_ok; }
 
 int solve_nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
                      const std::vector<double2>& ch, int chunk, double2* X, double2* sums, const ov_solve_opts& o,
                      SolveOut* so, cudaStream_t s, const std::function<int(int, int)>& per_chunk) {
-  if (fixed_point_fits(ctx, s))
+  if (fixed_point_fits(ctx))
     return nodes_coef<FX>(ctx, b_soa, nsrc, ns, zh, ch, chunk, X, sums, o, so, s, per_chunk);
   if (o.mode == OV_MODE_F32X2) {
     const int st = ensure_links_df(ctx, s);
@@ -2981,7 +2979,7 @@ int solve_nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const 
 
 int solve_sign_2pass(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int nsrc, const ov_solve_opts& o,
                      SolveOut* so, cudaStream_t s) {
-  if (o.mode != OV_MODE_FP64_REGEN && fixed_point_fits(ctx, s))
+  if (o.mode != OV_MODE_FP64_REGEN && fixed_point_fits(ctx))
     return solve_sign_coef<FX>(ctx, b_soa, out_soa, nsrc, o, so, s);
   if (o.mode == OV_MODE_F32X2) {
     const int st = ensure_links_df(ctx, s);
@@ -3201,7 +3199,9 @@ int lanczos_tridiag(ov_ctx* ctx, int steps, int squared, std::vector<double>& al
   if (st != OV_OK) return st;
   const size_t n12 = (size_t)12 * ctx->g.V;
   double2* b = (double2*)ws_get(ctx, "lz.b", sizeof(double2) * n12, &st);
-  double2* tmp = squared ? (double2*)ws_get(ctx, "lz.tmp", sizeof(double2) * n12, &st) : nullptr;
+  // the operator: through integers where they apply, else fused into K1 (H) or in FP64 (H^2)
+  const bool fx = ctx->fx_ok;
+  double2* tmp = squared || fx ? (double2*)ws_get(ctx, "lz.tmp", sizeof(double2) * n12, &st) : nullptr;
   double2* tmp2 = squared ? (double2*)ws_get(ctx, "lz.tmp2", sizeof(double2) * n12, &st) : nullptr;
   if (st != OV_OK) return st;
   start_vector_kernel<<<256, 256, 0, s>>>(b, n12);
@@ -3210,14 +3210,20 @@ int lanczos_tridiag(ov_ctx* ctx, int steps, int squared, std::vector<double>& al
   if (st != OV_OK) return st;
   for (int it = 0; it < steps; ++it) {
     SolveArgs<double> a = w.a;
-    if (squared) {
-      // H^2: apply H twice to U_i (ring slot i % 3, i = it + 1); K1 reads the result
-      const double2* Ui = w.a.ring + (size_t)((it + 1) % 3) * n12;
-      st = launch_hw64(ctx, Ui, tmp, 1, s);
-      if (st == OV_OK) st = launch_hw64(ctx, tmp, tmp2, 1, s);
-      if (st != OV_OK) return st;
+    // H or H^2 applied to U_i (ring slot i % 3, i = it + 1); K1 reads the result
+    const double2* Ui = w.a.ring + (size_t)((it + 1) % 3) * n12;
+    auto apply = [&](const double2* in, double2* out) {
+      return fx ? launch_hw64_fx(ctx, in, out, 1, false, s) : launch_hw64(ctx, in, out, 1, s);
+    };
+    if (squared || fx) {
+      st = apply(Ui, tmp);
+      a.stencil = tmp;
+    }
+    if (squared && st == OV_OK) {
+      st = apply(tmp, tmp2);
       a.stencil = tmp2;
     }
+    if (st != OV_OK) return st;
     lanczos_hw_kernel<double><<<k1_grid(w, 1), NT1, 0, s>>>(a);
     lanczos_update_kernel<double><<<dim3(w.nblk2u, 1), NT2, 0, s>>>(a);
   }
