@@ -401,7 +401,7 @@ int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream) {
 
 // FP32 stencil variants on float4 layouts, numbered after the structure-of-arrays ones:
 // layout P (right-hand-side pairs, 12 float4 per site and pair) or S (spin pairs, 6
-// float4 per site and RHS; its buffers alias the paired ones, 6 <= 12 per pair).
+// float4 per site and RHS; its buffer aliases the paired one, 6 <= 12 per pair).
 struct Float4Variant {
   bool paired;
   int form;              // P: launch_hw_pair12 form; S: unused (one S kernel)
@@ -414,20 +414,52 @@ constexpr Float4Variant kFloat4Variants[] = {
 };
 constexpr int kNFloat4Variants = sizeof(kFloat4Variants) / sizeof(kFloat4Variants[0]);
 
-static int fp32_float4_pack(ov_ctx* ctx, int v, const float2* in, float4* buf, int nrhs, cudaStream_t s) {
-  return kFloat4Variants[v].paired ? launch_pack_pair32(ctx, in, buf, nrhs, s) : launch_pack_s4(ctx, in, buf, nrhs, s);
-}
-
-static int fp32_float4_unpack(ov_ctx* ctx, int v, const float4* buf, float2* out, int nrhs, cudaStream_t s) {
-  return kFloat4Variants[v].paired ? launch_unpack_pair32(ctx, buf, out, nrhs, s)
-                                   : launch_unpack_s4(ctx, buf, out, nrhs, s);
-}
-
-static int fp32_float4_launch(ov_ctx* ctx, int v, const float4* in, float4* out, int nrhs, cudaStream_t s) {
-  const Float4Variant& f = kFloat4Variants[v];
+// out = H_W in in FP32 with variant k, canonical fields: the layout change, then the stencil
+// (which writes the canonical layout itself on the float4 layouts).
+static int apply_hw32(ov_ctx* ctx, int k, const float2* in, float2* out, int nrhs, cudaStream_t s) {
+  const size_t V = ctx->g.V;
+  int st = OV_OK;
+  if (k < hw32_variant_count()) {
+    float2* a = (float2*)ws_get(ctx, "hw.a32", sizeof(float2) * 12 * V * nrhs, &st);
+    float2* b = (float2*)ws_get(ctx, "hw.b32", sizeof(float2) * 12 * V * nrhs, &st);
+    if (st != OV_OK) return st;
+    if ((st = launch_pack32(ctx, in, a, nrhs, s))) return st;
+    if ((st = launch_hw32_soa(ctx, a, b, nrhs, s, k))) return st;
+    return launch_unpack32(ctx, b, out, nrhs, s);
+  }
+  const Float4Variant& f = kFloat4Variants[k - hw32_variant_count()];
   const int npair = (nrhs + 1) / 2;
-  if (!f.paired) return launch_hw32_s4(ctx, in, out, nrhs, s);
-  return launch_hw_pair12(ctx, in, out, npair, f.form, s);
+  float4* a = (float4*)ws_get(ctx, "hw.pa32", sizeof(float4) * 12 * V * npair, &st);
+  if (st != OV_OK) return st;
+  st = f.paired ? launch_pack_pair32(ctx, in, a, nrhs, s) : launch_pack_s4(ctx, in, a, nrhs, s);
+  if (st != OV_OK) return st;
+  return f.paired ? launch_hw_pair12(ctx, a, out, nrhs, f.form, s) : launch_hw32_s4(ctx, a, out, nrhs, s);
+}
+
+// The fastest variant for nrhs right-hand sides on this data (each timed three times after a
+// warm-up that builds its links).
+static int tune_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int* best) {
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  int st = OV_OK;
+  float best_ms = 1e30f;
+  *best = 0;
+  for (int k = 0; k < hw32_variant_count() + kNFloat4Variants && st == OV_OK; ++k) {
+    if ((st = apply_hw32(ctx, k, in, out, nrhs, s))) break;
+    cudaEventRecord(e0, s);
+    for (int rep = 0; rep < 3 && st == OV_OK; ++rep) st = apply_hw32(ctx, k, in, out, nrhs, s);
+    cudaEventRecord(e1, s);
+    cudaEventSynchronize(e1);
+    float ms = 0.f;
+    if (st == OV_OK && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best_ms) {
+      best_ms = ms;
+      *best = k;
+    }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  return st;
 }
 
 int ov_apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precision, void* stream) {
@@ -455,61 +487,17 @@ int ov_apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precision,
     if ((st = launch_hw64(ctx, a, b, nrhs, s))) return st;
     if ((st = launch_unpack64(ctx, b, (double2*)out, nrhs, s))) return st;
   } else {
-    const int npair = (nrhs + 1) / 2;
-    const int kpair = hw32_variant_count();
-    float2* a = (float2*)ws_get(ctx, "hw.a32", sizeof(float2) * n, &st);
-    float2* b = (float2*)ws_get(ctx, "hw.b32", sizeof(float2) * n, &st);
-    float4* pa = (float4*)ws_get(ctx, "hw.pa32", sizeof(float4) * 12 * (size_t)ctx->g.V * npair, &st);
-    float4* pb = (float4*)ws_get(ctx, "hw.pb32", sizeof(float4) * 12 * (size_t)ctx->g.V * npair, &st);
-    if (st != OV_OK) return st;
     int k = ctx->hw32_force;
     if (k < 0) {
       auto it = ctx->hw32_choice.find(nrhs);
       if (it != ctx->hw32_choice.end()) {
         k = it->second;
       } else {
-        // autotune: every structure-of-arrays variant, then the paired and spin-paired
-        // kernels, each timed on this data
-        if ((st = launch_pack32(ctx, (const float2*)in, a, nrhs, s))) return st;
-        int ksoa = 0;
-        float best = hw32_time_soa_variants(ctx, a, b, nrhs, s, &ksoa);
-        k = ksoa;
-        cudaEvent_t e0, e1;
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        for (int kk = kpair; kk < kpair + kNFloat4Variants; ++kk) {
-          if ((st = fp32_float4_pack(ctx, kk - kpair, (const float2*)in, pa, nrhs, s))) return st;
-          st = fp32_float4_launch(ctx, kk - kpair, pa, pb, nrhs, s);  // warm (builds the links)
-          if (st == OV_ERR_INVALID_ARG) {  // this lattice does not fit the variant
-            st = OV_OK;
-            continue;
-          }
-          if (st != OV_OK) return st;
-          cudaEventRecord(e0, s);
-          for (int rep = 0; rep < 3; ++rep) fp32_float4_launch(ctx, kk - kpair, pa, pb, nrhs, s);
-          cudaEventRecord(e1, s);
-          cudaEventSynchronize(e1);
-          float ms = 0.f;
-          cudaEventElapsedTime(&ms, e0, e1);
-          if (ms / 3 < best) {
-            best = ms / 3;
-            k = kk;
-          }
-        }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
+        if ((st = tune_hw32(ctx, (const float2*)in, (float2*)out, nrhs, s, &k))) return st;
         ctx->hw32_choice[nrhs] = k;
       }
     }
-    if (k >= kpair) {
-      if ((st = fp32_float4_pack(ctx, k - kpair, (const float2*)in, pa, nrhs, s))) return st;
-      if ((st = fp32_float4_launch(ctx, k - kpair, pa, pb, nrhs, s))) return st;
-      if ((st = fp32_float4_unpack(ctx, k - kpair, pb, (float2*)out, nrhs, s))) return st;
-    } else {
-      if ((st = launch_pack32(ctx, (const float2*)in, a, nrhs, s))) return st;
-      if ((st = launch_hw32_tuned(ctx, a, b, nrhs, s, k, nullptr))) return st;
-      if ((st = launch_unpack32(ctx, b, (float2*)out, nrhs, s))) return st;
-    }
+    return apply_hw32(ctx, k, (const float2*)in, (float2*)out, nrhs, s);
   }
   return OV_OK;
 }

@@ -5,6 +5,7 @@
 // Structure of arrays: a spinor is 12 planes of V complex numbers (plane k =
 // 3 * spin + colour), so consecutive threads (consecutive sites) read
 // consecutive 8- or 16-byte words of a plane; a gauge field is 4 x 9 planes.
+#include <algorithm>
 #include <cmath>
 
 #include "fixed.cuh"
@@ -34,37 +35,61 @@ __global__ void gauge_ingest_kernel(const double2* __restrict__ aos, double2* __
   }
 }
 
+// Canonical spinors <-> planes, one 32-site tile of a spinor (384 elements, contiguous in the
+// canonical layout) at a time through shared memory: both sides are read and written in
+// whole cache lines.  Rows of 13 elements keep the columns free of bank conflicts.
+constexpr int kTileNT = 384;
+constexpr int kTileRow = 13;
 template <typename T>
-__global__ void pack_kernel(const T* __restrict__ aos, T* __restrict__ soa, int V, int nrhs) {
-  const size_t n = (size_t)nrhs * V * 12;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    const size_t k = t % 12, q = t / 12;
-    const size_t site = q % V, r = q / V;
-    soa[(r * 12 + k) * V + site] = aos[t];
+__global__ void __launch_bounds__(kTileNT) pack_kernel(const T* __restrict__ aos, T* __restrict__ soa, int V,
+                                                       size_t ntiles) {
+  __shared__ T sh[32 * kTileRow];
+  const int t = threadIdx.x, nt = (V + 31) / 32;
+  for (size_t b = blockIdx.x; b < ntiles; b += gridDim.x) {
+    const size_t r = b / nt, s0 = b % nt * 32;
+    if (s0 + t / 12 < V) sh[t / 12 * kTileRow + t % 12] = aos[(r * V + s0) * 12 + t];
+    __syncthreads();
+    const size_t s = s0 + t % 32;
+    if (s < V) soa[(r * 12 + t / 32) * V + s] = sh[t % 32 * kTileRow + t / 32];
+    __syncthreads();
   }
 }
 
 template <typename T>
-__global__ void unpack_kernel(const T* __restrict__ soa, T* __restrict__ aos, int V, int nrhs) {
-  const size_t n = (size_t)nrhs * V * 12;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    const size_t k = t % 12, q = t / 12;
-    const size_t site = q % V, r = q / V;
-    aos[t] = soa[(r * 12 + k) * V + site];
+__global__ void __launch_bounds__(kTileNT) unpack_kernel(const T* __restrict__ soa, T* __restrict__ aos, int V,
+                                                         size_t ntiles) {
+  __shared__ T sh[32 * kTileRow];
+  const int t = threadIdx.x, nt = (V + 31) / 32;
+  for (size_t b = blockIdx.x; b < ntiles; b += gridDim.x) {
+    const size_t r = b / nt, s0 = b % nt * 32, s = s0 + t % 32;
+    if (s < V) sh[t % 32 * kTileRow + t / 32] = soa[(r * 12 + t / 32) * V + s];
+    __syncthreads();
+    if (s0 + t / 12 < V) aos[(r * V + s0) * 12 + t] = sh[t / 12 * kTileRow + t % 12];
+    __syncthreads();
   }
 }
 
-// out = (1+m)/2 b + (1-m)/2 gamma5 s ; b, out canonical; s structure of arrays
-__global__ void overlap_epilogue_kernel(const double2* __restrict__ b, const double2* __restrict__ s,
-                                        double2* __restrict__ out, double a, double c, int V, int nrhs) {
-  const size_t n = (size_t)nrhs * V * 12;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    const size_t k = t % 12, q = t / 12;
-    const size_t site = q % V, r = q / V;
-    const double2 sv = s[(r * 12 + k) * V + site];
-    const double g = (k < 6) ? c : -c;  // gamma5 = diag(1, 1, -1, -1) on spin = k / 3
-    const double2 bv = b[t];
-    out[t] = make_double2(fma(a, bv.x, g * sv.x), fma(a, bv.y, g * sv.y));
+// out = (1+m)/2 b + (1-m)/2 gamma5 s ; b, out canonical; s structure of arrays (tiles as in
+// unpack_kernel)
+__global__ void __launch_bounds__(kTileNT) overlap_epilogue_kernel(const double2* __restrict__ b,
+                                                                   const double2* __restrict__ s,
+                                                                   double2* __restrict__ out, double a, double c, int V,
+                                                                   size_t ntiles) {
+  __shared__ double2 sh[32 * kTileRow];
+  const int t = threadIdx.x, nt = (V + 31) / 32;
+  for (size_t q = blockIdx.x; q < ntiles; q += gridDim.x) {
+    const size_t r = q / nt, s0 = q % nt * 32, site = s0 + t % 32;
+    if (site < V) sh[t % 32 * kTileRow + t / 32] = s[(r * 12 + t / 32) * V + site];
+    __syncthreads();
+    if (s0 + t / 12 < V) {
+      const int k = t % 12;
+      const size_t e = (r * V + s0) * 12 + t;
+      const double2 sv = sh[t / 12 * kTileRow + k];
+      const double g = (k < 6) ? c : -c;  // gamma5 = diag(1, 1, -1, -1) on spin = k / 3
+      const double2 bv = b[e];
+      out[e] = make_double2(fma(a, bv.x, g * sv.x), fma(a, bv.y, g * sv.y));
+    }
+    __syncthreads();
   }
 }
 
@@ -152,16 +177,18 @@ int launch_gauge_ingest(ov_ctx* ctx, const double2* U_aos, cudaStream_t s) {
   return OV_OK;
 }
 
+static unsigned tile_grid(size_t ntiles) { return (unsigned)std::min<size_t>(ntiles, 152 * 64); }
+
 template <typename T>
 static int pack_impl(ov_ctx* ctx, const T* aos, T* soa, int nrhs, cudaStream_t s, bool unpack) {
-  const size_t n = (size_t)nrhs * ctx->g.V * 12;
+  const size_t n = (size_t)nrhs * ((ctx->g.V + 31) / 32);
   if (n == 0) return OV_OK;
   cudaEvent_t ev;
   kt_begin(ctx, KC_LAYOUT, s, &ev);
   if (unpack)
-    unpack_kernel<T><<<grid_for(n, 256), 256, 0, s>>>(aos, soa, ctx->g.V, nrhs);
+    unpack_kernel<T><<<tile_grid(n), kTileNT, 0, s>>>(aos, soa, ctx->g.V, n);
   else
-    pack_kernel<T><<<grid_for(n, 256), 256, 0, s>>>(aos, soa, ctx->g.V, nrhs);
+    pack_kernel<T><<<tile_grid(n), kTileNT, 0, s>>>(aos, soa, ctx->g.V, n);
   kt_end(ctx, KC_LAYOUT, s, ev);
   OV_CHECK_LAUNCH(ctx, unpack ? "unpack_kernel" : "pack_kernel");
   return OV_OK;
@@ -202,11 +229,11 @@ int launch_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream
 
 int launch_overlap_epilogue(ov_ctx* ctx, const double2* b_aos, const double2* s_soa, double2* out_aos,
                             double m_q, int nrhs, cudaStream_t s) {
-  const size_t n = (size_t)nrhs * ctx->g.V * 12;
+  const size_t n = (size_t)nrhs * ((ctx->g.V + 31) / 32);
   cudaEvent_t ev;
   kt_begin(ctx, KC_LAYOUT, s, &ev);
-  overlap_epilogue_kernel<<<grid_for(n, 256), 256, 0, s>>>(b_aos, s_soa, out_aos, 0.5 * (1.0 + m_q),
-                                                           0.5 * (1.0 - m_q), ctx->g.V, nrhs);
+  overlap_epilogue_kernel<<<tile_grid(n), kTileNT, 0, s>>>(b_aos, s_soa, out_aos, 0.5 * (1.0 + m_q),
+                                                           0.5 * (1.0 - m_q), ctx->g.V, n);
   kt_end(ctx, KC_LAYOUT, s, ev);
   OV_CHECK_LAUNCH(ctx, "overlap_epilogue_kernel");
   return OV_OK;

@@ -7,8 +7,9 @@
 //  * 12-real link compression: only rows 0 and 1 of each SU(3) link are stored;
 //    row 2 = conj(row0 x row1) (unitarity and det U = 1), rebuilt in registers.
 // With RT = 4 and compression the compulsory traffic is 192/4 + 192 = 240 B per site
-// and RHS.  The autotuner times the variants on the live problem once per
-// (lattice, nrhs) and keeps the fastest.
+// and RHS.  The autotuner (ov_apply_HW) times the variants, layout changes included, on
+// the live problem once per (lattice, nrhs) and keeps the fastest.
+#include <algorithm>
 #include <vector>
 
 #include "common.cuh"
@@ -207,52 +208,17 @@ static float2* compressed_links(ov_ctx* ctx, cudaStream_t s, int* st) {
   return c;
 }
 
-// Time every structure-of-arrays variant on the live data (3 launches each after a
-// warm-up); returns the best time per launch in ms and its index in *best.
-float hw32_time_soa_variants(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int* best) {
+// out = H_W in on planes with structure-of-arrays variant k.
+int launch_hw32_soa(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int k) {
   int st = OV_OK;
-  const float2* Uc = compressed_links(ctx, s, &st);
-  if (st != OV_OK) return 1e30f;
-  cudaEvent_t a, b;
-  cudaEventCreate(&a);
-  cudaEventCreate(&b);
-  const float diag = (float)(4.0 - ctx->m0);
-  float best_ms = 1e30f;
-  *best = 1;
-  for (int k = 0; k < kNCands; ++k) {
-    const Cand& c = kCands[k];
-    const float2* U = c.comp ? Uc : ctx->U32;
-    c.fn(in, out, U, ctx->g, diag, nrhs, s);  // warm
-    cudaEventRecord(a, s);
-    for (int rep = 0; rep < 3; ++rep) c.fn(in, out, U, ctx->g, diag, nrhs, s);
-    cudaEventRecord(b, s);
-    cudaEventSynchronize(b);
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, a, b);
-    if (cudaGetLastError() == cudaSuccess && ms / 3 < best_ms) {
-      best_ms = ms / 3;
-      *best = k;
-    }
-  }
-  cudaEventDestroy(a);
-  cudaEventDestroy(b);
-  return best_ms;
-}
-
-int launch_hw32_tuned(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int force_variant,
-                      int* used) {
-  int st = OV_OK;
-  const float2* Uc = compressed_links(ctx, s, &st);
-  if (st != OV_OK) return st;
-  int k = force_variant;
-  if (k < 0 || k >= kNCands) hw32_time_soa_variants(ctx, in, out, nrhs, s, &k);
   const Cand& c = kCands[k];
+  const float2* U = c.comp ? compressed_links(ctx, s, &st) : ctx->U32;
+  if (st != OV_OK) return st;
   cudaEvent_t ev;
   kt_begin(ctx, KC_DSLASH, s, &ev);
-  c.fn(in, out, c.comp ? Uc : ctx->U32, ctx->g, (float)(4.0 - ctx->m0), nrhs, s);
+  c.fn(in, out, U, ctx->g, (float)(4.0 - ctx->m0), nrhs, s);
   kt_end(ctx, KC_DSLASH, s, ev);
   OV_CHECK_LAUNCH(ctx, "hw32_tile_kernel");
-  if (used) *used = k;
   return OV_OK;
 }
 
@@ -341,59 +307,55 @@ __device__ __forceinline__ void hop_dir_s4(const float4* __restrict__ in, const 
 // registers, 97.3 us here).  The diagonal term is read before the hops, so that the x
 // and y neighbours, which share its cache lines, follow it through L1.
 constexpr int kS4NT = 128;
-__global__ void __launch_bounds__(kS4NT, 7) hw32_s4_kernel(const float4* __restrict__ in, float4* __restrict__ out,
+// The result goes to the canonical layout through shared memory.
+constexpr int kS4Row = 13;
+__global__ void __launch_bounds__(kS4NT, 7) hw32_s4_kernel(const float4* __restrict__ in, float2* __restrict__ out,
                                                            const float4* __restrict__ L, Geom g, float diag) {
-  const int s = blockIdx.x * kS4NT + threadIdx.x;
-  if (s >= g.V) return;
-  int c[4];
-  site_coords(g, s, c);
-  const int V = g.V;
-  const float4* inr = in + (size_t)blockIdx.y * 6 * V;
-  float4* outr = out + (size_t)blockIdx.y * 6 * V;
-  Cx<float> acc[12];
+  __shared__ float2 sh[kS4NT * kS4Row];
+  const int s0 = blockIdx.x * kS4NT, s = s0 + threadIdx.x, V = g.V;
+  if (s < V) {
+    int c[4];
+    site_coords(g, s, c);
+    const float4* inr = in + (size_t)blockIdx.y * 6 * V;
+    Cx<float> acc[12];
 #pragma unroll
-  for (int p = 0; p < 6; ++p) {
-    const int sp = p / 3, col = p % 3;
-    const float4 v = __ldg(inr + p * V + s);
-    acc[sp * 3 + col] = cscale(diag, Cx<float>{v.x, v.y});
-    acc[(sp + 2) * 3 + col] = cscale(diag, Cx<float>{v.z, v.w});
-  }
-  hop_dir_s4<0>(inr, L, g, s, c, acc);
-  hop_dir_s4<1>(inr, L, g, s, c, acc);
-  hop_dir_s4<2>(inr, L, g, s, c, acc);
-  hop_dir_s4<3>(inr, L, g, s, c, acc);
+    for (int p = 0; p < 6; ++p) {
+      const int sp = p / 3, col = p % 3;
+      const float4 v = __ldg(inr + p * V + s);
+      acc[sp * 3 + col] = cscale(diag, Cx<float>{v.x, v.y});
+      acc[(sp + 2) * 3 + col] = cscale(diag, Cx<float>{v.z, v.w});
+    }
+    hop_dir_s4<0>(inr, L, g, s, c, acc);
+    hop_dir_s4<1>(inr, L, g, s, c, acc);
+    hop_dir_s4<2>(inr, L, g, s, c, acc);
+    hop_dir_s4<3>(inr, L, g, s, c, acc);
 #pragma unroll
-  for (int p = 0; p < 6; ++p) {
-    const int sp = p / 3, col = p % 3;
-    const Cx<float> up = acc[sp * 3 + col], lo = acc[(sp + 2) * 3 + col];
-    // upper spin sp, lower spin sp + 2 (gamma5 = -1 on it)
-    outr[p * V + s] = make_float4(up.re, up.im, -lo.re, -lo.im);
+    for (int k = 0; k < 12; ++k)  // gamma5 = -1 on the lower spins
+      sh[threadIdx.x * kS4Row + k] = k < 6 ? make_float2(acc[k].re, acc[k].im) : make_float2(-acc[k].re, -acc[k].im);
   }
+  __syncthreads();
+  float2* po = out + ((size_t)blockIdx.y * V + s0) * 12;
+  const int n = min(kS4NT, V - s0) * 12;
+  for (int e = threadIdx.x; e < n; e += kS4NT) po[e] = sh[e / 12 * kS4Row + e % 12];
 }
 
-// canonical complex64 [rhs][site][12] <-> S4
-__global__ void pack_s4_kernel(const float2* __restrict__ aos, float4* __restrict__ s4, int V, int nrhs) {
-  const size_t n = (size_t)nrhs * 6 * V;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    const size_t site = t % V, q = t / V;
-    const size_t p = q % 6, r = q / 6;
-    const size_t sp = p / 3, col = p % 3;
-    const float2* a = aos + ((size_t)r * V + site) * 12;
-    const float2 u = a[sp * 3 + col], l = a[(sp + 2) * 3 + col];
-    s4[t] = make_float4(u.x, u.y, l.x, l.y);
-  }
-}
-
-__global__ void unpack_s4_kernel(const float4* __restrict__ s4, float2* __restrict__ aos, int V, int nrhs) {
-  const size_t n = (size_t)nrhs * 6 * V;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-    const size_t site = t % V, q = t / V;
-    const size_t p = q % 6, r = q / 6;
-    const size_t sp = p / 3, col = p % 3;
-    const float4 v = s4[t];
-    float2* a = aos + ((size_t)r * V + site) * 12;
-    a[sp * 3 + col] = make_float2(v.x, v.y);
-    a[(sp + 2) * 3 + col] = make_float2(v.z, v.w);
+// canonical complex64 [rhs][site][12] -> S4, one 32-site tile of a spinor at a time through
+// shared memory (as pack_kernel)
+__global__ void __launch_bounds__(384) pack_s4_kernel(const float2* __restrict__ aos, float4* __restrict__ s4, int V,
+                                                      size_t ntiles) {
+  __shared__ float2 sh[32 * kS4Row];
+  const int t = threadIdx.x, nt = (V + 31) / 32;
+  for (size_t b = blockIdx.x; b < ntiles; b += gridDim.x) {
+    const size_t r = b / nt, s0 = b % nt * 32;
+    if (s0 + t / 12 < V) sh[t / 12 * kS4Row + t % 12] = aos[(r * V + s0) * 12 + t];
+    __syncthreads();
+    const size_t s = s0 + t % 32;
+    const int p = t / 32;  // pair 3 spin + colour: components p and p + 6
+    if (p < 6 && s < V) {
+      const float2 u = sh[t % 32 * kS4Row + p], l = sh[t % 32 * kS4Row + p + 6];
+      s4[(r * 6 + p) * V + s] = make_float4(u.x, u.y, l.x, l.y);
+    }
+    __syncthreads();
   }
 }
 
@@ -420,14 +382,12 @@ int cap_grid32(size_t n) {
 }  // namespace
 
 int launch_pack_s4(ov_ctx* ctx, const float2* aos, float4* s4, int nrhs, cudaStream_t s) {
-  pack_s4_kernel<<<cap_grid32((size_t)nrhs * 6 * ctx->g.V), 256, 0, s>>>(aos, s4, ctx->g.V, nrhs);
+  const size_t n = (size_t)nrhs * ((ctx->g.V + 31) / 32);
+  cudaEvent_t ev;
+  kt_begin(ctx, KC_LAYOUT, s, &ev);
+  pack_s4_kernel<<<(unsigned)std::min<size_t>(n, 152 * 64), 384, 0, s>>>(aos, s4, ctx->g.V, n);
+  kt_end(ctx, KC_LAYOUT, s, ev);
   OV_CHECK_LAUNCH(ctx, "pack_s4_kernel");
-  return OV_OK;
-}
-
-int launch_unpack_s4(ov_ctx* ctx, const float4* s4, float2* aos, int nrhs, cudaStream_t s) {
-  unpack_s4_kernel<<<cap_grid32((size_t)nrhs * 6 * ctx->g.V), 256, 0, s>>>(s4, aos, ctx->g.V, nrhs);
-  OV_CHECK_LAUNCH(ctx, "unpack_s4_kernel");
   return OV_OK;
 }
 
@@ -444,7 +404,7 @@ const float4* s4_links(ov_ctx* ctx, cudaStream_t s, int* st) {
 }
 
 // out = H_W in on the S4 layout with the 12-real links, one RHS per thread.
-int launch_hw32_s4(ov_ctx* ctx, const float4* in, float4* out, int nrhs, cudaStream_t s) {
+int launch_hw32_s4(ov_ctx* ctx, const float4* in, float2* out, int nrhs, cudaStream_t s) {
   int st = OV_OK;
   const float4* l3 = s4_links(ctx, s, &st);
   if (st != OV_OK) return st;

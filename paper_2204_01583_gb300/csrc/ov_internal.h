@@ -175,12 +175,10 @@ int launch_unpack32(ov_ctx* ctx, const float2* soa, float2* aos, int nrhs, cudaS
 // out (SoA) = H_W in (SoA)
 int launch_hw64(ov_ctx* ctx, const double2* in, double2* out, int nrhs, cudaStream_t s);
 int launch_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s);
-// FP32 multi-RHS stencil (dslash32.cu): variant -1 = autotuned
-int launch_hw32_tuned(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int force_variant,
-                      int* used);
+// FP32 multi-RHS stencil on planes (dslash32.cu), structure-of-arrays variant k
+int launch_hw32_soa(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int k);
 int hw32_variant_count();  // SoA variants; index hw32_variant_count() is the paired kernel
 void hw32_variant_info(int k, int* rt, int* comp, int* nt);
-float hw32_time_soa_variants(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int* best);
 // double-float links for the FP32-pair solve (dslash.cu)
 int ensure_links_df(ov_ctx* ctx, cudaStream_t s);
 // Fixed-point links (dslash.cu): enqueues them and the copy of the check's verdict to
@@ -188,14 +186,12 @@ int ensure_links_df(ov_ctx* ctx, cudaStream_t s);
 bool launch_links_fx(ov_ctx* ctx, cudaStream_t s);
 // out = H_W in, FP64 fields (canonical or planes) through integers (hw64.cu); needs fx_ok
 int launch_hw64_fx(ov_ctx* ctx, const double2* in, double2* out, int nrhs, bool canonical, cudaStream_t s);
-// spin-paired float4 FP32 layout (dslash32.cu)
+// spin-paired float4 FP32 layout (dslash32.cu) and paired FP32 layout (pair32.cu): packing from
+// the canonical layout, H_W to the canonical layout
 int launch_pack_s4(ov_ctx* ctx, const float2* aos, float4* s4, int nrhs, cudaStream_t s);
-int launch_unpack_s4(ov_ctx* ctx, const float4* s4, float2* aos, int nrhs, cudaStream_t s);
-int launch_hw32_s4(ov_ctx* ctx, const float4* in, float4* out, int nrhs, cudaStream_t s);
-// paired FP32 layout (pair32.cu)
+int launch_hw32_s4(ov_ctx* ctx, const float4* in, float2* out, int nrhs, cudaStream_t s);
 int launch_pack_pair32(ov_ctx* ctx, const float2* aos, float4* pr, int nrhs, cudaStream_t s);
-int launch_unpack_pair32(ov_ctx* ctx, const float4* pr, float2* aos, int nrhs, cudaStream_t s);
-int launch_hw_pair12(ov_ctx* ctx, const float4* in, float4* out, int npair, int form, cudaStream_t s);
+int launch_hw_pair12(ov_ctx* ctx, const float4* in, float2* out, int nrhs, int form, cudaStream_t s);
 const float4* s4_links(ov_ctx* ctx, cudaStream_t s, int* st);
 // out(AoS) = (1+m)/2 b(AoS) + (1-m)/2 gamma5 s(SoA)
 int launch_overlap_epilogue(ov_ctx* ctx, const double2* b_aos, const double2* s_soa, double2* out_aos,
