@@ -19,8 +19,10 @@ void ellipse_rule(int n_q, double gamma, double rho, double alpha, int form, std
     // single contour: 2 P - 1; pair: + P_{Gamma+} - P_{Gamma-}
     const double scale = (form == OV_CONTOUR_PAIR) ? (k == 0 ? 1.0 : -1.0) : 2.0;
     for (int j = 1; j <= n_q; ++j) {
-      const double th = 2.0 * M_PI * (j - 0.5) / n_q;
-      const double ct = std::cos(th), sn = std::sin(th);
+      // node n_q + 1 - j is the conjugate of node j, exactly
+      const int jj = std::min(j, n_q + 1 - j);
+      const double th = 2.0 * M_PI * (jj - 0.5) / n_q;
+      const double ct = std::cos(th), sn = j == jj ? std::sin(th) : -std::sin(th);
       z.push_back(make_double2(centre + rho * ct, rho * alpha * sn));
       c.push_back(make_double2(scale * rho * alpha * ct / n_q, scale * rho * sn / n_q));
     }

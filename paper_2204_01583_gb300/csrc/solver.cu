@@ -1644,39 +1644,67 @@ __global__ void __launch_bounds__(NT2) fx_quantize_kernel(const __grid_constant_
 //   f_k = z - alpha_k,  f_i = z - alpha_i - beta_i^2 / f_{i+1};   y_1 = ||b|| / f_1,  y_{i+1} =
 //   beta_i y_i / f_{i+1}
 // (the factorisation from the last row up: |Im f_i| >= |Im z|).  Y[r][i][j] holds 1 / f, then y
-// / ||X_i||.  A serial chain of k complex reciprocals per thread, all nodes and sources at once
-// (on the host it took 8 us per source and node at 8^4, 2 of 10 ms of a 4-source solve).
+// / ||X_i||.  Two serial chains of k steps, all nodes and sources at once (on the host they
+// took 8 us per source and node at 8^4, 2 of 10 ms of a 4-source solve); the recurrence
+// scalars come from shared memory and the pivots of the way down a batch ahead, so that no
+// step waits for L2.
+constexpr int kCoefChunk = 512;
 __global__ void __launch_bounds__(32) fx_node_coef_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
                                                           double2* __restrict__ Y) {
-  const int r = blockIdx.y, j = blockIdx.x * 32 + threadIdx.x;
-  if (j >= ns) return;
+  __shared__ double sa[kCoefChunk], sb[kCoefChunk];
+  const int r = blockIdx.y, lane = threadIdx.x, j = min(blockIdx.x * 32 + lane, ns - 1);
+  const bool on = blockIdx.x * 32 + lane < ns;
   const SrcState* S = a.src + r;
   const int mi = a.prm->max_iter, k = S->iter - 1;
   const double *al = a.hist_a + (size_t)r * mi, *be = a.hist_b + (size_t)r * mi, *n2 = a.hist_n2 + (size_t)r * mi;
   double2* y = Y + (size_t)r * mi * ns + j;
   const double2 z = a.z[(size_t)r * ns + j];
   double2 f = make_double2(0.0, 0.0);  // 1 / f_{i+1}
-#pragma unroll 4
-  for (int i = k - 1; i >= 0; --i) {
-    const double b = be[i], b2 = i + 1 < k ? b * b : 0.0;
-    const double dx = fma(-b2, f.x, z.x - al[i]), dy = fma(-b2, f.y, z.y);
-    const double inv = __drcp_rn(fma(dx, dx, dy * dy));
-    f = make_double2(dx * inv, -dy * inv);
-    y[(size_t)i * ns] = f;
+  for (int hi = k; hi > 0; hi -= kCoefChunk) {
+    const int lo = max(0, hi - kCoefChunk);
+    __syncwarp();
+    for (int i = lo + lane; i < hi; i += 32) {
+      sa[i - lo] = al[i];
+      sb[i - lo] = i + 1 < k ? be[i] * be[i] : 0.0;
+    }
+    __syncwarp();
+    for (int i = hi - 1; i >= lo; --i) {
+      const double b2 = sb[i - lo], dx = fma(-b2, f.x, z.x - sa[i - lo]), dy = fma(-b2, f.y, z.y);
+      const double inv = __drcp_rn(fma(dx, dx, dy * dy));
+      f = make_double2(dx * inv, -dy * inv);
+      if (on) y[(size_t)i * ns] = f;
+    }
   }
   double2 v = make_double2(S->bnorm, 0.0);
-#pragma unroll 4
-  for (int i = 0; i < k; ++i) {
-    const double2 g = y[(size_t)i * ns];
-    const double b = i > 0 ? be[i - 1] : 1.0, rn = rsqrt(n2[i]);
-    v = cmul(v, make_double2(b * g.x, b * g.y));
-    y[(size_t)i * ns] = make_double2(v.x * rn, v.y * rn);
+  for (int lo = 0; lo < k; lo += kCoefChunk) {
+    const int hi = min(k, lo + kCoefChunk);
+    __syncwarp();
+    for (int i = lo + lane; i < hi; i += 32) {
+      sa[i - lo] = rsqrt(n2[i]);
+      sb[i - lo] = i > 0 ? be[i - 1] : 1.0;
+    }
+    __syncwarp();
+    constexpr int B = 8;
+    for (int i0 = lo; i0 < hi; i0 += B) {
+      double2 g[B];
+#pragma unroll
+      for (int t = 0; t < B; ++t) g[t] = y[(size_t)min(i0 + t, k - 1) * ns];
+#pragma unroll
+      for (int t = 0; t < B; ++t) {
+        if (i0 + t >= hi) break;
+        const double b = sb[i0 + t - lo], rn = sa[i0 + t - lo];
+        v = cmul(v, make_double2(b * g[t].x, b * g[t].y));
+        if (on) y[(size_t)(i0 + t) * ns] = make_double2(v.x * rn, v.y * rn);
+      }
+    }
   }
 }
 
-// w[0..k) at stride `ld` as integers of at most 2^57 (out), k from the whole block; returns the
-// factor of sum_i w_i X_i given as hh + x 2^-30 = 2^-60 sum_i out_i X_i.  *real: all imaginary
-// parts vanish up to rounding.
+// Coefficients w[0..k) as integers: at most 2^57, and so small that a sum over all k of
+// 2^-60 out_i X_i stays below 2^62 (k <= kFxSumMax; longer sums are cut into pieces of that
+// length).  Returns the factor that undoes the scale.  *real: all imaginary parts vanish up
+// to rounding.
+constexpr int kFxSumMax = 256;
 template <int NT, typename F>
 __device__ __forceinline__ double fx_quantise(F w, int k, int4* out, bool* real, int* sh) {
   int mr = 0, mi = 0;  // high words of the largest |re|, |im|
@@ -1689,7 +1717,9 @@ __device__ __forceinline__ double fx_quantise(F w, int k, int4* out, bool* real,
   __syncthreads();
   mi = block_max<NT>(mi, sh);
   *real = __hiloint2double(mi, 0) <= 1e-14 * __hiloint2double(mr, 0);
-  const int m = max(mr, mi) >> 20, e = m > 0 && m < 0x7ff ? 56 - (m - 1023) : 56;
+  // a complex sum adds two products per term: out < 2^(63 - log2 k)
+  const int bits = min(57, 62 - (31 - __clz(max(min(k, kFxSumMax), 1))));
+  const int m = max(mr, mi) >> 20, e = m > 0 && m < 0x7ff ? bits - 1 - (m - 1023) : bits - 1;
   for (int i = threadIdx.x; i < k; i += NT) {
     const double2 v = w(i);
     const FX re = fx_split(__double2ll_rn(ldexp(v.x, e))), im = fx_split(__double2ll_rn(ldexp(v.y, e)));
@@ -1703,21 +1733,15 @@ struct FxSumInfo {
   int k, real;
 };
 
-// G[r][i] = sum_j c_j Y[r][i][j] (one block per source) in integers.  Real coefficients come
-// from a node list closed under conjugation (basis_sum_kernel).
-constexpr int kCoefNT = 512;
-__global__ void __launch_bounds__(kCoefNT) fx_sum_coef_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
-                                                              const double2* __restrict__ Y, double2* __restrict__ g,
-                                                              int4* __restrict__ G, FxSumInfo* __restrict__ info) {
-  __shared__ int sh[kCoefNT / 32];
-  const int r = blockIdx.x, mi = a.prm->max_iter, k = a.src[r].iter - 1;
+// g[r][i] = sum_j c_j Y[r][i][j], a warp per i
+__global__ void __launch_bounds__(256) fx_sum_nodes_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
+                                                           const double2* __restrict__ Y, double2* __restrict__ g) {
+  const int r = blockIdx.y, mi = a.prm->max_iter, k = a.src[r].iter - 1, lane = threadIdx.x & 31;
   const double2* c = a.c + (size_t)r * ns;
-  g += (size_t)r * mi;
-  // a warp per i: lanes over the nodes
-  for (int i = threadIdx.x >> 5; i < k; i += kCoefNT / 32) {
+  for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < k; i += gridDim.x * 8) {
     const double2* y = Y + ((size_t)r * mi + i) * ns;
     double2 t = make_double2(0.0, 0.0);
-    for (int j = threadIdx.x & 31; j < ns; j += 32) {
+    for (int j = lane; j < ns; j += 32) {
       const double2 v = cmul(c[j], y[j]);
       t.x += v.x;
       t.y += v.y;
@@ -1727,11 +1751,21 @@ __global__ void __launch_bounds__(kCoefNT) fx_sum_coef_kernel(const __grid_const
       t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
       t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
     }
-    if ((threadIdx.x & 31) == 0) g[i] = t;
+    if (lane == 0) g[(size_t)r * mi + i] = t;
   }
-  __syncthreads();
+}
+
+// G = g in integers, one block per source.  Real coefficients come from a node list closed
+// under conjugation (basis_sum_kernel).
+constexpr int kCoefNT = 256;
+__global__ void __launch_bounds__(kCoefNT) fx_sum_quant_kernel(const __grid_constant__ SolveArgs<FX> a,
+                                                               const double2* __restrict__ g, int4* __restrict__ G,
+                                                               FxSumInfo* __restrict__ info) {
+  __shared__ int sh[kCoefNT / 32];
+  const int r = blockIdx.x, mi = a.prm->max_iter, k = a.src[r].iter - 1;
   bool real;
-  const double sc = fx_quantise<kCoefNT>([&](int i) { return g[i]; }, k, G + (size_t)r * mi, &real, sh);
+  const double sc =
+      fx_quantise<kCoefNT>([&](int i) { return g[(size_t)r * mi + i]; }, k, G + (size_t)r * mi, &real, sh);
   if (threadIdx.x == 0) info[r] = {sc, k, real ? 1 : 0};
 }
 
@@ -1748,30 +1782,31 @@ __global__ void __launch_bounds__(128) fx_node_quant_kernel(const __grid_constan
   if (threadIdx.x == 0) scale[o] = sc;
 }
 
-// K basis vectors' products added exactly, the group's sum in FP64
+// K basis vectors' products, their cross terms within 63 bits, added to re and im in units of
+// 2^60 over the scales.
 template <bool REAL, int K>
 __device__ __forceinline__ void fx_sum_group(const int4* __restrict__ w, const int4* __restrict__ B, size_t n12, int n,
-                                             double& re, double& im) {
-  long long rh = 0, rx = kFxHalf30, ih = 0, ix = kFxHalf30;
+                                             long long& re, long long& im) {
+  long long rx = kFxHalf30, ix = kFxHalf30;
 #pragma unroll
   for (int i = 0; i < K; ++i) {
     if (i < n) {
       const int4 g = __ldg(w + i), x = __ldg(B + (size_t)i * n12);
-      fx_mac(rh, rx, g.x, g.y, x.x, x.y);
-      fx_mac(ih, ix, g.x, g.y, x.z, x.w);
+      fx_mac(re, rx, g.x, g.y, x.x, x.y);
+      fx_mac(im, ix, g.x, g.y, x.z, x.w);
       if (!REAL) {
-        fx_mac(rh, rx, -g.z, -g.w, x.z, x.w);
-        fx_mac(ih, ix, g.z, g.w, x.x, x.y);
+        fx_mac(re, rx, -g.z, -g.w, x.z, x.w);
+        fx_mac(im, ix, g.z, g.w, x.x, x.y);
       }
     }
   }
-  re += (double)fx_value(rh, rx);
-  im += (double)fx_value(ih, ix);
+  re += rx >> 30;
+  im += ix >> 30;
 }
 
-// sum[r][e] += scale_r sum_i G_i X_i[e] (basis_sum_kernel in fixed point), G_i = g_i / ||X_i|| of
-// at most 2^57: groups of 8 products are summed exactly (their cross terms fit 63 bits), the
-// groups in FP64.  Reads 16 B per basis vector and element: HBM-bound.
+// sum[r][e] += scale_r sum_i G_i X_i[e] (basis_sum_kernel in fixed point), G_i = g_i / ||X_i||:
+// exact integer sums of up to kFxSumMax vectors.  Reads 16 B per basis vector and element:
+// HBM-bound.
 __global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restrict__ basis, int nslots,
                                                            const int4* __restrict__ G, int ldg,
                                                            const FxSumInfo* __restrict__ info,
@@ -1786,13 +1821,19 @@ __global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restric
   const FxSumInfo f = info[r];
   constexpr int K = 8;
   double re = 0.0, im = 0.0;
-  int i = 0;
-  if (f.real) {
-    for (; i + K <= f.k; i += K) fx_sum_group<true, K>(w + i, B + (size_t)i * n12, n12, K, re, im);
-  } else {
-    for (; i + K <= f.k; i += K) fx_sum_group<false, K>(w + i, B + (size_t)i * n12, n12, K, re, im);
+  for (int i0 = 0; i0 < f.k; i0 += kFxSumMax) {
+    const int end = min(f.k, i0 + kFxSumMax);
+    long long sr = 0, si = 0;
+    int i = i0;
+    if (f.real) {
+      for (; i + K <= end; i += K) fx_sum_group<true, K>(w + i, B + (size_t)i * n12, n12, K, sr, si);
+    } else {
+      for (; i + K <= end; i += K) fx_sum_group<false, K>(w + i, B + (size_t)i * n12, n12, K, sr, si);
+    }
+    if (i < end) fx_sum_group<false, K>(w + i, B + (size_t)i * n12, n12, end - i, sr, si);
+    re += (double)sr;
+    im += (double)si;
   }
-  if (i < f.k) fx_sum_group<false, K>(w + i, B + (size_t)i * n12, n12, f.k - i, re, im);
   double2* so = sum + ((size_t)r * 12 + tk % 12) * V + site;
   double2 sv = *so;
   sv.x = fma(f.scale, re, sv.x);
@@ -1800,58 +1841,82 @@ __global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restric
   *so = sv;
 }
 
-// Per-node solutions from a fixed-point basis (basis_nodes_kernel): Y per (source, node) with
-// its own scale, JT nodes per thread.
-template <int JT>
+// Per-node solutions from a fixed-point basis: x_j = A + i B with A = sum_i Re(Y_i) X_i, B = sum_i
+// Im(Y_i) X_i.  A node whose conjugate is also in the list needs no sums of its own: its
+// coefficients are the conjugates (T_k is real), its solution A - i B.  Two nodes or pairs per
+// thread (slot: node, partner or -1), Y per (source, node) with its own scale.  Bound by wide
+// multiply-adds, 12 per slot, element and basis vector.  (8^4, 2 sources, 48 nodes, 352
+// vectors: 4.4 ms with every node on its own and groups of 8 summed in FP64.)
 __global__ void __launch_bounds__(256) fx_basis_nodes_kernel(const int4* __restrict__ basis, int nslots,
                                                              const int4* __restrict__ Y,
                                                              const double* __restrict__ scale, int ns, int ldy,
-                                                             const FxSumInfo* __restrict__ info, int j0, int nc,
+                                                             const FxSumInfo* __restrict__ info,
+                                                             const int2* __restrict__ slot, int nslot, int j0, int nc,
                                                              double2* __restrict__ X, int V) {
-  const int r = blockIdx.y, jt = blockIdx.z * JT;
+  constexpr int JT = 2, K = 8;
+  const int r = blockIdx.y, q0 = blockIdx.z * JT;
   const size_t n12 = 12 * fx_padded(V), e = (size_t)blockIdx.x * blockDim.x + threadIdx.x, tk = e / kFxTile;
-  if (e >= n12 || jt >= nc) return;
+  if (e >= n12) return;
   const size_t site = tk / 12 * kFxTile + e % kFxTile;
   if (site >= V) return;
   const int4* B = basis + (size_t)r * nslots * n12 + n12 + e;
-  const int4* Yr = Y + ((size_t)r * ns + j0 + jt) * ldy;
-  const int k = info[r].k, nj = min(JT, nc - jt);
-  double re[JT], im[JT];
+  const int k = info[r].k;
+  int2 nd[JT];
+  const int4* y[JT];
 #pragma unroll
-  for (int t = 0; t < JT; ++t) re[t] = im[t] = 0.0;
-  for (int i0 = 0; i0 < k; i0 += 8) {
-    long long rh[JT], rx[JT], ih[JT], ix[JT];
+  for (int t = 0; t < JT; ++t) {
+    nd[t] = slot[min(q0 + t, nslot - 1)];
+    y[t] = Y + ((size_t)r * ns + nd[t].x) * ldy;
+  }
+  double s[JT][4];  // A.re, A.im, B.re, B.im
 #pragma unroll
-    for (int t = 0; t < JT; ++t) {
-      rh[t] = ih[t] = 0;
-      rx[t] = ix[t] = kFxHalf30;
-    }
-    const int n = min(8, k - i0);
-    for (int i = 0; i < n; ++i) {
-      const int4 x = __ldg(B + (size_t)(i0 + i) * n12);
+  for (int t = 0; t < JT; ++t)
 #pragma unroll
-      for (int t = 0; t < JT; ++t) {
-        if (t < nj) {
-          const int4 y = __ldg(Yr + (size_t)t * ldy + i0 + i);
-          fx_mac(rh[t], rx[t], y.x, y.y, x.x, x.y);
-          fx_mac(rh[t], rx[t], -y.z, -y.w, x.z, x.w);
-          fx_mac(ih[t], ix[t], y.x, y.y, x.z, x.w);
-          fx_mac(ih[t], ix[t], y.z, y.w, x.x, x.y);
+    for (int c = 0; c < 4; ++c) s[t][c] = 0.0;
+  for (int i0 = 0; i0 < k; i0 += kFxSumMax) {
+    const int end = min(k, i0 + kFxSumMax);
+    long long h[JT][4] = {};
+    for (int i = i0; i < end; i += K) {
+      long long x[JT][4];
+#pragma unroll
+      for (int t = 0; t < JT; ++t)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) x[t][c] = kFxHalf30;
+      auto add = [&](int m) {
+        const int4 u = __ldg(B + (size_t)(i + m) * n12);
+#pragma unroll
+        for (int t = 0; t < JT; ++t) {
+          const int4 w = __ldg(y[t] + i + m);
+          fx_mac(h[t][0], x[t][0], w.x, w.y, u.x, u.y);
+          fx_mac(h[t][1], x[t][1], w.x, w.y, u.z, u.w);
+          fx_mac(h[t][2], x[t][2], w.z, w.w, u.x, u.y);
+          fx_mac(h[t][3], x[t][3], w.z, w.w, u.z, u.w);
         }
+      };
+      if (i + K <= end) {
+#pragma unroll
+        for (int m = 0; m < K; ++m) add(m);
+      } else {
+        for (int m = 0; i + m < end; ++m) add(m);
       }
+#pragma unroll
+      for (int t = 0; t < JT; ++t)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) h[t][c] += x[t][c] >> 30;
     }
 #pragma unroll
-    for (int t = 0; t < JT; ++t) {
-      re[t] += (double)fx_value(rh[t], rx[t]);
-      im[t] += (double)fx_value(ih[t], ix[t]);
-    }
+    for (int t = 0; t < JT; ++t)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) s[t][c] += (double)h[t][c];
   }
 #pragma unroll
   for (int t = 0; t < JT; ++t) {
-    if (t < nj) {
-      const double sc = scale[(size_t)r * ns + j0 + jt + t];
-      X[(((size_t)r * nc + jt + t) * 12 + tk % 12) * V + site] = make_double2(sc * re[t], sc * im[t]);
-    }
+    if (q0 + t >= nslot) break;
+    const double sc = scale[(size_t)r * ns + nd[t].x];
+    double2* o = X + ((size_t)r * nc * 12 + tk % 12) * V + site;
+    const size_t st = (size_t)12 * V;
+    o[(nd[t].x - j0) * st] = make_double2(sc * (s[t][0] - s[t][3]), sc * (s[t][1] + s[t][2]));
+    if (nd[t].y >= 0) o[(nd[t].y - j0) * st] = make_double2(sc * (s[t][0] + s[t][3]), sc * (s[t][1] - s[t][2]));
   }
 }
 
@@ -2583,10 +2648,11 @@ static int fx_lanczos(ov_ctx* ctx, SolveWs<FX>& w, FxCoef& f, const double2* b_s
   cudaEvent_t ev;
   kt_begin(ctx, KC_MISC, s, &ev);
   fx_node_coef_kernel<<<dim3((ns + 31) / 32, nsrc), 32, 0, s>>>(w.a, ns, f.Y);
-  fx_sum_coef_kernel<<<nsrc, kCoefNT, 0, s>>>(w.a, ns, f.Y, f.g, f.G, f.info);
+  fx_sum_nodes_kernel<<<dim3(std::min((cap + 7) / 8, 64), nsrc), 256, 0, s>>>(w.a, ns, f.Y, f.g);
+  fx_sum_quant_kernel<<<nsrc, kCoefNT, 0, s>>>(w.a, f.g, f.G, f.info);
   kt_end(ctx, KC_MISC, s, ev);
   OV_CHECK_LAUNCH(ctx, "fx_node_coef_kernel");
-  *launches += 2.0;
+  *launches += 3.0;
   return OV_OK;
 }
 
@@ -2946,11 +3012,34 @@ int nodes_coef<FX>(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const st
   const int fst = finish_solve<FX>(ctx, w, nsrc, ns, zh, ch, so, s);
   if (fst != OV_OK && !(fst == OV_ERR_NOT_CONVERGED && cap >= o.max_iter)) return OV_ERR_INVALID_ARG;
   fx_node_quant_kernel<<<dim3(ns, nsrc), 128, 0, s>>>(w.a, ns, f.Y, Yq, Ysc);
-  constexpr int JT = 4;
+  int2* slotd = (int2*)ws_get(ctx, "fxs.slot", sizeof(int2) * ns, &st);
+  if (st != OV_OK) return st;
+  std::vector<int2> slot;
   for (int j0 = 0; j0 < ns; j0 += chunk) {
     const int nc = std::min(chunk, ns - j0);
-    fx_basis_nodes_kernel<JT><<<dim3((unsigned)((w.nvec + 255) / 256), nsrc, (nc + JT - 1) / JT), 256, 0, s>>>(
-        w.a.ring, cap + 3, Yq, Ysc, ns, cap, f.info, j0, nc, X, ctx->g.V);
+    // pairs of conjugate nodes (in every source's list) within the chunk
+    slot.clear();
+    std::vector<char> used(nc, 0);
+    for (int j = 0; j < nc; ++j) {
+      if (used[j]) continue;
+      int2 p = make_int2(j0 + j, -1);
+      for (int q = j + 1; q < nc && p.y < 0; ++q) {
+        bool conj = !used[q];
+        for (int r = 0; r < nsrc && conj; ++r) {
+          const double2 u = zh[(size_t)r * ns + j0 + j], v = zh[(size_t)r * ns + j0 + q];
+          conj = u.x == v.x && u.y == -v.y;
+        }
+        if (conj) p.y = j0 + q;
+      }
+      if (p.y >= 0) used[p.y - j0] = 1;
+      slot.push_back(p);
+    }
+    const cudaError_t e =
+        cudaMemcpyAsync(slotd, slot.data(), sizeof(int2) * slot.size(), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy node pairs");
+    const int nslot = (int)slot.size();
+    fx_basis_nodes_kernel<<<dim3((unsigned)((w.nvec + 255) / 256), nsrc, (nslot + 1) / 2), 256, 0, s>>>(
+        w.a.ring, cap + 3, Yq, Ysc, ns, cap, f.info, slotd, nslot, j0, nc, X, ctx->g.V);
     OV_CHECK_LAUNCH(ctx, "fx_basis_nodes_kernel");
     if ((st = per_chunk(j0, nc)) != OV_OK) return st;
   }
