@@ -178,6 +178,7 @@ struct SolveArgs {
   T* p;               // [src][nshift][12V]
   T* x;               // [src][nshift][12V] or null
   double2* sacc;      // [src][12V] weighted sum (FP64) or null
+  double2* sgrp;      // [src][groups - 1][12V] its parts from K2's other node groups or null
   T* ssum;            // [src][12V] regeneration-pass sum in the vector type (double-float) or null
   const T* stencil;   // optional pre-applied H U_i for K1 ([src][12V]) or null
   SrcState* src;
@@ -500,12 +501,16 @@ __global__ void __launch_bounds__(NT2) lanczos_update_kernel(SolveArgs<R> a) {
   T* base = a.ring + (size_t)r * a.prm->nslots * n12;
   const T* Ui = base + lz_slot(a.prm, i) * n12;
   T* W = base + lz_slot(a.prm, i + 1) * n12;
+  // node groups (blockIdx.z, k2_groups): group z takes the active nodes z, z + groups, ...;
+  // the first one also advances the Lanczos vector, the only reader and writer of w
+  const int z = blockIdx.z, nz = gridDim.z;
   const int na = a.prm->vec_shifts ? S->n_act : 0;
   const R inv_nR = scal<R>(S->inv_n, S->df + 0), anR = scal<R>(S->alpha_n, S->df + 6);
   typename Acc<R>::T nrm = Acc<R>::zero();
   double nrm_im = 0.0;  // FP64 vectors: the imaginary parts in a second, independent FMA chain
   size_t e0 = (size_t)blockIdx.x * NT2 + threadIdx.x;
   const size_t gs = (size_t)gridDim.x * NT2;
+  if (z >= na && z > 0) e0 = n12;  // fewer active nodes than groups
   if constexpr (!std::is_same<R, float>::value) {
     // scalar-only forms (no per-node vectors): four elements per thread in flight, their
     // loads issued before any arithmetic (the arithmetic and HBM overlap across them)
@@ -535,13 +540,15 @@ __global__ void __launch_bounds__(NT2) lanczos_update_kernel(SolveArgs<R> a) {
   // grid-stride: a few blocks per source (fewer partials and atomics than one block per chunk)
   for (size_t e = e0; e < n12; e += gs) {
     const Cx<R> ui = ld<R>(Ui + e);
-    const Cx<R> u = lz_next<R>(ld<R>(W + e), ui, anR);
-    st<R>(W + e, u);
-    if constexpr (std::is_same<R, double>::value) {
-      nrm = fma(u.re, u.re, nrm);
-      nrm_im = fma(u.im, u.im, nrm_im);
-    } else {
-      nrm = Acc<R>::dot(nrm, u, u);
+    if (z == 0) {
+      const Cx<R> u = lz_next<R>(ld<R>(W + e), ui, anR);
+      st<R>(W + e, u);
+      if constexpr (std::is_same<R, double>::value) {
+        nrm = fma(u.re, u.re, nrm);
+        nrm_im = fma(u.im, u.im, nrm_im);
+      } else {
+        nrm = Acc<R>::dot(nrm, u, u);
+      }
     }
     Cx<R> v = ui;  // v_i = U_i / ||U_i||, read only by the per-node direction updates
     if (na > 0) v = lz_v<R>(ui, inv_nR);
@@ -551,7 +558,7 @@ __global__ void __launch_bounds__(NT2) lanczos_update_kernel(SolveArgs<R> a) {
     const typename Coef<R>::T* al = a.act_l + (size_t)r * ns;
     const typename Coef<R>::T* acz = a.act_cz + (size_t)r * ns;
     const typename Coef<R>::T* az = a.act_z + (size_t)r * ns;
-    for (int k = 0; k < na; ++k) {
+    for (int k = z; k < na; k += nz) {
       const int j = __ldg(idx + k);
       T* P = a.p + ((size_t)r * ns + j) * n12 + e;
       Cx<R> pv = v;
@@ -575,7 +582,7 @@ __global__ void __launch_bounds__(NT2) lanczos_update_kernel(SolveArgs<R> a) {
         sre = (double)sdf.re;
         sim = (double)sdf.im;
       }
-      double2* Sx = a.sacc + (size_t)r * n12 + e;
+      double2* Sx = (z == 0 ? a.sacc + (size_t)r * n12 : a.sgrp + ((size_t)r * (nz - 1) + z - 1) * n12) + e;
       double2 sv = *Sx;
       sv.x += sre;
       sv.y += sim;
@@ -583,11 +590,13 @@ __global__ void __launch_bounds__(NT2) lanczos_update_kernel(SolveArgs<R> a) {
     }
   }
   if constexpr (std::is_same<R, double>::value) nrm += nrm_im;
-  double bs = Acc<R>::template total<NT2>(nrm, sh);
+  double bs = 0.0;
+  if (z == 0) bs = Acc<R>::template total<NT2>(nrm, sh);
+  __syncthreads();
   if (threadIdx.x == 0) {
-    a.part2[(size_t)r * gridDim.x + blockIdx.x] = bs;
+    if (z == 0) a.part2[(size_t)r * gridDim.x + blockIdx.x] = bs;
     __threadfence();
-    last = (atomicAdd(a.cnt + 2 * r + 1, 1u) == gridDim.x - 1);
+    last = (atomicAdd(a.cnt + 2 * r + 1, 1u) == gridDim.x * nz - 1);
   }
   __syncthreads();
   if (!last) return;
@@ -1981,6 +1990,7 @@ template <typename R>
 struct SolveWs {
   SolveArgs<R> a{};
   int nblk1 = 0, nblk2 = 0, nblk2u = 0;
+  int ngrp = 1;  // K2's node groups
   int nslots = 3;
   size_t nvec = 0;   // elements of one Lanczos vector (12 V, padded in fixed point)
   int nshift = 0;
@@ -2000,6 +2010,7 @@ SolveArgs<R> args_for_sources(const SolveWs<R>& w, int r0) {
   if (a.p) a.p += r * ns * n12;
   if (a.x) a.x += r * ns * n12;
   if (a.sacc) a.sacc += r * n12;
+  if (a.sgrp) a.sgrp += r * (w.ngrp - 1) * n12;
   if (a.ssum) a.ssum += r * n12;
   if (a.stencil) a.stencil += r * n12;
   a.src += r;
@@ -2087,6 +2098,15 @@ int capture_groups(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int G, F body, cu
   return OV_OK;
 }
 
+// Node groups of K2 with per-node vectors: small vectors leave most SMs idle while each block
+// runs every node through its SM's FP64 pipe.  The nodes then go over the grid's third
+// dimension until it holds four blocks per SM (the parts of the weighted sum, one per group
+// but the first, take at most 2.5 MB).  4^4, 1 source, 32 nodes: an iteration took 39 us with
+// the 12 blocks of one group and takes 26.5 us with 32 groups.
+inline int k2_groups(int nblk, int nsrc, int ns) {
+  return std::max(1, std::min(ns, 4 * 152 / std::max(1, nblk * nsrc)));
+}
+
 template <typename R>
 int setup_ws(ov_ctx* ctx, int nsrc, int ns, bool want_x, bool want_sacc, bool want_hist, int max_iter,
              SolveWs<R>* w, const char* tag, int nslots = 3, bool want_p = true) {
@@ -2118,6 +2138,10 @@ int setup_ws(ov_ctx* ctx, int nsrc, int ns, bool want_x, bool want_sacc, bool wa
   a.p = (ns && want_p) ? (T*)ws_get(ctx, (t + ".p").c_str(), sizeof(T) * n12 * (size_t)nsrc * ns, &st) : nullptr;
   a.x = (want_x && ns) ? (T*)ws_get(ctx, (t + ".x").c_str(), sizeof(T) * n12 * (size_t)nsrc * ns, &st) : nullptr;
   a.sacc = want_sacc ? (double2*)ws_get(ctx, (t + ".sacc").c_str(), sizeof(double2) * n12 * nsrc, &st) : nullptr;
+  w->ngrp = a.p && a.sacc ? k2_groups(w->nblk2u, nsrc, ns) : 1;
+  a.sgrp = w->ngrp > 1 ? (double2*)ws_get(ctx, (t + ".sgrp").c_str(),
+                                          sizeof(double2) * n12 * (size_t)nsrc * (w->ngrp - 1), &st)
+                       : nullptr;
   a.src = (SrcState*)ws_get(ctx, (t + ".src").c_str(), sizeof(SrcState) * nsrc, &st);
   const size_t nsh = (size_t)nsrc * (ns > 0 ? ns : 1);
   a.sh = (ShiftState*)ws_get(ctx, (t + ".sh").c_str(), sizeof(ShiftState) * nsh, &st);
@@ -2212,7 +2236,7 @@ int launch_iteration(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, cudaStream_t s,
   int n = launch_k1<R>(w, w.a, nsrc, s);
   kt_end(ctx, KC_LANCZOS_HW, s, ev);
   kt_begin(ctx, KC_SHIFT_UPDATE, s, &ev);
-  lanczos_update_kernel<R><<<dim3(w.nblk2u, nsrc), NT2, 0, s>>>(w.a);
+  lanczos_update_kernel<R><<<dim3(w.nblk2u, nsrc, w.ngrp), NT2, 0, s>>>(w.a);
   kt_end(ctx, KC_SHIFT_UPDATE, s, ev);
   ++n;
   if (w.defer && (it + 1) % kNodeCheck == 0) {
@@ -2252,7 +2276,7 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
             constexpr bool beside = std::is_same<R, FX>::value;
             for (int k = 0; k < chunk; ++k) {
               graph_launches += launch_k1<R>(w, a, n, cs) + 1;
-              lanczos_update_kernel<R><<<dim3(w.nblk2u, n), NT2, 0, cs>>>(a);
+              lanczos_update_kernel<R><<<dim3(w.nblk2u, n, w.ngrp), NT2, 0, cs>>>(a);
               if (!w.defer || (k + 1) % kNodeCheck != 0) continue;
               graph_launches += 1.0;
               if (beside) {
@@ -2352,6 +2376,8 @@ int init_solve(ov_ctx* ctx, SolveWs<R>& w, const double2* b_soa, int nsrc, int n
   }
   cudaMemsetAsync(w.a.cnt, 0, sizeof(unsigned) * 2 * nsrc, s);
   cudaMemsetAsync(w.a.done_count, 0, sizeof(int), s);
+  if (w.a.sgrp)
+    cudaMemsetAsync(w.a.sgrp, 0, sizeof(double2) * 12 * (size_t)w.a.g.V * nsrc * (w.ngrp - 1), s);
   if (w.a.bins1) cudaMemsetAsync(w.a.bins1, 0, sizeof(long long) * 4 * kFxBins * kFxWords * nsrc, s);
   if constexpr (!std::is_same<R, FX>::value) {  // fixed point keeps no per-node vectors
     const size_t n = (size_t)12 * ctx->g.V * nsrc * ns;
@@ -2409,6 +2435,20 @@ int finish_solve(ov_ctx* ctx, SolveWs<R>& w, int nsrc, int ns, const std::vector
 
 }  // namespace
 
+// out = the weighted sum, its node groups added up in order
+static __global__ void sum_groups_kernel(const double2* __restrict__ sacc, const double2* __restrict__ sgrp, int ngrp,
+                                         double2* __restrict__ out, size_t n12) {
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+  if (e >= n12) return;
+  double2 t = sacc[r * n12 + e];
+  for (int z = 0; z < ngrp - 1; ++z) {
+    const double2 q = sgrp[(r * (ngrp - 1) + z) * n12 + e];
+    t.x += q.x;
+    t.y += q.y;
+  }
+  out[r * n12 + e] = t;
+}
+
 // Shifted FP64 solve with an explicit node list per source (zh, ch: nsrc x ns): the
 // weighted sum c0 b + sum_j c_j y_j goes to out_soa (if not null) and, if xs_soa is
 // not null, every node's solution y_j to xs_soa[src][j][12V].
@@ -2431,9 +2471,10 @@ static int solve_nodes_t(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, co
   so->launches = launches + 2.0;  // pack + unpack/epilogue issued by the caller
   if (out_soa) {
     // the weighted sum, even when not converged (best iterate)
-    cudaError_t e = cudaMemcpyAsync(out_soa, w.a.sacc, sizeof(double2) * 12 * (size_t)ctx->g.V * nsrc,
-                                    cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy sum");
+    const size_t n12 = 12 * (size_t)ctx->g.V;
+    sum_groups_kernel<<<dim3((unsigned)((n12 + 255) / 256), nsrc), 256, 0, s>>>(w.a.sacc, w.a.sgrp, w.ngrp, out_soa, n12);
+    OV_CHECK_LAUNCH(ctx, "sum_groups_kernel");
+    so->launches += 1.0;
   }
   return st;
 }
