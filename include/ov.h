@@ -67,7 +67,10 @@ typedef enum { OV_FP64 = 0, OV_FP32 = 1 } ov_precision;
 typedef enum {
   /* FP64 shifted solve: one Lanczos process on H_W serves every node; each node
    * keeps its own FP64 search direction and the weighted sum of Eq. 7 is
-   * accumulated in the same pass (the paper's shift-solver structure). */
+   * accumulated in the same pass (the paper's shift-solver structure).
+   * Unitary links and |4 - m0| <= 4, where 29 more vectors per source fit: the Lanczos
+   * vectors are integers as in OV_MODE_FP64_2PASS, and the nodes' FP64 vectors take eight
+   * iterations at a time beside the next ones. */
   OV_MODE_FP64 = 0,
   /* Mixed precision: FP32 shifted solve, then batched per-node FP64 true
    * residuals and FP32 defect-correction solves over all nodes x sources in

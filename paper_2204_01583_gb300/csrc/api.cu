@@ -104,6 +104,15 @@ void ws_release_all(ov_ctx* ctx) {
   ctx->bufs.clear();
 }
 
+void ws_release(ov_ctx* ctx, const char* prefix) {
+  cudaDeviceSynchronize();
+  for (auto it = ctx->bufs.lower_bound(prefix); it != ctx->bufs.end() && it->first.rfind(prefix, 0) == 0;) {
+    if (it->second.p) cudaFree(it->second.p);
+    it = ctx->bufs.erase(it);
+  }
+  graphs_release(ctx);  // captured graphs may point at the buffers
+}
+
 void graphs_release(ov_ctx* ctx) {
   for (auto& kv : ctx->graphs) cudaGraphExecDestroy(kv.second);
   ctx->graphs.clear();

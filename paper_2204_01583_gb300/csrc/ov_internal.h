@@ -151,6 +151,7 @@ int ctx_fail(ov_ctx* ctx, int code, const std::string& msg);
 int ctx_cuda(ov_ctx* ctx, cudaError_t e, const char* what);
 void* ws_get(ov_ctx* ctx, const char* name, size_t bytes, int* status);
 void ws_release_all(ov_ctx* ctx);
+void ws_release(ov_ctx* ctx, const char* prefix);  // the buffers whose names start with prefix
 void graphs_release(ov_ctx* ctx);
 
 // Kernel timing: bracket a launch with events when ctx->timing is set.

@@ -28,7 +28,13 @@
 // the block partials in a fixed order, so reruns are bit-identical, and updates the
 // scalars.  The host only reads a done counter every few iterations, and replays
 // the per-iteration kernels from a CUDA graph.
+//
+// Unitary links and |4 - m0| <= 4: the Lanczos vectors are integers of one scale per vector
+// (fixed.cuh, the fx_ kernels), in the stored-basis forms and, with a ring of 32 of them, in
+// the vector-space form, whose per-node FP64 vectors then advance a batch of iterations at a
+// time (fx_node_update_kernel).
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <complex>
 #include <cstdio>
@@ -90,6 +96,7 @@ struct SrcState {
   int it1, it2;  // iteration K1 last ran, 0: none left to run (read by K2); iteration K1 runs
                  // next (written by K2)
   int e_in;      // X_1 = b 2^e_in
+  int upd_i, upd_n;  // per-node vectors: first iteration and most iterations of the next update
 };
 
 // exact double-float split of an FP64 value: hi = rn(x), lo = rn(x - hi)
@@ -145,6 +152,7 @@ struct SolveParams {
   // node_check_kernel every kNodeCheck iterations from the recorded alpha_i, beta_i,
   // not in the last blocks of K1 and K2 (which then only form alpha_i and beta_i)
   int defer_nodes;
+  int slot_mask;  // fixed point: X_i in slot i & slot_mask
 };
 
 // Iterations between per-node stopping checks of the scalar-only forms: a source runs at
@@ -199,6 +207,11 @@ struct SolveArgs {
   double* hist_b;
   double* hist_n2;    // fixed point: ||X_i||^2
   const double2* gco; // [src][max_iter] second-pass coefficients or null
+  // fixed point with per-node vectors (fx_node_update_kernel), else null
+  double2* pv;        // [src][nshift][12V padded] direction vectors, in the layout of X
+  double2* xv;        // [src][nshift][12V] node solutions or null
+  double2* nco;       // [src][nshift][kNodeRun][3] l_{i-1}, c_j zeta_i, zeta_i of the next update
+  double* nin;        // [src][kNodeRun] 1 / ||X_i||
   const RegenRec<R>* rrec;  // [src][max_iter] regeneration-pass scalars or null
   const double* tol_src;  // [src] per-source tolerance or null (then SolveParams::tol)
   const SolveParams* prm;
@@ -1269,9 +1282,9 @@ __global__ void __launch_bounds__(NT, NT == kFxNT ? 4 : 3) fx_lanczos_hw_kernel(
     SrcState* S = a.src + r;
     // the check of earlier iterations may set `done` while this runs: one answer per block
     if (__syncthreads_or(S->done)) continue;
-    const int i = S->it2, mi = a.prm->max_iter;
+    const int i = S->it2, mi = a.prm->max_iter, mask = a.prm->slot_mask;
     int4* base = a.ring + (size_t)r * a.prm->nslots * n12;
-    const int4* Xi = base + (size_t)i * n12;  // stored basis: slot i holds X_i
+    const int4* Xi = base + (size_t)(i & mask) * n12;  // stored basis: slot i holds X_i
     if (NT > kFxNT && wid == kFxNT / 32) {
       FxVec v;
       const bool end = fx_begin(a, S, r, i, tb == 0, &v);
@@ -1298,14 +1311,15 @@ __global__ void __launch_bounds__(NT, NT == kFxNT ? 4 : 3) fx_lanczos_hw_kernel(
       const bool low = wid >= 3;
       // 2^-q diag / 4 x - gam X_{i-1} = (hh 2^60 + x 2^30) / 2^60; gamma5 = -1 on the lower spins
       const FX dg = vec.dia, nd = FX{low ? -dg.hi : dg.hi, low ? -dg.lo : dg.lo}, ngm = vec.gam;
-      const int4* xp = Xi + fx_index(s, 12) + 2 * wid * kFxTile;
-      longlong2* wp = reinterpret_cast<longlong2*>(const_cast<int4*>(xp + n12));
+      const size_t o = fx_index(s, 12) + 2 * wid * kFxTile;
+      const int4 *xp = Xi + o, *up = base + (size_t)((i - 1) & mask) * n12 + o;
+      longlong2* wp = reinterpret_cast<longlong2*>(base + (size_t)((i + 1) & mask) * n12 + o);
       int4 xb[2], ub[2];
       longlong2 t[2];
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         xb[j] = __ldg(xp + j * kFxTile);
-        ub[j] = i > 1 ? __ldg(xp - n12 + j * kFxTile) : make_int4(0, 0, 0, 0);
+        ub[j] = i > 1 ? __ldg(up + j * kFxTile) : make_int4(0, 0, 0, 0);
         t[j] = fx_phase2(sm, 2 * wid + j, lane);
       }
       if (q > 0) {
@@ -1331,7 +1345,7 @@ __global__ void __launch_bounds__(NT, NT == kFxNT ? 4 : 3) fx_lanczos_hw_kernel(
         wp[j * kFxTile] = make_longlong2(w[0], w[1]);
       }
     } else if (wid < 6) {  // the padding of the last tile
-      int4* wp = base + (size_t)(i + 1) * n12 + fx_index(s, 12) + 2 * wid * kFxTile;
+      int4* wp = base + (size_t)((i + 1) & mask) * n12 + fx_index(s, 12) + 2 * wid * kFxTile;
       wp[0] = wp[kFxTile] = make_int4(0, 0, 0, 0);
     }
     // warp sums in words that cannot overflow 32 lanes: hh in 26 + 26 + 12 bits, the cross
@@ -1378,8 +1392,9 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
   if (__syncthreads_or(S->done) || i < 1) return;
   const size_t n12 = 12 * fx_padded(a.g.V);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int4* Xi = a.ring + ((size_t)r * a.prm->nslots + i) * n12;
-  int4* W = a.ring + ((size_t)r * a.prm->nslots + i + 1) * n12;
+  const int mask = a.prm->slot_mask;
+  const int4* Xi = a.ring + ((size_t)r * a.prm->nslots + (i & mask)) * n12;
+  int4* W = a.ring + ((size_t)r * a.prm->nslots + ((i + 1) & mask)) * n12;
   const size_t e0 = (size_t)blockIdx.x * NT2 + threadIdx.x, gs = (size_t)gridDim.x * NT2;
   constexpr int B = 2;  // elements in flight per thread
   int4 xb[B], wb[B];
@@ -1474,13 +1489,23 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
 // check intervals.  `final` (nothing runs beside it) takes them all, with the last beta from
 // K2's sums; so does a check that finds a source at the end of its Krylov space (beta = 0).
 // The count of iterations a source ends with does not depend on which check finds it.
+// With per-node vectors it also leaves what fx_node_update_kernel needs of these iterations.
+constexpr int kNodeRun = 32;   // most iterations between two updates (17: a check may run late)
+constexpr int kNodeBatch = 8;  // iterations fx_node_update_kernel takes at a time
 __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constant__ SolveArgs<FX> a, int final) {
   __shared__ int last_sh[NT1 / 32];
   const int r = blockIdx.y;
   SrcState* S = a.src + r;
-  if (S->done) return;  // set by this kernel only
+  const bool over = S->done;  // set by this kernel only
+  if (__syncthreads_or(over)) {
+    if (a.pv && threadIdx.x == 0) S->upd_n = 0;
+    return;
+  }
   const int ns = a.prm->nshift, mi = a.prm->max_iter;
-  const int ran = S->it2 - 1;  // iterations whose alpha is recorded; their betas but the last
+  __shared__ int it_sh;  // one answer for all threads: the iterations go on beside this
+  if (threadIdx.x == 0) it_sh = *(volatile int*)&S->it2;
+  __syncthreads();
+  const int ran = it_sh - 1;  // iterations whose alpha is recorded; their betas but the last
   int upto = ran / kNodeCheck * kNodeCheck - 1;
   if (__syncthreads_or(*(volatile int*)&S->it1 == 0 && ran >= 1)) upto = ran;  // K1 recorded the last beta, too
   __threadfence();
@@ -1500,21 +1525,26 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
   const double tol2 = a.prm->tol * a.prm->tol, inv_b2 = S->inv_b2;
   const double* ha = a.hist_a + (size_t)r * mi;
   const double* hb = a.hist_b + (size_t)r * mi;
-  int still = 0, last = 0;
+  const int i0 = S->upd_i + S->upd_n;  // with per-node vectors: the iteration every active node goes on with
+  if (a.pv) upto = min(upto, i0 + kNodeRun - 1);
+  int still = 0, last = 0, run = 0;
+  double updates = 0.0;
   for (int j0 = 0; j0 < ns; j0 += NT1) {
     const int j = j0 + threadIdx.x;
     bool act = false;
     if (j < ns) {
       ShiftState& q = a.sh[(size_t)r * ns + j];
+      if (a.pv) a.act_idx[(size_t)r * ns + j] = 0;
       if (q.active) {
         const double2 zj = a.z[(size_t)r * ns + j];
+        double2* co = a.pv ? a.nco + ((size_t)r * ns + j) * kNodeRun * 3 : nullptr;
         double2 invd = q.invd, om = q.omega, zeta = q.zeta;
         double res2 = q.res2;
         int i = q.last_iter + 1;
         act = true;
         for (; i <= upto; ++i) {
           const double alpha = __ldcg(ha + i - 1), beta = __ldcg(hb + i - 1);
-          double2 d;
+          double2 d, l = make_double2(0.0, 0.0);
           if (i == 1) {
             d = make_double2(zj.x - alpha, zj.y);
             om = make_double2(S->bnorm, 0.0);
@@ -1522,11 +1552,18 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
             const double bp = __ldcg(hb + i - 2);
             const double b2 = bp * bp;
             d = make_double2(zj.x - alpha - b2 * invd.x, zj.y - b2 * invd.y);
+            l = make_double2(-bp * invd.x, -bp * invd.y);
             om = cmul(make_double2(bp * invd.x, bp * invd.y), om);
           }
           const double inv = __drcp_rn(d.x * d.x + d.y * d.y);
           invd = make_double2(d.x * inv, -d.y * inv);
           zeta = cmul(om, invd);
+          if (co) {
+            double2* p = co + 3 * (i - i0);
+            p[0] = l;
+            p[1] = cmul(a.c[(size_t)r * ns + j], zeta);
+            p[2] = zeta;
+          }
           res2 = beta * beta * inv_b2 * (zeta.x * zeta.x + zeta.y * zeta.y);
           if (res2 <= tol2 || beta == 0.0) {
             if (beta == 0.0) res2 = 0.0;
@@ -1538,7 +1575,18 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
         q.omega = om;
         q.zeta = zeta;
         q.res2 = res2;
-        q.last_iter = act ? max(upto, 0) : i;
+        const int end = act ? max(upto, q.last_iter) : i, n = end - q.last_iter;
+        if (co) {
+          a.act_idx[(size_t)r * ns + j] = n;
+          // a batch's rest: p = 0 - (-1) p, nothing added
+          for (int t = n; t % kNodeBatch != 0; ++t) {
+            co[3 * t] = make_double2(-1.0, 0.0);
+            co[3 * t + 1] = co[3 * t + 2] = make_double2(0.0, 0.0);
+          }
+          updates += n;
+          run = max(run, n);
+        }
+        q.last_iter = end;
         q.active = act ? 1 : 0;
       }
       last = max(last, q.last_iter);
@@ -1546,6 +1594,22 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
     still += __syncthreads_count(act);
   }
   last = block_max<NT1>(last, last_sh);
+  if (a.pv) {
+    __syncthreads();
+    run = block_max<NT1>(run, last_sh);
+    if (updates > 0.0) atomicAdd(&S->node_updates, updates);  // whole numbers: exact in any order
+    for (int t = threadIdx.x; t < run; t += NT1)
+      a.nin[(size_t)r * kNodeRun + t] = 1.0 / sqrt(__ldcg(a.hist_n2 + (size_t)r * mi + i0 + t - 1));
+    if (threadIdx.x == 0) {
+      S->upd_i = i0;
+      S->upd_n = run;
+      if (still == 0) {
+        S->iter = last + 1;
+        mark_done(S, a.done_count, OV_OK);
+      }
+    }
+    return;
+  }
   if (threadIdx.x == 0 && ns > 0 && still == 0) {
     // The next multiple of the check interval after the last node's iteration, an even count:
     // the iterates of an indefinite operator alternate, and the sum over an odd number of
@@ -1553,6 +1617,64 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
     S->iter = min(ran, (last + kNodeCheck) / kNodeCheck * kNodeCheck) + 1;
     mark_done(S, a.done_count, OV_OK);
   }
+}
+
+// OV_MODE_FP64 in fixed point: p = v_i - l_{i-1} p, s += c_j zeta_i p, x_j += zeta_i p in FP64 for
+// the iterations that fx_node_check_kernel has just looked at, v_i = X_i / ||X_i||.  Runs beside
+// the next iterations.  Bound by the FP64 pipe (8 FMAs per node, iteration and element, 12 with
+// x_j); the p of a node stay in registers over a batch of iterations, an eighth of the traffic of
+// an update per iteration.  The nodes of small vectors go over the grid's third dimension as in
+// K2 (k2_groups).  4^4, 1 source, 32 nodes, against K1 and K2 in FP64 with K2 in node groups:
+// 6790 -> 3245 us per solve.
+template <bool X>
+__global__ void __launch_bounds__(256, 2) fx_node_update_kernel(const __grid_constant__ SolveArgs<FX> a) {
+  const int r = blockIdx.y, z = blockIdx.z, nz = gridDim.z, V = a.g.V, ns = a.prm->nshift;
+  const SrcState* S = a.src + r;
+  const int run = S->upd_n, i0 = S->upd_i, mask = a.prm->slot_mask;
+  const size_t np = 12 * fx_padded(V), n12 = (size_t)12 * V;
+  const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
+  const size_t tk = e / kFxTile, site = tk / 12 * kFxTile + e % kFxTile, pl = tk % 12 * V + site;
+  if (run == 0 || e >= np || site >= V) return;
+  const int4* B = a.ring + (size_t)r * a.prm->nslots * np + e;
+  const int* cnt = a.act_idx + (size_t)r * ns;
+  double sre = 0.0, sim = 0.0;
+  for (int b = 0; b < run; b += kNodeBatch) {
+    double2 v[kNodeBatch];
+#pragma unroll
+    for (int t = 0; t < kNodeBatch; ++t) {
+      v[t] = make_double2(0.0, 0.0);
+      if (b + t < run) {
+        const int4 x = __ldg(B + (size_t)((i0 + b + t) & mask) * np);
+        const double in = __ldg(a.nin + (size_t)r * kNodeRun + b + t);
+        v[t] = make_double2(fma((double)x.x, pow2(30), (double)x.y) * in, fma((double)x.z, pow2(30), (double)x.w) * in);
+      }
+    }
+    for (int j = z; j < ns; j += nz) {
+      if (__ldg(cnt + j) <= b) continue;
+      const size_t rj = (size_t)r * ns + j;
+      const double2* co = a.nco + (rj * kNodeRun + b) * 3;
+      double2* P = a.pv + rj * np + e;
+      double2 p = make_double2(0.0, 0.0), x = p;
+      if (i0 + b > 1) p = *P;
+      if (X) x = a.xv[rj * n12 + pl];
+#pragma unroll
+      for (int t = 0; t < kNodeBatch; ++t) {
+        const double2 l = __ldg(co + 3 * t), cz = __ldg(co + 3 * t + 1);
+        p = make_double2(fma(l.y, p.y, fma(-l.x, p.x, v[t].x)), fma(-l.y, p.x, fma(-l.x, p.y, v[t].y)));
+        sre = fma(-cz.y, p.y, fma(cz.x, p.x, sre));
+        sim = fma(cz.y, p.x, fma(cz.x, p.y, sim));
+        if (X) {
+          const double2 zt = __ldg(co + 3 * t + 2);
+          x = make_double2(fma(-zt.y, p.y, fma(zt.x, p.x, x.x)), fma(zt.y, p.x, fma(zt.x, p.y, x.y)));
+        }
+      }
+      *P = p;
+      if (X) a.xv[rj * n12 + pl] = x;
+    }
+  }
+  double2* s = (z == 0 ? a.sacc + (size_t)r * n12 : a.sgrp + ((size_t)r * (nz - 1) + z - 1) * n12) + pl;
+  const double2 sv = *s;
+  *s = make_double2(sv.x + sre, sv.y + sim);
 }
 
 // As the generic init, with the largest component of b for the scale of X_1 (written by
@@ -1621,6 +1743,8 @@ __global__ void __launch_bounds__(NT2) lanczos_init_kernel<FX>(SolveArgs<FX> a, 
   S->vec[1] = v;
   S->it1 = 0;
   S->it2 = 1;
+  S->upd_i = 1;
+  S->upd_n = 0;
   a.hist_n2[(size_t)r * a.prm->max_iter] = v.n2;
   S->status = OV_OK;
   S->n_act = 0;
@@ -1990,7 +2114,8 @@ template <typename R>
 struct SolveWs {
   SolveArgs<R> a{};
   int nblk1 = 0, nblk2 = 0, nblk2u = 0;
-  int ngrp = 1;  // K2's node groups
+  int ngrp = 1;  // node groups of K2 or of fx_node_update_kernel
+  int slot_mask = INT_MAX;
   int nslots = 3;
   size_t nvec = 0;   // elements of one Lanczos vector (12 V, padded in fixed point)
   int nshift = 0;
@@ -2011,6 +2136,10 @@ SolveArgs<R> args_for_sources(const SolveWs<R>& w, int r0) {
   if (a.x) a.x += r * ns * n12;
   if (a.sacc) a.sacc += r * n12;
   if (a.sgrp) a.sgrp += r * (w.ngrp - 1) * n12;
+  if (a.pv) a.pv += r * ns * w.nvec;
+  if (a.xv) a.xv += r * ns * n12;
+  if (a.nco) a.nco += r * ns * kNodeRun * 3;
+  if (a.nin) a.nin += r * kNodeRun;
   if (a.ssum) a.ssum += r * n12;
   if (a.stencil) a.stencil += r * n12;
   a.src += r;
@@ -2218,12 +2347,29 @@ int launch_k1(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s)
   }
 }
 
+// K2, in FP64 and double-float with the nodes in groups
 template <typename R>
-void launch_node_check(const SolveWs<R>& w, const SolveArgs<R>& a, int nsrc, cudaStream_t s, bool final = false) {
-  if constexpr (std::is_same<R, FX>::value)
+void launch_k2(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s) {
+  lanczos_update_kernel<R><<<dim3(w.nblk2u, n, std::is_same<R, FX>::value ? 1 : w.ngrp), NT2, 0, s>>>(a);
+}
+
+// Node checks and, in fixed point with per-node vectors, their updates.  Returns the number of
+// launches.
+template <typename R>
+int launch_node_check(const SolveWs<R>& w, const SolveArgs<R>& a, int nsrc, cudaStream_t s, bool final = false) {
+  if constexpr (std::is_same<R, FX>::value) {
     fx_node_check_kernel<<<dim3(1, nsrc), NT1, 0, s>>>(a, final);
-  else
+    if (!a.pv) return 1;
+    const dim3 grid((unsigned)((w.nvec + 255) / 256), nsrc, w.ngrp);
+    if (a.xv)
+      fx_node_update_kernel<true><<<grid, 256, 0, s>>>(a);
+    else
+      fx_node_update_kernel<false><<<grid, 256, 0, s>>>(a);
+    return 2;
+  } else {
     node_check_kernel<R><<<dim3(1, nsrc), NT1, 0, s>>>(a);
+    return 1;
+  }
 }
 
 // One Lanczos iteration (K1, K2); `it` counts iterations from 0 within the loop, and a
@@ -2236,12 +2382,11 @@ int launch_iteration(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, cudaStream_t s,
   int n = launch_k1<R>(w, w.a, nsrc, s);
   kt_end(ctx, KC_LANCZOS_HW, s, ev);
   kt_begin(ctx, KC_SHIFT_UPDATE, s, &ev);
-  lanczos_update_kernel<R><<<dim3(w.nblk2u, nsrc, w.ngrp), NT2, 0, s>>>(w.a);
+  launch_k2<R>(w, w.a, nsrc, s);
   kt_end(ctx, KC_SHIFT_UPDATE, s, ev);
   ++n;
   if (w.defer && (it + 1) % kNodeCheck == 0) {
-    launch_node_check<R>(w, w.a, nsrc, s);
-    ++n;
+    n += launch_node_check<R>(w, w.a, nsrc, s);
   }
   return n;
 }
@@ -2260,7 +2405,8 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
   double graph_launches = 0.0;  // per replay
   if (graph) {
     const int G = source_groups<R>(ctx, nsrc, w.nblk1);
-    GraphKey key{{(const void*)w.a.ring, (const void*)w.a.p, (const void*)w.a.x, (const void*)w.a.sacc},
+    GraphKey key{{(const void*)w.a.ring, w.a.pv ? (const void*)w.a.pv : (const void*)w.a.p,
+                  w.a.pv ? (const void*)w.a.xv : (const void*)w.a.x, (const void*)w.a.sacc},
                  nsrc, nshift, flavour * 128 + G, chunk, w.nslots, w.max_iter};
     auto it = ctx->graphs.find(key);
     if (it != ctx->graphs.end()) {
@@ -2276,17 +2422,16 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
             constexpr bool beside = std::is_same<R, FX>::value;
             for (int k = 0; k < chunk; ++k) {
               graph_launches += launch_k1<R>(w, a, n, cs) + 1;
-              lanczos_update_kernel<R><<<dim3(w.nblk2u, n, w.ngrp), NT2, 0, cs>>>(a);
+              launch_k2<R>(w, a, n, cs);
               if (!w.defer || (k + 1) % kNodeCheck != 0) continue;
-              graph_launches += 1.0;
               if (beside) {
                 if (k >= kNodeCheck) cudaStreamWaitEvent(cs, join, 0);
                 cudaEventRecord(fork, cs);
                 cudaStreamWaitEvent(side, fork, 0);
-                launch_node_check<R>(w, a, n, side);
+                graph_launches += launch_node_check<R>(w, a, n, side);
                 cudaEventRecord(join, side);
               } else {
-                launch_node_check<R>(w, a, n, cs);
+                graph_launches += launch_node_check<R>(w, a, n, cs);
               }
             }
             if (beside && w.defer) cudaStreamWaitEvent(cs, join, 0);
@@ -2317,9 +2462,8 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
     if (*ctx->host_flag >= nsrc) break;
   }
   if (w.defer) {  // the iterations since the last check (final node residuals and status)
-    launch_node_check<R>(w, w.a, nsrc, s, true);
+    *launches += launch_node_check<R>(w, w.a, nsrc, s, true);
     OV_CHECK_LAUNCH(ctx, "node_check_kernel");
-    *launches += 1.0;
   }
   return OV_OK;
 }
@@ -2365,7 +2509,7 @@ int init_solve(ov_ctx* ctx, SolveWs<R>& w, const double2* b_soa, int nsrc, int n
                double tol, int max_iter, cudaStream_t s, int vec_shifts = 1) {
   // scalar-only forms with nodes defer the per-node recurrences (they record alpha, beta)
   w.defer = (vec_shifts == 0 && ns > 0 && w.a.hist_a && w.a.hist_b);
-  SolveParams prm{tol, max_iter, ns, vec_shifts, w.nslots, w.nslots > 3 ? 1 : 0, w.defer ? 1 : 0};
+  SolveParams prm{tol, max_iter, ns, vec_shifts, w.nslots, w.nslots > 3 ? 1 : 0, w.defer ? 1 : 0, w.slot_mask};
   cudaError_t e = cudaMemcpyAsync(w.prm_dev, &prm, sizeof(prm), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy params");
   if (ns > 0) {
@@ -2479,9 +2623,64 @@ static int solve_nodes_t(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, co
   return st;
 }
 
+// solve_nodes_t with the Lanczos vectors in fixed point (a ring of kNodeRun of them) and the
+// per-node vectors in FP64.  OV_ERR_OUT_OF_MEMORY: its workspace, larger than the FP64 form's
+// by kNodeRun - 3 vectors per source, does not fit.
+static int solve_nodes_fx(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
+                          const std::vector<double2>& ch, double2 c0, double2* out_soa, double2* xs,
+                          const ov_solve_opts& o, SolveOut* so, cudaStream_t s) {
+  NvtxRange nvtx_("solve: vector space, fixed-point Lanczos vectors");
+  const size_t n12 = 12 * (size_t)ctx->g.V, nvec = vec_elems<FX>(ctx->g.V);
+  const char* const names[] = {"fxv.ring", "fxv.pv"};
+  const double need = (double)sizeof(double2) * nvec * nsrc * (kNodeRun + ns);
+  double held = 0.0;
+  for (const char* n : names) {
+    auto it = ctx->bufs.find(n);
+    if (it != ctx->bufs.end()) held += (double)it->second.bytes;
+  }
+  size_t freeb = 0, totalb = 0;
+  cudaMemGetInfo(&freeb, &totalb);
+  if (need > held && need - held > (double)freeb - 0.10 * (double)totalb) return OV_ERR_OUT_OF_MEMORY;
+  SolveWs<FX> w;
+  int st = setup_ws<FX>(ctx, nsrc, ns, false, true, true, o.max_iter, &w, "fxv", kNodeRun, false);
+  w.slot_mask = kNodeRun - 1;
+  w.ngrp = k2_groups((int)std::min<size_t>((nvec + 255) / 256, INT_MAX / nsrc), nsrc, ns);
+  w.a.sgrp = w.ngrp > 1 ? (double2*)ws_get(ctx, "fxv.sgrp", sizeof(double2) * n12 * (size_t)nsrc * (w.ngrp - 1), &st)
+                        : nullptr;
+  w.a.pv = (double2*)ws_get(ctx, "fxv.pv", sizeof(double2) * nvec * (size_t)nsrc * ns, &st);
+  w.a.nco = (double2*)ws_get(ctx, "fxv.nco", sizeof(double2) * 3 * kNodeRun * (size_t)nsrc * ns, &st);
+  w.a.nin = (double*)ws_get(ctx, "fxv.nin", sizeof(double) * kNodeRun * (size_t)nsrc, &st);
+  w.a.xv = xs;
+  if (st != OV_OK) return st;
+  if (xs) cudaMemsetAsync(xs, 0, sizeof(double2) * n12 * (size_t)nsrc * ns, s);
+  st = init_solve<FX>(ctx, w, b_soa, nsrc, ns, zh, ch, c0, o.tol, o.max_iter, s, 0);
+  if (st != OV_OK) return st;
+  double launches = 2.0;
+  st = run_iterations<FX>(ctx, w, nsrc, ns, xs ? 9 : 8, o.max_iter, o, s, &launches);
+  if (st != OV_OK) return st;
+  st = finish_solve<FX>(ctx, w, nsrc, ns, zh, ch, so, s);
+  so->launches = launches + 2.0;  // pack + unpack/epilogue issued by the caller
+  if (out_soa) {
+    sum_groups_kernel<<<dim3((unsigned)((n12 + 255) / 256), nsrc), 256, 0, s>>>(w.a.sacc, w.a.sgrp, w.ngrp, out_soa, n12);
+    OV_CHECK_LAUNCH(ctx, "sum_groups_kernel");
+    so->launches += 1.0;
+  }
+  return st;
+}
+
+// Whether the stored-basis and vector-space forms run in fixed point (fixed.cuh): links of norm 1 (the bounds
+// there) and |4 - m0| <= 4.  Other links and masses, and the persistent loop, keep the
+// FP64 and double-float kernels.
+static bool fixed_point_fits(const ov_ctx* ctx) { return ctx->no_coop && ctx->fx_ok; }
+
 int solve_nodes_soa(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
                     const std::vector<double2>& ch, double2 c0, double2* out_soa, double2* xs_soa,
                     const ov_solve_opts& o, SolveOut* so, cudaStream_t s) {
+  if (fixed_point_fits(ctx) && ns > 0) {
+    const int st = solve_nodes_fx(ctx, b_soa, nsrc, ns, zh, ch, c0, out_soa, xs_soa, o, so, s);
+    if (st != OV_ERR_OUT_OF_MEMORY) return st;
+    ws_release(ctx, "fxv.");
+  }
   return solve_nodes_t<double>(ctx, b_soa, nsrc, ns, zh, ch, c0, out_soa, xs_soa, o, so, s, "fp64");
 }
 
@@ -3088,11 +3287,6 @@ int nodes_coef<FX>(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const st
   if (so->converged) ctx->coef_iter_hint = so->iterations;
   return fst;
 }
-
-// Whether the stored-basis forms run in fixed point (fixed.cuh): links of norm 1 (the bounds
-// there) and |4 - m0| <= 4.  Other links and masses, and the persistent loop, keep the
-// FP64 and double-float kernels.
-static bool fixed_point_fits(const ov_ctx* ctx) { return ctx->no_coop && ctx->fx_ok; }
 
 int solve_nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
                      const std::vector<double2>& ch, int chunk, double2* X, double2* sums, const ov_solve_opts& o,
