@@ -1202,8 +1202,8 @@ __device__ __forceinline__ long long warp_sum(long long v) {
 }
 
 // The scalars of X_i (i >= 2) from ||X_i||^2 (K2's bins of iteration i - 1); a whole warp.
-// *beta: beta_{i-1}, *tot: ||X_i||^2.
-__device__ __forceinline__ FxVec fx_vec(const SolveArgs<FX>& a, const SrcState* S, int r, int i, double* beta) {
+// fx_close adds what K1 does not wait for: 1 / ||X_i||^2 and, returned, beta_{i-1}.
+__device__ __forceinline__ FxVec fx_vec(const SolveArgs<FX>& a, const SrcState* S, int r, int i, double* ratio, int* shift) {
   const long long* bins = fx_bins(a.bins2, r, i - 1) + (threadIdx.x & 31) * kFxWords;
   long long n[4];
 #pragma unroll
@@ -1212,46 +1212,46 @@ __device__ __forceinline__ FxVec fx_vec(const SolveArgs<FX>& a, const SrcState* 
   const int sh = p.q - S->k[(i - 1) & 1];
   FxVec v;
   v.n2 = fma((double)n[0], pow2(92), (double)n[1] * pow2(60)) + fma((double)n[2], pow2(38), (double)n[3] * 256.0);
-  v.inv_n2 = __drcp_rn(v.n2);
-  const double ratio = v.n2 * p.inv_n2;    // ||X_i||^2 / ||X_{i-1}||^2
-  *beta = sqrt(ratio) * pow2(2 + sh);
-  const double g1 = ratio * pow2(sh);      // beta_{i-1} ||X_i|| / (4 ||X_{i-1}||)
+  *ratio = v.n2 * p.inv_n2;                // ||X_i||^2 / ||X_{i-1}||^2, 0 if beta_{i-1} is
+  *shift = sh;
+  const double g1 = *ratio * pow2(sh);     // beta_{i-1} ||X_i|| / (4 ||X_{i-1}||)
   v.q = max(0, exponent_of(g1));           // g1 2^-q < 2
   v.gam = fx_split(-__double2ll_rn(g1 * pow2(60 - v.q)));
   v.dia = fx_split(__double2ll_rn(a.diag4 * pow2(60 - v.q)));
   return v;
 }
 
-// The start of an iteration by one warp: the scalars of X_i, recorded by the one warp that has
-// `record` set.  Returns true when no iteration is left to run.
-__device__ __forceinline__ bool fx_begin(const SolveArgs<FX>& a, SrcState* S, int r, int i, bool record, FxVec* out) {
+__device__ __forceinline__ double fx_close(FxVec* v, double ratio, int shift) {
+  v->inv_n2 = __drcp_rn(v->n2);
+  return sqrt(ratio) * pow2(2 + shift);
+}
+
+// What an iteration's start leaves for later kernels, by one warp per source.
+__device__ __forceinline__ void fx_record(const SolveArgs<FX>& a, SrcState* S, int r, int i, FxVec v, double ratio,
+                                          int shift, bool end) {
   const int lane = threadIdx.x & 31, mi = a.prm->max_iter;
-  double beta = 1.0;
-  const FxVec v = i > 1 ? fx_vec(a, S, r, i, &beta) : S->vec[1];
-  const bool end = beta == 0.0 || i > mi;
-  *out = v;
-  if (!record) return end;
   long long* z = fx_bins(a.bins2, r, i) + lane * kFxWords;
 #pragma unroll
   for (int k = 0; k < kFxWords; ++k) z[k] = 0;
-  if (lane == 0) {
-    if (i > 1) {
-      S->vec[i & 1] = v;
-      a.hist_b[(size_t)r * mi + i - 2] = beta;
-      if (i <= mi) a.hist_n2[(size_t)r * mi + i - 1] = v.n2;
-    }
-    __threadfence();  // a check running beside this reads the history once it1 is 0
-    *(volatile int*)&S->it1 = end ? 0 : i;
+  if (lane != 0) return;
+  if (i > 1) {
+    a.hist_b[(size_t)r * mi + i - 2] = fx_close(&v, ratio, shift);
+    S->vec[i & 1] = v;
+    if (i <= mi) a.hist_n2[(size_t)r * mi + i - 1] = v.n2;
   }
-  return end;
+  __threadfence();  // a check running beside this reads the history once it1 is 0
+  *(volatile int*)&S->it1 = end ? 0 : i;
 }
 
 // fx_begin ahead of K1 for grids of many blocks (one warp per source)
 __global__ void __launch_bounds__(32) fx_begin_kernel(const __grid_constant__ SolveArgs<FX> a) {
   SrcState* S = a.src + blockIdx.x;
   if (__any_sync(0xffffffffu, S->done)) return;
-  FxVec v;
-  fx_begin(a, S, blockIdx.x, S->it2, true, &v);
+  const int i = S->it2;
+  double ratio = 1.0;
+  int shift = 0;
+  const FxVec v = i > 1 ? fx_vec(a, S, blockIdx.x, i, &ratio, &shift) : S->vec[1];
+  fx_record(a, S, blockIdx.x, i, v, ratio, shift, ratio == 0.0 || i > a.prm->max_iter);
 }
 
 // A block takes one 32-site tile of `per` sources in turn (their links then come from L1).
@@ -1278,19 +1278,22 @@ __global__ void __launch_bounds__(NT, NT == kFxNT ? 4 : 3) fx_lanczos_hw_kernel(
   const int s = tb * kFxTile + lane;
   const bool in = s < V;
   const FxHops nbr = fx_hops(a.g, in ? s : 0, (wid >> 1) & 3);
+  if (NT > kFxNT) cudaGridDependencySynchronize();
   for (int r = r0; r < min(nsrc, r0 + per); ++r) {
     SrcState* S = a.src + r;
+    const int i = S->it2, mi = a.prm->max_iter, mask = a.prm->slot_mask, nslots = a.prm->nslots;
     // the check of earlier iterations may set `done` while this runs: one answer per block
     if (__syncthreads_or(S->done)) continue;
-    const int i = S->it2, mi = a.prm->max_iter, mask = a.prm->slot_mask;
-    int4* base = a.ring + (size_t)r * a.prm->nslots * n12;
+    FxVec next;  // the ninth warp's
+    double ratio = 1.0;
+    int shift = 0;
+    int4* base = a.ring + (size_t)r * nslots * n12;
     const int4* Xi = base + (size_t)(i & mask) * n12;  // stored basis: slot i holds X_i
     if (NT > kFxNT && wid == kFxNT / 32) {
-      FxVec v;
-      const bool end = fx_begin(a, S, r, i, tb == 0, &v);
+      next = i > 1 ? fx_vec(a, S, r, i, &ratio, &shift) : S->vec[1];
       if (lane == 0) {
-        vec = v;
-        stop = end;
+        vec = next;
+        stop = ratio == 0.0 || i > mi;
       }
     }
     if (NT == kFxNT && threadIdx.x == 0) {
@@ -1299,6 +1302,8 @@ __global__ void __launch_bounds__(NT, NT == kFxNT ? 4 : 3) fx_lanczos_hw_kernel(
     }
     if (in && i <= mi && wid < kFxNT / 32) fx_phase1(Xi, a.U, wid, s, nbr, sm + (wid >> 1) * 12 * kFxTile + lane);
     __syncthreads();
+    if (NT > kFxNT) cudaTriggerProgrammaticLaunchCompletion();
+    if (NT > kFxNT && wid == kFxNT / 32 && tb == 0) fx_record(a, S, r, i, next, ratio, shift, stop);
     if (stop) {
       __syncthreads();
       continue;
@@ -1388,13 +1393,13 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
   __shared__ int k_sh;
   const int r = blockIdx.y;
   SrcState* S = a.src + r;
-  const int i = S->it1;
+  cudaGridDependencySynchronize();
+  const int i = S->it1, mask = a.prm->slot_mask, nslots = a.prm->nslots;
   if (__syncthreads_or(S->done) || i < 1) return;
   const size_t n12 = 12 * fx_padded(a.g.V);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int mask = a.prm->slot_mask;
-  const int4* Xi = a.ring + ((size_t)r * a.prm->nslots + (i & mask)) * n12;
-  int4* W = a.ring + ((size_t)r * a.prm->nslots + ((i + 1) & mask)) * n12;
+  const int4* Xi = a.ring + ((size_t)r * nslots + (i & mask)) * n12;
+  int4* W = a.ring + ((size_t)r * nslots + ((i + 1) & mask)) * n12;
   const size_t e0 = (size_t)blockIdx.x * NT2 + threadIdx.x, gs = (size_t)gridDim.x * NT2;
   constexpr int B = 2;  // elements in flight per thread
   int4 xb[B], wb[B];
@@ -1475,6 +1480,7 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
     if (lane == 0) red[wid][j] = n[j];
   }
   __syncthreads();
+  cudaTriggerProgrammaticLaunchCompletion();
   if (threadIdx.x < 4) {
     long long t = 0;
 #pragma unroll
@@ -1512,10 +1518,11 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
   if (final) {
     upto = ran;
     if (ran >= 1 && threadIdx.x < 32) {
-      double beta;
-      const FxVec v = fx_vec(a, S, r, ran + 1, &beta);
+      double ratio;
+      int shift;
+      FxVec v = fx_vec(a, S, r, ran + 1, &ratio, &shift);
       if (threadIdx.x == 0) {
-        a.hist_b[(size_t)r * mi + ran - 1] = beta;
+        a.hist_b[(size_t)r * mi + ran - 1] = fx_close(&v, ratio, shift);
         if (ran < mi) a.hist_n2[(size_t)r * mi + ran] = v.n2;
         S->iter = ran + 1;
       }
@@ -2327,15 +2334,41 @@ dim3 k1_grid(const SolveWs<R>& w, int n) {
 // links then come from L1), fewer while the grid would not fill the GPU; grids of at most
 // three blocks per SM form the scalars themselves.  Returns the number of launches.
 constexpr int kFxPerBlock = 6;
+
+// A launch that may become resident while the kernel before it in the stream ends: K1 (288
+// threads) and K2 in fixed point wait for that kernel (its memory included) before they read
+// anything, and let their successor in late, when K1 has its hops and K2 its vector stored:
+// blocks that wait keep others' branches out.  Solves at 4^4 with 1 source 3268 -> 2963 us, 8^4
+// with 4 6570 -> 5923, 6 x 10 x 4 x 14 with 3 5700 -> 5250; let in from the start: 3033, 5908,
+// 5638, and a gradient at 8^4 11690 -> 12195 instead of 11419.  With fx_begin_kernel ahead of
+// K1, in large grids, it costs 3 %: ordinary launches there.
+template <typename... P, typename... A>
+void launch_early(void (*k)(P...), dim3 grid, int nt, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(nt);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
 template <typename R>
-int launch_k1(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s) {
+int launch_k1(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s, bool joined = false) {
   if constexpr (std::is_same<R, FX>::value) {
     int ng = (n + kFxPerBlock - 1) / kFxPerBlock;
     while (ng < n && (size_t)w.nblk1 * ng < 4 * 4 * 152) ++ng;
     const int per = (n + ng - 1) / ng;
     const unsigned grid = (unsigned)w.nblk1 * ((n + per - 1) / per);
     if (grid <= 3 * 152) {
-      fx_lanczos_hw_kernel<kFxNT + 32><<<grid, kFxNT + 32, 0, s>>>(a, n, per);
+      // two branches meet ahead of it (`joined`): an ordinary launch
+      if (joined)
+        fx_lanczos_hw_kernel<kFxNT + 32><<<grid, kFxNT + 32, 0, s>>>(a, n, per);
+      else
+        launch_early(fx_lanczos_hw_kernel<kFxNT + 32>, grid, kFxNT + 32, s, a, n, per);
       return 1;
     }
     fx_begin_kernel<<<n, 32, 0, s>>>(a);
@@ -2349,8 +2382,14 @@ int launch_k1(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s)
 
 // K2, in FP64 and double-float with the nodes in groups
 template <typename R>
-void launch_k2(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s) {
-  lanczos_update_kernel<R><<<dim3(w.nblk2u, n, std::is_same<R, FX>::value ? 1 : w.ngrp), NT2, 0, s>>>(a);
+void launch_k2(const SolveWs<R>& w, const SolveArgs<R>& a, int n, cudaStream_t s, bool early = false) {
+  if constexpr (std::is_same<R, FX>::value) {
+    if (early)
+      launch_early(lanczos_update_kernel<FX>, dim3(w.nblk2u, n), NT2, s, a);
+    else
+      lanczos_update_kernel<R><<<dim3(w.nblk2u, n), NT2, 0, s>>>(a);
+  } else
+    lanczos_update_kernel<R><<<dim3(w.nblk2u, n, w.ngrp), NT2, 0, s>>>(a);
 }
 
 // Node checks and, in fixed point with per-node vectors, their updates.  Returns the number of
@@ -2421,8 +2460,9 @@ int run_iterations(ov_ctx* ctx, const SolveWs<R>& w, int nsrc, int nshift, int f
             // fixed point: the node checks run on a side branch beside the next interval
             constexpr bool beside = std::is_same<R, FX>::value;
             for (int k = 0; k < chunk; ++k) {
-              graph_launches += launch_k1<R>(w, a, n, cs) + 1;
-              launch_k2<R>(w, a, n, cs);
+              const int n1 = launch_k1<R>(w, a, n, cs, beside && k % kNodeCheck == 0);
+              launch_k2<R>(w, a, n, cs, n1 == 1);
+              graph_launches += n1 + 1;
               if (!w.defer || (k + 1) % kNodeCheck != 0) continue;
               if (beside) {
                 if (k >= kNodeCheck) cudaStreamWaitEvent(cs, join, 0);
