@@ -207,6 +207,9 @@ struct SolveArgs {
   double* hist_b;
   double* hist_n2;    // fixed point: ||X_i||^2
   const double2* gco; // [src][max_iter] second-pass coefficients or null
+  // fixed point with a stored basis: rows of every node's LDL^T, else null
+  double2* fd;        // [src][max_iter][nshift] 1 / d_i
+  double2* fz;        // [src][max_iter][nshift] zeta_i
   // fixed point with per-node vectors (fx_node_update_kernel), else null
   double2* pv;        // [src][nshift][12V padded] direction vectors, in the layout of X
   double2* xv;        // [src][nshift][12V] node solutions or null
@@ -1495,7 +1498,8 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
 // check intervals.  `final` (nothing runs beside it) takes them all, with the last beta from
 // K2's sums; so does a check that finds a source at the end of its Krylov space (beta = 0).
 // The count of iterations a source ends with does not depend on which check finds it.
-// With per-node vectors it also leaves what fx_node_update_kernel needs of these iterations.
+// With per-node vectors it also leaves what fx_node_update_kernel needs of these iterations,
+// with a stored basis the rows of every node's factorisation, stopped ones included.
 constexpr int kNodeRun = 32;   // most iterations between two updates (17: a check may run late)
 constexpr int kNodeBatch = 8;  // iterations fx_node_update_kernel takes at a time
 __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constant__ SolveArgs<FX> a, int final) {
@@ -1532,7 +1536,7 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
   const double tol2 = a.prm->tol * a.prm->tol, inv_b2 = S->inv_b2;
   const double* ha = a.hist_a + (size_t)r * mi;
   const double* hb = a.hist_b + (size_t)r * mi;
-  const int i0 = S->upd_i + S->upd_n;  // with per-node vectors: the iteration every active node goes on with
+  const int i0 = S->upd_i + S->upd_n;  // the iteration all nodes go on with
   if (a.pv) upto = min(upto, i0 + kNodeRun - 1);
   int still = 0, last = 0, run = 0;
   double updates = 0.0;
@@ -1542,14 +1546,14 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
     if (j < ns) {
       ShiftState& q = a.sh[(size_t)r * ns + j];
       if (a.pv) a.act_idx[(size_t)r * ns + j] = 0;
-      if (q.active) {
+      act = q.active != 0;
+      if (act || !a.pv) {
         const double2 zj = a.z[(size_t)r * ns + j];
         double2* co = a.pv ? a.nco + ((size_t)r * ns + j) * kNodeRun * 3 : nullptr;
         double2 invd = q.invd, om = q.omega, zeta = q.zeta;
         double res2 = q.res2;
-        int i = q.last_iter + 1;
-        act = true;
-        for (; i <= upto; ++i) {
+        int end = act ? max(upto, q.last_iter) : q.last_iter;
+        for (int i = i0; i <= upto; ++i) {
           const double alpha = __ldcg(ha + i - 1), beta = __ldcg(hb + i - 1);
           double2 d, l = make_double2(0.0, 0.0);
           if (i == 1) {
@@ -1570,20 +1574,26 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
             p[0] = l;
             p[1] = cmul(a.c[(size_t)r * ns + j], zeta);
             p[2] = zeta;
+          } else {
+            const size_t o = ((size_t)r * mi + i - 1) * ns + j;
+            a.fd[o] = invd;
+            a.fz[o] = zeta;
           }
+          if (!act) continue;
           res2 = beta * beta * inv_b2 * (zeta.x * zeta.x + zeta.y * zeta.y);
           if (res2 <= tol2 || beta == 0.0) {
             if (beta == 0.0) res2 = 0.0;
             act = false;
-            break;
+            end = i;
+            if (co) break;
           }
         }
         q.invd = invd;
         q.omega = om;
         q.zeta = zeta;
         q.res2 = res2;
-        const int end = act ? max(upto, q.last_iter) : i, n = end - q.last_iter;
         if (co) {
+          const int n = end - q.last_iter;
           a.act_idx[(size_t)r * ns + j] = n;
           // a batch's rest: p = 0 - (-1) p, nothing added
           for (int t = n; t % kNodeBatch != 0; ++t) {
@@ -1617,6 +1627,7 @@ __global__ void __launch_bounds__(NT1) fx_node_check_kernel(const __grid_constan
     }
     return;
   }
+  if (threadIdx.x == 0) S->upd_i = max(i0, upto + 1);
   if (threadIdx.x == 0 && ns > 0 && still == 0) {
     // The next multiple of the check interval after the last node's iteration, an even count:
     // the iterates of an indefinite operator alternate, and the sum over an odd number of
@@ -1780,61 +1791,74 @@ __global__ void __launch_bounds__(NT2) fx_quantize_kernel(const __grid_constant_
   }
 }
 
-// Coefficients y = (z_j - T_k)^-1 e_1 ||b|| of every node, one thread per node:
-//   f_k = z - alpha_k,  f_i = z - alpha_i - beta_i^2 / f_{i+1};   y_1 = ||b|| / f_1,  y_{i+1} =
-//   beta_i y_i / f_{i+1}
-// (the factorisation from the last row up: |Im f_i| >= |Im z|).  Y[r][i][j] holds 1 / f, then y
-// / ||X_i||.  Two serial chains of k steps, all nodes and sources at once (on the host they
-// took 8 us per source and node at 8^4, 2 of 10 ms of a 4-source solve); the recurrence
-// scalars come from shared memory and the pivots of the way down a batch ahead, so that no
-// step waits for L2.
+// Coefficients y = (z_j - T_k)^-1 e_1 ||b|| of every node, one thread per node, from the rows of
+// its LDL^T that the node checks left (fd, fz); rows behind the last check, at most a check
+// interval of them, come first.
+//   y_k = zeta_k,  y_i = zeta_i + beta_i / d_i y_{i+1};   fz[i] becomes y_i / ||X_i||
+// A serial chain of two FMAs a step; rows come a batch ahead, the scalars from shared memory.
+// (A factorisation from the last row up, which needs no stored rows, has a reciprocal in the
+// chain: 280 us for 352 steps.)
 constexpr int kCoefChunk = 512;
-__global__ void __launch_bounds__(32) fx_node_coef_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
-                                                          double2* __restrict__ Y) {
+__global__ void __launch_bounds__(32) fx_node_coef_kernel(const __grid_constant__ SolveArgs<FX> a, int ns) {
   __shared__ double sa[kCoefChunk], sb[kCoefChunk];
   const int r = blockIdx.y, lane = threadIdx.x, j = min(blockIdx.x * 32 + lane, ns - 1);
   const bool on = blockIdx.x * 32 + lane < ns;
   const SrcState* S = a.src + r;
   const int mi = a.prm->max_iter, k = S->iter - 1;
   const double *al = a.hist_a + (size_t)r * mi, *be = a.hist_b + (size_t)r * mi, *n2 = a.hist_n2 + (size_t)r * mi;
-  double2* y = Y + (size_t)r * mi * ns + j;
+  double2 *fd = a.fd + (size_t)r * mi * ns + j, *fz = a.fz + (size_t)r * mi * ns + j;
   const double2 z = a.z[(size_t)r * ns + j];
-  double2 f = make_double2(0.0, 0.0);  // 1 / f_{i+1}
+  for (int i = S->upd_i; i <= k; ++i) {
+    double2 d = make_double2(z.x - al[i - 1], z.y), om = make_double2(S->bnorm, 0.0);
+    if (i > 1) {
+      const double bp = be[i - 2], b2 = bp * bp;
+      const double2 g = fd[(size_t)(i - 2) * ns], zp = fz[(size_t)(i - 2) * ns];
+      d = make_double2(d.x - b2 * g.x, d.y - b2 * g.y);
+      om = make_double2(bp * zp.x, bp * zp.y);
+    }
+    const double inv = __drcp_rn(d.x * d.x + d.y * d.y);
+    const double2 g = make_double2(d.x * inv, -d.y * inv);
+    __syncwarp();  // lanes beyond ns share the last node's rows
+    if (on) {
+      fd[(size_t)(i - 1) * ns] = g;
+      fz[(size_t)(i - 1) * ns] = cmul(om, g);
+    }
+    __syncwarp();
+  }
+  constexpr int B = 8;
+  double2 y = make_double2(0.0, 0.0), g[B], zt[B];
+  auto load = [&](int i) {  // rows i - 1, i - 2, ...
+#pragma unroll
+    for (int t = 0; t < B; ++t) {
+      const size_t o = (size_t)max(i - 1 - t, 0) * ns;
+      g[t] = fd[o];
+      zt[t] = fz[o];
+    }
+  };
+  if (k > 0) load(k);
   for (int hi = k; hi > 0; hi -= kCoefChunk) {
     const int lo = max(0, hi - kCoefChunk);
     __syncwarp();
     for (int i = lo + lane; i < hi; i += 32) {
-      sa[i - lo] = al[i];
-      sb[i - lo] = i + 1 < k ? be[i] * be[i] : 0.0;
-    }
-    __syncwarp();
-    for (int i = hi - 1; i >= lo; --i) {
-      const double b2 = sb[i - lo], dx = fma(-b2, f.x, z.x - sa[i - lo]), dy = fma(-b2, f.y, z.y);
-      const double inv = __drcp_rn(fma(dx, dx, dy * dy));
-      f = make_double2(dx * inv, -dy * inv);
-      if (on) y[(size_t)i * ns] = f;
-    }
-  }
-  double2 v = make_double2(S->bnorm, 0.0);
-  for (int lo = 0; lo < k; lo += kCoefChunk) {
-    const int hi = min(k, lo + kCoefChunk);
-    __syncwarp();
-    for (int i = lo + lane; i < hi; i += 32) {
       sa[i - lo] = rsqrt(n2[i]);
-      sb[i - lo] = i > 0 ? be[i - 1] : 1.0;
+      sb[i - lo] = i + 1 < k ? be[i] : 0.0;
     }
     __syncwarp();
-    constexpr int B = 8;
-    for (int i0 = lo; i0 < hi; i0 += B) {
-      double2 g[B];
-#pragma unroll
-      for (int t = 0; t < B; ++t) g[t] = y[(size_t)min(i0 + t, k - 1) * ns];
+    for (int i0 = hi; i0 > lo; i0 -= B) {
+      double2 gb[B], zb[B];
 #pragma unroll
       for (int t = 0; t < B; ++t) {
-        if (i0 + t >= hi) break;
-        const double b = sb[i0 + t - lo], rn = sa[i0 + t - lo];
-        v = cmul(v, make_double2(b * g[t].x, b * g[t].y));
-        if (on) y[(size_t)(i0 + t) * ns] = make_double2(v.x * rn, v.y * rn);
+        const double b = i0 - t > lo ? sb[i0 - 1 - t - lo] : 0.0;
+        gb[t] = make_double2(b * g[t].x, b * g[t].y);
+        zb[t] = zt[t];
+      }
+      load(i0 - min(B, i0 - lo));
+#pragma unroll
+      for (int t = 0; t < B; ++t) {
+        if (i0 - t <= lo) break;
+        const double rn = sa[i0 - 1 - t - lo];
+        y = make_double2(fma(-gb[t].y, y.y, fma(gb[t].x, y.x, zb[t].x)), fma(gb[t].y, y.x, fma(gb[t].x, y.y, zb[t].y)));
+        if (on) fz[(size_t)(i0 - 1 - t) * ns] = make_double2(y.x * rn, y.y * rn);
       }
     }
   }
@@ -2143,6 +2167,8 @@ SolveArgs<R> args_for_sources(const SolveWs<R>& w, int r0) {
   if (a.x) a.x += r * ns * n12;
   if (a.sacc) a.sacc += r * n12;
   if (a.sgrp) a.sgrp += r * (w.ngrp - 1) * n12;
+  if (a.fd) a.fd += r * w.max_iter * ns;
+  if (a.fz) a.fz += r * w.max_iter * ns;
   if (a.pv) a.pv += r * ns * w.nvec;
   if (a.xv) a.xv += r * ns * n12;
   if (a.nco) a.nco += r * ns * kNodeRun * 3;
@@ -2917,6 +2943,8 @@ static int fx_lanczos(ov_ctx* ctx, SolveWs<FX>& w, FxCoef& f, const double2* b_s
   f.g = (double2*)ws_get(ctx, "fxs.gd", sizeof(double2) * (size_t)nsrc * cap, &st);
   f.G = (int4*)ws_get(ctx, "fxs.g", sizeof(int4) * (size_t)nsrc * cap, &st);
   f.info = (FxSumInfo*)ws_get(ctx, "fxs.info", sizeof(FxSumInfo) * nsrc, &st);
+  w.a.fd = (double2*)ws_get(ctx, "fxs.D", sizeof(double2) * (size_t)nsrc * cap * ns, &st);
+  w.a.fz = f.Y;
   if (st != OV_OK) return st;
   w.a.sacc = sums;  // c0 b, written by the init kernel only
   st = init_solve<FX>(ctx, w, b_soa, nsrc, ns, zh, ch, c0, o.tol, cap, s, 0);
@@ -2927,7 +2955,7 @@ static int fx_lanczos(ov_ctx* ctx, SolveWs<FX>& w, FxCoef& f, const double2* b_s
   if (st != OV_OK) return st;
   cudaEvent_t ev;
   kt_begin(ctx, KC_MISC, s, &ev);
-  fx_node_coef_kernel<<<dim3((ns + 31) / 32, nsrc), 32, 0, s>>>(w.a, ns, f.Y);
+  fx_node_coef_kernel<<<dim3((ns + 31) / 32, nsrc), 32, 0, s>>>(w.a, ns);
   fx_sum_nodes_kernel<<<dim3(std::min((cap + 7) / 8, 64), nsrc), 256, 0, s>>>(w.a, ns, f.Y, f.g);
   fx_sum_quant_kernel<<<nsrc, kCoefNT, 0, s>>>(w.a, f.g, f.G, f.info);
   kt_end(ctx, KC_MISC, s, ev);

@@ -94,3 +94,22 @@ def test_non_finite_link_breaks_down(gpu_lib, mode, bad):
     with pytest.raises(gpu_lib.OvError) as e:
         sgn_gpu(ctx, S.gaussian_spinor(dims, 3152), mode=mode)
     assert e.value.code == gpu_lib.OV_ERR_BREAKDOWN
+
+
+@pytest.mark.parametrize("imag", [0.9, 0.22, 0.12])
+def test_coefficients_of_short_and_long_recurrences(gpu_lib, imag):
+    """Nodes that stop early beside one at distance `imag`, which decides the count: within
+    one pass of the coefficient recurrence (512 rows), and beyond it.  Both forms stop at
+    residual tol ||b||: at most 2 sum_j |c_j / Im z_j| tol ||b|| apart."""
+    dims = (4, 4, 4, 6)
+    ctx, _ = make_ctx(gpu_lib, dims, 0.5, 3181)
+    z = np.array([0.3 + 1j * imag, -2.0 + 3.0j, 1.0 - 6.0j, 5.0 + 2.0j])
+    c = np.array([0.4 - 0.3j, -0.7 + 0.2j, 0.5 + 0.1j, 0.2j])
+    ctx.set_contour(z, c, 0.1)
+    b = S.gaussian_spinor(dims, 3182, n=3)
+    want, _ = sgn_gpu(ctx, b, nrhs=3, tol=TOL, mode="fp64_regen")
+    got, st = sgn_gpu(ctx, b, nrhs=3, tol=TOL, mode="fp64_2pass")
+    assert (st["iterations"] > 512) == (imag < 0.2) and st["iterations"] < 1024
+    bound = 2 * np.sum(np.abs(c / z.imag)) * TOL
+    for k in range(3):
+        assert np.linalg.norm(got[k] - want[k]) <= bound * np.linalg.norm(b[k])
