@@ -78,19 +78,22 @@ __device__ __noinline__ double2 hw64_component(const double2* in, size_t ks, siz
 }
 
 __device__ __forceinline__ double2 hw64_scale(longlong2 w, int e) {
-  // (double) w 2^e; a product with a power of two inside the normal range
+  // (double) w 2^e; inside the normal range by an addition to the exponent
   const double x = (double)w.x, y = (double)w.y;
   if (e >= -900 && e <= 900) {
-    const double f = __longlong_as_double((long long)(e + 1023) << 52);
-    return make_double2(x * f, y * f);
+    const int a = e << 20;
+    return make_double2(__hiloint2double(__double2hiint(x) + (w.x != 0 ? a : 0), __double2loint(x)),
+                        __hiloint2double(__double2hiint(y) + (w.y != 0 ? a : 0), __double2loint(y)));
   }
   return make_double2(ldexp(x, e), ldexp(y, e));
 }
 
 // out = H_W in: phase 1 as in fx_lanczos_hw_kernel, each direction's partials at the larger
-// scale of its two neighbours, phase 2 at the largest of the nine; 4 blocks per SM.
+// scale of its two neighbours, phase 2 at the largest of the nine.  3 blocks per SM: 761 us for
+// 12 right-hand sides at 16^3 x 32, where 4 (64 registers, spills) take 843 and 2 take 938.  With
+// the FP64 path of a non-finite site inside the loop over components, 4 took 783.
 template <bool AOS>
-__global__ void __launch_bounds__(kFxNT, 4) hw64_fx_kernel(const int4* __restrict__ X, const int* __restrict__ scale,
+__global__ void __launch_bounds__(kFxNT, 3) hw64_fx_kernel(const int4* __restrict__ X, const int* __restrict__ scale,
                                                            const int4* __restrict__ U, const double2* __restrict__ in,
                                                            const double2* __restrict__ U64, double2* __restrict__ out,
                                                            const __grid_constant__ Geom g, FX diag, double diag64,
@@ -123,26 +126,31 @@ __global__ void __launch_bounds__(kFxNT, 4) hw64_fx_kernel(const int4* __restric
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int k = 2 * wid + j;
-        double2 v;
-        if (e == kExpBad) {
-          const double2* inr = in + (size_t)r * 12 * V;
-          v = hw64_component(inr, AOS ? 1 : V, AOS ? 12 : 1, U64, g, s, k, diag64);
-        } else {
-          const int4 x = __ldg(Xr + fx_index(s, 12) + k * kFxTile);
-          longlong2 w = fx_phase2_scaled(sm, k, lane, k0, k1, k2, k3);
-          long long hh = 0, xx = kFxHalf30;
-          fx_mac(hh, xx, d.hi, d.lo, x.x, x.y);
-          w.x += fx_sar(fx_value(hh, xx), ko);
-          hh = 0;
-          xx = kFxHalf30;
-          fx_mac(hh, xx, d.hi, d.lo, x.z, x.w);
-          w.y += fx_sar(fx_value(hh, xx), ko);
-          v = hw64_scale(w, e + 2);
-        }
+        const int4 x = __ldg(Xr + fx_index(s, 12) + k * kFxTile);
+        longlong2 w = fx_phase2_scaled(sm, k, lane, k0, k1, k2, k3);
+        long long hh = 0, xx = kFxHalf30;
+        fx_mac(hh, xx, d.hi, d.lo, x.x, x.y);
+        w.x += fx_sar(fx_value(hh, xx), ko);
+        hh = 0;
+        xx = kFxHalf30;
+        fx_mac(hh, xx, d.hi, d.lo, x.z, x.w);
+        w.y += fx_sar(fx_value(hh, xx), ko);
+        const double2 v = hw64_scale(w, e + 2);
         if (AOS)
           so[lane * kRow + k] = v;
         else
           out[((size_t)r * 12 + k) * V + s] = v;
+      }
+      if (e == kExpBad) {  // overwrites the two components
+        const double2* inr = in + (size_t)r * 12 * V;
+#pragma unroll 1
+        for (int k = 2 * wid; k < 2 * wid + 2; ++k) {
+          const double2 v = hw64_component(inr, AOS ? 1 : V, AOS ? 12 : 1, U64, g, s, k, diag64);
+          if (AOS)
+            so[lane * kRow + k] = v;
+          else
+            out[((size_t)r * 12 + k) * V + s] = v;
+        }
       }
     }
     if (!AOS) {
