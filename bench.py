@@ -48,6 +48,13 @@ UNIT = "applies/s"
 
 # FP64 arithmetic peak of one GB300 (profiling recipe's nominal table); HBM from MEASURED_PEAKS.json
 FP64_PEAK_TFLOPS = 1.25
+# Wide integer multiply-adds (32 x 32 + 64 bits): 32 lanes per clock and SM (measured loop) x
+# 152 SMs x 2.07 GHz.  Unitary links and |4 - m0| <= 4, as in every workload here: the solver's
+# vectors are integers except in the regeneration and FP32 forms; its stencil kernel needs
+# 1730 such operations per source-iteration and site.
+INT_MAC_PEAK_TERA = 10.07
+INT_MODES = ("fp64", "fp64_2pass", "f32x2")
+INT_MACS_HW = 1730.0
 HBM_FALLBACK_GBS = 6800.0
 
 # The contour of the sign workloads: one explicit single ellipse, the same for both arms
@@ -625,7 +632,8 @@ def roofline(wl, mode, ktimes, kstats, nsrc):
             continue
         d = {"launches": n, "ms": ms, "avg_us": ms / n * 1e3}
         if mode in ("fp64", "fp64_2pass", "fp64_regen", "f32x2") and k in FP64_WORK:
-            uk = dict(units, ls=n * V)
+            # with integer vectors the node updates are not the update kernel's
+            uk = dict(units, ls=n * V, nu=0 if mode in INT_MODES else units["nu"])
             fl = sum(uk[u] * w[0] for u, w in FP64_WORK[k].items())
             by = sum(uk[u] * w[1] for u, w in FP64_WORK[k].items())
             d["tflops"] = fl / (ms / 1e3) / 1e12
@@ -635,10 +643,14 @@ def roofline(wl, mode, ktimes, kstats, nsrc):
         return None, out
     dom = max(out, key=lambda k: out[k]["ms"])
     d = out[dom]
-    if "tflops" in d and mode == "f32x2":
-        # double-float vectors occupy 16 B per complex like FP64: the same algorithmic bytes;
-        # the kernel itself is bound by the FP32 issue rate (about 10 FP32 instructions per
-        # FP64-equivalent flop), so the HBM fraction says how far it is from streaming
+    if "tflops" in d and mode in INT_MODES and dom == "lanczos_hw_kernel":
+        macs = INT_MACS_HW * units["si"] / (d["ms"] / 1e3) / 1e12
+        roof = {"bound": "alu", "achieved": macs, "peak": INT_MAC_PEAK_TERA, "unit": "T wide integer MAC/s",
+                "frac": macs / INT_MAC_PEAK_TERA, "traffic": stored_traffic(dom, wl_name_of(wl)), "kernel": dom,
+                "peak_source": "measured loop: 32 lanes per clock and SM",
+                "fp64_equivalent_tflops": d["tflops"], "hbm_gbs_algorithmic": d["gbs"],
+                "hbm_frac_of_measured": d["gbs"] / hbm, "launch_avg_us": d["avg_us"]}
+    elif "tflops" in d and mode in INT_MODES:
         roof = {"bound": "hbm", "achieved": d["gbs"], "peak": hbm, "unit": "GB/s", "frac": d["gbs"] / hbm,
                 "traffic": stored_traffic(dom, wl_name_of(wl)), "kernel": dom, "peak_source": hbm_src,
                 "fp64_equivalent_tflops": d["tflops"], "launch_avg_us": d["avg_us"]}

@@ -6,7 +6,7 @@
 // every partial sum at 2^-53), however the magnitude varies over the lattice.  A site with a
 // non-finite component among these nine is computed in FP64.
 //
-// 16^3 x 32, 12 right-hand sides, canonical layout: 2655 -> 809 us (packing 134, stencil 676),
+// 16^3 x 32, 12 right-hand sides, canonical layout: 2655 -> 761 us (packing 134, stencil 627),
 // error against 64-bit values 1.9e-16 -> 1.4e-16; 4^4, one right-hand side: 41 -> 10 us.  The
 // stencil is bound by instruction issue (53% of cycles; wide multiply-adds on 53% of theirs).
 #include <cmath>

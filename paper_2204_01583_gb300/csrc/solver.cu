@@ -1261,8 +1261,8 @@ __global__ void __launch_bounds__(32) fx_begin_kernel(const __grid_constant__ So
 // Bound by the wide multiply-adds (one warp instruction per cycle and SM, 1300 per 32 sites
 // for the hops and 430 for the rest, half of the time) and the L2 latency of the neighbour
 // loads.  One source at 16^3 x 32: 63 us, where the FP64 kernel takes 227 us and the
-// double-float one 66 us; 6 sources in one launch: 6 x 45 us (links from L1).  4 blocks per
-// SM (64 registers): 375 ms per 12-source FP64 solve, 393 ms at 3.  NT = 288, for small grids
+// double-float one 66 us; 6 sources in one launch: 6 x 43 us (links from L1).  4 blocks per
+// SM (64 registers): 334 ms per 12-source FP64 solve, 363 at 3, 366 at 5.  NT = 288, for small grids
 // where nothing else covers it: a ninth warp forms the scalars while the others run phase 1
 // (8^4, 4 sources: 8.0 -> 6.5 ms per solve against a last block's serial end); NT = 256: from
 // fx_begin_kernel (formed in every block, 16^3 x 32 took 374 ms instead of 366).
