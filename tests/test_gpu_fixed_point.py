@@ -113,3 +113,17 @@ def test_coefficients_of_short_and_long_recurrences(gpu_lib, imag):
     bound = 2 * np.sum(np.abs(c / z.imag)) * TOL
     for k in range(3):
         assert np.linalg.norm(got[k] - want[k]) <= bound * np.linalg.norm(b[k])
+
+
+@pytest.mark.parametrize("dims,steps", [((4, 4, 4, 4), 4), ((3, 5, 4, 6), 7), ((8, 8, 8, 8), 40), ((12, 12, 12, 16), 24)])
+def test_spectral_bounds(gpu_lib, dims, steps):
+    """The Lanczos bounds from integer vectors (default) and, with the persistent loop enabled,
+    from FP64 vectors.  Over so few steps no Ritz value has converged, so the tridiagonals
+    differ by rounding alone, amplified by at most some thousands: 1e-11 ||H||."""
+    ctx, _ = make_ctx(gpu_lib, dims, 0.5, 3191)
+    got = ctx.place_contour(8, steps=steps)
+    ctx.set_persistent(1)
+    want = ctx.place_contour(8, steps=steps)
+    assert got["steps"] == want["steps"] == steps
+    for key in ("lambda_min", "lambda_max", "abs_max_bound"):
+        assert abs(got[key] - want[key]) <= 1e-11 * 8
