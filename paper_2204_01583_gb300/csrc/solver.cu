@@ -3625,7 +3625,11 @@ static int lanczos_tridiag_fx(ov_ctx* ctx, int steps, std::vector<double>& alpha
 
 int lanczos_tridiag(ov_ctx* ctx, int steps, int squared, std::vector<double>& alpha, std::vector<double>& beta,
                     cudaStream_t s) {
-  if (!squared && fixed_point_fits(ctx)) return lanczos_tridiag_fx(ctx, steps, alpha, beta, s);
+  if (!squared && fixed_point_fits(ctx)) {
+    const int st = lanczos_tridiag_fx(ctx, steps, alpha, beta, s);
+    if (st != OV_ERR_OUT_OF_MEMORY) return st;
+    ws_release(ctx, "lzx.");
+  }
   SolveWs<double> w;
   int st = setup_ws<double>(ctx, 1, 0, false, false, true, steps, &w, "lz");
   if (st != OV_OK) return st;
