@@ -15,8 +15,11 @@
 // Bounds, for links whose rows and columns have norm at most 1 (kFxRowMax) and
 // |4 - m0| <= 4: the real and imaginary parts of a projected component and their sum fit 31
 // bits (hi) and 32 bits (lo); a row's cross terms are below 2^62.3; H_W / 4 is at most
-// (19.6 + 4) / 4 = 5.9 times the largest component, the Lanczos terms add at most 2 + 2 times,
-// so that every sum stays below 2^62.
+// (19.6 + 4) / 4 = 5.9 times the largest component.  The Lanczos coefficients: gam (of X_{i-1})
+// is below 2 by the choice of the shift q; a = <X, w> / <X, X> is at most ||H_W|| / 4 <=
+// (4 + 4 ||U||) / 4, and ||U|| <= 1.733, the Frobenius norm of such a link (all entries
+// 1 / sqrt(3) reach it): |a| <= 2.74, kept in units of 2^-59.  The terms together are at most
+// 5.9 + 2 + 2.74 times the largest component, so that every sum stays below 2^62.
 #pragma once
 
 #include "common.cuh"

@@ -68,7 +68,7 @@ constexpr bool kHalvedLinks = std::is_same<R, double>::value || std::is_same<R, 
 // Fixed point: what the kernels of iteration i know of X_i.
 struct FxVec {
   double n2, inv_n2;  // ||X_i||^2 in integer units and its reciprocal
-  FX dia, gam;        // coefficients of X_i and X_{i-1} in w, unit 2^-60
+  FX dia, gam;        // coefficients of X_i and X_{i-1} in w, unit 2^-60 (both below 2)
   int q;              // w = (H X_i / 4) 2^-q - ...
 };
 
@@ -1428,7 +1428,7 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
     const double bound = fma(fabs(a1), pow2(kFxBits), (double)(m + 1LL) * 4294967296.0);
     const int k = kFxBits - 1 - exponent_of(bound);
     if (lane == 0) {
-      alf_sh = fx_split(-__double2ll_rn(a1 * pow2(60)));
+      alf_sh = fx_split(-__double2ll_rn(a1 * pow2(59)));  // |a1| < 4 (fixed.cuh): a unit more than gam's
       k_sh = k;
     }
     if (blockIdx.x == 0) {
@@ -1460,10 +1460,11 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
       FX o[2];
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
-        // w - a X = w + (ah 2^60 + ax 2^30) / 2^60
-        long long ah = wv[c], ax = kFxHalf30;
-        fx_mac(ah, ax, alf.hi, alf.lo, xv[2 * c], xv[2 * c + 1]);
-        const long long y = fx_shr(fx_shl(fx_value(ah, ax), kl) + rnd, kr);
+        // w - a X = w + 2 hi X.hi + (hi X.lo + lo X.hi) / 2^29
+        long long ah = wv[c] + (long long)alf.hi * (2 * xv[2 * c]), ax = kFxHalf30 >> 1;
+        ax += (long long)alf.hi * xv[2 * c + 1];
+        ax += (long long)alf.lo * xv[2 * c];
+        const long long y = fx_shr(fx_shl(ah + (ax >> 29), kl) + rnd, kr);
         o[c].hi = (int)(y >> 30);
         o[c].lo = ((int)y & 0x3fffffff) - (1 << 29);
         hh += (long long)o[c].hi * o[c].hi;

@@ -1,0 +1,67 @@
+"""Integer Lanczos vectors at the limits of what their dispatch admits (GPU).
+
+An eigenvector of H_W, H b = lambda b, has the closed form S_N b = r_N(lambda) b with
+r_N(lambda) = c0 + sum_j c_j / (z_j - lambda), exact up to the node residuals: at most
+sum_j |c_j / Im z_j| tol ||b|| < 4 tol ||b|| for the nodes below.
+"""
+import numpy as np
+import pytest
+
+import synthetic as S
+from tests.gpu_common import sgn_gpu, to_dev
+
+pytestmark = pytest.mark.gpu
+
+Z = np.array([0.3 + 0.9j, 0.3 - 0.9j, -1.5 + 1.1j, -1.5 - 1.1j, 4.0 + 2.0j])
+C = np.array([0.4 - 0.3j, 0.4 + 0.3j, -0.7 + 0.2j, -0.7 - 0.2j, 0.5 + 0.1j])
+C0 = 0.2
+TOL = 1e-12
+MODES = ("fp64", "fp64_2pass", "f32x2", "fp64_regen")
+
+
+def _r(lam):
+    return C0 + np.sum(C / (Z - lam))
+
+
+def _staggered(dims):
+    lx, ly, lz, lt = dims
+    t, z, y, x = np.meshgrid(np.arange(lt), np.arange(lz), np.arange(ly), np.arange(lx), indexing="ij")
+    return (-1.0) ** (x + y + z + t)
+
+
+def _ctx(lib, dims, U, m0):
+    ctx = lib.Context(dims, bc_t=1, m0=m0)
+    ctx.set_gauge(to_dev(U))
+    ctx.set_contour(Z, C, C0)
+    return ctx
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("spin", [0, 1, 2, 3])
+@pytest.mark.parametrize("dims,m0", [((4, 4, 4, 4), 0.0), ((2, 4, 6, 4), 0.0), ((4, 4, 4, 4), 8.0), ((3, 5, 4, 6), 8.0)])
+def test_eigenvalues_of_modulus_8(gpu_lib, dims, m0, spin, mode):
+    """||H_W|| = |4 - m0| + 4 = 8 at both ends of the masses: free links, periodic time; a
+    constant field has lambda = gamma5 (-m0), a staggered one gamma5 (8 - m0)."""
+    field = np.ones(dims[::-1]) if m0 == 8.0 else _staggered(dims)
+    lam = (-m0 if m0 == 8.0 else 8.0) * (1 if spin < 2 else -1)
+    b = np.zeros(dims[::-1] + (4, 3), dtype=np.complex128)
+    b[..., spin, :] = field[..., None] * np.array([0.7 - 0.2j, -1.1, 0.4j])
+    ctx = _ctx(gpu_lib, dims, S.unit_links(dims), m0)
+    got, st = sgn_gpu(ctx, b, tol=TOL, mode=mode)
+    assert st["converged"] == 1
+    assert np.linalg.norm(got - _r(lam) * b) <= 4 * TOL * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("spin", [0, 2])
+def test_links_of_unit_rows_and_larger_norm(gpu_lib, spin, mode):
+    """All entries 1 / sqrt(3): rows and columns of norm 1, operator norm sqrt(3), and an
+    eigenvalue of modulus 4 - m0 + 4 sqrt(3) = 9.33 on staggered colour singlets."""
+    dims, m0 = (4, 4, 4, 4), 1.6
+    lam = (4.0 - m0 + 4.0 * np.sqrt(3.0)) * (1 if spin < 2 else -1)
+    b = np.zeros(dims[::-1] + (4, 3), dtype=np.complex128)
+    b[..., spin, :] = _staggered(dims)[..., None]
+    ctx = _ctx(gpu_lib, dims, np.full((4,) + dims[::-1] + (3, 3), 3.0**-0.5, dtype=np.complex128), m0)
+    got, st = sgn_gpu(ctx, b, tol=TOL, mode=mode)
+    assert st["converged"] == 1
+    assert np.linalg.norm(got - _r(lam) * b) <= 4 * TOL * np.linalg.norm(b)
