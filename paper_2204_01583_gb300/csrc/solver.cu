@@ -1214,7 +1214,7 @@ __device__ __forceinline__ FxVec fx_vec(const SolveArgs<FX>& a, const SrcState* 
   const FxVec p = S->vec[(i - 1) & 1];
   const int sh = p.q - S->k[(i - 1) & 1];
   FxVec v;
-  v.n2 = fma((double)n[0], pow2(92), (double)n[1] * pow2(60)) + fma((double)n[2], pow2(38), (double)n[3] * 256.0);
+  v.n2 = fma((double)n[0], pow2(92), (double)n[1] * pow2(60)) + fma((double)n[2], pow2(62), (double)n[3] * pow2(30));
   *ratio = v.n2 * p.inv_n2;                // ||X_i||^2 / ||X_{i-1}||^2, 0 if beta_{i-1} is
   *shift = sh;
   const double g1 = *ratio * pow2(sh);     // beta_{i-1} ||X_i|| / (4 ||X_{i-1}||)
@@ -1447,7 +1447,9 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
   const int kl = max(k_sh, 0), kr = max(-k_sh, 0);  // below 32 both
   // 2^k y rounded, plus 2^29 (hi then comes out of a plain shift by 30)
   const long long rnd = (kr > 0 ? 1LL << (kr - 1) : 0) + (kFxHalf30 << kr);
-  // ||X||^2 = n[0] 2^92 + n[1] 2^60 + n[2] 2^38 + n[3] 2^8 (what is dropped is far below 2^-53)
+  // ||X||^2 = n[0] 2^92 + n[1] 2^60 + n[2] 2^62 + n[3] 2^30: high and low words of the hi hi
+  // products and of the rest, whose sums over the largest lattice stay within 63 bits (2^33
+  // reals, one addition of at most 2^32 per four of them) however the components are correlated
   long long n[4] = {0, 0, 0, 0};
   for (size_t eb = e0; eb < n12; eb += B * gs) {
     if (eb != e0) load(eb);
@@ -1473,10 +1475,11 @@ __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX
       }
       if (eb + t * gs < n12) W[eb + t * gs] = make_int4(o[0].hi, o[0].lo, o[1].hi, o[1].lo);
     }
+    xx += ll >> 30;
     n[0] += hh >> 32;
     n[1] += (unsigned)hh;
-    n[2] += xx >> 8;
-    n[3] += ll >> 8;
+    n[2] += xx >> 32;
+    n[3] += (unsigned)xx;
   }
 #pragma unroll
   for (int j = 0; j < 4; ++j) {

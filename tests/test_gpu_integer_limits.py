@@ -65,3 +65,20 @@ def test_links_of_unit_rows_and_larger_norm(gpu_lib, spin, mode):
     got, st = sgn_gpu(ctx, b, tol=TOL, mode=mode)
     assert st["converged"] == 1
     assert np.linalg.norm(got - _r(lam) * b) <= 4 * TOL * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (16, 16, 16, 16), (16, 16, 16, 32)])
+def test_norms_of_constant_vectors(gpu_lib, dims):
+    """A constant field on free links stays constant: no component's low limb differs from
+    site to site, and the sums of the norm add up without cancellation.  Upper spins have
+    lambda = -m0, lower ones m0, so that the Krylov space ends after two vectors."""
+    m0 = 1.6
+    b = np.zeros(dims[::-1] + (4, 3), dtype=np.complex128)
+    b[..., 0, 0], b[..., 1, 2], b[..., 2, 1] = 0.77123, 0.3j, 1.234567
+    want = b.copy()
+    want[..., :2, :] *= _r(-m0)
+    want[..., 2:, :] *= _r(m0)
+    ctx = _ctx(gpu_lib, dims, S.unit_links(dims), m0)
+    got, st = sgn_gpu(ctx, b, tol=TOL, mode="fp64")
+    assert st["converged"] == 1 and st["iterations"] == 2
+    assert np.linalg.norm(got - want) <= 4 * TOL * np.linalg.norm(b)
