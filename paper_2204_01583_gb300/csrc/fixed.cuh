@@ -140,9 +140,11 @@ __device__ __forceinline__ FxHops fx_hops(const Geom& g, int s, int mu) {
 // the vector / 4 (factor -1/2 in the links): u_f + u_b for the upper spin, -A_mu^dag (u_b -
 // u_f) for the lower one.
 constexpr int kFxNT = 256;
+// Products are rounded to nearest and exact zeros stay: a point source's empty components
+// would otherwise collect units of its one large component in every step.
 // SCALED (fields with a scale per site, ov_apply_HW): u_f and u_b are shifted right by sf and
-// sb, products are rounded to nearest and negations exact, so that exact zeros stay.  The
-// Lanczos kernels round down and negate to -v - 1 (a unit of 2^-58; 3% faster).
+// sb before their sums.  Without it negations are to -v - 1, and the reader of the sums over the
+// directions adds the units (fx_negations): an addition of 64 bits less per direction and component.
 template <bool SCALED = false>
 __device__ __forceinline__ void fx_phase1(const int4* __restrict__ in, const int4* __restrict__ U, int mu_spin,
                                           int s, const FxHops& nb, longlong2* out, FxShift sf = {0, 0},
@@ -173,8 +175,8 @@ __device__ __forceinline__ void fx_phase1(const int4* __restrict__ in, const int
     for (int i = 0; i < 3; ++i) {
       // a complex product from three real ones: re = a - b, im = c - a - b with a = l_re h_re,
       // b = l_im h_im, c = (l_re + l_im)(h_re + h_im): 27 wide multiply-adds per row, not 36
-      constexpr long long rnd = SCALED ? kFxHalf30 : 0;
-      long long ah = 0, ax = 0, bh = 0, bx = 0, ch = 0, cx = rnd;
+      // (half a unit in ax rounds re, the second one in cx im)
+      long long ah = 0, ax = kFxHalf30, bh = 0, bx = 0, ch = 0, cx = 2 * kFxHalf30;
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
         const int4 m = l[3 * i + j];
@@ -182,7 +184,7 @@ __device__ __forceinline__ void fx_phase1(const int4* __restrict__ in, const int
         fx_mac(bh, bx, m.z, m.w, h[j].z, h[j].w);
         fx_mac(ch, cx, m.x + m.z, m.y + m.w, hs[j].x, hs[j].y);
       }
-      longlong2 u = make_longlong2(fx_value(ah - bh, ax - bx + rnd), fx_value(ch - ah - bh, cx - ax - bx));
+      longlong2 u = make_longlong2(fx_value(ah - bh, ax - bx), fx_value(ch - ah - bh, cx - ax - bx));
       if (SCALED) {
         u.x = fx_sar(u.x, dir == 0 ? sf : sb);
         u.y = fx_sar(u.y, dir == 0 ? sf : sb);
@@ -200,12 +202,19 @@ __device__ __forceinline__ void fx_phase1(const int4* __restrict__ in, const int
   }
 }
 
+// The directions whose partial of component k is a negation (dre, dim of fx_projection; those
+// of a lower spin only).
+__device__ __forceinline__ int2 fx_negations(int k) {
+  return k < 6 ? make_int2(0, 0) : make_int2(k < 9 ? 4 : 2, 2);
+}
+
 // Component k of gamma5 times the hopping part of H_W x / 4: the sum of the partials.
 __device__ __forceinline__ longlong2 fx_phase2(const longlong2* sm, int k, int lane) {
   constexpr int D = 12 * kFxTile;
   const longlong2* p = sm + k * kFxTile + lane;
   const longlong2 x = p[0], y = p[D], z = p[2 * D], t = p[3 * D];
-  return make_longlong2((x.x + y.x) + (z.x + t.x), (x.y + y.y) + (z.y + t.y));
+  const int2 n = fx_negations(k);
+  return make_longlong2((x.x + y.x) + (z.x + t.x) + n.x, (x.y + y.y) + (z.y + t.y) + n.y);
 }
 // The same with the direction's partials shifted right by k0 .. k3.
 __device__ __forceinline__ longlong2 fx_phase2_scaled(const longlong2* sm, int k, int lane, FxShift k0, FxShift k1,

@@ -67,6 +67,31 @@ def test_links_of_unit_rows_and_larger_norm(gpu_lib, spin, mode):
     assert np.linalg.norm(got - _r(lam) * b) <= 4 * TOL * np.linalg.norm(b)
 
 
+def _against_fp64_vectors(lib, dims, eps, b, modes):
+    """Both forms run to node residuals far below rounding (tol 1e-16), so that rounding is all
+    they differ by.  FP64 vectors commit about 2 units of 2^-53 per Lanczos step, independent
+    of one another: 2 sqrt(500) 2^-53 < 5e-15 over the 500 steps of this contour, which the
+    integer forms have to keep as well."""
+    ctx = lib.Context(dims, bc_t=-1, m0=1.6)
+    ctx.set_gauge(to_dev(S.su3_links(dims, eps, 6001)))
+    ctx.set_contour_ellipse(64, 3.36, 3.36, 0.25)
+    n = b.shape[0]
+    want, _ = sgn_gpu(ctx, b, tol=1e-16, mode="fp64_regen")
+    for mode in modes:
+        got, st = sgn_gpu(ctx, b, tol=1e-16, mode=mode)
+        assert st["converged"] == 1
+        d, w = (got - want).reshape(n, -1), want.reshape(n, -1)
+        assert np.all(np.linalg.norm(d, axis=1) <= 5e-15 * np.linalg.norm(w, axis=1)), mode
+
+
+@pytest.mark.parametrize("dims,eps", [((8, 8, 8, 8), 0.5), ((16, 16, 16, 16), 0.5)])
+def test_point_sources_round_as_fp64_vectors(gpu_lib, dims, eps):
+    """A point source's largest component is its whole norm: noise in units of it on every
+    other component of the lattice adds up to sqrt(24 V) units."""
+    b = S.point_sources(dims, site=(1, 2, 3, 0))[[0, 7]]
+    _against_fp64_vectors(gpu_lib, dims, eps, b, ("fp64",))
+
+
 @pytest.mark.parametrize("dims", [(4, 4, 4, 4), (16, 16, 16, 16), (16, 16, 16, 32)])
 def test_norms_of_constant_vectors(gpu_lib, dims):
     """A constant field on free links stays constant: no component's low limb differs from
