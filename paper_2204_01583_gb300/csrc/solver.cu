@@ -2738,15 +2738,18 @@ static int solve_nodes_fx(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, c
   return st;
 }
 
-// Whether the stored-basis and vector-space forms run in fixed point (fixed.cuh): links of norm 1 (the bounds
-// there) and |4 - m0| <= 4.  Other links and masses, and the persistent loop, keep the
-// FP64 and double-float kernels.
-static bool fixed_point_fits(const ov_ctx* ctx) { return ctx->no_coop && ctx->fx_ok; }
+// Whether the stored-basis and vector-space forms of a solver mode run in fixed point
+// (fixed.cuh): links of norm 1 (the bounds there) and |4 - m0| <= 4.  Other links and masses,
+// the persistent loop and OV_MODE_FP64_REGEN (its gradients included) keep the FP64 and
+// double-float kernels.
+static bool fixed_point_fits(const ov_ctx* ctx, int mode) {
+  return ctx->no_coop && ctx->fx_ok && mode != OV_MODE_FP64_REGEN;
+}
 
 int solve_nodes_soa(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
                     const std::vector<double2>& ch, double2 c0, double2* out_soa, double2* xs_soa,
                     const ov_solve_opts& o, SolveOut* so, cudaStream_t s) {
-  if (fixed_point_fits(ctx) && ns > 0) {
+  if (fixed_point_fits(ctx, o.mode) && ns > 0) {
     const int st = solve_nodes_fx(ctx, b_soa, nsrc, ns, zh, ch, c0, out_soa, xs_soa, o, so, s);
     if (st != OV_ERR_OUT_OF_MEMORY) return st;
     ws_release(ctx, "fxv.");
@@ -3363,7 +3366,7 @@ int nodes_coef<FX>(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const st
 int solve_nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const std::vector<double2>& zh,
                      const std::vector<double2>& ch, int chunk, double2* X, double2* sums, const ov_solve_opts& o,
                      SolveOut* so, cudaStream_t s, const std::function<int(int, int)>& per_chunk) {
-  if (fixed_point_fits(ctx))
+  if (fixed_point_fits(ctx, o.mode))
     return nodes_coef<FX>(ctx, b_soa, nsrc, ns, zh, ch, chunk, X, sums, o, so, s, per_chunk);
   if (o.mode == OV_MODE_F32X2) {
     const int st = ensure_links_df(ctx, s);
@@ -3375,7 +3378,7 @@ int solve_nodes_coef(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const 
 
 int solve_sign_2pass(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int nsrc, const ov_solve_opts& o,
                      SolveOut* so, cudaStream_t s) {
-  if (o.mode != OV_MODE_FP64_REGEN && fixed_point_fits(ctx))
+  if (fixed_point_fits(ctx, o.mode))
     return solve_sign_coef<FX>(ctx, b_soa, out_soa, nsrc, o, so, s);
   if (o.mode == OV_MODE_F32X2) {
     const int st = ensure_links_df(ctx, s);
@@ -3629,7 +3632,7 @@ static int lanczos_tridiag_fx(ov_ctx* ctx, int steps, std::vector<double>& alpha
 
 int lanczos_tridiag(ov_ctx* ctx, int steps, int squared, std::vector<double>& alpha, std::vector<double>& beta,
                     cudaStream_t s) {
-  if (!squared && fixed_point_fits(ctx)) {
+  if (!squared && fixed_point_fits(ctx, OV_MODE_FP64)) {
     const int st = lanczos_tridiag_fx(ctx, steps, alpha, beta, s);
     if (st != OV_ERR_OUT_OF_MEMORY) return st;
     ws_release(ctx, "lzx.");

@@ -92,6 +92,25 @@ def test_point_sources_round_as_fp64_vectors(gpu_lib, dims, eps):
     _against_fp64_vectors(gpu_lib, dims, eps, b, ("fp64",))
 
 
+def test_gradients_of_the_regeneration_form_keep_fp64_vectors(gpu_lib):
+    """S_N is hermitian on nodes in conjugate pairs: the gradient of Re<eta, S_N b> in b is
+    S_N eta, here from OV_MODE_FP64_REGEN on both sides."""
+    import torch
+
+    dims = (8, 8, 8, 8)
+    ctx = gpu_lib.Context(dims, bc_t=-1, m0=1.6)
+    ctx.set_gauge(to_dev(S.su3_links(dims, 0.5, 6001)))
+    ctx.set_contour_ellipse(64, 3.36, 3.36, 0.25)
+    eta = S.point_sources(dims, site=(1, 2, 3, 0))[7]
+    want, _ = sgn_gpu(ctx, eta, tol=1e-16, mode="fp64_regen")
+    ed, grad_b = to_dev(eta), torch.empty(dims[::-1] + (4, 3), dtype=torch.complex128, device="cuda")
+    st = ctx.sgn_vjp(ed, to_dev(S.gaussian_spinor(dims, 6002)), grad_b, None, ctx.opts(tol=1e-16, mode="fp64_regen"))
+    torch.cuda.synchronize()
+    assert st["converged"] == 1
+    d = grad_b.cpu().numpy() - want
+    assert np.linalg.norm(d) <= 5e-15 * np.linalg.norm(want)  # as in _against_fp64_vectors
+
+
 @pytest.mark.parametrize("dims", [(4, 4, 4, 4), (16, 16, 16, 16), (16, 16, 16, 32)])
 def test_norms_of_constant_vectors(gpu_lib, dims):
     """A constant field on free links stays constant: no component's low limb differs from
