@@ -1868,36 +1868,43 @@ __global__ void __launch_bounds__(32) fx_node_coef_kernel(const __grid_constant_
   }
 }
 
-// Coefficients w[0..k) as integers: at most 2^57, and so small that a sum over all k of
-// 2^-60 out_i X_i stays below 2^62 (k <= kFxSumMax; longer sums are cut into pieces of that
-// length).  Returns the factor that undoes the scale.  *real: all imaginary parts vanish up
-// to rounding.
-constexpr int kFxSumMax = 256;
+// Coefficients of a sum over basis vectors as integers, a scale per group of vectors: up to the
+// 1st, 2nd, 4th, 8th and 64th one, then 256 at a time.  G_i = g_i / ||X_i|| falls by orders of
+// magnitude while a point source spreads (||X_1|| is one component, ||X_i|| as many as the source
+// has reached); with one scale for all, each of the later vectors' components was rounded to
+// a unit of the first one's coefficient: 2.3e-12 of a sum over the 16^4 lattice, now 8e-16 as
+// with FP64 vectors.  Few groups, since each costs a conversion to FP64 per sum.
+// A group's sum is one of n terms of at most 2^bits 2^58 / 2^60 (two per vector if complex)
+// below 2^62: bits = 64 - log2 n, 59 at most for the cross terms' sake, one less if complex.
+constexpr int kFxGroup = 256;
+__host__ __device__ constexpr int fx_group_end(int g) { return g < 4 ? 1 << g : 64 + kFxGroup * (g - 4); }
+constexpr int fx_groups(int k) { return 5 + (k + kFxGroup - 1) / kFxGroup; }  // at most, for k vectors
+
+// out = w[0..k) in integers, a warp per group; scale: what undoes each group's
 template <int NT, typename F>
-__device__ __forceinline__ double fx_quantise(F w, int k, int4* out, bool* real, int* sh) {
-  int mr = 0, mi = 0;  // high words of the largest |re|, |im|
-  for (int i = threadIdx.x; i < k; i += NT) {
-    const double2 v = w(i);
-    mr = max(mr, __double2hiint(v.x) & 0x7fffffff);
-    mi = max(mi, __double2hiint(v.y) & 0x7fffffff);
+__device__ __forceinline__ void fx_quantise(F w, int k, bool complex_sum, int4* out, double* scale) {
+  const int lane = threadIdx.x & 31;
+  for (int g = threadIdx.x >> 5;; g += NT / 32) {
+    const int i0 = g > 0 ? fx_group_end(g - 1) : 0, end = min(k, fx_group_end(g));
+    if (i0 >= k) break;
+    int hi = 0;  // high word of the largest |re|, |im|
+    for (int i = i0 + lane; i < end; i += 32) {
+      const double2 v = w(i);
+      hi = max(hi, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
+    }
+    const int bits = min(59, 32 + __clz(end - i0 - 1)) - (complex_sum ? 1 : 0);
+    const int m = __reduce_max_sync(0xffffffffu, hi) >> 20;
+    const int e = m > 0 && m < 0x7ff ? bits - 1 - (m - 1023) : bits - 1;
+    for (int i = i0 + lane; i < end; i += 32) {
+      const double2 v = w(i);
+      const FX re = fx_split(__double2ll_rn(ldexp(v.x, e))), im = fx_split(__double2ll_rn(ldexp(v.y, e)));
+      out[i] = make_int4(re.hi, re.lo, im.hi, im.lo);
+    }
+    if (lane == 0) scale[g] = ldexp(1.0, 60 - e);
   }
-  mr = block_max<NT>(mr, sh);
-  __syncthreads();
-  mi = block_max<NT>(mi, sh);
-  *real = __hiloint2double(mi, 0) <= 1e-14 * __hiloint2double(mr, 0);
-  // a complex sum adds two products per term: out < 2^(63 - log2 k)
-  const int bits = min(57, 62 - (31 - __clz(max(min(k, kFxSumMax), 1))));
-  const int m = max(mr, mi) >> 20, e = m > 0 && m < 0x7ff ? bits - 1 - (m - 1023) : bits - 1;
-  for (int i = threadIdx.x; i < k; i += NT) {
-    const double2 v = w(i);
-    const FX re = fx_split(__double2ll_rn(ldexp(v.x, e))), im = fx_split(__double2ll_rn(ldexp(v.y, e)));
-    out[i] = make_int4(re.hi, re.lo, im.hi, im.lo);
-  }
-  return ldexp(1.0, 60 - e);
 }
 
 struct FxSumInfo {
-  double scale;
   int k, real;
 };
 
@@ -1923,31 +1930,38 @@ __global__ void __launch_bounds__(256) fx_sum_nodes_kernel(const __grid_constant
   }
 }
 
-// G = g in integers, one block per source.  Real coefficients come from a node list closed
-// under conjugation (basis_sum_kernel).
+// G = g in integers, one block per source.  Real coefficients (of unit vectors, up to rounding)
+// come from a node list closed under conjugation (basis_sum_kernel).
 constexpr int kCoefNT = 256;
 __global__ void __launch_bounds__(kCoefNT) fx_sum_quant_kernel(const __grid_constant__ SolveArgs<FX> a,
                                                                const double2* __restrict__ g, int4* __restrict__ G,
+                                                               double* __restrict__ scale, int ng,
                                                                FxSumInfo* __restrict__ info) {
-  __shared__ int sh[kCoefNT / 32];
+  __shared__ int sh[2][kCoefNT / 32];
   const int r = blockIdx.x, mi = a.prm->max_iter, k = a.src[r].iter - 1;
-  bool real;
-  const double sc =
-      fx_quantise<kCoefNT>([&](int i) { return g[(size_t)r * mi + i]; }, k, G + (size_t)r * mi, &real, sh);
-  if (threadIdx.x == 0) info[r] = {sc, k, real ? 1 : 0};
+  const double2* gr = g + (size_t)r * mi;
+  const double* n2 = a.hist_n2 + (size_t)r * mi;
+  int mr = 0, mm = 0;  // high words of the largest |re|, |im|
+  for (int i = threadIdx.x; i < k; i += kCoefNT) {
+    const double n = sqrt(n2[i]);
+    mr = max(mr, __double2hiint(gr[i].x * n) & 0x7fffffff);
+    mm = max(mm, __double2hiint(gr[i].y * n) & 0x7fffffff);
+  }
+  mr = block_max<kCoefNT>(mr, sh[0]);
+  mm = block_max<kCoefNT>(mm, sh[1]);
+  const bool real = __hiloint2double(mm, 0) <= 1e-14 * __hiloint2double(mr, 0);
+  fx_quantise<kCoefNT>([&](int i) { return gr[i]; }, k, !real, G + (size_t)r * mi, scale + (size_t)r * ng);
+  if (threadIdx.x == 0) info[r] = {k, real ? 1 : 0};
 }
 
 // Yq[r][j][i] = Y[r][i][j] in integers, one block per (node, source)
 __global__ void __launch_bounds__(128) fx_node_quant_kernel(const __grid_constant__ SolveArgs<FX> a, int ns,
                                                             const double2* __restrict__ Y, int4* __restrict__ Yq,
-                                                            double* __restrict__ scale) {
-  __shared__ int sh[128 / 32];
+                                                            double* __restrict__ scale, int ng) {
   const int r = blockIdx.y, j = blockIdx.x, mi = a.prm->max_iter, k = a.src[r].iter - 1;
   const double2* y = Y + (size_t)r * mi * ns + j;
-  bool real;
   const size_t o = (size_t)r * ns + j;
-  const double sc = fx_quantise<128>([&](int i) { return y[(size_t)i * ns]; }, k, Yq + o * mi, &real, sh);
-  if (threadIdx.x == 0) scale[o] = sc;
+  fx_quantise<128>([&](int i) { return y[(size_t)i * ns]; }, k, false, Yq + o * mi, scale + o * ng);
 }
 
 // K basis vectors' products, their cross terms within 63 bits, added to re and im in units of
@@ -1972,11 +1986,12 @@ __device__ __forceinline__ void fx_sum_group(const int4* __restrict__ w, const i
   im += ix >> 30;
 }
 
-// sum[r][e] += scale_r sum_i G_i X_i[e] (basis_sum_kernel in fixed point), G_i = g_i / ||X_i||:
-// exact integer sums of up to kFxSumMax vectors.  Reads 16 B per basis vector and element:
-// HBM-bound.
+// sum[r][e] += sum_i G_i X_i[e] (basis_sum_kernel in fixed point), G_i = g_i / ||X_i||: exact
+// integer sums of a group of vectors, the groups added in FP64.  Reads 16 B per basis vector and
+// element: HBM-bound.
 __global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restrict__ basis, int nslots,
                                                            const int4* __restrict__ G, int ldg,
+                                                           const double* __restrict__ scale, int ng,
                                                            const FxSumInfo* __restrict__ info,
                                                            double2* __restrict__ sum, int V) {
   const int r = blockIdx.y;
@@ -1986,38 +2001,55 @@ __global__ void __launch_bounds__(256) fx_basis_sum_kernel(const int4* __restric
   if (site >= V) return;
   const int4* B = basis + (size_t)r * nslots * n12 + n12 + e;
   const int4* w = G + (size_t)r * ldg;
+  const double* sc = scale + (size_t)r * ng;
   const FxSumInfo f = info[r];
   constexpr int K = 8;
   double re = 0.0, im = 0.0;
-  for (int i0 = 0; i0 < f.k; i0 += kFxSumMax) {
-    const int end = min(f.k, i0 + kFxSumMax);
+  auto close = [&](int g, long long sr, long long si) {
+    const double s = __ldg(sc + g);
+    re = fma(s, (double)sr, re);
+    im = fma(s, (double)si, im);
+  };
+  int g = 0, i = 0;
+  if (f.k >= K) {  // the groups of 1, 1, 2 and 4, their loads together
+    long long s[4][2] = {};
+    fx_sum_group<false, 1>(w, B, n12, 1, s[0][0], s[0][1]);
+    fx_sum_group<false, 1>(w + 1, B + n12, n12, 1, s[1][0], s[1][1]);
+    fx_sum_group<false, 2>(w + 2, B + 2 * n12, n12, 2, s[2][0], s[2][1]);
+    fx_sum_group<false, 4>(w + 4, B + 4 * n12, n12, 4, s[3][0], s[3][1]);
+    for (; g < 4; ++g) close(g, s[g][0], s[g][1]);
+    i = K;
+  }
+  for (; i < f.k; ++g) {
+    const int end = min(f.k, fx_group_end(g));
     long long sr = 0, si = 0;
-    int i = i0;
     if (f.real) {
       for (; i + K <= end; i += K) fx_sum_group<true, K>(w + i, B + (size_t)i * n12, n12, K, sr, si);
     } else {
       for (; i + K <= end; i += K) fx_sum_group<false, K>(w + i, B + (size_t)i * n12, n12, K, sr, si);
     }
     if (i < end) fx_sum_group<false, K>(w + i, B + (size_t)i * n12, n12, end - i, sr, si);
-    re += (double)sr;
-    im += (double)si;
+    i = end;
+    close(g, sr, si);
   }
   double2* so = sum + ((size_t)r * 12 + tk % 12) * V + site;
   double2 sv = *so;
-  sv.x = fma(f.scale, re, sv.x);
-  sv.y = fma(f.scale, im, sv.y);
+  sv.x += re;
+  sv.y += im;
   *so = sv;
 }
 
 // Per-node solutions from a fixed-point basis: x_j = A + i B with A = sum_i Re(Y_i) X_i, B = sum_i
 // Im(Y_i) X_i.  A node whose conjugate is also in the list needs no sums of its own: its
 // coefficients are the conjugates (T_k is real), its solution A - i B.  Two nodes or pairs per
-// thread (slot: node, partner or -1), Y per (source, node) with its own scale.  Bound by wide
-// multiply-adds, 12 per slot, element and basis vector.  (8^4, 2 sources, 48 nodes, 352
-// vectors: 4.4 ms with every node on its own and groups of 8 summed in FP64.)
-__global__ void __launch_bounds__(256) fx_basis_nodes_kernel(const int4* __restrict__ basis, int nslots,
+// thread (slot: node, partner or -1), Y per (source, node) with its own scales.  Bound by wide
+// multiply-adds, 12 per slot, element and basis vector.  Three blocks per SM cover the FP64
+// conversions between groups (8^4, 2 sources, 48 nodes, 352 vectors: 1.66 ms, 2.14 with two blocks;
+// 1.89 with two and a single scale; 4.4 with every node on its own and groups of 8 summed in
+// FP64).
+__global__ void __launch_bounds__(256, 3) fx_basis_nodes_kernel(const int4* __restrict__ basis, int nslots,
                                                              const int4* __restrict__ Y,
-                                                             const double* __restrict__ scale, int ns, int ldy,
+                                                             const double* __restrict__ scale, int ng, int ns, int ldy,
                                                              const FxSumInfo* __restrict__ info,
                                                              const int2* __restrict__ slot, int nslot, int j0, int nc,
                                                              double2* __restrict__ X, int V) {
@@ -2041,50 +2073,71 @@ __global__ void __launch_bounds__(256) fx_basis_nodes_kernel(const int4* __restr
   for (int t = 0; t < JT; ++t)
 #pragma unroll
     for (int c = 0; c < 4; ++c) s[t][c] = 0.0;
-  for (int i0 = 0; i0 < k; i0 += kFxSumMax) {
-    const int end = min(k, i0 + kFxSumMax);
-    long long h[JT][4] = {};
-    for (int i = i0; i < end; i += K) {
-      long long x[JT][4];
+  long long h[JT][4] = {};
+  // h += the products of vectors i .. i + n - 1 (N of them, n in a tail)
+  auto add = [&](auto count, int i, int n) {
+    constexpr int N = decltype(count)::value;
+    long long x[JT][4];
 #pragma unroll
-      for (int t = 0; t < JT; ++t)
+    for (int t = 0; t < JT; ++t)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) x[t][c] = kFxHalf30;
-      auto add = [&](int m) {
-        const int4 u = __ldg(B + (size_t)(i + m) * n12);
+      for (int c = 0; c < 4; ++c) x[t][c] = kFxHalf30;
 #pragma unroll
-        for (int t = 0; t < JT; ++t) {
-          const int4 w = __ldg(y[t] + i + m);
-          fx_mac(h[t][0], x[t][0], w.x, w.y, u.x, u.y);
-          fx_mac(h[t][1], x[t][1], w.x, w.y, u.z, u.w);
-          fx_mac(h[t][2], x[t][2], w.z, w.w, u.x, u.y);
-          fx_mac(h[t][3], x[t][3], w.z, w.w, u.z, u.w);
-        }
-      };
-      if (i + K <= end) {
+    for (int m = 0; m < N; ++m) {
+      if (m >= n) break;
+      const int4 u = __ldg(B + (size_t)(i + m) * n12);
 #pragma unroll
-        for (int m = 0; m < K; ++m) add(m);
-      } else {
-        for (int m = 0; i + m < end; ++m) add(m);
+      for (int t = 0; t < JT; ++t) {
+        const int4 v = __ldg(y[t] + i + m);
+        fx_mac(h[t][0], x[t][0], v.x, v.y, u.x, u.y);
+        fx_mac(h[t][1], x[t][1], v.x, v.y, u.z, u.w);
+        fx_mac(h[t][2], x[t][2], v.z, v.w, u.x, u.y);
+        fx_mac(h[t][3], x[t][3], v.z, v.w, u.z, u.w);
       }
-#pragma unroll
-      for (int t = 0; t < JT; ++t)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) h[t][c] += x[t][c] >> 30;
     }
 #pragma unroll
     for (int t = 0; t < JT; ++t)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) s[t][c] += (double)h[t][c];
+      for (int c = 0; c < 4; ++c) h[t][c] += x[t][c] >> 30;
+  };
+  auto close = [&](int g) {
+#pragma unroll
+    for (int t = 0; t < JT; ++t) {
+      const double sc = __ldg(scale + ((size_t)r * ns + nd[t].x) * ng + g);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        s[t][c] = fma(sc, (double)h[t][c], s[t][c]);
+        h[t][c] = 0;
+      }
+    }
+  };
+  int g = 0, i = 0;
+  if (k >= K) {  // the groups of 1, 1, 2 and 4, their loads together
+    add(std::integral_constant<int, 1>(), 0, 1);
+    close(0);
+    add(std::integral_constant<int, 1>(), 1, 1);
+    close(1);
+    add(std::integral_constant<int, 2>(), 2, 2);
+    close(2);
+    add(std::integral_constant<int, 4>(), 4, 4);
+    close(3);
+    g = 4;
+    i = K;
+  }
+  for (; i < k; ++g) {
+    const int end = min(k, fx_group_end(g));
+    for (; i + K <= end; i += K) add(std::integral_constant<int, K>(), i, K);
+    if (i < end) add(std::integral_constant<int, K>(), i, end - i);
+    i = end;
+    close(g);
   }
 #pragma unroll
   for (int t = 0; t < JT; ++t) {
     if (q0 + t >= nslot) break;
-    const double sc = scale[(size_t)r * ns + nd[t].x];
     double2* o = X + ((size_t)r * nc * 12 + tk % 12) * V + site;
     const size_t st = (size_t)12 * V;
-    o[(nd[t].x - j0) * st] = make_double2(sc * (s[t][0] - s[t][3]), sc * (s[t][1] + s[t][2]));
-    if (nd[t].y >= 0) o[(nd[t].y - j0) * st] = make_double2(sc * (s[t][0] + s[t][3]), sc * (s[t][1] - s[t][2]));
+    o[(nd[t].x - j0) * st] = make_double2(s[t][0] - s[t][3], s[t][1] + s[t][2]);
+    if (nd[t].y >= 0) o[(nd[t].y - j0) * st] = make_double2(s[t][0] + s[t][3], s[t][1] - s[t][2]);
   }
 }
 
@@ -2936,6 +2989,8 @@ int solve_sign_stored(ov_ctx* ctx, const double2* b_soa, double2* out_soa, int n
 struct FxCoef {
   double2 *Y = nullptr, *g = nullptr;
   int4* G = nullptr;
+  double* scale = nullptr;  // [src][ng] of G's groups
+  int ng = 0;
   FxSumInfo* info = nullptr;
 };
 
@@ -2949,6 +3004,8 @@ static int fx_lanczos(ov_ctx* ctx, SolveWs<FX>& w, FxCoef& f, const double2* b_s
   f.Y = (double2*)ws_get(ctx, "fxs.Y", sizeof(double2) * (size_t)nsrc * cap * ns, &st);
   f.g = (double2*)ws_get(ctx, "fxs.gd", sizeof(double2) * (size_t)nsrc * cap, &st);
   f.G = (int4*)ws_get(ctx, "fxs.g", sizeof(int4) * (size_t)nsrc * cap, &st);
+  f.ng = fx_groups(cap);
+  f.scale = (double*)ws_get(ctx, "fxs.gs", sizeof(double) * (size_t)nsrc * f.ng, &st);
   f.info = (FxSumInfo*)ws_get(ctx, "fxs.info", sizeof(FxSumInfo) * nsrc, &st);
   w.a.fd = (double2*)ws_get(ctx, "fxs.D", sizeof(double2) * (size_t)nsrc * cap * ns, &st);
   w.a.fz = f.Y;
@@ -2964,7 +3021,7 @@ static int fx_lanczos(ov_ctx* ctx, SolveWs<FX>& w, FxCoef& f, const double2* b_s
   kt_begin(ctx, KC_MISC, s, &ev);
   fx_node_coef_kernel<<<dim3((ns + 31) / 32, nsrc), 32, 0, s>>>(w.a, ns);
   fx_sum_nodes_kernel<<<dim3(std::min((cap + 7) / 8, 64), nsrc), 256, 0, s>>>(w.a, ns, f.Y, f.g);
-  fx_sum_quant_kernel<<<nsrc, kCoefNT, 0, s>>>(w.a, f.g, f.G, f.info);
+  fx_sum_quant_kernel<<<nsrc, kCoefNT, 0, s>>>(w.a, f.g, f.G, f.scale, f.ng, f.info);
   kt_end(ctx, KC_MISC, s, ev);
   OV_CHECK_LAUNCH(ctx, "fx_node_coef_kernel");
   *launches += 3.0;
@@ -2975,8 +3032,8 @@ static int launch_fx_basis_sum(ov_ctx* ctx, const SolveWs<FX>& w, const FxCoef& 
                                cudaStream_t s) {
   cudaEvent_t ev;
   kt_begin(ctx, KC_BASIS_SUM, s, &ev);
-  fx_basis_sum_kernel<<<dim3((unsigned)((w.nvec + 255) / 256), nsrc), 256, 0, s>>>(w.a.ring, cap + 3, f.G, cap, f.info,
-                                                                                sums, ctx->g.V);
+  fx_basis_sum_kernel<<<dim3((unsigned)((w.nvec + 255) / 256), nsrc), 256, 0, s>>>(w.a.ring, cap + 3, f.G, cap, f.scale,
+                                                                                f.ng, f.info, sums, ctx->g.V);
   kt_end(ctx, KC_BASIS_SUM, s, ev);
   OV_CHECK_LAUNCH(ctx, "fx_basis_sum_kernel");
   return OV_OK;
@@ -3321,12 +3378,12 @@ int nodes_coef<FX>(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const st
   double launches = 0.0;
   int st = fx_lanczos(ctx, w, f, b_soa, nsrc, ns, zh, ch, make_double2(0.0, 0.0), sums, o, s, cap, 7, &launches);
   int4* Yq = (int4*)ws_get(ctx, "fxs.Yq", sizeof(int4) * (size_t)nsrc * ns * cap, &st);
-  double* Ysc = (double*)ws_get(ctx, "fxs.Ysc", sizeof(double) * (size_t)nsrc * ns, &st);
+  double* Ysc = (double*)ws_get(ctx, "fxs.Ysc", sizeof(double) * (size_t)nsrc * ns * f.ng, &st);
   if (st == OV_OK) st = launch_fx_basis_sum(ctx, w, f, nsrc, cap, sums, s);
   if (st != OV_OK) return st;
   const int fst = finish_solve<FX>(ctx, w, nsrc, ns, zh, ch, so, s);
   if (fst != OV_OK && !(fst == OV_ERR_NOT_CONVERGED && cap >= o.max_iter)) return OV_ERR_INVALID_ARG;
-  fx_node_quant_kernel<<<dim3(ns, nsrc), 128, 0, s>>>(w.a, ns, f.Y, Yq, Ysc);
+  fx_node_quant_kernel<<<dim3(ns, nsrc), 128, 0, s>>>(w.a, ns, f.Y, Yq, Ysc, f.ng);
   int2* slotd = (int2*)ws_get(ctx, "fxs.slot", sizeof(int2) * ns, &st);
   if (st != OV_OK) return st;
   std::vector<int2> slot;
@@ -3354,7 +3411,7 @@ int nodes_coef<FX>(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, const st
     if (e != cudaSuccess) return ctx_cuda(ctx, e, "copy node pairs");
     const int nslot = (int)slot.size();
     fx_basis_nodes_kernel<<<dim3((unsigned)((w.nvec + 255) / 256), nsrc, (nslot + 1) / 2), 256, 0, s>>>(
-        w.a.ring, cap + 3, Yq, Ysc, ns, cap, f.info, slotd, nslot, j0, nc, X, ctx->g.V);
+        w.a.ring, cap + 3, Yq, Ysc, f.ng, ns, cap, f.info, slotd, nslot, j0, nc, X, ctx->g.V);
     OV_CHECK_LAUNCH(ctx, "fx_basis_nodes_kernel");
     if ((st = per_chunk(j0, nc)) != OV_OK) return st;
   }

@@ -92,6 +92,39 @@ def test_point_sources_round_as_fp64_vectors(gpu_lib, dims, eps):
     _against_fp64_vectors(gpu_lib, dims, eps, b, ("fp64",))
 
 
+@pytest.mark.parametrize("kind", ["point", "gauss"])
+@pytest.mark.parametrize("dims", [(8, 8, 8, 8), (16, 16, 16, 16)])
+def test_sums_over_the_stored_basis_round_as_fp64_vectors(gpu_lib, dims, kind):
+    """The coefficients of a point source's first vectors are orders of magnitude above those
+    of the later ones, which reach the whole lattice."""
+    b = S.point_sources(dims, site=(1, 2, 3, 0))[[0, 7]] if kind == "point" else S.gaussian_spinor(dims, 6003, n=2)
+    _against_fp64_vectors(gpu_lib, dims, 0.5, b, ("fp64_2pass", "f32x2"))
+
+
+@pytest.mark.parametrize("mode", ["fp64_2pass", "f32x2"])
+def test_node_solutions_round_as_fp64_vectors(gpu_lib, mode):
+    """The same for the per-node solutions behind the link force: products of two solutions,
+    each within 5e-15 of the FP64 form (_against_fp64_vectors)."""
+    import torch
+
+    dims = (8, 8, 8, 8)
+    ctx = gpu_lib.Context(dims, bc_t=-1, m0=1.6)
+    ctx.set_gauge(to_dev(S.su3_links(dims, 0.5, 6001)))
+    ctx.set_contour_ellipse(64, 3.36, 3.36, 0.25)
+    pt = S.point_sources(dims, site=(1, 2, 3, 0))
+    out = {}
+    for m in ("fp64_regen", mode):
+        gb = torch.empty(dims[::-1] + (4, 3), dtype=torch.complex128, device="cuda")
+        gl = torch.empty((4,) + dims[::-1] + (8,), dtype=torch.float64, device="cuda")
+        st = ctx.sgn_vjp(to_dev(pt[7]), to_dev(pt[0]), gb, gl, ctx.opts(tol=1e-16, mode=m))
+        torch.cuda.synchronize()
+        assert st["converged"] == 1
+        out[m] = gb.cpu().numpy(), gl.cpu().numpy()
+    (b1, l1), (b0, l0) = out[mode], out["fp64_regen"]
+    assert np.linalg.norm(b1 - b0) <= 5e-15 * np.linalg.norm(b0)
+    assert np.linalg.norm(l1 - l0) <= 1e-14 * np.linalg.norm(l0)
+
+
 def test_gradients_of_the_regeneration_form_keep_fp64_vectors(gpu_lib):
     """S_N is hermitian on nodes in conjugate pairs: the gradient of Re<eta, S_N b> in b is
     S_N eta, here from OV_MODE_FP64_REGEN on both sides."""
