@@ -49,7 +49,7 @@ UNIT = "applies/s"
 # FP64 arithmetic peak of one GB300 (profiling recipe's nominal table); HBM from MEASURED_PEAKS.json
 FP64_PEAK_TFLOPS = 1.25
 # Wide integer multiply-adds (32 x 32 + 64 bits): 32 lanes per clock and SM (measured loop) x
-# 152 SMs x 2.07 GHz.  Unitary links and |4 - m0| <= 4, as in every workload here: the solver's
+# 152 SMs x 2.07 GHz.  SU(3) links and |4 - m0| <= 4, as in every workload here: the solver's
 # vectors are integers except in the regeneration and FP32 forms; its stencil kernel needs
 # 1730 such operations per source-iteration and site.
 INT_MAC_PEAK_TERA = 10.07

@@ -68,9 +68,9 @@ typedef enum {
   /* FP64 shifted solve: one Lanczos process on H_W serves every node; each node
    * keeps its own FP64 search direction and the weighted sum of Eq. 7 is
    * accumulated in the same pass (the paper's shift-solver structure).
-   * Unitary links and |4 - m0| <= 4, where 29 more vectors per source fit: the Lanczos
-   * vectors are integers as in OV_MODE_FP64_2PASS, and the nodes' FP64 vectors take eight
-   * iterations at a time beside the next ones. */
+   * Links of unit norm (see ov_set_gauge) and |4 - m0| <= 4, where 29 more vectors per
+   * source fit: the Lanczos vectors are integers as in OV_MODE_FP64_2PASS, and the nodes'
+   * FP64 vectors take eight iterations at a time beside the next ones. */
   OV_MODE_FP64 = 0,
   /* Mixed precision: FP32 shifted solve, then batched per-node FP64 true
    * residuals and FP32 defect-correction solves over all nodes x sources in
@@ -82,7 +82,7 @@ typedef enum {
    * memory when min(max_iter, 1024) vectors per source fit a quarter of it (the sum is
    * then one read of the basis); otherwise a second Lanczos pass regenerates it.
    * Same result as OV_MODE_FP64 up to rounding; vector work independent of N.
-   * Unitary links and |4 - m0| <= 4: the vectors of the stored basis are 58-bit integers
+   * Links of unit norm and |4 - m0| <= 4: the vectors of the stored basis are 58-bit integers
    * of one scale per vector, products and sums of them exact to 2^-58 of the vector's
    * largest component (GB300's FP64 rate is a fourteenth of its integer multiply rate);
    * recurrence scalars and the result stay FP64.  Other links and masses: FP64 vectors. */
@@ -90,7 +90,7 @@ typedef enum {
   /* As OV_MODE_FP64_2PASS, always regenerating the basis (memory: three vectors per
    * source). */
   OV_MODE_FP64_REGEN = 3,
-  /* As OV_MODE_FP64_2PASS; where its integer vectors do not apply (links not unitary, or
+  /* As OV_MODE_FP64_2PASS; where its integer vectors do not apply (other links, or
    * |4 - m0| > 4) or a stored basis does not fit, every vector operation -- the H_W
    * stencil, the Lanczos updates and the basis -- is in FP32-pair (double-float)
    * arithmetic on the FP32 units: each real is an unevaluated sum of two floats (~48-bit significand), sums
@@ -169,14 +169,17 @@ const char* ov_last_error(const ov_ctx* ctx);
  * experiments").  Canonical layout U[mu][t][z][y][x][3][3], V*4*9 complex doubles.
  * U may be a host (on_device = 0) or device (on_device = 1) pointer; it is copied on
  * `stream` and not retained.  The library keeps FP64, FP32 and double-float
- * structure-of-arrays copies.  Any cached contour placement is invalidated (explicit
+ * structure-of-arrays copies and, where every row and every column of every link has a
+ * norm between 1/2 and 1 (up to 1.00045: SU(3) links, and shortened ones), a 58-bit
+ * integer copy: "links of unit norm" below.  Other links take FP64, double-float and
+ * FP32 arithmetic only.  Any cached contour placement is invalidated (explicit
  * contours are kept).  Errors: INVALID_ARG (null U), OUT_OF_MEMORY, CUDA. */
 int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream);
 
 /* out = H_W in (Eq. 1 and the definition of H_W = gamma5 D_W(-m0) after it) for nrhs
  * spinors in the canonical layout psi[rhs][t][z][y][x][4][3], device pointers, in the
- * given precision (OV_FP64: complex double, OV_FP32: complex float).  FP64 with unitary
- * links and |4 - m0| <= 4 is computed in integers, exact to about 2^-57 of the largest
+ * given precision (OV_FP64: complex double, OV_FP32: complex float).  FP64 with links
+ * of unit norm and |4 - m0| <= 4 is computed in integers, exact to about 2^-57 of the largest
  * component of each output's site and its eight neighbours (non-finite components
  * propagate as in FP64 arithmetic); other links and masses in FP64.  in and out must
  * not alias.  nrhs = 0 is a no-op.  Errors: INVALID_ARG, NO_GAUGE, OUT_OF_MEMORY, CUDA. */

@@ -124,8 +124,8 @@ __global__ void links_df_kernel(const double2* __restrict__ u64, float4* __restr
 }
 
 // FP64 solver links (-1/2 U, boundary sign included) -> fixed-point tiles of unit 2^-58; *bad
-// is set when a link's rows or columns exceed the norm the fixed-point bounds assume (not
-// unitary, or not finite)
+// is set when a link's rows or columns are longer than the fixed-point bounds assume (or not
+// finite) or shorter than kFxRowMin
 __global__ void links_fx_kernel(const double2* __restrict__ u, int4* __restrict__ ufx,
                                 int V, int* __restrict__ bad) {
   const size_t n = 4 * fx_padded(V);
@@ -144,7 +144,10 @@ __global__ void links_fx_kernel(const double2* __restrict__ u, int4* __restrict_
     }
     bool ok = true;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) ok = ok && row[k] <= 0.25 * kFxRowMax && col[k] <= 0.25 * kFxRowMax;
+    for (int k = 0; k < 3; ++k) {
+      ok = ok && row[k] <= 0.25 * kFxRowMax && col[k] <= 0.25 * kFxRowMax;
+      ok = ok && row[k] >= 0.25 * kFxRowMin && col[k] >= 0.25 * kFxRowMin;
+    }
     if (!ok) {  // also for NaN
       atomicOr(bad, 1);
       continue;

@@ -34,6 +34,10 @@ struct Store<FX> {
 
 constexpr int kFxBits = 58;           // vectors: |x| <= 2^58
 constexpr double kFxRowMax = 1.0009;  // largest squared norm of a link row or column
+// ... and the smallest: products of shorter links are small against the unit that they are
+// rounded to (H_W b with m0 = 4, no diagonal term, and 0.3 / 0.01 / 1e-6 of an SU(3) field: off by
+// 2.0e-16, 3.9e-15, 3.9e-11; by 1.6e-16 with the whole one)
+constexpr double kFxRowMin = 0.25;
 constexpr double kFxDiagMax = 4.0;    // largest |4 - m0|
 
 __host__ __device__ __forceinline__ FX fx_split(long long v) {

@@ -29,7 +29,7 @@
 // scalars.  The host only reads a done counter every few iterations, and replays
 // the per-iteration kernels from a CUDA graph.
 //
-// Unitary links and |4 - m0| <= 4: the Lanczos vectors are integers of one scale per vector
+// Links of about unit norm and |4 - m0| <= 4: the Lanczos vectors are integers of one scale per vector
 // (fixed.cuh, the fx_ kernels), in the stored-basis forms and, with a ring of 32 of them, in
 // the vector-space form, whose per-node FP64 vectors then advance a batch of iterations at a
 // time (fx_node_update_kernel).
@@ -2792,7 +2792,7 @@ static int solve_nodes_fx(ov_ctx* ctx, const double2* b_soa, int nsrc, int ns, c
 }
 
 // Whether the stored-basis and vector-space forms of a solver mode run in fixed point
-// (fixed.cuh): links of norm 1 (the bounds there) and |4 - m0| <= 4.  Other links and masses,
+// (fixed.cuh): links of about unit norm (the bounds there) and |4 - m0| <= 4.  Other links and masses,
 // the persistent loop and OV_MODE_FP64_REGEN (its gradients included) keep the FP64 and
 // double-float kernels.
 static bool fixed_point_fits(const ov_ctx* ctx, int mode) {

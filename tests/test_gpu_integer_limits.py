@@ -144,6 +144,32 @@ def test_gradients_of_the_regeneration_form_keep_fp64_vectors(gpu_lib):
     assert np.linalg.norm(d) <= 5e-15 * np.linalg.norm(want)  # as in _against_fp64_vectors
 
 
+@pytest.mark.parametrize("factor", [1e-6, 1e-2, 0.6, 1.0])
+def test_short_links(gpu_lib, factor):
+    """At m0 = 4 H_W is its hopping term alone, as small as the links: results are held to its
+    size.  The stencil: 2^-43 of the largest component times the factor (the bound of the FP64
+    kernels, whose partial sums all scale with it).  A solve with nodes that scale alike: as
+    _against_fp64_vectors."""
+    import torch
+
+    dims, m0 = (4, 4, 4, 6), 4.0
+    U = to_dev(factor * S.su3_links(dims, 0.5, 6011))
+    ctx = gpu_lib.Context(dims, bc_t=-1, m0=m0)
+    ctx.set_gauge(U)
+    ctx.set_contour(factor * Z, factor * C, C0)
+    b = S.gaussian_spinor(dims, 6012, n=2)
+    x = to_dev(b)
+    got, want = torch.empty_like(x), torch.empty_like(x)
+    ctx.apply_HW(x, got, 2, gpu_lib.OV_FP64)
+    assert gpu_lib.apply_HW_noalloc(dims, -1, m0, U, x, want, 2) == gpu_lib.OV_OK
+    torch.cuda.synchronize()
+    assert (got - want).abs().max().item() <= 2.0**-43 * factor * np.abs(b).max()
+    want, _ = sgn_gpu(ctx, b, tol=1e-16, mode="fp64_regen")
+    for mode in ("fp64", "fp64_2pass"):
+        got, _ = sgn_gpu(ctx, b, tol=1e-16, mode=mode)
+        assert np.linalg.norm(got - want) <= 5e-15 * np.linalg.norm(want), mode
+
+
 @pytest.mark.parametrize("dims", [(4, 4, 4, 4), (16, 16, 16, 16), (16, 16, 16, 32)])
 def test_norms_of_constant_vectors(gpu_lib, dims):
     """A constant field on free links stays constant: no component's low limb differs from
