@@ -105,12 +105,16 @@ void ws_release_all(ov_ctx* ctx) {
 }
 
 void ws_release(ov_ctx* ctx, const char* prefix) {
-  cudaDeviceSynchronize();
-  for (auto it = ctx->bufs.lower_bound(prefix); it != ctx->bufs.end() && it->first.rfind(prefix, 0) == 0;) {
-    if (it->second.p) cudaFree(it->second.p);
-    it = ctx->bufs.erase(it);
+  bool held = false;
+  auto first = ctx->bufs.lower_bound(prefix), last = first;
+  for (; last != ctx->bufs.end() && last->first.rfind(prefix, 0) == 0; ++last) held = held || last->second.p;
+  if (held) {  // else neither a wait for the device nor new graphs
+    cudaDeviceSynchronize();
+    for (auto it = first; it != last; ++it)
+      if (it->second.p) cudaFree(it->second.p);
+    graphs_release(ctx);  // captured graphs may point at the buffers
   }
-  graphs_release(ctx);  // captured graphs may point at the buffers
+  ctx->bufs.erase(first, last);
 }
 
 void graphs_release(ov_ctx* ctx) {
