@@ -3687,21 +3687,15 @@ static int lanczos_tridiag_fx(ov_ctx* ctx, int steps, std::vector<double>& alpha
   return read_tridiag<FX>(ctx, w, alpha, beta, s);
 }
 
-int lanczos_tridiag(ov_ctx* ctx, int steps, int squared, std::vector<double>& alpha, std::vector<double>& beta,
-                    cudaStream_t s) {
-  if (!squared && fixed_point_fits(ctx, OV_MODE_FP64)) {
-    const int st = lanczos_tridiag_fx(ctx, steps, alpha, beta, s);
-    if (st != OV_ERR_OUT_OF_MEMORY) return st;
-    ws_release(ctx, "lzx.");
-  }
+// The tridiagonal of H or H^2 with FP64 vectors.  The operator: with fx in integers of a scale per
+// site, else fused into K1 (H) or in FP64 (H^2).
+static int lanczos_tridiag_fp64(ov_ctx* ctx, int steps, int squared, bool fx, std::vector<double>& alpha,
+                                std::vector<double>& beta, cudaStream_t s) {
   SolveWs<double> w;
   int st = setup_ws<double>(ctx, 1, 0, false, false, true, steps, &w, "lz");
   if (st != OV_OK) return st;
   const size_t n12 = (size_t)12 * ctx->g.V;
   double2* b = (double2*)ws_get(ctx, "lz.b", sizeof(double2) * n12, &st);
-  // the operator: in integers of a scale per site where they apply (H^2, and H beside the
-  // persistent loop), else fused into K1 (H) or in FP64 (H^2)
-  const bool fx = ctx->fx_ok;
   double2* tmp = squared || fx ? (double2*)ws_get(ctx, "lz.tmp", sizeof(double2) * n12, &st) : nullptr;
   double2* tmp2 = squared ? (double2*)ws_get(ctx, "lz.tmp2", sizeof(double2) * n12, &st) : nullptr;
   if (st != OV_OK) return st;
@@ -3730,4 +3724,20 @@ int lanczos_tridiag(ov_ctx* ctx, int steps, int squared, std::vector<double>& al
   }
   OV_CHECK_LAUNCH(ctx, "lanczos bound kernels");
   return read_tridiag<double>(ctx, w, alpha, beta, s);
+}
+
+// Integers where they apply: the solver's kernels for H, the stencil beside FP64 vectors for H^2
+// (and for H beside the persistent loop).  Where their vectors do not fit (5 and 7 to the 4 and
+// 6 of the FP64 forms, and what the call before left), FP64.
+int lanczos_tridiag(ov_ctx* ctx, int steps, int squared, std::vector<double>& alpha, std::vector<double>& beta,
+                    cudaStream_t s) {
+  int st = OV_ERR_OUT_OF_MEMORY;
+  if (!squared && fixed_point_fits(ctx, OV_MODE_FP64))
+    st = lanczos_tridiag_fx(ctx, steps, alpha, beta, s);
+  else if (ctx->fx_ok)
+    st = lanczos_tridiag_fp64(ctx, steps, squared, true, alpha, beta, s);
+  if (st != OV_ERR_OUT_OF_MEMORY) return st;
+  ws_release(ctx, "lzx.");
+  ws_release(ctx, "hw.fx");
+  return lanczos_tridiag_fp64(ctx, steps, squared, false, alpha, beta, s);
 }

@@ -50,3 +50,30 @@ def test_vector_space_solves_without_room_for_the_integer_ring(gpu_lib, ballast)
     torch.cuda.synchronize()
     assert running
     assert again["iterations"] == st["iterations"] and again["converged"] == 1
+
+
+_LARGE = (32, 32, 32, 64)  # 402 MB per FP64 vector: what the allocator keeps for itself is small beside it
+_VEC = 192 * 32**3 * 64
+
+
+@pytest.mark.parametrize("vectors", [6, 8, 10, 12])
+def test_spectral_bounds_without_room_for_integer_vectors(gpu_lib, ballast, vectors):
+    """The FP64 forms of H^2 take a ring of three vectors, the start vector and two products; the
+    integer ones more.  Over 8 steps no Ritz value has converged, and rounding differs by less
+    than 1e-11 ||H|| (||H||^2 in the squared one, whose root the gap is)."""
+    import torch
+
+    U = torch.eye(3, dtype=torch.complex128, device="cuda").expand((4,) + _LARGE[::-1] + (3, 3)).contiguous()
+    ctx = gpu_lib.Context(_LARGE, bc_t=-1, m0=1.6)
+    ctx.set_gauge(U)
+    want = ctx.place_contour(8, steps=8)
+    ctx.close()
+    ctx = gpu_lib.Context(_LARGE, bc_t=-1, m0=1.6)
+    ctx.set_gauge(U)
+    ballast(vectors * _VEC + (300 << 20))
+    got = ctx.place_contour(8, steps=8)
+    assert got["steps"] == want["steps"] == 8
+    for key in ("lambda_min", "lambda_max", "abs_max_bound"):
+        assert abs(got[key] - want[key]) <= 1e-11 * 8
+    assert abs(got["gap"] ** 2 - want["gap"] ** 2) <= 1e-11 * 64
+    ctx.close()
