@@ -171,7 +171,8 @@ const char* ov_last_error(const ov_ctx* ctx);
  * `stream` and not retained.  The library keeps FP64, FP32 and double-float
  * structure-of-arrays copies and, where every row and every column of every link has a
  * norm between 1/2 and 1 (up to 1.00045: SU(3) links, and shortened ones), a 58-bit
- * integer copy: "links of unit norm" below.  Other links take FP64, double-float and
+ * integer copy (576 bytes per site, given up where it or a later call would not fit in
+ * memory with it): "links of unit norm" below.  Other links take FP64, double-float and
  * FP32 arithmetic only.  Any cached contour placement is invalidated (explicit
  * contours are kept).  Errors: INVALID_ARG (null U), OUT_OF_MEMORY, CUDA. */
 int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream);

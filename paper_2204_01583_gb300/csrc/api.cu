@@ -117,6 +117,21 @@ void ws_release(ov_ctx* ctx, const char* prefix) {
   ctx->bufs.erase(first, last);
 }
 
+int or_without_integers(ov_ctx* ctx, cudaStream_t s, const std::function<int()>& call) {
+  int st = call();
+  if (st != OV_ERR_OUT_OF_MEMORY || !ctx || !ctx->fx_ok) return st;
+  DeviceGuard dg(ctx->device);
+  ctx->fx_ok = false;
+  for (const char* prefix : {"fx", "lzx.", "hw.fx", "gauge.fx"}) ws_release(ctx, prefix);
+  st = call();
+  if (st != OV_ERR_OUT_OF_MEMORY) return st;
+  const std::string err = ctx->err;
+  const bool fx = launch_links_fx(ctx, s);
+  ctx->fx_ok = cudaStreamSynchronize(s) == cudaSuccess && fx && ctx->host_flag[1] == 0;
+  ctx->err = err;
+  return st;
+}
+
 void graphs_release(ov_ctx* ctx) {
   for (auto& kv : ctx->graphs) cudaGraphExecDestroy(kv.second);
   ctx->graphs.clear();
@@ -475,8 +490,7 @@ static int tune_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaS
   return st;
 }
 
-int ov_apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precision, void* stream) {
-  NvtxRange nvtx_("ov_apply_HW");
+static int apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precision, void* stream) {
   if (!ctx) return OV_ERR_INVALID_ARG;
   if (!ctx->have_gauge) return ctx_fail(ctx, OV_ERR_NO_GAUGE, "ov_set_gauge has not been called");
   if (nrhs < 0 || (nrhs > 0 && (!in || !out)) || in == out)
@@ -513,6 +527,12 @@ int ov_apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precision,
     return apply_hw32(ctx, k, (const float2*)in, (float2*)out, nrhs, s);
   }
   return OV_OK;
+}
+
+int ov_apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precision, void* stream) {
+  NvtxRange nvtx_("ov_apply_HW");
+  return or_without_integers(ctx, (cudaStream_t)stream,
+                             [&] { return apply_HW(ctx, in, out, nrhs, precision, stream); });
 }
 
 int ov_set_contour(ov_ctx* ctx, int n, const double* z, const double* c, double c0_re, double c0_im) {
@@ -606,7 +626,8 @@ int ov_place_contour(ov_ctx* ctx, int n_q, int steps, ov_spectrum* out, void* st
   cudaStream_t s = (cudaStream_t)stream;
   double lo, hi, amax, gap, gap_lo;
   int nsteps = 0;
-  int st = spectral_bounds(ctx, steps, s, &lo, &hi, &amax, &gap, &gap_lo, &nsteps);
+  int st = or_without_integers(
+      ctx, s, [&] { return spectral_bounds(ctx, steps, s, &lo, &hi, &amax, &gap, &gap_lo, &nsteps); });
   if (st != OV_OK) return st;
   // single ellipse from 0 to 1.05 * amax; alpha minimises the predicted method error
   const double R = 1.05 * amax;
@@ -687,7 +708,8 @@ int ov_place_zolotarev(ov_ctx* ctx, int n_poles, int steps, ov_spectrum* out, vo
   cudaStream_t s = (cudaStream_t)stream;
   double lo, hi, amax, gap, gap_lo, delta = 0.0;
   int nsteps = 0;
-  int st = spectral_bounds(ctx, steps, s, &lo, &hi, &amax, &gap, &gap_lo, &nsteps);
+  int st = or_without_integers(
+      ctx, s, [&] { return spectral_bounds(ctx, steps, s, &lo, &hi, &amax, &gap, &gap_lo, &nsteps); });
   if (st != OV_OK) return st;
   st = ov_set_contour_zolotarev(ctx, n_poles, gap_lo, amax, &delta);
   if (st != OV_OK) return st;
@@ -746,13 +768,17 @@ static int sign_or_overlap(ov_ctx* ctx, bool overlap, double m_q, const void* b,
 int ov_sgn_HW_apply(ov_ctx* ctx, const void* b, void* out, int nrhs, const ov_solve_opts* opts, ov_stats* stats,
                     void* stream) {
   NvtxRange nvtx_("ov_sgn_HW_apply");
-  return sign_or_overlap(ctx, false, 0.0, b, out, nrhs, opts, stats, stream);
+  return or_without_integers(ctx, (cudaStream_t)stream, [&] {
+    return sign_or_overlap(ctx, false, 0.0, b, out, nrhs, opts, stats, stream);
+  });
 }
 
 int ov_overlap_apply(ov_ctx* ctx, double m_q, const void* b, void* out, int nrhs, const ov_solve_opts* opts,
                      ov_stats* stats, void* stream) {
   NvtxRange nvtx_("ov_overlap_apply");
-  return sign_or_overlap(ctx, true, m_q, b, out, nrhs, opts, stats, stream);
+  return or_without_integers(ctx, (cudaStream_t)stream, [&] {
+    return sign_or_overlap(ctx, true, m_q, b, out, nrhs, opts, stats, stream);
+  });
 }
 
 }  // extern "C"
@@ -910,15 +936,19 @@ extern "C" {
 
 int ov_sgn_vjp(ov_ctx* ctx, const void* eta, const void* b, void* grad_b, double* grad_links,
                const ov_solve_opts* opts, ov_stats* stats, void* stream) {
-  return vjp_core(ctx, 0.0, 1.0, 1.0, false, eta, b, grad_b, grad_links, opts, stats, stream);
+  return or_without_integers(ctx, (cudaStream_t)stream, [&] {
+    return vjp_core(ctx, 0.0, 1.0, 1.0, false, eta, b, grad_b, grad_links, opts, stats, stream);
+  });
 }
 
 int ov_overlap_vjp(ov_ctx* ctx, double m_q, const void* eta, const void* b, void* grad_b, double* grad_links,
                    const ov_solve_opts* opts, ov_stats* stats, void* stream) {
   if (!std::isfinite(m_q)) return ctx_fail(ctx, OV_ERR_INVALID_ARG, "m_q is not finite");
   // L = Re<eta, (1+m)/2 b> + (1-m)/2 Re<gamma5 eta, S_N b>
-  return vjp_core(ctx, 0.5 * (1.0 + m_q), 0.5 * (1.0 - m_q), 0.5 * (1.0 - m_q), true, eta, b, grad_b, grad_links,
-                  opts, stats, stream);
+  return or_without_integers(ctx, (cudaStream_t)stream, [&] {
+    return vjp_core(ctx, 0.5 * (1.0 + m_q), 0.5 * (1.0 - m_q), 0.5 * (1.0 - m_q), true, eta, b, grad_b, grad_links,
+                    opts, stats, stream);
+  });
 }
 
 int ov_set_hw32_variant(ov_ctx* ctx, int k) {

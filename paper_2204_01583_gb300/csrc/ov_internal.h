@@ -153,6 +153,10 @@ void* ws_get(ov_ctx* ctx, const char* name, size_t bytes, int* status);
 void ws_release_all(ov_ctx* ctx);
 void ws_release(ov_ctx* ctx, const char* prefix);  // the buffers whose names start with prefix
 void graphs_release(ov_ctx* ctx);
+// call(), and if it runs out of memory beside the integer links, once more without them: they
+// and the integer forms' buffers are released until the next ov_set_gauge.  (Kept if the call does
+// not fit either way.)  call has to be repeatable: no outputs before its last allocation.
+int or_without_integers(ov_ctx* ctx, cudaStream_t s, const std::function<int()>& call);
 
 // Kernel timing: bracket a launch with events when ctx->timing is set.
 void kt_begin(ov_ctx* ctx, int cls, cudaStream_t s, cudaEvent_t* a);

@@ -147,9 +147,8 @@ int dot(CgCtx& c, const double2* u, const double2* v, std::vector<double>& out) 
 
 }  // namespace
 
-extern "C" int ov_overlap_solve(ov_ctx* ctx, double m_q, const void* b, void* x, int nrhs, const ov_solve_opts* inner,
-                                double tol, int max_iter, ov_stats* stats, void* stream) {
-  NvtxRange nvtx_("ov_overlap_solve");
+static int overlap_solve(ov_ctx* ctx, double m_q, const void* b, void* x, int nrhs, const ov_solve_opts* inner,
+                         double tol, int max_iter, ov_stats* stats, void* stream) {
   const double t0 = now_ms();
   if (!ctx) return OV_ERR_INVALID_ARG;
   if (!ctx->have_gauge) return ctx_fail(ctx, OV_ERR_NO_GAUGE, "ov_set_gauge has not been called");
@@ -270,4 +269,12 @@ extern "C" int ov_overlap_solve(ov_ctx* ctx, double m_q, const void* b, void* x,
   kt_collect(ctx);
   fill_stats(stats, so, now_ms() - t0);
   return so.converged ? OV_OK : ctx_fail(ctx, OV_ERR_NOT_CONVERGED, "overlap CG did not reach tol in max_iter");
+}
+
+extern "C" int ov_overlap_solve(ov_ctx* ctx, double m_q, const void* b, void* x, int nrhs, const ov_solve_opts* inner,
+                                double tol, int max_iter, ov_stats* stats, void* stream) {
+  NvtxRange nvtx_("ov_overlap_solve");
+  return or_without_integers(ctx, (cudaStream_t)stream, [&] {
+    return overlap_solve(ctx, m_q, b, x, nrhs, inner, tol, max_iter, stats, stream);
+  });
 }

@@ -77,3 +77,42 @@ def test_spectral_bounds_without_room_for_integer_vectors(gpu_lib, ballast, vect
         assert abs(got[key] - want[key]) <= 1e-11 * 8
     assert abs(got["gap"] ** 2 - want["gap"] ** 2) <= 1e-11 * 64
     ctx.close()
+
+
+@pytest.mark.parametrize("call,vectors", [("hw", 0), ("bounds", 3), ("sgn", 4)])
+def test_integer_links_give_way(gpu_lib, ballast, call, vectors):
+    """The integer copy of the links takes three vectors' memory.  A call that fits without it and
+    not beside it runs in FP64: the stencil within 2^-43 of the largest component of the integer
+    one, a solve within its tolerance (two solves: 8 tol ||b||, sum_j |c_j / Im z_j| < 4)."""
+    import torch
+
+    U = torch.eye(3, dtype=torch.complex128, device="cuda").expand((4,) + _LARGE[::-1] + (3, 3)).contiguous()
+    gen = torch.Generator(device="cuda").manual_seed(7011)
+    b = torch.randn(_LARGE[::-1] + (4, 3), dtype=torch.complex128, device="cuda", generator=gen)
+    z = np.array([0.3 + 0.9j, 0.3 - 0.9j, -1.5 + 1.1j, -1.5 - 1.1j])
+    c = np.array([0.4 - 0.3j, 0.4 + 0.3j, -0.7 + 0.2j, -0.7 - 0.2j])
+    out = []
+    for limit in (False, True):
+        ctx = gpu_lib.Context(_LARGE, bc_t=-1, m0=1.6)
+        ctx.set_gauge(U)
+        ctx.set_contour(z, c, 0.2)
+        x = torch.empty_like(b)
+        if limit:
+            ballast(vectors * _VEC + (300 << 20))
+        if call == "hw":
+            ctx.apply_HW(b, x, 1, gpu_lib.OV_FP64)
+        elif call == "sgn":
+            ctx.sgn(b, x, 1, ctx.opts(mode="fp64_2pass", tol=1e-12))
+        else:
+            r = ctx.place_contour(8, steps=8)
+            x = torch.tensor([r["lambda_min"], r["lambda_max"], r["gap"] ** 2])
+        torch.cuda.synchronize()
+        out.append(x)
+        ctx.close()
+    d = (out[1] - out[0]).abs()
+    if call == "hw":
+        assert d.max().item() <= 2.0**-43 * b.abs().max().item()
+    elif call == "sgn":
+        assert torch.linalg.norm(d).item() <= 8e-12 * torch.linalg.norm(b).item()
+    else:
+        assert d.max().item() <= 1e-11 * 64
