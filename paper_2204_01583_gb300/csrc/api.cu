@@ -464,29 +464,42 @@ static int apply_hw32(ov_ctx* ctx, int k, const float2* in, float2* out, int nrh
   return f.paired ? launch_hw_pair12(ctx, a, out, nrhs, f.form, s) : launch_hw32_s4(ctx, a, out, nrhs, s);
 }
 
-// The fastest variant for nrhs right-hand sides on this data (each timed three times after a
-// warm-up that builds its links).
+// The fastest variant for nrhs right-hand sides on this data: each is run twice, the first time
+// to build its links and buffers, all in a row and with one wait at the end.  (The first call of a
+// context and count, in us, with this / with four runs and a wait per variant / when the trials
+// left the layout passes out: 4^4, 1 source 234 / 415 / 290; 16^3 x 32, 12 sources 3138 / 5956 / 3717.)
 static int tune_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int* best) {
-  cudaEvent_t e0, e1;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
-  int st = OV_OK;
+  constexpr int kMax = 16;
+  const int n = std::min(hw32_variant_count() + kNFloat4Variants, kMax);
+  cudaEvent_t ev[2 * kMax];
+  int nev = 0, st = OV_OK;
+  for (; nev < 2 * n && st == OV_OK; ++nev) {
+    const cudaError_t e = cudaEventCreate(ev + nev);
+    if (e != cudaSuccess) {
+      st = ctx_cuda(ctx, e, "cudaEventCreate");
+      break;
+    }
+  }
+  for (int k = 0; k < n && st == OV_OK; ++k) {
+    if ((st = apply_hw32(ctx, k, in, out, nrhs, s))) break;
+    cudaEventRecord(ev[2 * k], s);
+    st = apply_hw32(ctx, k, in, out, nrhs, s);
+    cudaEventRecord(ev[2 * k + 1], s);
+  }
+  if (st == OV_OK) {
+    const cudaError_t e = cudaEventSynchronize(ev[2 * n - 1]);
+    if (e != cudaSuccess) st = ctx_cuda(ctx, e, "FP32 stencil variants");
+  }
   float best_ms = 1e30f;
   *best = 0;
-  for (int k = 0; k < hw32_variant_count() + kNFloat4Variants && st == OV_OK; ++k) {
-    if ((st = apply_hw32(ctx, k, in, out, nrhs, s))) break;
-    cudaEventRecord(e0, s);
-    for (int rep = 0; rep < 3 && st == OV_OK; ++rep) st = apply_hw32(ctx, k, in, out, nrhs, s);
-    cudaEventRecord(e1, s);
-    cudaEventSynchronize(e1);
+  for (int k = 0; k < n && st == OV_OK; ++k) {
     float ms = 0.f;
-    if (st == OV_OK && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best_ms) {
+    if (cudaEventElapsedTime(&ms, ev[2 * k], ev[2 * k + 1]) == cudaSuccess && ms < best_ms) {
       best_ms = ms;
       *best = k;
     }
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
+  while (nev > 0) cudaEventDestroy(ev[--nev]);
   return st;
 }
 

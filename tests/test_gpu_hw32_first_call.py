@@ -1,0 +1,35 @@
+"""The first FP32 ov_apply_HW of a context and source count, which tries every variant (GPU)."""
+import time
+
+import numpy as np
+import pytest
+
+from tests.gpu_common import make_ctx
+
+pytestmark = pytest.mark.gpu
+
+
+def test_trials_cost_less_than_thirty_calls(gpu_lib):
+    """Two runs of each of the six variants, the slowest of which takes twice the time of the
+    fastest at this size: 19 calls of the chosen one, and allocations."""
+    import torch
+
+    dims, n = (16, 16, 16, 32), 12
+    x = torch.randn((n,) + dims[::-1] + (4, 3), dtype=torch.complex64, device="cuda")
+    y = torch.empty_like(x)
+
+    def seconds(ctx, calls):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        for _ in range(calls):
+            ctx.apply_HW(x, y, n, gpu_lib.OV_FP32)
+        torch.cuda.synchronize()
+        return (time.perf_counter() - t) / calls
+
+    first, later = [], []
+    for k in range(6):
+        ctx, _ = make_ctx(gpu_lib, dims, 0.0, 0)
+        first.append(seconds(ctx, 1))
+        later.append(seconds(ctx, 20))
+        ctx.close()
+    assert np.median(first[1:]) <= 30 * np.median(later)  # the very first one loads the kernels
