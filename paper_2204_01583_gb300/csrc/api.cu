@@ -473,6 +473,8 @@ static int tune_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaS
   const int n = std::min(hw32_variant_count() + kNFloat4Variants, kMax);
   cudaEvent_t ev[2 * kMax];
   int nev = 0, st = OV_OK;
+  const bool timing = ctx->timing;
+  ctx->timing = false;  // trials are not calls: they stay out of ov_kernel_times
   for (; nev < 2 * n && st == OV_OK; ++nev) {
     const cudaError_t e = cudaEventCreate(ev + nev);
     if (e != cudaSuccess) {
@@ -500,6 +502,7 @@ static int tune_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaS
     }
   }
   while (nev > 0) cudaEventDestroy(ev[--nev]);
+  ctx->timing = timing;
   return st;
 }
 

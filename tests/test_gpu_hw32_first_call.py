@@ -33,3 +33,16 @@ def test_trials_cost_less_than_thirty_calls(gpu_lib):
         later.append(seconds(ctx, 20))
         ctx.close()
     assert np.median(first[1:]) <= 30 * np.median(later)  # the very first one loads the kernels
+
+
+def test_trials_stay_out_of_the_kernel_times(gpu_lib):
+    import torch
+
+    dims, n = (6, 4, 4, 5), 3
+    ctx, _ = make_ctx(gpu_lib, dims, 0.3, 8001)
+    x = torch.randn((n,) + dims[::-1] + (4, 3), dtype=torch.complex64, device="cuda")
+    ctx.set_kernel_timing(True)
+    ctx.apply_HW(x, torch.empty_like(x), n, gpu_lib.OV_FP32)
+    torch.cuda.synchronize()
+    times = ctx.kernel_times()
+    assert times["hw_kernel"][0] == 1 and times["layout_kernels"][0] in (1, 2)  # unpacking: some variants
