@@ -28,7 +28,6 @@ __device__ __forceinline__ P2 ldp(const float4* p) {
   const float4 v = __ldg(p);
   return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
 }
-__device__ __forceinline__ void stp(float4* p, P2 v) { *p = make_float4(v.re.x, v.re.y, v.im.x, v.im.y); }
 
 // a + S b for a compile-time sign S = +-1 (one paired instruction)
 template <int S>
