@@ -400,6 +400,10 @@ int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream) {
         cudaMalloc(&ctx->U32, sizeof(float2) * n) != cudaSuccess ||
         cudaMalloc(&ctx->U64h, sizeof(double2) * n) != cudaSuccess) {
       cudaGetLastError();
+      cudaFree(ctx->U64);  // the next call allocates all three again
+      cudaFree(ctx->U32);
+      ctx->U64 = nullptr;
+      ctx->U32 = nullptr;
       return ctx_fail(ctx, OV_ERR_OUT_OF_MEMORY, "gauge field allocation failed");
     }
   }

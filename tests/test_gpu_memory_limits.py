@@ -20,6 +20,7 @@ def ballast():
         torch.cuda.empty_cache()
         held.append(torch.empty(torch.cuda.mem_get_info()[0] - int(leave), dtype=torch.uint8, device="cuda"))
 
+    take.release = held.clear
     yield take
     held.clear()
     torch.cuda.empty_cache()
@@ -116,3 +117,26 @@ def test_integer_links_give_way(gpu_lib, ballast, call, vectors):
         assert torch.linalg.norm(d).item() <= 8e-12 * torch.linalg.norm(b).item()
     else:
         assert d.max().item() <= 1e-11 * 64
+
+
+def test_set_gauge_after_one_that_did_not_fit(gpu_lib, ballast):
+    """The first of three link fields fits and the second does not: an error, and a later call
+    with room for all of them starts anew."""
+    import torch
+
+    U = torch.eye(3, dtype=torch.complex128, device="cuda").expand((4,) + _LARGE[::-1] + (3, 3)).contiguous()
+    b = torch.ones(_LARGE[::-1] + (4, 3), dtype=torch.complex128, device="cuda")
+    x = torch.empty_like(b)
+    ctx = gpu_lib.Context(_LARGE, bc_t=1, m0=1.6)
+    ballast(U.numel() * 16 + (300 << 20))
+    with pytest.raises(gpu_lib.OvError) as e:
+        ctx.set_gauge(U)
+    assert e.value.code == gpu_lib.OV_ERR_OUT_OF_MEMORY
+    ballast.release()
+    torch.cuda.empty_cache()
+    ctx.set_gauge(U)
+    ctx.apply_HW(b, x, 1, gpu_lib.OV_FP64)
+    torch.cuda.synchronize()
+    ctx.close()
+    want = b * torch.tensor([-1.6, -1.6, 1.6, 1.6], dtype=torch.float64, device="cuda")[:, None]  # gamma5 (-m0) on a constant field
+    assert (x - want).abs().max().item() <= 2.0**-43
