@@ -7,10 +7,13 @@
 //
 //     x = hi 2^30 + lo,   lo in [-2^29, 2^29),   |x| <= 2^58,
 //
-// the largest component just below 2^58 (a power-of-two scale chosen anew for every vector), links as integers of unit 2^-58 (carrying the hop factor -1/2 and the time
-// boundary sign).  Products drop lo * lo only (2^-60 of the full scale), all sums are
-// exact, and one rounding to an integer ends each hop: errors of about 2^-58 of the
-// vector's largest component, where FP64 rounds every partial sum at 2^-54 of its size.
+// the largest component just below 2^58 (a power-of-two scale chosen anew for every vector),
+// links as integers of unit 2^-58 (carrying the hop factor -1/2 and the time boundary sign).
+// Products drop lo * lo only (2^-60 of the full scale), all sums are exact, and one rounding to
+// nearest ends each hop: errors of a few 2^-58 of the vector's largest component, zeros exact.
+// FP64 rounds every partial sum at 2^-53 of its own size: more where components are of one
+// size, less far below the largest.  In norm, S_N b of point and Gaussian sources (8^4 to
+// 16^3 x 32) is within 0.7e-15 to 1.1e-15 of FP64 vectors, as two FP64 forms are of one another.
 //
 // Bounds, for links whose rows and columns have norm at most 1 (kFxRowMax) and
 // |4 - m0| <= 4: the real and imaginary parts of a projected component and their sum fit 31
