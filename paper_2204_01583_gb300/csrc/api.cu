@@ -418,7 +418,7 @@ int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream) {
   }
   st = launch_gauge_ingest(ctx, src, s);
   if (st != OV_OK) return st;
-  const bool fx = launch_links_fx(ctx, s);
+  const bool fx = launch_links_fx(ctx, s), su3 = launch_links_su3(ctx, s);
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return ctx_cuda(ctx, e, "ov_set_gauge");
   kt_collect(ctx);
@@ -428,6 +428,7 @@ int ov_set_gauge(ov_ctx* ctx, const double* U, int on_device, void* stream) {
   ctx->have_s4 = false;
   ctx->have_df = false;
   ctx->fx_ok = fx && ctx->host_flag[1] == 0;
+  ctx->su3 = su3 && ctx->host_flag[2] == 0;
   return OV_OK;
 }
 
@@ -468,6 +469,14 @@ static int apply_hw32(ov_ctx* ctx, int k, const float2* in, float2* out, int nrh
   return f.paired ? launch_hw_pair12(ctx, a, out, nrhs, f.form, s) : launch_hw32_s4(ctx, a, out, nrhs, s);
 }
 
+// Whether variant k gives H_W on the links at hand.
+static bool hw32_admits(const ov_ctx* ctx, int k) {
+  if (ctx->su3) return true;
+  int rt, comp = 1, nt;
+  if (k < hw32_variant_count()) hw32_variant_info(k, &rt, &comp, &nt);  // every float4 form: 12-real links
+  return comp == 0;
+}
+
 // The fastest variant for nrhs right-hand sides on this data: each is run twice, the first time
 // to build its links and buffers, all in a row and with one wait at the end.  (The first call of a
 // context and count, in us, with this / with four runs and a wait per variant / when the trials
@@ -486,19 +495,23 @@ static int tune_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaS
       break;
     }
   }
+  int last = 0;
   for (int k = 0; k < n && st == OV_OK; ++k) {
+    if (!hw32_admits(ctx, k)) continue;
+    last = k;
     if ((st = apply_hw32(ctx, k, in, out, nrhs, s))) break;
     cudaEventRecord(ev[2 * k], s);
     st = apply_hw32(ctx, k, in, out, nrhs, s);
     cudaEventRecord(ev[2 * k + 1], s);
   }
   if (st == OV_OK) {
-    const cudaError_t e = cudaEventSynchronize(ev[2 * n - 1]);
+    const cudaError_t e = cudaEventSynchronize(ev[2 * last + 1]);
     if (e != cudaSuccess) st = ctx_cuda(ctx, e, "FP32 stencil variants");
   }
   float best_ms = 1e30f;
-  *best = 0;
+  *best = last;
   for (int k = 0; k < n && st == OV_OK; ++k) {
+    if (!hw32_admits(ctx, k)) continue;
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, ev[2 * k], ev[2 * k + 1]) == cudaSuccess && ms < best_ms) {
       best_ms = ms;
@@ -536,12 +549,13 @@ static int apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precis
   } else {
     int k = ctx->hw32_force;
     if (k < 0) {
-      auto it = ctx->hw32_choice.find(nrhs);
-      if (it != ctx->hw32_choice.end()) {
+      auto& choice = ctx->hw32_choice[ctx->su3];
+      auto it = choice.find(nrhs);
+      if (it != choice.end()) {
         k = it->second;
       } else {
         if ((st = tune_hw32(ctx, (const float2*)in, (float2*)out, nrhs, s, &k))) return st;
-        ctx->hw32_choice[nrhs] = k;
+        choice[nrhs] = k;
       }
     }
     return apply_hw32(ctx, k, (const float2*)in, (float2*)out, nrhs, s);

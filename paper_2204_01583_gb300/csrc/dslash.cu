@@ -160,6 +160,27 @@ __global__ void links_fx_kernel(const double2* __restrict__ u, int4* __restrict_
   }
 }
 
+// *bad is set when row 2 of a link is not conj(row 0 x row 1) to 2^-21 (a few times what links
+// rounded to FP32 are off by): the FP32 forms with 12-real links rebuild it so
+__global__ void links_su3_kernel(const double2* __restrict__ u, int V, int* __restrict__ bad) {
+  const size_t n = (size_t)4 * V;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
+    const double2* l = u + t / V * 9 * V + t % V;
+    double2 v[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) v[e] = l[(size_t)e * V];
+    bool ok = true;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const double2 a = v[(e + 1) % 3], b = v[3 + (e + 2) % 3], c = v[(e + 2) % 3], d = v[3 + (e + 1) % 3];
+      const double re = a.x * b.x - a.y * b.y - (c.x * d.x - c.y * d.y);
+      const double im = a.x * b.y + a.y * b.x - (c.x * d.y + c.y * d.x);
+      ok = ok && fabs(v[6 + e].x - re) <= 0x1p-21 && fabs(v[6 + e].y + im) <= 0x1p-21;  // false for NaN
+    }
+    if (!ok) atomicOr(bad, 1);
+  }
+}
+
 int grid_for(size_t n, int nt) {
   size_t b = (n + nt - 1) / nt;
   if (b > 152 * 16) b = 152 * 16;
@@ -260,6 +281,19 @@ int ensure_links_df(ov_ctx* ctx, cudaStream_t s) {
     ctx->have_df = true;
   }
   return OV_OK;
+}
+
+bool launch_links_su3(ov_ctx* ctx, cudaStream_t s) {
+  int st = OV_OK;
+  int* bad = (int*)ws_get(ctx, "gauge.su3bad", sizeof(int), &st);
+  if (st != OV_OK) return false;
+  cudaMemsetAsync(bad, 0, sizeof(int), s);
+  cudaEvent_t ev;
+  kt_begin(ctx, KC_LAYOUT, s, &ev);
+  links_su3_kernel<<<grid_for((size_t)4 * ctx->g.V, 256), 256, 0, s>>>(ctx->U64, ctx->g.V, bad);
+  kt_end(ctx, KC_LAYOUT, s, ev);
+  return cudaGetLastError() == cudaSuccess &&
+         cudaMemcpyAsync(ctx->host_flag + 2, bad, sizeof(int), cudaMemcpyDeviceToHost, s) == cudaSuccess;
 }
 
 bool launch_links_fx(ov_ctx* ctx, cudaStream_t s) {

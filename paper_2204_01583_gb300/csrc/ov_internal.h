@@ -115,7 +115,8 @@ struct ov_ctx {
   bool have_df = false;
   int4* Ufx = nullptr;                 // fixed-point links (workspace "gauge.fx") when fx_ok
   bool fx_ok = false;                  // links and mass fit the fixed-point bounds
-  std::map<int, int> hw32_choice;      // nrhs -> autotuned FP32 stencil variant
+  bool su3 = false;                    // row 2 of every link is conj(row 0 x row 1): 12-real forms
+  std::map<int, int> hw32_choice[2];   // nrhs -> autotuned FP32 stencil variant, by su3
   int hw32_force = -1;                 // ov_set_hw32_variant
   bool no_coop = true;                 // ov_set_persistent(ctx, 1) enables the persistent loop
   int groups = 0;                      // ov_set_concurrency: source groups per graph (0 = auto)
@@ -189,6 +190,9 @@ int ensure_links_df(ov_ctx* ctx, cudaStream_t s);
 // Fixed-point links (dslash.cu): enqueues them and the copy of the check's verdict to
 // ctx->host_flag[1] (0: every link fits); false when they do not apply or do not fit in memory.
 bool launch_links_fx(ov_ctx* ctx, cudaStream_t s);
+// Enqueues the check behind ctx->su3 and the copy of its verdict to ctx->host_flag[2] (0: SU(3));
+// false when it could not.
+bool launch_links_su3(ov_ctx* ctx, cudaStream_t s);
 // out = H_W in, FP64 fields (canonical or planes) through integers (hw64.cu); needs fx_ok
 int launch_hw64_fx(ov_ctx* ctx, const double2* in, double2* out, int nrhs, bool canonical, cudaStream_t s);
 // spin-paired float4 FP32 layout (dslash32.cu) and paired FP32 layout (pair32.cu): packing from

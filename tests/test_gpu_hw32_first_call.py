@@ -4,7 +4,8 @@ import time
 import numpy as np
 import pytest
 
-from tests.gpu_common import make_ctx
+import synthetic as S
+from tests.gpu_common import make_ctx, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -46,3 +47,22 @@ def test_trials_stay_out_of_the_kernel_times(gpu_lib):
     torch.cuda.synchronize()
     times = ctx.kernel_times()
     assert times["hw_kernel"][0] == 1 and times["layout_kernels"][0] in (1, 2)  # unpacking: some variants
+
+
+@pytest.mark.parametrize("dims,n", [((4, 4, 4, 4), 1), ((8, 8, 8, 8), 2), ((16, 16, 16, 16), 12)])
+def test_links_that_are_not_su3(gpu_lib, dims, n):
+    """The forms that rebuild row 2 of a link from rows 0 and 1 are left out on links of another
+    norm, and come back with SU(3) ones.  FP32 against FP64: 2e-6, the oracle tests' bound."""
+    import torch
+
+    U = to_dev(S.su3_links(dims, 0.5, 8011))
+    ctx = gpu_lib.Context(dims, bc_t=-1, m0=1.6)
+    x = torch.randn((n,) + dims[::-1] + (4, 3), dtype=torch.complex64, device="cuda")
+    y, x64 = torch.empty_like(x), x.to(torch.complex128)
+    want = torch.empty_like(x64)
+    for factor in (1.0, 0.7, 1.2, 1.0):
+        ctx.set_gauge(factor * U)
+        ctx.apply_HW(x, y, n, gpu_lib.OV_FP32)
+        ctx.apply_HW(x64, want, n, gpu_lib.OV_FP64)
+        torch.cuda.synchronize()
+        assert (y.to(torch.complex128) - want).abs().max().item() <= 2e-6 * want.abs().max().item(), factor
