@@ -288,7 +288,8 @@ int ov_overlap_solve(ov_ctx* ctx, double m_q, const void* b, void* x, int nrhs, 
  * stencil of Eq. 1; the paper has no counterpart).  Variants differ in layout, right-hand
  * sides per thread (link loads reused across them) and 12-real link compression (row 2
  * rebuilt as conj(row0 x row1)).  k = -1 (default): autotune -- each variant is timed
- * once on the live data per right-hand-side count and the fastest is kept; on links that
+ * once on the live data per right-hand-side count and the fastest is kept (up to 32768
+ * sites times right-hand sides the spin-paired kernel without trials); on links that
  * are not SU(3) (row 2 further than 2^-21 from conj(row0 x row1)) those with plain links
  * only.  A variant set here runs on any links.
  * ov_hw32_variants returns the number of variants and, for 0 <= k < count, describes

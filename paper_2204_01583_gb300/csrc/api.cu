@@ -477,10 +477,17 @@ static bool hw32_admits(const ov_ctx* ctx, int k) {
   return comp == 0;
 }
 
+// Sites times right-hand sides up to which nothing is tried: a call is the latency of its
+// launches, two with the float4 layouts and three with planes, and one timed run of each does not
+// tell the variants apart.  Calls of 4^4 with 1 to 12 sources to 8^4 with 4 and 6 x 10 x 7 x 9 with
+// 5: spin-paired 9.7 to 10.9 us, paired 9.7 to 12.5, planes 12 to 16.7.  Above: 6 x 10 x 7 x 9 with 12
+// 13.6 / 13.7, 8^4 with 12 14.4 / 12.6.
+constexpr size_t kHw32Untried = 32768;
+
 // The fastest variant for nrhs right-hand sides on this data: each is run twice, the first time
 // to build its links and buffers, all in a row and with one wait at the end.  (The first call of a
 // context and count, in us, with this / with four runs and a wait per variant / when the trials
-// left the layout passes out: 4^4, 1 source 234 / 415 / 290; 16^3 x 32, 12 sources 3138 / 5956 / 3717.)
+// left the layout passes out: 8^4, 12 sources 461 / 778 / 627; 16^3 x 32, 12 sources 3138 / 5956 / 3717.)
 static int tune_hw32(ov_ctx* ctx, const float2* in, float2* out, int nrhs, cudaStream_t s, int* best) {
   constexpr int kMax = 16;
   const int n = std::min(hw32_variant_count() + kNFloat4Variants, kMax);
@@ -553,6 +560,8 @@ static int apply_HW(ov_ctx* ctx, const void* in, void* out, int nrhs, int precis
       auto it = choice.find(nrhs);
       if (it != choice.end()) {
         k = it->second;
+      } else if (ctx->su3 && (size_t)ctx->g.V * nrhs <= kHw32Untried) {
+        k = hw32_variant_count();  // the spin-paired kernel
       } else {
         if ((st = tune_hw32(ctx, (const float2*)in, (float2*)out, nrhs, s, &k))) return st;
         choice[nrhs] = k;

@@ -39,7 +39,7 @@ def test_trials_cost_less_than_thirty_calls(gpu_lib):
 def test_trials_stay_out_of_the_kernel_times(gpu_lib):
     import torch
 
-    dims, n = (6, 4, 4, 5), 3
+    dims, n = (8, 8, 8, 9), 8  # beyond the size up to which nothing is tried
     ctx, _ = make_ctx(gpu_lib, dims, 0.3, 8001)
     x = torch.randn((n,) + dims[::-1] + (4, 3), dtype=torch.complex64, device="cuda")
     ctx.set_kernel_timing(True)
@@ -66,3 +66,23 @@ def test_links_that_are_not_su3(gpu_lib, dims, n):
         ctx.apply_HW(x64, want, n, gpu_lib.OV_FP64)
         torch.cuda.synchronize()
         assert (y.to(torch.complex128) - want).abs().max().item() <= 2e-6 * want.abs().max().item(), factor
+
+
+@pytest.mark.parametrize("dims,n", [((4, 4, 4, 4), 1), ((6, 10, 7, 9), 5), ((8, 8, 8, 8), 8), ((3, 5, 4, 6), 91)])
+def test_small_calls_try_nothing(gpu_lib, dims, n):
+    """Up to 32768 sites times sources one kernel is taken unseen: results do not depend on the
+    context, and are within FP32 rounding (2e-6) of FP64."""
+    import torch
+
+    x = torch.randn((n,) + dims[::-1] + (4, 3), dtype=torch.complex64, device="cuda")
+    out = []
+    for _ in range(4):
+        ctx, _ = make_ctx(gpu_lib, dims, 0.5, 8021)
+        out.append(torch.empty_like(x))
+        ctx.apply_HW(x, out[-1], n, gpu_lib.OV_FP32)
+    x64 = x.to(torch.complex128)
+    want = torch.empty_like(x64)
+    ctx.apply_HW(x64, want, n, gpu_lib.OV_FP64)
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, out[0]) for o in out)
+    assert (out[0].to(torch.complex128) - want).abs().max().item() <= 2e-6 * want.abs().max().item()
