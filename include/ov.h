@@ -290,7 +290,7 @@ int ov_overlap_solve(ov_ctx* ctx, double m_q, const void* b, void* x, int nrhs, 
  * rebuilt as conj(row0 x row1)).  k = -1 (default): autotune -- each variant is timed
  * once on the live data per right-hand-side count and the fastest is kept (up to 32768
  * sites times right-hand sides the spin-paired kernel without trials); on links that
- * are not SU(3) (row 2 further than 2^-21 from conj(row0 x row1)) those with plain links
+ * are not SU(3) (row 2 further than 2^-20 from conj(row0 x row1)) those with plain links
  * only.  A variant set here runs on any links.
  * ov_hw32_variants returns the number of variants and, for 0 <= k < count, describes
  * variant k.  Structure-of-arrays float2 layout: compressed 0 plain links, 1 12-real
