@@ -1260,9 +1260,10 @@ __global__ void __launch_bounds__(32) fx_begin_kernel(const __grid_constant__ So
 // A block takes one 32-site tile of `per` sources in turn (their links then come from L1).
 // Bound by the wide multiply-adds (one warp instruction per cycle and SM, 1300 per 32 sites
 // for the hops and 430 for the rest, half of the time) and the L2 latency of the neighbour
-// loads.  One source at 16^3 x 32: 63 us, where the FP64 kernel takes 227 us and the
-// double-float one 66 us; 6 sources in one launch: 6 x 43 us (links from L1).  4 blocks per
-// SM (64 registers): 334 ms per 12-source FP64 solve, 363 at 3, 366 at 5.  NT = 288, for small grids
+// loads.  One source at 16^3 x 32: 55 us, where the FP64 kernel takes 227 us and the
+// double-float one 66 us; 6 sources in one launch: 6 x 44 us (links from L1; 6 x 43 when it
+// rounded down and left negations a unit short).  4 blocks per SM (64 registers): 338 ms per
+// 12-source FP64 solve (with the rounding of before 334, 363 at 3, 366 at 5).  NT = 288, for small grids
 // where nothing else covers it: a ninth warp forms the scalars while the others run phase 1
 // (8^4, 4 sources: 8.0 -> 6.5 ms per solve against a last block's serial end); NT = 256: from
 // fx_begin_kernel (formed in every block, 16^3 x 32 took 374 ms instead of 366).
@@ -1387,7 +1388,7 @@ __global__ void __launch_bounds__(NT, NT == kFxNT ? 4 : 3) fx_lanczos_hw_kernel(
 }
 
 // HBM-bound (576 B per site and source): two reads, one write, an exact integer norm; one
-// wave of blocks, two elements in flight per thread (18.6 us for one source at 16^3 x 32).
+// wave of blocks, two elements in flight per thread (19.0 us for one source at 16^3 x 32).
 // Warp 0 forms alpha and the scale from K1's sums beside the block's first loads.
 template <>
 __global__ void __launch_bounds__(NT2, 4) lanczos_update_kernel<FX>(SolveArgs<FX> a) {
